@@ -17,6 +17,7 @@
 
 #include "nb_common.cuh"
 #include "nb_symsched.cuh"
+#include "nb_tri.cuh"
 
 namespace nb {
 
@@ -222,6 +223,15 @@ size_t force_bytes(const Plan &pl, int mode, int64_t n, bool extra_pos, bool phi
   return c.off + 256;
 }
 
+// The pair kernel of a plan: the FP32-pipe half-pair kernel where it serves
+// the call (nb_tri.cu), else the kernels of nb_pair.cu and nb_sym.cu.
+cudaError_t launch_pairs(const Plan &pl, int mode, int64_t n, const double *x, const double *y, const double *z,
+                         const double *q, const PosF32 &pf, double soft2, double *part, unsigned *err,
+                         cudaStream_t st) {
+  if (tri_serves(pl, mode, soft2)) return launch_pair_tri(pl, n, x, y, z, q, part, err, st);
+  return launch_pair_force(pl, mode, n, x, y, z, q, pf, soft2, part, err, st);
+}
+
 // Force evaluation at positions (x, y, z) into `part`.
 nb_status pair_forces(const Plan &pl, int mode, int64_t n, const double *x, const double *y,
                       const double *z, const double *q, double soft2, double *part, float *split,
@@ -233,7 +243,7 @@ nb_status pair_forces(const Plan &pl, int mode, int64_t n, const double *x, cons
     pf = PosF32{split, split + n, split + 2 * n, split + 3 * n, split + 4 * n, split + 5 * n};
   }
   timing_begin(st);
-  NB_CUDA_TRY(launch_pair_force(pl, mode, n, x, y, z, q, pf, soft2, part, err, st));
+  NB_CUDA_TRY(launch_pairs(pl, mode, n, x, y, z, q, pf, soft2, part, err, st));
   timing_end(st);
   count_launches(1);
   return NB_OK;
@@ -471,7 +481,7 @@ nb_status nb_forces(const nb_params *params, const nb_system *sys, double *phi, 
   if (n == 0) return NB_OK;
   cudaStream_t st = (cudaStream_t)stream;
   const int mode = params->precision;
-  const Plan pl = make_plan(n, mode, 0);
+  const Plan pl = make_force_plan(n, mode, params->soft2);
   const Plan plp = make_plan(n, MODE_FP64, 1);
   Arena *a = nullptr;
   NB_TRY(get_arena(st, force_bytes(pl, mode, n, false, phi != nullptr, plp), &a));
@@ -508,7 +518,7 @@ nb_status nb_step(const nb_params *params, nb_system *sys, int64_t nsteps, void 
   }
   cudaStream_t st = (cudaStream_t)stream;
   const int mode = params->precision;
-  const Plan pl = make_plan(n, mode, 0);
+  const Plan pl = make_force_plan(n, mode, params->soft2);
   Arena *a = nullptr;
   if (use_small_steps(pl, mode, n)) {
     NvtxRange sub_("nb_step: single-block steps");
@@ -881,7 +891,7 @@ nb_status nb_plan_info(int32_t kind, int32_t precision, int64_t n, int64_t out[8
   if (kind < 0 || kind > 2) return fail(NB_EINVAL, "kind must be 0 (force), 1 (potential) or 2 (VJP)");
   if (precision < NB_FP64 || precision > NB_MIXED_SPLIT_RSQ) return fail(NB_EINVAL, "bad precision");
   if (n < 1) return fail(NB_EINVAL, "n must be >= 1");
-  const Plan pl = make_plan(n, kind == 0 ? precision : MODE_FP64, kind);
+  const Plan pl = kind == 0 ? make_force_plan(n, precision, 0.0) : make_plan(n, MODE_FP64, kind);
   out[0] = pl.block;
   out[1] = pl.R;
   out[2] = pl.jchunk;
@@ -1037,7 +1047,7 @@ extern "C" nb_status nb_traj_backward(const nb_params *params, const nb_system *
   if (gscale && !aligned8(gscale)) return fail(NB_EINVAL, "gscale is not 8-byte aligned");
   cudaStream_t st = (cudaStream_t)stream;
   const int mode = params->precision;  // the forward's force arithmetic, for the recompute
-  const Plan pl = make_plan(n, mode, 0);
+  const Plan pl = make_force_plan(n, mode, params->soft2);
   const Plan plv = make_plan(n, MODE_FP64, 2);
   const int64_t S = n_segments(nsteps, every);
   const int64_t slots = std::min(every, std::max<int64_t>(nsteps, 1)) + 2;
@@ -1088,7 +1098,7 @@ extern "C" nb_status nb_traj_backward(const nb_params *params, const nb_system *
       count_launches(1);
       for (int64_t m = 0; m < len; ++m) {
         const auto P = slot(m + 1), Nx = slot(m + 2);
-        NB_CUDA_TRY(launch_pair_force(pl, mode, n, P[0], P[1], P[2], sys->q, nopf, params->soft2, fpart, a->err, st));
+        NB_CUDA_TRY(launch_pairs(pl, mode, n, P[0], P[1], P[2], sys->q, nopf, params->soft2, fpart, a->err, st));
         NB_CUDA_TRY(launch_epi_step(p, sv, P[0], P[1], P[2], fpart, pl.n_jc, start + m + 1, Nx[0], Nx[1], Nx[2],
                                     a->err, st));
         count_launches(2);

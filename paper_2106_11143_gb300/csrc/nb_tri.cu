@@ -1,0 +1,431 @@
+// nb_tri.cu -- half-pair force kernel of the FP64-class precisions (fp64,
+// df64) on the FP32 pipe (nb_tri.cuh).
+//
+// Work items and output are those of the half-pair kernels (nb_symsched.cuh):
+// a block pair (P, Q), P <= Q, of BI = 32 G ions.  Each warp owns one P-tile of
+// 64 V ions, 2 V per lane as V packed pairs, whose words stay in its registers
+// for the whole item, and visits Q-tiles of 32 ions.  Q words sit in shared
+// memory, each tile twice back to back, so that rotation r of a tile is a fixed
+// offset; the Q side's sums rotate one lane per iteration by shuffle, one
+// packed double-float per component (the low half sums the terms of the even
+// P-ions of the lane, the high half the odd ones).  32 rotations evaluate every
+// pair of the two tiles once.  The sums are double-floats within a tile and are
+// added to FP64 accumulators in shared memory after it: the warp's own for P,
+// and for Q the block's, which the warps visit in a staggered order with a
+// barrier between steps.  Everything is in units of L; the output applies L^-2.
+//
+// Diagonal items (P == Q) run the same tiles one-sided (ONE).
+//
+// What bounds it: the FMA pipe, 126 lane-cycles per evaluation (21 for d, 18
+// for r^2, 18 for r^-3, 12 for the products, 48 for the two ions' TwoSum sums,
+// 9 to keep them normalised), 76 % busy at n = 32768 with issue at 48 %, ALU
+// 9 % and the FP64 pipe 23 % (the tiles' sums into FP64); most stalls wait for
+// the FMA pipe.  The half-pair kernel on the FP64 pipe (nb_sym.cu: 10.3 FP64
+// instructions per evaluation in fp64, 3.4 in df64) took 91.0 ms (fp64) and
+// 34.0 ms (df64) at n = 1e5; this one takes 19.2 ms for both.  Conditioned
+// error over all ions at n = 1e5: rms 2^-50.4, largest 2^-45.2, against
+// 2^-50.1 and 2^-44.9 (fp64) and 2^-49.2 and 2^-43.9 (df64) there.
+//
+// Measured and not kept: one pair of P-ions per lane (V = 1: twice the
+// shuffles per evaluation, 5-8 % slower; kept for 64-ion blocks, which it
+// needs); ordering the summands by FSETP/FSEL so that a Fast2Sum does (18
+// FMA lane-cycles fewer, 2-6 % slower: the halves of a packed pair are moved
+// apart and together); 256 threads and two blocks per SM instead of 128 and
+// four (3-4 % slower at 256-ion blocks); unrolling 4 or 8 rotations (level).
+#include <algorithm>
+#include <mutex>
+
+#include "nb_symsched.cuh"
+#include "nb_tri.cuh"
+
+namespace nb {
+
+template <int V>
+struct TriIons {  // 2 V ions of a lane: words and, with weights, the weight's (hi, lo)
+  f32x2 h[V][3], m[V][3], l[V][3], wh[V], wl[V];
+};
+
+// A staged tile: word k of entry e (64 entries, the tile twice) at
+// [k * 64 + e], the weight's high and low parts in the w of words 0 and 1.
+constexpr int TRI_TILE4 = 3 * 64;
+
+// One tile step: this lane's P-ions against the 32 Q-ions of `qt` (lane's
+// entry).  Returns the largest 1/r met.  self: the lane's P-ion (0 .. 2 V - 1)
+// that is Q-ion 0 of the rotation itself, or -1 (ONE only).
+template <int V, bool W, bool ONE>
+__device__ __forceinline__ float tri_tile(const TriIons<V> &p, const float4 *qt, int lane, int self, f32x2 ah[V][3],
+                                          f32x2 al[V][3], f32x2 bh[3], f32x2 bl[3]) {
+  float ymax = 0.0f;
+  const int next = (lane + 1) & 31;
+#pragma unroll 1
+  for (int r0 = 0; r0 < 32; r0 += 2) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const float4 q0 = qt[r0 + s], q1 = qt[64 + r0 + s], q2 = qt[128 + r0 + s];
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        f32x2 dh[3], dl[3], h, l, sh, sl;
+        tri_diff(p.h[v][0], p.m[v][0], p.l[v][0], pk1(q0.x), pk1(q1.x), pk1(q2.x), dh[0], dl[0]);
+        tri_diff(p.h[v][1], p.m[v][1], p.l[v][1], pk1(q0.y), pk1(q1.y), pk1(q2.y), dh[1], dl[1]);
+        tri_diff(p.h[v][2], p.m[v][2], p.l[v][2], pk1(q0.z), pk1(q1.z), pk1(q2.z), dh[2], dl[2]);
+        tri_r2(dh, dl, h, l);
+        float ha, hb;
+        upk(h, ha, hb);
+        float ya = rsqrt_approx(ha), yb = rsqrt_approx(hb);
+        if (ONE) {
+          // the ion itself: d = 0 gives a zero term with any finite y
+          ymax = fmaxf(ymax, s == 0 && r0 == 0 && self == 2 * v ? 0.0f : ya);
+          ymax = fmaxf(ymax, s == 0 && r0 == 0 && self == 2 * v + 1 ? 0.0f : yb);
+          ya = fminf(ya, TRI_YMAX_GRID);
+          yb = fminf(yb, TRI_YMAX_GRID);
+        } else {
+          ymax = fmaxf(ymax, fmaxf(ya, yb));
+        }
+        tri_rinv3(h, l, pk(ya, yb), sh, sl);
+        f32x2 sph = sh, spl = sl, sqh = sh, sql = sl;
+        if (W) ptwo_prod(sh, sl, pk1(q0.w), pk1(q1.w), sph, spl);
+        if (W && !ONE) ptwo_prod(sh, sl, p.wh[v], p.wl[v], sqh, sql);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          f32x2 th, tl;
+          ptwo_prod(dh[c], dl[c], sph, spl, th, tl);
+          pacc(ah[v][c], al[v][c], th, tl);
+          if (!ONE) {
+            if (W) ptwo_prod(dh[c], dl[c], sqh, sql, th, tl);
+            pacc_sub(bh[c], bl[c], th, tl);
+          }
+          // the low sums stay at an ulp of the high ones, so that adding to
+          // them rounds at 2^-49 of the sum
+          if (s == 1) pfast2(ah[v][c], al[v][c]);
+        }
+      }
+      if (!ONE)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          if (V == 2 || s == 1) pfast2(bh[c], bl[c]);
+          bh[c] = pshfl(bh[c], next);
+          bl[c] = pshfl(bl[c], next);
+        }
+    }
+  }
+  return ymax;
+}
+
+// The same tile step in FP64 from the caller's positions, for tiles the FP32
+// path leaves: ions [i0, i0 + ni) (the P-tile) against [j0, j0 + 32), those
+// below n.  `sc` takes a force from its own units to the accumulators'.
+template <bool ONE>
+__device__ __noinline__ void tri_tile_fp64(int64_t n, const double *x, const double *y, const double *z,
+                                           const double *q, int64_t i0, int ni, int64_t j0, double sc, double *accP,
+                                           int ldp, double *accQ, int ldq) {
+  const int lane = threadIdx.x & 31;
+  for (int u = 0; u < ni; u += 32) {
+    const int64_t i = i0 + u + lane;
+    double a[3] = {0.0, 0.0, 0.0}, b[3] = {0.0, 0.0, 0.0};
+    for (int r = 0; r < 32; ++r) {
+      const int64_t j = j0 + ((lane + r) & 31);
+      if (i < n && j < n && i != j) {
+        const double dx = x[i] - x[j], dy = y[i] - y[j], dz = z[i] - z[j];
+        const double s = rinv3_fp64(dx, dy, dz, 0.0);
+        const double sp = (q ? s * q[j] : s), sq = (q ? s * q[i] : s);
+        a[0] = fma(dx, sp, a[0]);
+        a[1] = fma(dy, sp, a[1]);
+        a[2] = fma(dz, sp, a[2]);
+        b[0] = fma(-dx, sq, b[0]);
+        b[1] = fma(-dy, sq, b[1]);
+        b[2] = fma(-dz, sq, b[2]);
+      }
+      if (!ONE)
+        for (int c = 0; c < 3; ++c) b[c] = __shfl_sync(0xffffffffu, b[c], (lane + 1) & 31);
+    }
+    for (int c = 0; c < 3; ++c) {
+      accP[c * ldp + u + lane] += a[c] * sc;
+      if (!ONE) accQ[c * ldq + lane] += b[c] * sc;
+    }
+  }
+}
+
+// The item's scale: the largest biased exponent of a coordinate in em, the
+// weights' in ew; false when the item is left to FP64.  Ends with a barrier.
+template <int NT, bool QARR>
+__device__ __forceinline__ bool tri_scale(int64_t p0, int np, int64_t q0, int nq, const double *x, const double *y,
+                                          const double *z, const double *q, int &em, int &ew) {
+  __shared__ int red[3][NT / 32];
+  int mx = 0, wx = 0, wn = 0x7fffffff;
+  for (int i = threadIdx.x; i < np + nq; i += NT) {
+    const int64_t g = i < np ? p0 + i : q0 + (i - np);
+    mx = max(mx, __double2hiint(x[g]) & 0x7fffffff);
+    mx = max(mx, __double2hiint(y[g]) & 0x7fffffff);
+    mx = max(mx, __double2hiint(z[g]) & 0x7fffffff);
+    if (QARR) {
+      const int w = __double2hiint(q[g]) & 0x7fffffff;
+      wx = max(wx, w);
+      if (q[g] != 0.0) wn = min(wn, w);
+    }
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (QARR) {
+    wx = __reduce_max_sync(0xffffffffu, wx);
+    wn = __reduce_min_sync(0xffffffffu, wn);
+  }
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    red[0][w] = mx;
+    red[1][w] = wx;
+    red[2][w] = wn;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NT / 32; ++k) {
+    mx = max(mx, red[0][k]);
+    wx = max(wx, red[1][k]);
+    wn = min(wn, red[2][k]);
+  }
+  em = mx >> 20;
+  ew = 1023;
+  bool ok = em >= TRI_EMIN && em <= TRI_EMAX;
+  if (QARR) {
+    ew = wx >> 20;
+    ok = ok && ew >= 1023 - 400 && ew <= 1023 + 400 && ew - (wn >> 20) <= TRI_WSPREAD;
+  }
+  return ok;
+}
+
+// Words of ion g (or a padding ion on side `far`) with its weight.
+template <bool QARR>
+__device__ __forceinline__ void tri_ion(int64_t g, bool real, const double *x, const double *y, const double *z,
+                                        const double *q, int em, int ew, float far, float w0[4], float w1[4],
+                                        float w2[4]) {
+  w0[3] = w1[3] = w2[3] = 0.0f;
+  if (real) {
+    float t[3];
+    tri_words(x[g], em, t);
+    w0[0] = t[0]; w1[0] = t[1]; w2[0] = t[2];
+    tri_words(y[g], em, t);
+    w0[1] = t[0]; w1[1] = t[1]; w2[1] = t[2];
+    tri_words(z[g], em, t);
+    w0[2] = t[0]; w1[2] = t[1]; w2[2] = t[2];
+    if (QARR && q[g] != 0.0) split_f64_scaled(q[g], ew - 1023, w0[3], w1[3]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      w0[c] = far;
+      w1[c] = w2[c] = 0.0f;
+    }
+  }
+}
+
+template <int V, bool QARR, int NT, int NB, bool INPLACE>
+__global__ void __launch_bounds__(NT, NB)
+    k_pair_sym_tri(int64_t n, int nbk, int G, const double *__restrict__ x, const double *__restrict__ y,
+                   const double *__restrict__ z, const double *__restrict__ q, double *__restrict__ out,
+                   int *__restrict__ sync, unsigned *err) {
+  constexpr int NW = NT / 32, PI = 64 * V;  // warps; ions of a P-tile
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int BI = 32 * G;
+  float4 *qs = reinterpret_cast<float4 *>(smem_raw);                 // [G][TRI_TILE4]
+  double *accQ = reinterpret_cast<double *>(qs + G * TRI_TILE4);     // [3][BI]
+  double *accP = accQ + 3 * BI;                                      // [NW][3][PI]
+  const SymItem it = sym_block_item(INPLACE, sync, nbk);
+  const int64_t p0 = (int64_t)it.P * BI, q0 = (int64_t)it.Q * BI;
+  const int np = (int)min((int64_t)BI, n - p0), nq = (int)min((int64_t)BI, n - q0);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool diag = it.P == it.Q;
+  int em, ew;
+  const bool fast = tri_scale<NT, QARR>(p0, np, q0, diag ? 0 : nq, x, y, z, q, em, ew);
+  // units: a coordinate is L X with L = 2^(em - 1022), a weight 2^(ew - 1023) w
+  const int kl = fast ? em - 1022 : 0, kw = fast ? ew - 1023 : 0;
+
+  const int PT = BI / PI, NG = NW / PT, nqt = G / NG;  // P-tiles, warps per P-tile, Q-tiles per warp
+  const int pt = warp % PT, grp = warp / PT;
+  TriIons<V> p;
+  int low = 0;  // an l word is set
+  if (fast) {
+    for (int i = tid; i < BI; i += NT) {
+      float w0[4], w1[4], w2[4];
+      tri_ion<QARR>(q0 + i, i < nq, x, y, z, q, em, ew, -TRI_FAR, w0, w1, w2);
+      float4 *e = qs + (i >> 5) * TRI_TILE4 + (i & 31);
+      e[0] = e[32] = make_float4(w0[0], w0[1], w0[2], w0[3]);
+      e[64] = e[96] = make_float4(w1[0], w1[1], w1[2], w1[3]);
+      e[128] = e[160] = make_float4(w2[0], w2[1], w2[2], w2[3]);
+      low |= w2[0] != 0.0f || w2[1] != 0.0f || w2[2] != 0.0f;
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      float w0[2][4], w1[2][4], w2[2][4];
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const int i = pt * PI + v * 64 + b * 32 + lane;
+        tri_ion<QARR>(p0 + i, i < np, x, y, z, q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
+        low |= w2[b][0] != 0.0f || w2[b][1] != 0.0f || w2[b][2] != 0.0f;
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        p.h[v][c] = pk(w0[0][c], w0[1][c]);
+        p.m[v][c] = pk(w1[0][c], w1[1][c]);
+        p.l[v][c] = pk(w2[0][c], w2[1][c]);
+      }
+      p.wh[v] = pk(w0[0][3], w0[1][3]);
+      p.wl[v] = pk(w1[0][3], w1[1][3]);
+    }
+  }
+  for (int i = tid; i < 3 * BI; i += NT) accQ[i] = 0.0;
+  for (int i = tid; i < NW * 3 * PI; i += NT) accP[i] = 0.0;
+  const float ylim = __syncthreads_or(low) ? TRI_YMAX : TRI_YMAX_GRID;
+
+  double *aP = accP + warp * 3 * PI;
+  const double back = pow2d(2 * kl - kw);  // own units -> the accumulators'
+  const bool live = pt * PI < np;          // the P-tile holds ions
+  for (int k = 0; k < nqt; ++k) {
+    // distinct over the P-tiles of a step: nqt >= PT
+    const int t = grp * nqt + (k + pt) % nqt;
+    if (k > 0) __syncthreads();  // the Q sums of the last step are written
+    double *aQ = accQ + t * 32;
+    if (!live || t * 32 >= nq) continue;
+    bool done = false;
+    if (fast) {
+      f32x2 ah[V][3], al[V][3], bh[3], bl[3];
+      const f32x2 zero = pk1(0.0f);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        bh[c] = bl[c] = zero;
+#pragma unroll
+        for (int v = 0; v < V; ++v) ah[v][c] = al[v][c] = zero;
+      }
+      const float4 *qt = qs + t * TRI_TILE4 + lane;
+      float ymax;
+      if (diag) {
+        const int u = t - pt * 2 * V;  // the lane's own ion in this Q-tile, if any
+        ymax = tri_tile<V, QARR, true>(p, qt, lane, u >= 0 && u < 2 * V ? u : -1, ah, al, bh, bl);
+      } else {
+        ymax = tri_tile<V, QARR, false>(p, qt, lane, -1, ah, al, bh, bl);
+      }
+      done = !__any_sync(0xffffffffu, !(ymax <= ylim));
+      if (done) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          float h0, h1, l0, l1;
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            upk(ah[v][c], h0, h1);
+            upk(al[v][c], l0, l1);
+            double *d = aP + c * PI + v * 64 + lane;
+            d[0] += (double)h0 + (double)l0;
+            d[32] += (double)h1 + (double)l1;
+          }
+          if (!diag) {
+            upk(bh[c], h0, h1);
+            upk(bl[c], l0, l1);
+            aQ[c * BI + lane] += ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
+          }
+        }
+      }
+    }
+    if (!done) {
+      if (diag)
+        tri_tile_fp64<true>(n, x, y, z, q, p0 + pt * PI, PI, q0 + t * 32, back, aP, PI, aQ, BI);
+      else
+        tri_tile_fp64<false>(n, x, y, z, q, p0 + pt * PI, PI, q0 + t * 32, back, aP, PI, aQ, BI);
+    }
+  }
+  __syncthreads();
+  const double fwd = pow2d(kw - 2 * kl);
+  sym_output<NT>(INPLACE, it, n, p0, np, q0, nq, out, sync, err,
+                 [&](int c, int i) {
+                   double v = 0.0;
+                   const double *s = accP + (i / PI) * 3 * PI + c * PI + i % PI;
+                   for (int g = 0; g < NG; ++g) v += s[g * PT * 3 * PI];
+                   return v * fwd;
+                 },
+                 [&](int c, int i) { return accQ[c * BI + i] * fwd; });
+}
+
+// ---------------------------------------------------------------------------
+template <int V, int NT>
+static size_t tri_smem(int G) {
+  return (size_t)G * TRI_TILE4 * sizeof(float4) + (size_t)3 * 32 * G * sizeof(double) +
+         (size_t)(NT / 32) * 3 * 64 * V * sizeof(double);
+}
+
+template <int V, int NT, int NB>
+static cudaError_t launch_tri(int64_t n, int nbk, int G, const double *x, const double *y, const double *z,
+                              const double *q, double *part, int *sync, unsigned *err, bool inplace,
+                              cudaStream_t st) {
+  static std::mutex mu;
+  static bool done[64] = {false};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!done[dev]) {
+      const void *fns[4] = {(const void *)k_pair_sym_tri<V, true, NT, NB, true>,
+                            (const void *)k_pair_sym_tri<V, false, NT, NB, true>,
+                            (const void *)k_pair_sym_tri<V, true, NT, NB, false>,
+                            (const void *)k_pair_sym_tri<V, false, NT, NB, false>};
+      for (int k = 0; k < 4 && e == cudaSuccess; ++k)
+        e = cudaFuncSetAttribute(fns[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem<V, NT>(32));
+      if (e != cudaSuccess) return e;
+      done[dev] = true;
+    }
+  }
+  if (inplace) {
+    e = cudaMemsetAsync(sync, 0, sizeof(int) * sym_sync_ints(nbk), st);
+    if (e != cudaSuccess) return e;
+  }
+  const int items = nbk * (nbk + 1) / 2;
+  const size_t smem = tri_smem<V, NT>(G);
+#define NB_TRI_LAUNCH(QA, IP) \
+  k_pair_sym_tri<V, QA, NT, NB, IP><<<items, NT, smem, st>>>(n, nbk, G, x, y, z, q, part, sync, err)
+  if (inplace) {
+    if (q) NB_TRI_LAUNCH(true, true); else NB_TRI_LAUNCH(false, true);
+  } else {
+    if (q) NB_TRI_LAUNCH(true, false); else NB_TRI_LAUNCH(false, false);
+  }
+#undef NB_TRI_LAUNCH
+  return cudaGetLastError();
+}
+
+// 32-ion blocks (set_tuning only) and softened sums stay with nb_sym.cu.
+static bool tri_sums(const Plan &pl, int mode, double soft2) {
+  return pl.sym && soft2 == 0.0 && (mode == MODE_FP64 || mode == MODE_DF64);
+}
+bool tri_serves(const Plan &pl, int mode, double soft2) { return tri_sums(pl, mode, soft2) && pl.G >= 2; }
+
+// Block sizes, the fastest measured over n = 1500 .. 150000 (us per nb_forces
+// call, fp64): 64 ions below 2800 (30.0 against 33.1 with 128 at n = 2000),
+// 128 up to 12160 (82 against 107 with 256 at 5003, 239 against 270 at 10000),
+// where 96 blocks would take the in-place output, whose chain of commits these
+// short items do not hide (628 against 454 at 14000), 256 above (19245 against
+// 19989 with 512 at 1e5).
+Plan make_force_plan(int64_t n, int mode, double soft2) {
+  Plan pl = make_plan(n, mode, 0);
+  int tb = 0, tr = 0, tbps = 0;
+  if (!tri_sums(pl, mode, soft2) || tuning_lookup(4, mode, n, &tb, &tr, &tbps)) return pl;
+  int G = n > 12160 ? 8 : (n >= 2800 ? 4 : 2);
+  while (G < 32 && (n + 32 * G - 1) / (32 * G) > 60000) G *= 2;  // the schedule's block limit
+  pl.G = G;
+  pl.nbk = (int)((n + 32 * G - 1) / (32 * G));
+  // the output rule of the half-pair kernels: in place from 96 blocks or 1 GB of partials
+  pl.n_jc = pl.nbk >= 96 || (double)pl.nbk * 3.0 * (double)n * 8.0 > 1e9 ? 1 : pl.nbk;
+  return pl;
+}
+
+cudaError_t launch_pair_tri(const Plan &pl, int64_t n, const double *x, const double *y, const double *z,
+                            const double *q, double *part, unsigned *err, cudaStream_t st) {
+  int *sync = part_sync(pl, part, n, 3);
+  const bool inplace = pl.n_jc == 1;
+#define NB_TRI(V, NT, NB) launch_tri<V, NT, NB>(n, pl.nbk, pl.G, x, y, z, q, part, sync, err, inplace, st)
+  switch (pl.G) {
+    case 2: return NB_TRI(1, 64, 10);
+    case 4:
+    case 8: return NB_TRI(2, 128, 4);
+    case 16:
+    case 32: return NB_TRI(2, 256, 2);
+    default: return cudaErrorInvalidValue;
+  }
+#undef NB_TRI
+}
+
+}  // namespace nb

@@ -1,0 +1,219 @@
+// nb_tri.cuh -- FP64-class pair terms (Eq. 1) formed entirely on the FP32
+// pipe, from positions carried as three FP32 words on a common grid.
+//
+// GB300's FP64 pipe retires 2 lanes per clock per SM against 128 on the FP32
+// pipe, so even the three FP64 subtractions of a displacement take longer than
+// about 100 FP32 instructions.  Here a work item (two blocks of ions) picks one
+// power of two L above every coordinate it touches and cuts each coordinate's
+// bits, in units of L, into
+//   h: a multiple of 2^-22,  m: a multiple of 2^-45 below 2^-22,
+//   l: a multiple of 2^-69 below 2^-45   (all with the coordinate's sign).
+// A FP64 coordinate of at least 2^-16 L is represented exactly, a smaller one
+// to 2^-69 L.  The words' differences are exact in FP32 (at most 24 bits on
+// the word's own grid), so d = dh + dm + dl is exact, and one Fast2Sum makes
+// it the double-float (RN(dh + dm), rest): 7 FP32 operations per component,
+// all of which exist as packed .f32x2 instructions.
+//
+// A pair closer than 2^-20 L (where the 2^-69 L cut would pass 2^-49 of the
+// distance, and dl stops being small against dm) makes its tile fall back to
+// FP64 arithmetic; the test is the largest 1/r met, one FMNMX per pair.  When
+// no coordinate of the item has bits in l (positions on a grid), d is exact
+// and normal at any distance, and only FP32's range sets a limit, 2^-40 L.
+// Items whose scale or weights are far from the ordinary (below) take the
+// FP64 path as a whole.
+#pragma once
+
+#include "nb_common.cuh"
+
+namespace nb {
+
+// Packed FP32 pairs (.f32x2): the same IEEE operation on both halves in one
+// issue slot and two cycles of the FMA pipe.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ f32x2 pk1(float v) { return pk(v, v); }
+__device__ __forceinline__ void upk(f32x2 v, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 padd(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 psub(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 pmul(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 pfma(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 pneg(f32x2 v) {
+  float a, b;
+  upk(v, a, b);
+  return pk(-a, -b);
+}
+
+// s + e = a + b and a - b exactly (Knuth TwoSum).
+__device__ __forceinline__ void ptwo_sum(f32x2 a, f32x2 b, f32x2 &s, f32x2 &e) {
+  s = padd(a, b);
+  const f32x2 bb = psub(s, a);
+  e = padd(psub(a, psub(s, bb)), psub(b, bb));
+}
+__device__ __forceinline__ void ptwo_diff(f32x2 a, f32x2 b, f32x2 &s, f32x2 &e) {
+  s = psub(a, b);
+  const f32x2 bb = psub(s, a);  // about -b
+  e = psub(psub(a, psub(s, bb)), padd(b, bb));
+}
+
+// The words of coordinate x in units of L = 2^(em - 1022), em at least x's
+// biased exponent: w[0] + w[1] + w[2] = x / L to 2^-69.
+__device__ __forceinline__ void tri_words(double x, int em, float w[3]) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  const unsigned t1 = e ? (0x80000000u | ((hi & 0xfffffu) << 11) | (lo >> 21)) : 0u, t0 = e ? lo << 11 : 0u;
+  const int s = em - e, k = s & 31, j = s >> 5;  // the mantissa (t1:t0) moves down s bits
+  const unsigned a0 = t1 >> k, a1 = __funnelshift_r(t0, t1, k), a2 = __funnelshift_r(0u, t0, k);
+  const unsigned w0 = j == 0 ? a0 : 0u;
+  const unsigned w1 = j == 0 ? a1 : (j == 1 ? a0 : 0u);
+  const unsigned w2 = j == 0 ? a2 : (j == 1 ? a1 : (j == 2 ? a0 : 0u));
+  const float sg = __uint_as_float(0x3f800000u | (hi & 0x80000000u));
+  w[0] = (float)(int)(w0 >> 10) * (sg * 0x1p-22f);
+  w[1] = (float)(int)(((w0 & 0x3ffu) << 13) | (w1 >> 19)) * (sg * 0x1p-45f);
+  w[2] = (float)(int)(((w1 & 0x7ffffu) << 5) | (w2 >> 27)) * (sg * 0x1p-69f);
+}
+
+// A padding ion's coordinate, in units of L: far enough that every term with
+// it underflows to zero (y^3 < 2^-149), near enough that r^2 stays finite.  The
+// two sides use opposite signs, so two padding ions never coincide.
+constexpr float TRI_FAR = 1e18f;
+
+// Largest 1/r (units of 1/L) of the FP32 path, and where no l word is set.
+constexpr float TRI_YMAX = 0x1p20f, TRI_YMAX_GRID = 0x1p40f;
+
+// Scales the path accepts: L within 2^+-200 (so that L^2, L^-2 and their
+// products with a force stay far inside FP64), and weights within 2^40 of the
+// item's largest (so that a double-float weight keeps its 48 bits).
+constexpr int TRI_EMIN = 1023 - 200, TRI_EMAX = 1023 + 200, TRI_WSPREAD = 40;
+
+// d = p - q as a double-float: the word differences are exact; Fast2Sum holds
+// because dh is 0 or at least 2^-22 > |dm|.
+__device__ __forceinline__ void tri_diff(f32x2 ph, f32x2 pm, f32x2 pl, f32x2 qh, f32x2 qm, f32x2 ql, f32x2 &h,
+                                         f32x2 &l) {
+  const f32x2 dh = psub(ph, qh), dm = psub(pm, qm), dl = psub(pl, ql);
+  h = padd(dh, dm);
+  l = padd(psub(dm, psub(h, dh)), dl);
+}
+
+// s + e = a + b exactly for |a| >= |b| (Fast2Sum).
+__device__ __forceinline__ void pfast2(f32x2 &a, f32x2 &b) {
+  const f32x2 s = padd(a, b);
+  b = psub(b, psub(s, a));
+  a = s;
+}
+
+// r^2 of the double-float displacement (dh, dl) as the double-float (h, l).
+// The largest component's square comes first, so every partial sum a + b^2
+// has a >= b^2 and its rounding error is one exact difference and one FMA
+// (FMNMX runs on the ALU pipe, which the pair loop leaves idle).  The
+// dl^2 terms are there against a bias: without them r^2 is short by 2^-50.
+__device__ __forceinline__ void tri_r2(const f32x2 dh[3], const f32x2 dl[3], f32x2 &h, f32x2 &l) {
+  float x[2], y[2], z[2], M[2], m1[2], m2[2];
+  upk(dh[0], x[0], x[1]);
+  upk(dh[1], y[0], y[1]);
+  upk(dh[2], z[0], z[1]);
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    const float t = fmaxf(fabsf(x[b]), fabsf(y[b]));
+    m1[b] = fminf(fabsf(x[b]), fabsf(y[b]));
+    M[b] = fmaxf(t, fabsf(z[b]));
+    m2[b] = fminf(t, fabsf(z[b]));
+  }
+  const f32x2 A = pk(M[0], M[1]), B = pk(m1[0], m1[1]), C = pk(m2[0], m2[1]);
+  const f32x2 p = pmul(A, A);
+  const f32x2 e0 = pfma(A, A, pneg(p));
+  const f32x2 h1 = pfma(B, B, p);
+  const f32x2 t1 = pfma(B, B, psub(p, h1));
+  h = pfma(C, C, h1);
+  const f32x2 t2 = pfma(C, C, psub(h1, h));
+  const f32x2 q = pfma(dh[2], dl[2], pfma(dh[1], dl[1], pmul(dh[0], dl[0])));
+  const f32x2 d2 = pfma(dl[2], dl[2], pfma(dl[1], dl[1], pmul(dl[0], dl[0])));
+  l = pfma(pk1(2.0f), q, padd(padd(e0, t1), padd(t2, d2)));
+}
+
+// r^-3 as the double-float (sh, sl) from r^2 = h + l and the seed y of
+// 1/sqrt(h) (relative error below 2^-22.9).  With w = RN(y^2) and e = y^2 - w
+// exactly, the residual is rho = 1 - (h + l) w (its first FMA is all but
+// exact) and
+//   r^-3 = w^(3/2) (1 - rho)^(-3/2),  w^(1/2) = y (1 - e / (2 y^2)) to e^2,
+// so that r^-3 = (w y - y e / 2) (1 + 3/2 t), t = rho + 5/4 rho^2, with w y kept
+// as a double-float.  3/2 t goes in as t + t/2 (a product 1.5 t would round
+// once more), and (sh, sl) is left normalised, so that the products with it
+// lose nothing to a long sl.
+__device__ __forceinline__ void tri_rinv3(f32x2 h, f32x2 l, f32x2 y, f32x2 &sh, f32x2 &sl) {
+  const f32x2 w = pmul(y, y), nw = pneg(w);
+  const f32x2 e = pfma(y, y, nw);
+  const f32x2 rho = pfma(l, nw, pfma(h, nw, pk1(1.0f)));
+  const f32x2 t = pfma(pmul(rho, pk1(1.25f)), rho, rho);
+  sh = pmul(w, y);
+  f32x2 low = pfma(e, pmul(y, pk1(-0.5f)), pfma(w, y, pneg(sh)));
+  low = pfma(pmul(low, pk1(1.5f)), rho, low);
+  sl = pfma(sh, t, pfma(pmul(sh, pk1(0.5f)), t, low));
+  pfast2(sh, sl);
+}
+
+// (h, l) = (ah + al) (bh + bl) as a double-float.
+__device__ __forceinline__ void ptwo_prod(f32x2 ah, f32x2 al, f32x2 bh, f32x2 bl, f32x2 &h, f32x2 &l) {
+  h = pmul(ah, bh);
+  l = pfma(ah, bl, pfma(al, bh, pfma(ah, bh, pneg(h))));
+}
+
+// Double-float sums: (h, l) += (th, tl) and -= (th, tl).
+__device__ __forceinline__ void pacc(f32x2 &h, f32x2 &l, f32x2 th, f32x2 tl) {
+  f32x2 s, e;
+  ptwo_sum(h, th, s, e);
+  h = s;
+  l = padd(l, padd(e, tl));
+}
+__device__ __forceinline__ void pacc_sub(f32x2 &h, f32x2 &l, f32x2 th, f32x2 tl) {
+  f32x2 s, e;
+  ptwo_diff(h, th, s, e);
+  h = s;
+  l = padd(l, psub(e, tl));
+}
+
+__device__ __forceinline__ f32x2 pshfl(f32x2 v, int lane) {
+  float a, b;
+  upk(v, a, b);
+  return pk(__shfl_sync(0xffffffffu, a, lane), __shfl_sync(0xffffffffu, b, lane));
+}
+
+__device__ __forceinline__ float rsqrt_approx(float v) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(v));
+  return y;
+}
+
+// 2^k as FP64 (|k| <= 1000).
+__device__ __forceinline__ double pow2d(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+
+// The plan of a force evaluation: make_plan's, with this file's kernel's own
+// block sizes where it serves the call (nb_tri.cu).
+Plan make_force_plan(int64_t n, int mode, double soft2);
+// Whether the kernel serves a plan, and its launch.
+bool tri_serves(const Plan &pl, int mode, double soft2);
+cudaError_t launch_pair_tri(const Plan &pl, int64_t n, const double *x, const double *y, const double *z,
+                            const double *q, double *part, unsigned *err, cudaStream_t st);
+
+}  // namespace nb
