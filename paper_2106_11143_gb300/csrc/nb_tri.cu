@@ -1,5 +1,6 @@
-// nb_tri.cu -- half-pair force kernel of the FP64-class precisions (fp64,
-// df64) on the FP32 pipe (nb_tri.cuh).
+// nb_tri.cu -- half-pair force kernels whose pair loop has no FP64
+// instruction: the FP64-class precisions (fp64, df64) and the literal mixed
+// form, from three-word positions on the FP32 pipe (nb_tri.cuh).
 //
 // Work items and output are those of the half-pair kernels (nb_symsched.cuh):
 // a block pair (P, Q), P <= Q, of BI = 32 G ions.  Each warp owns one P-tile of
@@ -32,6 +33,17 @@
 // FMA lane-cycles fewer, 2-6 % slower: the halves of a packed pair are moved
 // apart and together); 256 threads and two blocks per SM instead of 128 and
 // four (3-4 % slower at 256-ion blocks); unrolling 4 or 8 rotations (level).
+//
+// The literal mixed form (MIX) takes the same words: its displacement, formed
+// exactly and rounded once to FP32, is the FP64 difference cast to FP32, at 8
+// FMA lane-cycles per component.  With 38 lane-cycles per evaluation it runs
+// 6.95 ms at n = 1e5 (FMA pipe 69 % by that count), where three FP64
+// differences per evaluation took 31.9 ms (nb_sym.cu), and gives its sums to
+// FP64 rounding: every FP32 operation and partial sum is the same, in the same
+// order (norm of the difference at most 2e-11 of the result over n = 2000 ..
+// 1e5; FP32 ties of a displacement may round the other way).  A pairwise
+// order of the FP32 sums would be 20 % faster and as accurate, but would change
+// results in their eighth digit.
 #include <algorithm>
 #include <mutex>
 
@@ -45,6 +57,12 @@ struct TriIons {  // 2 V ions of a lane: words and, with weights, the weight's (
   f32x2 h[V][3], m[V][3], l[V][3], wh[V], wl[V];
 };
 
+// The sums of a tile step: double-floats, or FP32 (MIX) in the high words.
+template <int V>
+struct TriSums {
+  f32x2 ah[V][3], al[V][3], bh[3], bl[3];
+};
+
 // A staged tile: word k of entry e (64 entries, the tile twice) at
 // [k * 64 + e], the weight's high and low parts in the w of words 0 and 1.
 constexpr int TRI_TILE4 = 3 * 64;
@@ -53,8 +71,8 @@ constexpr int TRI_TILE4 = 3 * 64;
 // entry).  Returns the largest 1/r met.  self: the lane's P-ion (0 .. 2 V - 1)
 // that is Q-ion 0 of the rotation itself, or -1 (ONE only).
 template <int V, bool W, bool ONE>
-__device__ __forceinline__ float tri_tile(const TriIons<V> &p, const float4 *qt, int lane, int self, f32x2 ah[V][3],
-                                          f32x2 al[V][3], f32x2 bh[3], f32x2 bl[3]) {
+__device__ __forceinline__ float tri_tile(const TriIons<V> &p, const float4 *qt, int lane, int self, TriSums<V> &t) {
+  f32x2(&ah)[V][3] = t.ah, (&al)[V][3] = t.al, (&bh)[3] = t.bh, (&bl)[3] = t.bl;
   float ymax = 0.0f;
   const int next = (lane + 1) & 31;
 #pragma unroll 1
@@ -106,6 +124,59 @@ __device__ __forceinline__ float tri_tile(const TriIons<V> &p, const float4 *qt,
           bh[c] = pshfl(bh[c], next);
           bl[c] = pshfl(bl[c], next);
         }
+    }
+  }
+  return ymax;
+}
+
+// The tile step of the literal mixed form, operation for operation that of the
+// FP64-difference kernel (sym_step_mixed and the diagonal loop of nb_sym.cu):
+// the displacement rounded once to FP32 (h + l is exact, so RN(h + l) is), the
+// arithmetic of f32_rinv3, and one FP32 sum of 32 terms per ion and 32 x 32
+// tile pair, in the order of the rotations, or (ONE) of the partners.  Q sums,
+// with the sign reversed: bh for the ions of pair 0, bl for pair 1.
+template <int V, bool W, bool ONE>
+__device__ __forceinline__ float tri_tile_mixed(const TriIons<V> &p, const float4 *qt, int lane, int self,
+                                                TriSums<V> &t) {
+  static_assert(V <= 2, "one Q sum per pair of P-ions");
+  float ymax = 0.0f;
+  const int next = (lane + 1) & 31;
+  const f32x2 m15 = pk1(-1.5f), p15 = pk1(1.5f);
+#pragma unroll 4
+  for (int r = 0; r < 32; ++r) {
+    const float4 q0 = qt[r], q1 = qt[64 + r], q2 = qt[128 + r];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      f32x2 d[3], h, l;
+      tri_diff(p.h[v][0], p.m[v][0], p.l[v][0], pk1(q0.x), pk1(q1.x), pk1(q2.x), h, l);
+      d[0] = padd(h, l);
+      tri_diff(p.h[v][1], p.m[v][1], p.l[v][1], pk1(q0.y), pk1(q1.y), pk1(q2.y), h, l);
+      d[1] = padd(h, l);
+      tri_diff(p.h[v][2], p.m[v][2], p.l[v][2], pk1(q0.z), pk1(q1.z), pk1(q2.z), h, l);
+      d[2] = padd(h, l);
+      const f32x2 r2 = pfma(d[0], d[0], pfma(d[1], d[1], pmul(d[2], d[2])));
+      float ra, rb;
+      upk(r2, ra, rb);
+      float ya = rsqrt_approx(ra), yb = rsqrt_approx(rb);
+      if (ONE) {
+        ymax = fmaxf(ymax, r == lane && self == 2 * v ? 0.0f : ya);
+        ymax = fmaxf(ymax, r == lane && self == 2 * v + 1 ? 0.0f : yb);
+        ya = fminf(ya, TRI_YMAX_GRID);
+        yb = fminf(yb, TRI_YMAX_GRID);
+      } else {
+        ymax = fmaxf(ymax, fmaxf(ya, yb));
+      }
+      const f32x2 y = pk(ya, yb), y2 = pmul(y, y), y3 = pmul(y2, y);
+      const f32x2 s = pfma(y3, pfma(pmul(m15, r2), y2, p15), y3);
+      const f32x2 sp = W ? pmul(s, pk1(q0.w)) : s, sq = W && !ONE ? pmul(s, p.wh[v]) : s;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        t.ah[v][c] = pfma(d[c], sp, t.ah[v][c]);
+        if (!ONE) {
+          f32x2 &b = v == 0 ? t.bh[c] : t.bl[c];
+          b = pshfl(pfma(d[c], sq, b), next);
+        }
+      }
     }
   }
   return ymax;
@@ -215,9 +286,79 @@ __device__ __forceinline__ void tri_ion(int64_t g, bool real, const double *x, c
   }
 }
 
-template <int V, bool QARR, int NT, int NB, bool INPLACE>
+// The item's in-place output of the mixed form (sym_commit, nb_symsched.cuh,
+// laid out for short items): the sums are formed before the wait for the
+// previous round, and all of a thread's old values are loaded before the first
+// is stored, so that a commit costs one trip to L2 instead of one per value.
+// At n = 40000 (157 rounds of 256-ion blocks) the chain of commits bounded the
+// mixed form: 24 % per evaluation against sym_commit.  The fp64
+// items are three times as long and hide the chain: there sym_commit, with
+// fewer registers, is faster (19.2 against 19.7 ms at n = 1e5).
+template <int NT, class FP, class FQ>
+__device__ __forceinline__ void tri_commit(const SymItem &it, int64_t n, int BI, int64_t p0, int np, int64_t q0,
+                                           int nq, double *out, int *sync, unsigned *err, FP sumP, FQ sumQ) {
+  __shared__ int s_ok;
+  const int tid = threadIdx.x;
+  const bool two = it.P != it.Q;
+  const bool first = it.round == 0;
+  for (int i0 = tid; i0 < BI; i0 += 2 * NT) {
+    double vp[2][3], vq[2][3];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const int i = i0 + k * NT;
+        vp[k][c] = i < np ? sumP(c, i) : 0.0;
+        vq[k][c] = two && i < nq ? sumQ(c, i) : 0.0;
+      }
+    if (i0 < 2 * NT) {  // the first pass, every thread: BI >= NT
+      if (tid == 0) {
+        bool ok = true;
+        if (it.round > 0) ok = sym_wait(sync, it.P, it.round, err) && (!two || sym_wait(sync, it.Q, it.round, err));
+        if (!ok) atomicOr(err, ERR_TIMEOUT);
+        s_ok = ok;
+      }
+      __syncthreads();
+    }
+    if (!s_ok) continue;
+    if (!first) {
+      double op[2][3], oq[2][3];
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const int i = i0 + k * NT;
+          op[k][c] = i < np ? __ldcg(out + c * n + p0 + i) : 0.0;
+          oq[k][c] = two && i < nq ? __ldcg(out + c * n + q0 + i) : 0.0;
+        }
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          vp[k][c] += op[k][c];
+          vq[k][c] += oq[k][c];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const int i = i0 + k * NT;
+        if (i < np) __stcg(out + c * n + p0 + i, vp[k][c]);
+        if (two && i < nq) __stcg(out + c * n + q0 + i, vq[k][c]);
+      }
+  }
+  __syncthreads();  // every thread's adds happen before thread 0's release
+  if (tid == 0) {
+    __threadfence();
+    st_release(sync + 1 + it.P, it.round + 1);
+    if (two) st_release(sync + 1 + it.Q, it.round + 1);
+  }
+}
+
+template <bool MIX, int V, bool QARR, int NT, int NB, bool INPLACE>
 __global__ void __launch_bounds__(NT, NB)
-    k_pair_sym_tri(int64_t n, int nbk, int G, const double *__restrict__ x, const double *__restrict__ y,
+    k_pair_sym_tri(int64_t n, int nbk, int G, int SB, const double *__restrict__ x, const double *__restrict__ y,
                    const double *__restrict__ z, const double *__restrict__ q, double *__restrict__ out,
                    int *__restrict__ sync, unsigned *err) {
   constexpr int NW = NT / 32, PI = 64 * V;  // warps; ions of a P-tile
@@ -271,7 +412,8 @@ __global__ void __launch_bounds__(NT, NB)
   }
   for (int i = tid; i < 3 * BI; i += NT) accQ[i] = 0.0;
   for (int i = tid; i < NW * 3 * PI; i += NT) accP[i] = 0.0;
-  const float ylim = __syncthreads_or(low) ? TRI_YMAX : TRI_YMAX_GRID;
+  // FP32 rounding of d leaves the 2^-69 L cut far behind at any distance (MIX)
+  const float ylim = __syncthreads_or(low) && !MIX ? TRI_YMAX : TRI_YMAX_GRID;
 
   double *aP = accP + warp * 3 * PI;
   const double back = pow2d(2 * kl - kw);  // own units -> the accumulators'
@@ -282,23 +424,31 @@ __global__ void __launch_bounds__(NT, NB)
     if (k > 0) __syncthreads();  // the Q sums of the last step are written
     double *aQ = accQ + t * 32;
     if (!live || t * 32 >= nq) continue;
+    // a diagonal item's tile pairs are one-sided; in the mixed form only within
+    // a sub-block of SB tiles, and across sub-blocks each pair is taken once,
+    // from the lower one
+    const int sp = pt * 2 * V / SB, sq = t / SB;
+    const bool one = diag && (!MIX || sp == sq);
+    if (MIX && diag && sp > sq) continue;
     bool done = false;
     if (fast) {
-      f32x2 ah[V][3], al[V][3], bh[3], bl[3];
+      TriSums<V> ts;
       const f32x2 zero = pk1(0.0f);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        bh[c] = bl[c] = zero;
+        ts.bh[c] = ts.bl[c] = zero;
 #pragma unroll
-        for (int v = 0; v < V; ++v) ah[v][c] = al[v][c] = zero;
+        for (int v = 0; v < V; ++v) ts.ah[v][c] = ts.al[v][c] = zero;
       }
       const float4 *qt = qs + t * TRI_TILE4 + lane;
       float ymax;
-      if (diag) {
+      if (one) {
         const int u = t - pt * 2 * V;  // the lane's own ion in this Q-tile, if any
-        ymax = tri_tile<V, QARR, true>(p, qt, lane, u >= 0 && u < 2 * V ? u : -1, ah, al, bh, bl);
+        const int self = u >= 0 && u < 2 * V ? u : -1;
+        ymax = MIX ? tri_tile_mixed<V, QARR, true>(p, qt - lane, lane, self, ts)
+                   : tri_tile<V, QARR, true>(p, qt, lane, self, ts);
       } else {
-        ymax = tri_tile<V, QARR, false>(p, qt, lane, -1, ah, al, bh, bl);
+        ymax = MIX ? tri_tile_mixed<V, QARR, false>(p, qt, lane, -1, ts) : tri_tile<V, QARR, false>(p, qt, lane, -1, ts);
       }
       done = !__any_sync(0xffffffffu, !(ymax <= ylim));
       if (done) {
@@ -307,22 +457,25 @@ __global__ void __launch_bounds__(NT, NB)
           float h0, h1, l0, l1;
 #pragma unroll
           for (int v = 0; v < V; ++v) {
-            upk(ah[v][c], h0, h1);
-            upk(al[v][c], l0, l1);
+            upk(ts.ah[v][c], h0, h1);
+            upk(ts.al[v][c], l0, l1);
             double *d = aP + c * PI + v * 64 + lane;
-            d[0] += (double)h0 + (double)l0;
-            d[32] += (double)h1 + (double)l1;
+            d[0] += MIX ? f32_to_f64(h0) : (double)h0 + (double)l0;
+            d[32] += MIX ? f32_to_f64(h1) : (double)h1 + (double)l1;
           }
-          if (!diag) {
-            upk(bh[c], h0, h1);
-            upk(bl[c], l0, l1);
-            aQ[c * BI + lane] += ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
+          if (!one) {
+            upk(ts.bh[c], h0, h1);
+            upk(ts.bl[c], l0, l1);
+            if (MIX)
+              aQ[c * BI + lane] -= (f32_to_f64(h0) + f32_to_f64(h1)) + (f32_to_f64(l0) + f32_to_f64(l1));
+            else
+              aQ[c * BI + lane] += ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
           }
         }
       }
     }
     if (!done) {
-      if (diag)
+      if (one)
         tri_tile_fp64<true>(n, x, y, z, q, p0 + pt * PI, PI, q0 + t * 32, back, aP, PI, aQ, BI);
       else
         tri_tile_fp64<false>(n, x, y, z, q, p0 + pt * PI, PI, q0 + t * 32, back, aP, PI, aQ, BI);
@@ -330,14 +483,18 @@ __global__ void __launch_bounds__(NT, NB)
   }
   __syncthreads();
   const double fwd = pow2d(kw - 2 * kl);
-  sym_output<NT>(INPLACE, it, n, p0, np, q0, nq, out, sync, err,
-                 [&](int c, int i) {
-                   double v = 0.0;
-                   const double *s = accP + (i / PI) * 3 * PI + c * PI + i % PI;
-                   for (int g = 0; g < NG; ++g) v += s[g * PT * 3 * PI];
-                   return v * fwd;
-                 },
-                 [&](int c, int i) { return accQ[c * BI + i] * fwd; });
+  auto sumP = [&](int c, int i) {
+    double v = 0.0;
+    const double *s = accP + (i / PI) * 3 * PI + c * PI + i % PI;
+    for (int g = 0; g < NG; ++g) v += s[g * PT * 3 * PI];
+    if (MIX && diag) v += accQ[c * BI + i];  // across its sub-blocks
+    return v * fwd;
+  };
+  auto sumQ = [&](int c, int i) { return accQ[c * BI + i] * fwd; };
+  if (MIX && INPLACE)
+    tri_commit<NT>(it, n, BI, p0, np, q0, nq, out, sync, err, sumP, sumQ);
+  else
+    sym_output<NT>(INPLACE, it, n, p0, np, q0, nq, out, sync, err, sumP, sumQ);
 }
 
 // ---------------------------------------------------------------------------
@@ -347,8 +504,8 @@ static size_t tri_smem(int G) {
          (size_t)(NT / 32) * 3 * 64 * V * sizeof(double);
 }
 
-template <int V, int NT, int NB>
-static cudaError_t launch_tri(int64_t n, int nbk, int G, const double *x, const double *y, const double *z,
+template <bool MIX, int V, int NT, int NB>
+static cudaError_t launch_tri(int64_t n, int nbk, int G, int SB, const double *x, const double *y, const double *z,
                               const double *q, double *part, int *sync, unsigned *err, bool inplace,
                               cudaStream_t st) {
   static std::mutex mu;
@@ -360,10 +517,10 @@ static cudaError_t launch_tri(int64_t n, int nbk, int G, const double *x, const 
     std::lock_guard<std::mutex> lk(mu);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!done[dev]) {
-      const void *fns[4] = {(const void *)k_pair_sym_tri<V, true, NT, NB, true>,
-                            (const void *)k_pair_sym_tri<V, false, NT, NB, true>,
-                            (const void *)k_pair_sym_tri<V, true, NT, NB, false>,
-                            (const void *)k_pair_sym_tri<V, false, NT, NB, false>};
+      const void *fns[4] = {(const void *)k_pair_sym_tri<MIX, V, true, NT, NB, true>,
+                            (const void *)k_pair_sym_tri<MIX, V, false, NT, NB, true>,
+                            (const void *)k_pair_sym_tri<MIX, V, true, NT, NB, false>,
+                            (const void *)k_pair_sym_tri<MIX, V, false, NT, NB, false>};
       for (int k = 0; k < 4 && e == cudaSuccess; ++k)
         e = cudaFuncSetAttribute(fns[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem<V, NT>(32));
       if (e != cudaSuccess) return e;
@@ -377,7 +534,7 @@ static cudaError_t launch_tri(int64_t n, int nbk, int G, const double *x, const 
   const int items = nbk * (nbk + 1) / 2;
   const size_t smem = tri_smem<V, NT>(G);
 #define NB_TRI_LAUNCH(QA, IP) \
-  k_pair_sym_tri<V, QA, NT, NB, IP><<<items, NT, smem, st>>>(n, nbk, G, x, y, z, q, part, sync, err)
+  k_pair_sym_tri<MIX, V, QA, NT, NB, IP><<<items, NT, smem, st>>>(n, nbk, G, SB, x, y, z, q, part, sync, err)
   if (inplace) {
     if (q) NB_TRI_LAUNCH(true, true); else NB_TRI_LAUNCH(false, true);
   } else {
@@ -387,9 +544,11 @@ static cudaError_t launch_tri(int64_t n, int nbk, int G, const double *x, const 
   return cudaGetLastError();
 }
 
-// 32-ion blocks (set_tuning only) and softened sums stay with nb_sym.cu.
+// Softened sums stay with nb_sym.cu, and so do 32-ion blocks (the mixed form
+// below n = 2000, where 16-term FP32 sums are more accurate than 32-term ones at
+// the same speed; elsewhere by set_tuning only).
 static bool tri_sums(const Plan &pl, int mode, double soft2) {
-  return pl.sym && soft2 == 0.0 && (mode == MODE_FP64 || mode == MODE_DF64);
+  return pl.sym && soft2 == 0.0 && (mode == MODE_FP64 || mode == MODE_DF64 || mode == MODE_MIXED);
 }
 bool tri_serves(const Plan &pl, int mode, double soft2) { return tri_sums(pl, mode, soft2) && pl.G >= 2; }
 
@@ -398,12 +557,16 @@ bool tri_serves(const Plan &pl, int mode, double soft2) { return tri_sums(pl, mo
 // 128 up to 12160 (82 against 107 with 256 at 5003, 239 against 270 at 10000),
 // where 96 blocks would take the in-place output, whose chain of commits these
 // short items do not hide (628 against 454 at 14000), 256 above (19245 against
-// 19989 with 512 at 1e5).
+// 19989 with 512 at 1e5).  The mixed form's lines lie close by, from n = 2000;
+// its FP32 sums run one-sided within a diagonal block, so its block (or
+// sub-block, see launch_pair_tri) stays that of make_plan: 64 ions below 3000,
+// 128 below 32768, 256 below 60000, 512 above.
 Plan make_force_plan(int64_t n, int mode, double soft2) {
   Plan pl = make_plan(n, mode, 0);
   int tb = 0, tr = 0, tbps = 0;
-  if (!tri_sums(pl, mode, soft2) || tuning_lookup(4, mode, n, &tb, &tr, &tbps)) return pl;
+  if (!tri_sums(pl, mode, soft2) || (mode == MODE_MIXED && n < 2000) || tuning_lookup(4, mode, n, &tb, &tr, &tbps)) return pl;
   int G = n > 12160 ? 8 : (n >= 2800 ? 4 : 2);
+  if (mode == MODE_MIXED) G = n >= 60000 ? 16 : (n > 12160 ? 8 : (n >= 3000 ? 4 : 2));
   while (G < 32 && (n + 32 * G - 1) / (32 * G) > 60000) G *= 2;  // the schedule's block limit
   pl.G = G;
   pl.nbk = (int)((n + 32 * G - 1) / (32 * G));
@@ -412,17 +575,31 @@ Plan make_force_plan(int64_t n, int mode, double soft2) {
   return pl;
 }
 
-cudaError_t launch_pair_tri(const Plan &pl, int64_t n, const double *x, const double *y, const double *z,
+cudaError_t launch_pair_tri(const Plan &pl, int mode, int64_t n, const double *x, const double *y, const double *z,
                             const double *q, double *part, unsigned *err, cudaStream_t st) {
   int *sync = part_sync(pl, part, n, 3);
   const bool inplace = pl.n_jc == 1;
-#define NB_TRI(V, NT, NB) launch_tri<V, NT, NB>(n, pl.nbk, pl.G, x, y, z, q, part, sync, err, inplace, st)
+#define NB_TRI(MIX, V, NT, NB) launch_tri<MIX, V, NT, NB>(n, pl.nbk, pl.G, SB, x, y, z, q, part, sync, err, inplace, st)
+  // The mixed form's FP32 sums keep the order they have with make_plan's
+  // blocks: one-sided within 128 ions for n < 32768 (whose items of 256 ions
+  // from n = 12161 on only change where FP64 sums are added), else within the
+  // item.  The fp64 form has no such order to keep; halving its diagonal items
+  // this way cost 2 % at n = 1e5 (a second inlined tile step in the branch).
+  const int SB = mode == MODE_MIXED && n < 32768 ? std::min(pl.G, 4) : pl.G;
+  if (mode == MODE_MIXED) switch (pl.G) {
+      case 2: return NB_TRI(true, 1, 64, 12);
+      case 4:
+      case 8: return NB_TRI(true, 2, 128, 4);
+      case 16: return NB_TRI(true, 2, 128, 3);
+      case 32: return NB_TRI(true, 2, 256, 2);
+      default: return cudaErrorInvalidValue;
+    }
   switch (pl.G) {
-    case 2: return NB_TRI(1, 64, 10);
+    case 2: return NB_TRI(false, 1, 64, 10);
     case 4:
-    case 8: return NB_TRI(2, 128, 4);
+    case 8: return NB_TRI(false, 2, 128, 4);
     case 16:
-    case 32: return NB_TRI(2, 256, 2);
+    case 32: return NB_TRI(false, 2, 256, 2);
     default: return cudaErrorInvalidValue;
   }
 #undef NB_TRI

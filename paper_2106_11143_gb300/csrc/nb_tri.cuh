@@ -213,7 +213,7 @@ __device__ __forceinline__ double pow2d(int k) { return __hiloint2double((1023 +
 Plan make_force_plan(int64_t n, int mode, double soft2);
 // Whether the kernel serves a plan, and its launch.
 bool tri_serves(const Plan &pl, int mode, double soft2);
-cudaError_t launch_pair_tri(const Plan &pl, int64_t n, const double *x, const double *y, const double *z,
+cudaError_t launch_pair_tri(const Plan &pl, int mode, int64_t n, const double *x, const double *y, const double *z,
                             const double *q, double *part, unsigned *err, cudaStream_t st);
 
 }  // namespace nb
