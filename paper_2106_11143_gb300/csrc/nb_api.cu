@@ -228,7 +228,7 @@ size_t force_bytes(const Plan &pl, int mode, int64_t n, bool extra_pos, bool phi
 cudaError_t launch_pairs(const Plan &pl, int mode, int64_t n, const double *x, const double *y, const double *z,
                          const double *q, const PosF32 &pf, double soft2, double *part, unsigned *err,
                          cudaStream_t st) {
-  if (tri_serves(pl, mode, soft2)) return launch_pair_tri(pl, mode, n, x, y, z, q, part, err, st);
+  if (tri_serves(pl, mode, soft2)) return launch_pair_tri(pl, mode, n, x, y, z, q, soft2, part, err, st);
   return launch_pair_force(pl, mode, n, x, y, z, q, pf, soft2, part, err, st);
 }
 

@@ -18,8 +18,9 @@
 // kernel by value (__grid_constant__), so a launch needs no host-to-device
 // copy and can be captured in a CUDA graph.
 //
-// Instances of at most 4096 ions use a half-pair force phase (bsym_forces
-// below); larger instances use the one-sided phase.
+// Instances of at most 4096 ions use a half-pair force phase: btri_forces
+// below, which has no FP64 in its pair loop, or bsym_forces for unusual
+// scales; larger instances use the one-sided phase.
 // Either way the arithmetic of an ion depends only on its instance (a fixed
 // pair order and accumulation order per ion), not on the schedule or the block
 // size, so results are bitwise reproducible.
@@ -27,6 +28,7 @@
 #include <mutex>
 #include <vector>
 
+#include "nb_tri.cuh"
 #include "nb_verlet.cuh"
 
 namespace nb {
@@ -39,7 +41,7 @@ constexpr int BATCH_MAX_INST = 1024;
 constexpr int BATCH_MAX_BINS = 1024;
 static_assert(BATCH_MAX_INST == BATCH_LIMIT_INST, "schedule arrays sized for the validated instance limit");
 // ions per instance (BATCH_LIMIT_N, checked on the host): 32 B each in shared memory
-static_assert(sizeof(Phys) % 16 == 0 && sizeof(Phys) + BATCH_LIMIT_N * sizeof(BD4) <= 227 * 1024,
+static_assert(sizeof(Phys) % 16 == 0 && sizeof(Phys) + BATCH_LIMIT_N * sizeof(BD4) <= 227 * 1024 - 1024,
               "an instance's parameters and positions fit one block's shared memory");
 
 struct BatchSched {
@@ -49,6 +51,31 @@ struct BatchSched {
   unsigned short order[BATCH_MAX_INST];             // instances, grouped by bin
   unsigned short bin_start[BATCH_MAX_BINS + 1];     // bin b = order[bin_start[b] .. bin_start[b+1])
 };
+
+// An instance's ions: positions in shared memory, charges in the caller's
+// array (nullptr: one species).
+struct BIons {
+  const double *x, *y, *z, *q;
+  int n;
+};
+// Ion i with its weight as the pair terms take it (an FP64 value for fp64, an
+// FP32 (hi, lo) pair for df64); past the end a weight-0 dummy far away.
+template <bool QARR, bool DF>
+__device__ __forceinline__ BD4 bion(const BIons &v, int i) {
+  BD4 r{1e18, 1e18, 1e18, 0.0};
+  if (i < v.n) {
+    r.x = v.x[i];
+    r.y = v.y[i];
+    r.z = v.z[i];
+    r.w = QARR ? v.q[i] : 1.0;
+    if (DF) {
+      float qh = 1.0f, ql = 0.0f;
+      if (QARR) split_f64(v.q[i], qh, ql);
+      *reinterpret_cast<float2 *>(&r.w) = make_float2(qh, ql);
+    }
+  }
+  return r;
+}
 
 // FP64 pair term, identical arithmetic to the single-system force kernel.
 template <bool QARR>
@@ -105,8 +132,11 @@ __device__ __forceinline__ void bpair_df64(double xi, double yi, double zi, cons
 // and rotates tile b's accumulators by shuffle.  The order of every sum is
 // fixed by the schedule, not by the block size.
 constexpr int BATCH_SYM_N = 4096;
-static_assert(sizeof(Phys) + BATCH_SYM_N * (sizeof(BD4) + 3 * sizeof(double)) <= 227 * 1024,
-              "the half-pair phase's accumulators fit beside the positions");
+constexpr int BATCH_THREADS_MAX = 512;
+constexpr int BTRI_STAGE4 = 3 * 32;  // float4 per warp: a Q-tile's words
+static_assert(sizeof(Phys) + BATCH_SYM_N * 6 * sizeof(double) + BATCH_THREADS_MAX / 32 * BTRI_STAGE4 * sizeof(float4) <=
+                  227 * 1024 - 1024,
+              "the half-pair phase's accumulators and staged tiles fit beside the positions");
 
 __device__ __forceinline__ double bshfl_next(double v, int lane) {
   return __shfl_sync(0xffffffffu, v, (lane + 1) & 31);
@@ -181,14 +211,14 @@ __device__ __forceinline__ void round_pair(int rho, int k, int Tp, int &a, int &
 // The force phase: acc[c * npad + i] = sum_j w_j (r_i - r_j) / |r_i - r_j|^3
 // for the instance's np32 staged entries (n real ions, weights in w: an FP64
 // value for fp64, an FP32 (hi, lo) pair for df64).
-template <bool W, bool DF>
-__device__ __forceinline__ void bsym_tile_pair(const BD4 &pp, const BD4 *qt, int lane, double soft2,
+template <bool QARR, bool W, bool DF>
+__device__ __forceinline__ void bsym_tile_pair(const BIons &v, const BD4 &pp, int q0, int lane, double soft2,
                                                float s2h, float s2l, double a[3], double b[3]) {
   if (DF) {
     float ah[3] = {0, 0, 0}, al[3] = {0, 0, 0}, bh[3] = {0, 0, 0}, bl[3] = {0, 0, 0};
 #pragma unroll 2
     for (int r = 0; r < 32; ++r) {
-      bsym_eval_df64<W>(pp, qt[(lane + r) & 31], s2h, s2l, ah, al, bh, bl);
+      bsym_eval_df64<W>(pp, bion<QARR, DF>(v, q0 + ((lane + r) & 31)), s2h, s2l, ah, al, bh, bl);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         bh[c] = __shfl_sync(0xffffffffu, bh[c], (lane + 1) & 31);
@@ -204,7 +234,7 @@ __device__ __forceinline__ void bsym_tile_pair(const BD4 &pp, const BD4 *qt, int
     a[0] = a[1] = a[2] = b[0] = b[1] = b[2] = 0.0;
 #pragma unroll 2
     for (int r = 0; r < 32; ++r) {
-      bsym_eval<W>(pp, qt[(lane + r) & 31], soft2, a, b);
+      bsym_eval<W>(pp, bion<QARR, DF>(v, q0 + ((lane + r) & 31)), soft2, a, b);
       b[0] = bshfl_next(b[0], lane);
       b[1] = bshfl_next(b[1], lane);
       b[2] = bshfl_next(b[2], lane);
@@ -213,15 +243,15 @@ __device__ __forceinline__ void bsym_tile_pair(const BD4 &pp, const BD4 *qt, int
 }
 
 template <bool QARR, bool DF>
-__device__ void bsym_forces(const BD4 *sp, double *acc, int npad, int n, int np32, double soft2,
-                            float s2h, float s2l) {
+__device__ __noinline__ void bsym_forces(const BIons v, double *acc, int npad, double soft2, float s2h, float s2l) {
+  const int n = v.n, np32 = (n + 31) & ~31;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5;
   const int T = np32 >> 5;
   const bool ragged = (n & 31) != 0;
   // diagonal tiles, one-sided (the self pair gives 0)
   for (int t = warp; t < T; t += NW) {
     const int i = t * 32 + lane;
-    const BD4 pi = sp[i];
+    const BD4 pi = bion<QARR, DF>(v, i);
     double a[3] = {0.0, 0.0, 0.0};
     const bool w = QARR || (ragged && t == T - 1);
     if (DF) {
@@ -229,18 +259,18 @@ __device__ void bsym_forces(const BD4 *sp, double *acc, int npad, int n, int np3
       for (int j = 0; j < 32; ++j) {
         bh[0] = bh[1] = bh[2] = bl[0] = bl[1] = bl[2] = 0.0f;  // the partner side is not used
         if (w)
-          bsym_eval_df64<true>(pi, sp[t * 32 + j], s2h, s2l, ah, al, bh, bl);
+          bsym_eval_df64<true>(pi, bion<QARR, DF>(v, t * 32 + j), s2h, s2l, ah, al, bh, bl);
         else
-          bsym_eval_df64<false>(pi, sp[t * 32 + j], s2h, s2l, ah, al, bh, bl);
+          bsym_eval_df64<false>(pi, bion<QARR, DF>(v, t * 32 + j), s2h, s2l, ah, al, bh, bl);
       }
 #pragma unroll
       for (int c = 0; c < 3; ++c) a[c] = f32_to_f64(ah[c]) + f32_to_f64(al[c]);
     } else {
       double dummy[3];
       if (w) {
-        for (int j = 0; j < 32; ++j) bsym_eval<true>(pi, sp[t * 32 + j], soft2, a, dummy);
+        for (int j = 0; j < 32; ++j) bsym_eval<true>(pi, bion<QARR, DF>(v, t * 32 + j), soft2, a, dummy);
       } else {
-        for (int j = 0; j < 32; ++j) bsym_eval<false>(pi, sp[t * 32 + j], soft2, a, dummy);
+        for (int j = 0; j < 32; ++j) bsym_eval<false>(pi, bion<QARR, DF>(v, t * 32 + j), soft2, a, dummy);
       }
     }
 #pragma unroll
@@ -253,13 +283,12 @@ __device__ void bsym_forces(const BD4 *sp, double *acc, int npad, int n, int np3
       int ta, tb;
       round_pair(rho, k, Tp, ta, tb);
       if (ta >= T || tb >= T) continue;  // the bye of an odd tile count
-      const BD4 pp = sp[ta * 32 + lane];
-      const BD4 *qt = sp + tb * 32;
+      const BD4 pp = bion<QARR, DF>(v, ta * 32 + lane);
       double a[3], b[3];
       if (QARR || (ragged && (ta == T - 1 || tb == T - 1)))
-        bsym_tile_pair<true, DF>(pp, qt, lane, soft2, s2h, s2l, a, b);
+        bsym_tile_pair<QARR, true, DF>(v, pp, tb * 32, lane, soft2, s2h, s2l, a, b);
       else
-        bsym_tile_pair<false, DF>(pp, qt, lane, soft2, s2h, s2l, a, b);
+        bsym_tile_pair<QARR, false, DF>(v, pp, tb * 32, lane, soft2, s2h, s2l, a, b);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         acc[c * npad + ta * 32 + lane] += a[c];
@@ -270,14 +299,223 @@ __device__ void bsym_forces(const BD4 *sp, double *acc, int npad, int n, int np3
   }
 }
 
+// ---------------------------------------------------------------------------
+// The half-pair force phase on the FP32 pipe (nb_tri.cuh), both precisions.
+//
+// The instance is cut into S super-tiles of 128 ions, four 32-ion tiles each.
+// A task (A, B, t) takes the 128 ions of A as the P side (four per lane) and
+// tile t of B as the Q side; B = A is one-sided.  Tasks are numbered round by
+// round: round 0 holds the S diagonal super-tiles, rounds 1 .. pair every two
+// super-tiles once (circle method, as above), four tasks to a pair.  Each warp
+// takes one task of every NW.  The arithmetic only reads positions; the sums
+// are then added to the accumulators in the order of the rounds and, on a pair's
+// A, of its four tasks, so that every ion's sum has one order whatever the
+// number of warps.  That order is kept by a counter per super-tile of the tasks
+// that have added to it: a task waits for its turn on A and, on B, for the
+// earlier rounds, and no barrier stands between tasks, so a warp's FP64 adds
+// overlap the others' pair arithmetic.  A task waits only for lower-numbered
+// ones, which warps take in order, so the lowest unfinished never waits; the
+// wait is bounded all the same (ERR_TIMEOUT).
+//
+// What bounds it: the FMA pipe, as in nb_tri.cu, with 16 warps per SM (the
+// registers' limit); the words are cut from the FP64 positions at every task
+// (450 instructions against 10 400 of pair arithmetic), diagonal super-tiles are
+// one-sided, and below about 500 ions there are fewer tasks than warps.  Two
+// steps of 512 instances of 32 .. 4096 ions: 14.2 ms (421 G pairs/s) against
+// 59.9 (fp64) and 25.8 ms (df64) with bsym_forces; 152 instances of 4096: 10.7
+// against 45.9 and 18.7 ms.  With the tasks' adds between barriers instead of
+// counters the FP64 adds of all 16 warps coincided: 18.8 ms.
+constexpr int BTRI_PI = 128;
+
+// A tile of a task in FP64 (nb_tri.cuh's limits): the P side's 128 ions
+// against tile q0 .. q0 + 31, added to acc.
+template <bool QARR>
+__device__ __noinline__ void btri_tile_fp64(const BIons v, int p0, int q0, bool one, double soft2, double sc,
+                                            double *acc, int npad) {
+  const int lane = threadIdx.x & 31;
+  for (int u = 0; u < BTRI_PI; u += 32) {
+    const int i = p0 + u + lane;
+    double a[3] = {0.0, 0.0, 0.0}, b[3] = {0.0, 0.0, 0.0};
+    for (int r = 0; r < 32; ++r) {
+      const int j = q0 + ((lane + r) & 31);
+      if (i < v.n && j < v.n && i != j) {
+        const BD4 pi = bion<QARR, false>(v, i), pj = bion<QARR, false>(v, j);
+        bsym_eval<QARR>(pi, pj, soft2, a, b);
+      }
+      for (int c = 0; c < 3; ++c) b[c] = bshfl_next(b[c], lane);
+    }
+    for (int c = 0; c < 3; ++c) {
+      if (i < v.n) acc[c * npad + i] += a[c] * sc;
+      __syncwarp();
+      if (!one && q0 + lane < v.n) acc[c * npad + q0 + lane] += b[c] * sc;
+    }
+  }
+}
+
+// Bounded wait of a warp for counter c to reach v (about a second).
+constexpr int BTRI_SPIN_LIMIT = 1 << 24;
+__device__ __forceinline__ bool btri_wait(const int *c, int v) {
+  bool ok = false;
+  if ((threadIdx.x & 31) == 0)
+    for (int k = 0; k < BTRI_SPIN_LIMIT && !ok; ++k) {
+      ok = *(const volatile int *)c >= v;
+      if (!ok) __nanosleep(32);
+    }
+  ok = __shfl_sync(0xffffffffu, ok, 0);
+  __threadfence_block();
+  return ok;
+}
+
+// One task: the pair arithmetic of the P side's 64 V ions from p0 against tile
+// q0 .. q0 + 31, then, in its turn, the adds to acc.  wait() takes the turn
+// (false: it gave up); self as in tri_tile, or -1 for two super-tiles.
+template <int V, bool QARR, class WAIT>
+__device__ __forceinline__ bool btri_task(const BIons &v, double *acc, int npad, float4 *st, int em, int ew,
+                                          double soft2, int p0, int q0, int self, WAIT wait) {
+  const int lane = threadIdx.x & 31, n = v.n;
+  const bool one = self >= 0;
+  float w0[2][4], w1[2][4], w2[2][4];
+  __syncwarp();  // every lane is done with the last tile
+  tri_ion<QARR>(q0 + lane, q0 + lane < n, v.x, v.y, v.z, v.q, em, ew, -TRI_FAR, w0[0], w1[0], w2[0]);
+  st[lane] = make_float4(w0[0][0], w0[0][1], w0[0][2], w0[0][3]);
+  st[32 + lane] = make_float4(w1[0][0], w1[0][1], w1[0][2], w1[0][3]);
+  st[64 + lane] = make_float4(w2[0][0], w2[0][1], w2[0][2], w2[0][3]);
+  TriIons<V> p;
+#pragma unroll
+  for (int u = 0; u < V; ++u) {
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int i = p0 + u * 64 + b * 32 + lane;
+      tri_ion<QARR>(i, i < n, v.x, v.y, v.z, v.q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      p.h[u][c] = pk(w0[0][c], w0[1][c]);
+      p.m[u][c] = pk(w1[0][c], w1[1][c]);
+      p.l[u][c] = pk(w2[0][c], w2[1][c]);
+    }
+    p.wh[u] = pk(w0[0][3], w0[1][3]);
+    p.wl[u] = pk(w1[0][3], w1[1][3]);
+  }
+  TriSums<V> ts;
+  const f32x2 zero = pk1(0.0f);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    ts.bh[c] = ts.bl[c] = zero;
+#pragma unroll
+    for (int u = 0; u < V; ++u) ts.ah[u][c] = ts.al[u][c] = zero;
+  }
+  __syncwarp();
+  auto ld = [&](int r, float4 &f0, float4 &f1, float4 &f2) {
+    const float4 *e = st + ((lane + r) & 31);
+    f0 = e[0];
+    f1 = e[32];
+    f2 = e[64];
+  };
+  float ymax;
+  if (soft2 != 0.0) {
+    float sh, sl;
+    split_f64_scaled(soft2, 2 * (em - 1022), sh, sl);
+    ymax = one ? tri_tile<V, QARR, true, true>(p, ld, lane, self, pk1(sh), pk1(sl), ts)
+               : tri_tile<V, QARR, false, true>(p, ld, lane, -1, pk1(sh), pk1(sl), ts);
+  } else {
+    ymax = one ? tri_tile<V, QARR, true, false>(p, ld, lane, self, zero, zero, ts)
+               : tri_tile<V, QARR, false, false>(p, ld, lane, -1, zero, zero, ts);
+  }
+  const bool done = !__any_sync(0xffffffffu, !(ymax <= TRI_YMAX));
+  if (!wait()) return false;
+  if (!done) {
+    btri_tile_fp64<QARR>(v, p0, q0, one, soft2, pow2d(2 * (em - 1022) - (ew - 1023)), acc, npad);
+    return true;
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float h0, h1, l0, l1;
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      upk(ts.ah[u][c], h0, h1);
+      upk(ts.al[u][c], l0, l1);
+      const int i = p0 + u * 64 + lane;
+      if (i < n) acc[c * npad + i] += (double)h0 + (double)l0;
+      if (i + 32 < n) acc[c * npad + i + 32] += (double)h1 + (double)l1;
+    }
+    if (!one && q0 + lane < n) {
+      upk(ts.bh[c], h0, h1);
+      upk(ts.bl[c], l0, l1);
+      acc[c * npad + q0 + lane] += ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
+    }
+  }
+  return true;
+}
+
+template <bool QARR>
+__device__ __forceinline__ void btri_forces(const BIons &v, double *acc, int npad, float4 *stage, int *cnt, int em,
+                                            int ew, double soft2, unsigned *err) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5;
+  const int n = v.n, S = (n + BTRI_PI - 1) / BTRI_PI, odd = S & 1;
+  const int per = 4 * (S >> 1);  // tasks of a round
+  const int M = 4 * S + (S > 1 ? (S - 1 + odd) * per : 0);
+  float4 *st = stage + warp * BTRI_STAGE4;
+  for (int m = warp; m < M; m += NW) {
+    const int k = m & 3;  // 4 S and per are multiples of 4
+    int A = m >> 2, B = A, rd = 0;
+    if (m >= 4 * S) {
+      const int u = m - 4 * S, rho = u / per;
+      rd = 1 + rho;
+      round_pair(rho, ((u - rho * per) >> 2) + odd, S + odd, A, B);  // an odd S: pair 0 is the bye
+    }
+    const int p0 = A * BTRI_PI, q0 = B * BTRI_PI + 32 * k;
+    const bool one = A == B;
+    // rounds before this one that X has taken part in: all but its own bye
+    auto before = [&](int X) { return rd - (odd && X < rd - 1 ? 1 : 0); };
+    auto wait = [&]() {
+      const bool a = btri_wait(cnt + A, 4 * before(A) + k);
+      return (one || btri_wait(cnt + B, 4 * before(B))) && a;
+    };
+    // a super-tile of at most 64 ions (the last one, or a small instance) has
+    // one pair of P-ions per lane: 8.9 to 6.1 ms for 50 steps of 1024 instances
+    // of 16 .. 64 ions
+    bool ok;
+    if (q0 >= n)
+      ok = wait();
+    else if (p0 + 64 < n)
+      ok = btri_task<2, QARR>(v, acc, npad, st, em, ew, soft2, p0, q0, one ? k : -1, wait);
+    else
+      ok = btri_task<1, QARR>(v, acc, npad, st, em, ew, soft2, p0, q0, one ? k : -1, wait);
+    if (!ok && lane == 0) atomicOr(err, ERR_TIMEOUT);
+    __threadfence_block();
+    __syncwarp();
+    if (lane == 0) {
+      atomicAdd(cnt + A, 1);
+      if (!one) atomicAdd(cnt + B, 1);
+    }
+  }
+  __syncthreads();
+}
+
+// The largest (or with MIN the smallest) of a value over the block; red holds
+// one int per warp and is free again after the caller's next barrier.
+template <bool MIN>
+__device__ __forceinline__ int block_extreme(int v, int *red) {
+  v = MIN ? __reduce_min_sync(0xffffffffu, v) : __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = MIN ? min(v, red[w]) : max(v, red[w]);
+  return v;
+}
+
 template <bool QARR, bool DF, bool SYM>
 __global__ void __launch_bounds__(512, 1) k_batched(Phys pall, const Phys *__restrict__ ptab, StateView s,
                                                   const __grid_constant__ BatchSched sch,
                                                   int64_t step0, int64_t nsteps, int npad, unsigned *err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Phys &pinst = *reinterpret_cast<Phys *>(smem_raw);  // the running instance's parameters
-  BD4 *sp = reinterpret_cast<BD4 *>(smem_raw + sizeof(Phys));
-  double *acc = reinterpret_cast<double *>(sp + npad);  // SYM: [3][npad]
+  double *sx = reinterpret_cast<double *>(smem_raw + sizeof(Phys)), *sy = sx + npad, *sz = sy + npad;
+  double *acc = sz + npad;                                       // SYM: [3][npad]
+  float4 *stage = reinterpret_cast<float4 *>(acc + 3 * npad);    // SYM: BTRI_STAGE4 per warp
+  double *sw = sz + npad;                                        // one-sided: the weights
+  __shared__ int red[3][BATCH_THREADS_MAX / 32];
+  __shared__ int cnt[BATCH_SYM_N / BTRI_PI];  // tasks that have added to each super-tile
   const int T = blockDim.x;
   const int tid = threadIdx.x;
   bool bad = false;
@@ -297,21 +535,26 @@ __global__ void __launch_bounds__(512, 1) k_batched(Phys pall, const Phys *__res
         pinst.instance = pall.instance + (unsigned)inst;
       }
     }
-    const int np32 = (n + 31) & ~31;
-    if (SYM)
-      for (int i = n + tid; i < np32; i += T) sp[i] = BD4{1e18, 1e18, 1e18, 0.0};  // weight-0 dummies
+    const BIons ions{sx, sy, sz, QARR ? s.q + i0 : nullptr, n};
+    int wx = 0, wn = 0x7fffffff;  // the weights' largest and smallest exponent words
     for (int i = tid; i < n; i += T) {
-      BD4 r;
-      r.x = s.x[i0 + i]; r.y = s.y[i0 + i]; r.z = s.z[i0 + i];
-      r.w = QARR ? s.q[i0 + i] : 1.0;
-      if (DF && QARR) {  // q as an FP32 (hi, lo) pair for the double-float pair term
-        float qh, ql;
-        split_f64(s.q[i0 + i], qh, ql);
-        *reinterpret_cast<float2 *>(&r.w) = make_float2(qh, ql);
-      } else if (DF) {
-        *reinterpret_cast<float2 *>(&r.w) = make_float2(1.0f, 0.0f);
+      sx[i] = s.x[i0 + i];
+      sy[i] = s.y[i0 + i];
+      sz[i] = s.z[i0 + i];
+      if (SYM && QARR && s.q[i0 + i] != 0.0) {
+        const int w = __double2hiint(s.q[i0 + i]) & 0x7fffffff;
+        wx = max(wx, w);
+        wn = min(wn, w);
       }
-      sp[i] = r;
+      if (!SYM) sw[i] = bion<QARR, DF>(ions, i).w;
+    }
+    int ew = 1023;
+    bool tri_w = true;  // the weights' range suits the FP32 path
+    if (SYM && QARR) {
+      wx = block_extreme<false>(wx, red[0]);
+      wn = block_extreme<true>(wn, red[1]);
+      ew = wx >> 20;
+      tri_w = ew >= 1023 - 400 && ew <= 1023 + 400 && ew - (wn >> 20) <= TRI_WSPREAD;
     }
     __syncthreads();
     const Phys &p = pinst;
@@ -327,31 +570,51 @@ __global__ void __launch_bounds__(512, 1) k_batched(Phys pall, const Phys *__res
       const int64_t snew = step0 + st + 1;
       const double t = p.t0 + (double)snew * dt;
       // drift: r+ = r + v dt + a dt^2/2 (each thread its own ions)
+      int mx = 0;
+      if (SYM)
+        for (int i = tid; i < BATCH_SYM_N / BTRI_PI; i += T) cnt[i] = 0;
       for (int i = tid; i < n; i += T) {
-        BD4 r = sp[i];
-        r.x = r.x + s.vx[i0 + i] * dt + hdt2 * s.ax[i0 + i];
-        r.y = r.y + s.vy[i0 + i] * dt + hdt2 * s.ay[i0 + i];
-        r.z = r.z + s.vz[i0 + i] * dt + hdt2 * s.az[i0 + i];
-        sp[i] = r;
+        const double rx = sx[i] + s.vx[i0 + i] * dt + hdt2 * s.ax[i0 + i];
+        const double ry = sy[i] + s.vy[i0 + i] * dt + hdt2 * s.ay[i0 + i];
+        const double rz = sz[i] + s.vz[i0 + i] * dt + hdt2 * s.az[i0 + i];
+        sx[i] = rx;
+        sy[i] = ry;
+        sz[i] = rz;
+        if (SYM) {
+          mx = max(mx, max(__double2hiint(rx) & 0x7fffffff,
+                           max(__double2hiint(ry) & 0x7fffffff, __double2hiint(rz) & 0x7fffffff)));
+          acc[i] = acc[npad + i] = acc[2 * npad + i] = 0.0;
+        }
       }
-      __syncthreads();
       // forces at r+ and the kick
-      if (SYM) bsym_forces<QARR, DF>(sp, acc, npad, n, np32, soft2, s2h, s2l);
+      double fwd = 1.0;  // the accumulators' unit
+      if (SYM) {
+        const int em = block_extreme<false>(mx, red[2]) >> 20;
+        if (tri_w && tri_scale_ok(em, soft2)) {
+          fwd = pow2d((ew - 1023) - 2 * (em - 1022));
+          btri_forces<QARR>(ions, acc, npad, stage, cnt, em, ew, soft2, err);
+        } else {
+          bsym_forces<QARR, DF>(ions, acc, npad, soft2, s2h, s2l);
+        }
+      } else {
+        __syncthreads();
+      }
       for (int ib = 0; ib < n; ib += T) {
         const int i = ib + tid;
-        const BD4 ri = sp[min(i, n - 1)];
+        const int ic = min(i, n - 1);
+        const BD4 ri{sx[ic], sy[ic], sz[ic], 0.0};
         double a0 = 0.0, a1 = 0.0, a2 = 0.0;
         if (SYM) {
           if (i < n) {
-            a0 = acc[i];
-            a1 = acc[npad + i];
-            a2 = acc[2 * npad + i];
+            a0 = acc[i] * fwd;
+            a1 = acc[npad + i] * fwd;
+            a2 = acc[2 * npad + i] * fwd;
           }
         } else if (DF) {
           float ah[3] = {0.0f, 0.0f, 0.0f}, al[3] = {0.0f, 0.0f, 0.0f};
           for (int j0 = 0; j0 < n; j0 += 256) {  // double-float sums flushed every 256 partners
             const int j1 = min(n, j0 + 256);
-            for (int j = j0; j < j1; ++j) bpair_df64<QARR>(ri.x, ri.y, ri.z, sp[j], s2h, s2l, ah, al);
+            for (int j = j0; j < j1; ++j) bpair_df64<QARR>(ri.x, ri.y, ri.z, BD4{sx[j], sy[j], sz[j], sw[j]}, s2h, s2l, ah, al);
             a0 += f32_to_f64(ah[0]) + f32_to_f64(al[0]);
             a1 += f32_to_f64(ah[1]) + f32_to_f64(al[1]);
             a2 += f32_to_f64(ah[2]) + f32_to_f64(al[2]);
@@ -359,7 +622,7 @@ __global__ void __launch_bounds__(512, 1) k_batched(Phys pall, const Phys *__res
           }
         } else {
 #pragma unroll 2
-          for (int j = 0; j < n; ++j) bpair<QARR>(ri.x, ri.y, ri.z, sp[j], soft2, a0, a1, a2);
+          for (int j = 0; j < n; ++j) bpair<QARR>(ri.x, ri.y, ri.z, BD4{sx[j], sy[j], sz[j], sw[j]}, soft2, a0, a1, a2);
         }
         if (i < n) {
           const int64_t gi = i0 + i;
@@ -386,9 +649,9 @@ __global__ void __launch_bounds__(512, 1) k_batched(Phys pall, const Phys *__res
       __syncthreads();
     }
     for (int i = tid; i < n; i += T) {
-      s.x[i0 + i] = sp[i].x;
-      s.y[i0 + i] = sp[i].y;
-      s.z[i0 + i] = sp[i].z;
+      s.x[i0 + i] = sx[i];
+      s.y[i0 + i] = sy[i];
+      s.z[i0 + i] = sz[i];
     }
   }
   if (bad) atomicOr(err, ERR_NONFINITE);
@@ -442,8 +705,9 @@ cudaError_t launch_batched(const Phys &p, const Phys *ptab, const StateView &s, 
   const bool df = p.precision == MODE_DF64;
   const bool sym = allow_sym && maxn <= BATCH_SYM_N;
   const int npad = (std::max(maxn, 1) + 31) & ~31;
-  const size_t need = sizeof(Phys) + (sym ? (size_t)npad * (sizeof(BD4) + 3 * sizeof(double))
-                                          : (size_t)std::max(maxn, 1) * sizeof(BD4));
+  const size_t need = sizeof(Phys) + (sym ? (size_t)npad * 6 * sizeof(double) +
+                                                (size_t)(threads / 32) * BTRI_STAGE4 * sizeof(float4)
+                                          : (size_t)npad * 4 * sizeof(double));
   // At least 120 KB of shared memory per CTA, so no SM holds two bins: each
   // bin then owns one SM, which is what the LPT packing assumes.
   const size_t smem = std::max(need, (size_t)120 * 1024);
@@ -456,7 +720,7 @@ cudaError_t launch_batched(const Phys &p, const Phys *ptab, const StateView &s, 
     std::lock_guard<std::mutex> lk(mu);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!attr_done[dev]) {
-      const int lim = 227 * 1024;
+      const int lim = 227 * 1024 - 1024;  // beside the block's static shared memory
       const void *fns[8] = {(const void *)k_batched<true, false, false>, (const void *)k_batched<false, false, false>,
                             (const void *)k_batched<true, true, false>,  (const void *)k_batched<false, true, false>,
                             (const void *)k_batched<true, false, true>,  (const void *)k_batched<false, false, true>,

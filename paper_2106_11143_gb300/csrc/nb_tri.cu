@@ -52,82 +52,9 @@
 
 namespace nb {
 
-template <int V>
-struct TriIons {  // 2 V ions of a lane: words and, with weights, the weight's (hi, lo)
-  f32x2 h[V][3], m[V][3], l[V][3], wh[V], wl[V];
-};
-
-// The sums of a tile step: double-floats, or FP32 (MIX) in the high words.
-template <int V>
-struct TriSums {
-  f32x2 ah[V][3], al[V][3], bh[3], bl[3];
-};
-
 // A staged tile: word k of entry e (64 entries, the tile twice) at
 // [k * 64 + e], the weight's high and low parts in the w of words 0 and 1.
 constexpr int TRI_TILE4 = 3 * 64;
-
-// One tile step: this lane's P-ions against the 32 Q-ions of `qt` (lane's
-// entry).  Returns the largest 1/r met.  self: the lane's P-ion (0 .. 2 V - 1)
-// that is Q-ion 0 of the rotation itself, or -1 (ONE only).
-template <int V, bool W, bool ONE>
-__device__ __forceinline__ float tri_tile(const TriIons<V> &p, const float4 *qt, int lane, int self, TriSums<V> &t) {
-  f32x2(&ah)[V][3] = t.ah, (&al)[V][3] = t.al, (&bh)[3] = t.bh, (&bl)[3] = t.bl;
-  float ymax = 0.0f;
-  const int next = (lane + 1) & 31;
-#pragma unroll 1
-  for (int r0 = 0; r0 < 32; r0 += 2) {
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const float4 q0 = qt[r0 + s], q1 = qt[64 + r0 + s], q2 = qt[128 + r0 + s];
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        f32x2 dh[3], dl[3], h, l, sh, sl;
-        tri_diff(p.h[v][0], p.m[v][0], p.l[v][0], pk1(q0.x), pk1(q1.x), pk1(q2.x), dh[0], dl[0]);
-        tri_diff(p.h[v][1], p.m[v][1], p.l[v][1], pk1(q0.y), pk1(q1.y), pk1(q2.y), dh[1], dl[1]);
-        tri_diff(p.h[v][2], p.m[v][2], p.l[v][2], pk1(q0.z), pk1(q1.z), pk1(q2.z), dh[2], dl[2]);
-        tri_r2(dh, dl, h, l);
-        float ha, hb;
-        upk(h, ha, hb);
-        float ya = rsqrt_approx(ha), yb = rsqrt_approx(hb);
-        if (ONE) {
-          // the ion itself: d = 0 gives a zero term with any finite y
-          ymax = fmaxf(ymax, s == 0 && r0 == 0 && self == 2 * v ? 0.0f : ya);
-          ymax = fmaxf(ymax, s == 0 && r0 == 0 && self == 2 * v + 1 ? 0.0f : yb);
-          ya = fminf(ya, TRI_YMAX_GRID);
-          yb = fminf(yb, TRI_YMAX_GRID);
-        } else {
-          ymax = fmaxf(ymax, fmaxf(ya, yb));
-        }
-        tri_rinv3(h, l, pk(ya, yb), sh, sl);
-        f32x2 sph = sh, spl = sl, sqh = sh, sql = sl;
-        if (W) ptwo_prod(sh, sl, pk1(q0.w), pk1(q1.w), sph, spl);
-        if (W && !ONE) ptwo_prod(sh, sl, p.wh[v], p.wl[v], sqh, sql);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          f32x2 th, tl;
-          ptwo_prod(dh[c], dl[c], sph, spl, th, tl);
-          pacc(ah[v][c], al[v][c], th, tl);
-          if (!ONE) {
-            if (W) ptwo_prod(dh[c], dl[c], sqh, sql, th, tl);
-            pacc_sub(bh[c], bl[c], th, tl);
-          }
-          // the low sums stay at an ulp of the high ones, so that adding to
-          // them rounds at 2^-49 of the sum
-          if (s == 1) pfast2(ah[v][c], al[v][c]);
-        }
-      }
-      if (!ONE)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          if (V == 2 || s == 1) pfast2(bh[c], bl[c]);
-          bh[c] = pshfl(bh[c], next);
-          bl[c] = pshfl(bl[c], next);
-        }
-    }
-  }
-  return ymax;
-}
 
 // The tile step of the literal mixed form, operation for operation that of the
 // FP64-difference kernel (sym_step_mixed and the diagonal loop of nb_sym.cu):
@@ -158,13 +85,11 @@ __device__ __forceinline__ float tri_tile_mixed(const TriIons<V> &p, const float
       float ra, rb;
       upk(r2, ra, rb);
       float ya = rsqrt_approx(ra), yb = rsqrt_approx(rb);
+      const bool me0 = ONE && r == lane && self == 2 * v, me1 = ONE && r == lane && self == 2 * v + 1;
+      ymax = fmaxf(ymax, fmaxf(me0 ? 0.0f : ya, me1 ? 0.0f : yb));
       if (ONE) {
-        ymax = fmaxf(ymax, r == lane && self == 2 * v ? 0.0f : ya);
-        ymax = fmaxf(ymax, r == lane && self == 2 * v + 1 ? 0.0f : yb);
         ya = fminf(ya, TRI_YMAX_GRID);
         yb = fminf(yb, TRI_YMAX_GRID);
-      } else {
-        ymax = fmaxf(ymax, fmaxf(ya, yb));
       }
       const f32x2 y = pk(ya, yb), y2 = pmul(y, y), y3 = pmul(y2, y);
       const f32x2 s = pfma(y3, pfma(pmul(m15, r2), y2, p15), y3);
@@ -187,8 +112,8 @@ __device__ __forceinline__ float tri_tile_mixed(const TriIons<V> &p, const float
 // below n.  `sc` takes a force from its own units to the accumulators'.
 template <bool ONE>
 __device__ __noinline__ void tri_tile_fp64(int64_t n, const double *x, const double *y, const double *z,
-                                           const double *q, int64_t i0, int ni, int64_t j0, double sc, double *accP,
-                                           int ldp, double *accQ, int ldq) {
+                                           const double *q, double soft2, int64_t i0, int ni, int64_t j0, double sc,
+                                           double *accP, int ldp, double *accQ, int ldq) {
   const int lane = threadIdx.x & 31;
   for (int u = 0; u < ni; u += 32) {
     const int64_t i = i0 + u + lane;
@@ -197,7 +122,7 @@ __device__ __noinline__ void tri_tile_fp64(int64_t n, const double *x, const dou
       const int64_t j = j0 + ((lane + r) & 31);
       if (i < n && j < n && i != j) {
         const double dx = x[i] - x[j], dy = y[i] - y[j], dz = z[i] - z[j];
-        const double s = rinv3_fp64(dx, dy, dz, 0.0);
+        const double s = rinv3_fp64(dx, dy, dz, soft2);
         const double sp = (q ? s * q[j] : s), sq = (q ? s * q[i] : s);
         a[0] = fma(dx, sp, a[0]);
         a[1] = fma(dy, sp, a[1]);
@@ -220,7 +145,7 @@ __device__ __noinline__ void tri_tile_fp64(int64_t n, const double *x, const dou
 // weights' in ew; false when the item is left to FP64.  Ends with a barrier.
 template <int NT, bool QARR>
 __device__ __forceinline__ bool tri_scale(int64_t p0, int np, int64_t q0, int nq, const double *x, const double *y,
-                                          const double *z, const double *q, int &em, int &ew) {
+                                          const double *z, const double *q, double soft2, int &em, int &ew) {
   __shared__ int red[3][NT / 32];
   int mx = 0, wx = 0, wn = 0x7fffffff;
   for (int i = threadIdx.x; i < np + nq; i += NT) {
@@ -254,36 +179,12 @@ __device__ __forceinline__ bool tri_scale(int64_t p0, int np, int64_t q0, int nq
   }
   em = mx >> 20;
   ew = 1023;
-  bool ok = em >= TRI_EMIN && em <= TRI_EMAX;
+  bool ok = tri_scale_ok(em, soft2);
   if (QARR) {
     ew = wx >> 20;
     ok = ok && ew >= 1023 - 400 && ew <= 1023 + 400 && ew - (wn >> 20) <= TRI_WSPREAD;
   }
   return ok;
-}
-
-// Words of ion g (or a padding ion on side `far`) with its weight.
-template <bool QARR>
-__device__ __forceinline__ void tri_ion(int64_t g, bool real, const double *x, const double *y, const double *z,
-                                        const double *q, int em, int ew, float far, float w0[4], float w1[4],
-                                        float w2[4]) {
-  w0[3] = w1[3] = w2[3] = 0.0f;
-  if (real) {
-    float t[3];
-    tri_words(x[g], em, t);
-    w0[0] = t[0]; w1[0] = t[1]; w2[0] = t[2];
-    tri_words(y[g], em, t);
-    w0[1] = t[0]; w1[1] = t[1]; w2[1] = t[2];
-    tri_words(z[g], em, t);
-    w0[2] = t[0]; w1[2] = t[1]; w2[2] = t[2];
-    if (QARR && q[g] != 0.0) split_f64_scaled(q[g], ew - 1023, w0[3], w1[3]);
-  } else {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      w0[c] = far;
-      w1[c] = w2[c] = 0.0f;
-    }
-  }
 }
 
 // The item's in-place output of the mixed form (sym_commit, nb_symsched.cuh,
@@ -356,10 +257,10 @@ __device__ __forceinline__ void tri_commit(const SymItem &it, int64_t n, int BI,
   }
 }
 
-template <bool MIX, int V, bool QARR, int NT, int NB, bool INPLACE>
+template <bool MIX, int V, bool QARR, int NT, int NB, bool INPLACE, bool SOFT>
 __global__ void __launch_bounds__(NT, NB)
     k_pair_sym_tri(int64_t n, int nbk, int G, int SB, const double *__restrict__ x, const double *__restrict__ y,
-                   const double *__restrict__ z, const double *__restrict__ q, double *__restrict__ out,
+                   const double *__restrict__ z, const double *__restrict__ q, double soft2, double *__restrict__ out,
                    int *__restrict__ sync, unsigned *err) {
   constexpr int NW = NT / 32, PI = 64 * V;  // warps; ions of a P-tile
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -373,7 +274,7 @@ __global__ void __launch_bounds__(NT, NB)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool diag = it.P == it.Q;
   int em, ew;
-  const bool fast = tri_scale<NT, QARR>(p0, np, q0, diag ? 0 : nq, x, y, z, q, em, ew);
+  const bool fast = tri_scale<NT, QARR>(p0, np, q0, diag ? 0 : nq, x, y, z, q, soft2, em, ew);
   // units: a coordinate is L X with L = 2^(em - 1022), a weight 2^(ew - 1023) w
   const int kl = fast ? em - 1022 : 0, kw = fast ? ew - 1023 : 0;
 
@@ -414,6 +315,13 @@ __global__ void __launch_bounds__(NT, NB)
   for (int i = tid; i < NW * 3 * PI; i += NT) accP[i] = 0.0;
   // FP32 rounding of d leaves the 2^-69 L cut far behind at any distance (MIX)
   const float ylim = __syncthreads_or(low) && !MIX ? TRI_YMAX : TRI_YMAX_GRID;
+  f32x2 s2h = 0, s2l = 0;
+  if (SOFT) {
+    float sh, sl;
+    split_f64_scaled(soft2, 2 * kl, sh, sl);
+    s2h = pk1(sh);
+    s2l = pk1(sl);
+  }
 
   double *aP = accP + warp * 3 * PI;
   const double back = pow2d(2 * kl - kw);  // own units -> the accumulators'
@@ -441,14 +349,20 @@ __global__ void __launch_bounds__(NT, NB)
         for (int v = 0; v < V; ++v) ts.ah[v][c] = ts.al[v][c] = zero;
       }
       const float4 *qt = qs + t * TRI_TILE4 + lane;
+      auto ld = [&](int r, float4 &q0, float4 &q1, float4 &q2) {
+        q0 = qt[r];
+        q1 = qt[64 + r];
+        q2 = qt[128 + r];
+      };
       float ymax;
       if (one) {
         const int u = t - pt * 2 * V;  // the lane's own ion in this Q-tile, if any
         const int self = u >= 0 && u < 2 * V ? u : -1;
         ymax = MIX ? tri_tile_mixed<V, QARR, true>(p, qt - lane, lane, self, ts)
-                   : tri_tile<V, QARR, true>(p, qt, lane, self, ts);
+                   : tri_tile<V, QARR, true, SOFT>(p, ld, lane, self, s2h, s2l, ts);
       } else {
-        ymax = MIX ? tri_tile_mixed<V, QARR, false>(p, qt, lane, -1, ts) : tri_tile<V, QARR, false>(p, qt, lane, -1, ts);
+        ymax = MIX ? tri_tile_mixed<V, QARR, false>(p, qt, lane, -1, ts)
+                   : tri_tile<V, QARR, false, SOFT>(p, ld, lane, -1, s2h, s2l, ts);
       }
       done = !__any_sync(0xffffffffu, !(ymax <= ylim));
       if (done) {
@@ -476,9 +390,9 @@ __global__ void __launch_bounds__(NT, NB)
     }
     if (!done) {
       if (one)
-        tri_tile_fp64<true>(n, x, y, z, q, p0 + pt * PI, PI, q0 + t * 32, back, aP, PI, aQ, BI);
+        tri_tile_fp64<true>(n, x, y, z, q, soft2, p0 + pt * PI, PI, q0 + t * 32, back, aP, PI, aQ, BI);
       else
-        tri_tile_fp64<false>(n, x, y, z, q, p0 + pt * PI, PI, q0 + t * 32, back, aP, PI, aQ, BI);
+        tri_tile_fp64<false>(n, x, y, z, q, soft2, p0 + pt * PI, PI, q0 + t * 32, back, aP, PI, aQ, BI);
     }
   }
   __syncthreads();
@@ -504,9 +418,9 @@ static size_t tri_smem(int G) {
          (size_t)(NT / 32) * 3 * 64 * V * sizeof(double);
 }
 
-template <bool MIX, int V, int NT, int NB>
+template <bool MIX, int V, int NT, int NB, bool SOFT = false>
 static cudaError_t launch_tri(int64_t n, int nbk, int G, int SB, const double *x, const double *y, const double *z,
-                              const double *q, double *part, int *sync, unsigned *err, bool inplace,
+                              const double *q, double soft2, double *part, int *sync, unsigned *err, bool inplace,
                               cudaStream_t st) {
   static std::mutex mu;
   static bool done[64] = {false};
@@ -517,10 +431,10 @@ static cudaError_t launch_tri(int64_t n, int nbk, int G, int SB, const double *x
     std::lock_guard<std::mutex> lk(mu);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!done[dev]) {
-      const void *fns[4] = {(const void *)k_pair_sym_tri<MIX, V, true, NT, NB, true>,
-                            (const void *)k_pair_sym_tri<MIX, V, false, NT, NB, true>,
-                            (const void *)k_pair_sym_tri<MIX, V, true, NT, NB, false>,
-                            (const void *)k_pair_sym_tri<MIX, V, false, NT, NB, false>};
+      const void *fns[4] = {(const void *)k_pair_sym_tri<MIX, V, true, NT, NB, true, SOFT>,
+                            (const void *)k_pair_sym_tri<MIX, V, false, NT, NB, true, SOFT>,
+                            (const void *)k_pair_sym_tri<MIX, V, true, NT, NB, false, SOFT>,
+                            (const void *)k_pair_sym_tri<MIX, V, false, NT, NB, false, SOFT>};
       for (int k = 0; k < 4 && e == cudaSuccess; ++k)
         e = cudaFuncSetAttribute(fns[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem<V, NT>(32));
       if (e != cudaSuccess) return e;
@@ -534,7 +448,7 @@ static cudaError_t launch_tri(int64_t n, int nbk, int G, int SB, const double *x
   const int items = nbk * (nbk + 1) / 2;
   const size_t smem = tri_smem<V, NT>(G);
 #define NB_TRI_LAUNCH(QA, IP) \
-  k_pair_sym_tri<MIX, V, QA, NT, NB, IP><<<items, NT, smem, st>>>(n, nbk, G, SB, x, y, z, q, part, sync, err)
+  k_pair_sym_tri<MIX, V, QA, NT, NB, IP, SOFT><<<items, NT, smem, st>>>(n, nbk, G, SB, x, y, z, q, soft2, part, sync, err)
   if (inplace) {
     if (q) NB_TRI_LAUNCH(true, true); else NB_TRI_LAUNCH(false, true);
   } else {
@@ -544,11 +458,11 @@ static cudaError_t launch_tri(int64_t n, int nbk, int G, int SB, const double *x
   return cudaGetLastError();
 }
 
-// Softened sums stay with nb_sym.cu, and so do 32-ion blocks (the mixed form
+// The softened mixed form stays with nb_sym.cu, and so do 32-ion blocks (mixed
 // below n = 2000, where 16-term FP32 sums are more accurate than 32-term ones at
 // the same speed; elsewhere by set_tuning only).
 static bool tri_sums(const Plan &pl, int mode, double soft2) {
-  return pl.sym && soft2 == 0.0 && (mode == MODE_FP64 || mode == MODE_DF64 || mode == MODE_MIXED);
+  return pl.sym && (mode == MODE_FP64 || mode == MODE_DF64 || (mode == MODE_MIXED && soft2 == 0.0));
 }
 bool tri_serves(const Plan &pl, int mode, double soft2) { return tri_sums(pl, mode, soft2) && pl.G >= 2; }
 
@@ -576,10 +490,12 @@ Plan make_force_plan(int64_t n, int mode, double soft2) {
 }
 
 cudaError_t launch_pair_tri(const Plan &pl, int mode, int64_t n, const double *x, const double *y, const double *z,
-                            const double *q, double *part, unsigned *err, cudaStream_t st) {
+                            const double *q, double soft2, double *part, unsigned *err, cudaStream_t st) {
   int *sync = part_sync(pl, part, n, 3);
   const bool inplace = pl.n_jc == 1;
-#define NB_TRI(MIX, V, NT, NB) launch_tri<MIX, V, NT, NB>(n, pl.nbk, pl.G, SB, x, y, z, q, part, sync, err, inplace, st)
+  // softened: 8 more lane-cycles per evaluation, kernels of their own so that the
+  // others' pair loop has no branch (2 % of it at n = 1e5)
+#define NB_TRI(...) launch_tri<__VA_ARGS__>(n, pl.nbk, pl.G, SB, x, y, z, q, soft2, part, sync, err, inplace, st)
   // The mixed form's FP32 sums keep the order they have with make_plan's
   // blocks: one-sided within 128 ions for n < 32768 (whose items of 256 ions
   // from n = 12161 on only change where FP64 sums are added), else within the
@@ -592,6 +508,14 @@ cudaError_t launch_pair_tri(const Plan &pl, int mode, int64_t n, const double *x
       case 8: return NB_TRI(true, 2, 128, 4);
       case 16: return NB_TRI(true, 2, 128, 3);
       case 32: return NB_TRI(true, 2, 256, 2);
+      default: return cudaErrorInvalidValue;
+    }
+  if (soft2 != 0.0) switch (pl.G) {
+      case 2: return NB_TRI(false, 1, 64, 10, true);
+      case 4:
+      case 8: return NB_TRI(false, 2, 128, 4, true);
+      case 16:
+      case 32: return NB_TRI(false, 2, 256, 2, true);
       default: return cudaErrorInvalidValue;
     }
   switch (pl.G) {

@@ -16,7 +16,7 @@
 //
 // A pair closer than 2^-20 L (where the 2^-69 L cut would pass 2^-49 of the
 // distance, and dl stops being small against dm) makes its tile fall back to
-// FP64 arithmetic; the test is the largest 1/r met, one FMNMX per pair.  When
+// FP64 arithmetic; the test is the smallest r^2 met, one FMNMX per pair.  When
 // no coordinate of the item has bits in l (positions on a grid), d is exact
 // and normal at any distance, and only FP32's range sets a limit, 2^-40 L.
 // Items whose scale or weights are far from the ordinary (below) take the
@@ -106,6 +106,11 @@ constexpr float TRI_YMAX = 0x1p20f, TRI_YMAX_GRID = 0x1p40f;
 // products with a force stay far inside FP64), and weights within 2^40 of the
 // item's largest (so that a double-float weight keeps its 48 bits).
 constexpr int TRI_EMIN = 1023 - 200, TRI_EMAX = 1023 + 200, TRI_WSPREAD = 40;
+// and a softening length up to 2^10 L (far above it the terms' low parts would
+// leave FP32's range).
+__device__ __forceinline__ bool tri_scale_ok(int em, double soft2) {
+  return em >= TRI_EMIN && em <= TRI_EMAX && ((__double2hiint(soft2) >> 20) & 0x7ff) - 2 * (em - 1022) <= 1023 + 20;
+}
 
 // d = p - q as a double-float: the word differences are exact; Fast2Sum holds
 // because dh is 0 or at least 2^-22 > |dm|.
@@ -208,12 +213,120 @@ __device__ __forceinline__ float rsqrt_approx(float v) {
 // 2^k as FP64 (|k| <= 1000).
 __device__ __forceinline__ double pow2d(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
+template <int V>
+struct TriIons {  // 2 V ions of a lane: words and, with weights, the weight's (hi, lo)
+  f32x2 h[V][3], m[V][3], l[V][3], wh[V], wl[V];
+};
+
+// The sums of a tile step: double-floats, or FP32 (MIX) in the high words.
+template <int V>
+struct TriSums {
+  f32x2 ah[V][3], al[V][3], bh[3], bl[3];
+};
+
+// One tile step: this lane's P-ions against the 32 Q-ions of a tile;
+// ld(r, q0, q1, q2) loads the three words (with the weight's parts in the w of
+// q0 and q1) of Q-ion (lane + r) mod 32.  Returns the largest 1/r met
+// (with a softening, of the distance without it).  self: the lane's P-ion (0 ..
+// 2 V - 1) that is Q-ion 0 of the rotation itself, or -1 (ONE only).  SOFT: the
+// softening soft2 L^-2 as the double-float (s2h, s2l).
+template <int V, bool W, bool ONE, bool SOFT, class LD>
+__device__ __forceinline__ float tri_tile(const TriIons<V> &p, LD ld, int lane, int self, f32x2 s2h, f32x2 s2l,
+                                          TriSums<V> &t) {
+  f32x2(&ah)[V][3] = t.ah, (&al)[V][3] = t.al, (&bh)[3] = t.bh, (&bl)[3] = t.bl;
+  float ymax = 0.0f, rmin = __int_as_float(0x7f800000);
+  const int next = (lane + 1) & 31;
+#pragma unroll 1
+  for (int r0 = 0; r0 < 32; r0 += 2) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      float4 q0, q1, q2;
+      ld(r0 + s, q0, q1, q2);
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        f32x2 dh[3], dl[3], h, l, sh, sl;
+        tri_diff(p.h[v][0], p.m[v][0], p.l[v][0], pk1(q0.x), pk1(q1.x), pk1(q2.x), dh[0], dl[0]);
+        tri_diff(p.h[v][1], p.m[v][1], p.l[v][1], pk1(q0.y), pk1(q1.y), pk1(q2.y), dh[1], dl[1]);
+        tri_diff(p.h[v][2], p.m[v][2], p.l[v][2], pk1(q0.z), pk1(q1.z), pk1(q2.z), dh[2], dl[2]);
+        tri_r2(dh, dl, h, l);
+        float ha, hb;
+        upk(h, ha, hb);
+        // the ion itself is left out: its d = 0 gives a zero term with any finite y
+        const bool me0 = ONE && s == 0 && r0 == 0 && self == 2 * v;
+        const bool me1 = ONE && s == 0 && r0 == 0 && self == 2 * v + 1;
+        if (SOFT) {
+          rmin = fminf(rmin, fminf(me0 ? rmin : ha, me1 ? rmin : hb));
+          f32x2 e;
+          ptwo_sum(h, s2h, h, e);
+          l = padd(l, padd(e, s2l));
+          upk(h, ha, hb);
+        }
+        float ya = rsqrt_approx(ha), yb = rsqrt_approx(hb);
+        if (!SOFT) ymax = fmaxf(ymax, fmaxf(me0 ? 0.0f : ya, me1 ? 0.0f : yb));
+        if (ONE) {
+          ya = fminf(ya, TRI_YMAX_GRID);
+          yb = fminf(yb, TRI_YMAX_GRID);
+        }
+        tri_rinv3(h, l, pk(ya, yb), sh, sl);
+        f32x2 sph = sh, spl = sl, sqh = sh, sql = sl;
+        if (W) ptwo_prod(sh, sl, pk1(q0.w), pk1(q1.w), sph, spl);
+        if (W && !ONE) ptwo_prod(sh, sl, p.wh[v], p.wl[v], sqh, sql);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          f32x2 th, tl;
+          ptwo_prod(dh[c], dl[c], sph, spl, th, tl);
+          pacc(ah[v][c], al[v][c], th, tl);
+          if (!ONE) {
+            if (W) ptwo_prod(dh[c], dl[c], sqh, sql, th, tl);
+            pacc_sub(bh[c], bl[c], th, tl);
+          }
+          // the low sums stay at an ulp of the high ones, so that adding to
+          // them rounds at 2^-49 of the sum
+          if (s == 1) pfast2(ah[v][c], al[v][c]);
+        }
+      }
+      if (!ONE)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          if (V == 2 || s == 1) pfast2(bh[c], bl[c]);
+          bh[c] = pshfl(bh[c], next);
+          bl[c] = pshfl(bl[c], next);
+        }
+    }
+  }
+  return SOFT ? rsqrt_approx(rmin) : ymax;
+}
+
+// Words of ion g (or a padding ion on side `far`) with its weight.
+template <bool QARR>
+__device__ __forceinline__ void tri_ion(int64_t g, bool real, const double *x, const double *y, const double *z,
+                                        const double *q, int em, int ew, float far, float w0[4], float w1[4],
+                                        float w2[4]) {
+  w0[3] = w1[3] = w2[3] = 0.0f;
+  if (real) {
+    float t[3];
+    tri_words(x[g], em, t);
+    w0[0] = t[0]; w1[0] = t[1]; w2[0] = t[2];
+    tri_words(y[g], em, t);
+    w0[1] = t[0]; w1[1] = t[1]; w2[1] = t[2];
+    tri_words(z[g], em, t);
+    w0[2] = t[0]; w1[2] = t[1]; w2[2] = t[2];
+    if (QARR && q[g] != 0.0) split_f64_scaled(q[g], ew - 1023, w0[3], w1[3]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      w0[c] = far;
+      w1[c] = w2[c] = 0.0f;
+    }
+  }
+}
+
 // The plan of a force evaluation: make_plan's, with this file's kernel's own
 // block sizes where it serves the call (nb_tri.cu).
 Plan make_force_plan(int64_t n, int mode, double soft2);
 // Whether the kernel serves a plan, and its launch.
 bool tri_serves(const Plan &pl, int mode, double soft2);
 cudaError_t launch_pair_tri(const Plan &pl, int mode, int64_t n, const double *x, const double *y, const double *z,
-                            const double *q, double *part, unsigned *err, cudaStream_t st);
+                            const double *q, double soft2, double *part, unsigned *err, cudaStream_t st);
 
 }  // namespace nb
