@@ -318,8 +318,9 @@ nb_status nb_plan_batched(int32_t n_inst, const int64_t *offsets, int32_t n_bins
                           double *mean_load);
 
 /* Host-only: the launch plan a call at n ions would use, for kind 0 (the
- * force kernel of nb_forces / nb_step in `precision`), 1 (the potential
- * kernel) or 2 (the VJP kernel, fp64 and df64 alike; for kinds 1 and 2
+ * force kernel of nb_forces / nb_step in `precision`; softened mixed sums take
+ * the block sizes of the other precisions' tables), 1 (the one-sided potential
+ * kernel, used below n = 2000 or with a kind-1 override) or 2 (the VJP kernel, fp64 and df64 alike; for kinds 1 and 2
  * `precision` is validated but does not change the plan), with the current tuning overrides:
  * out[0] threads per block (one-sided) or 256 / 128 (symmetric), out[1] ions
  * per thread R, out[2] partners per j-chunk, out[3] i-tiles (one-sided) or

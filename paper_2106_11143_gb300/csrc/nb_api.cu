@@ -214,12 +214,12 @@ StateView to_view(const nb_system *s) {
 namespace {
 
 // Scratch need of one force evaluation.
-size_t force_bytes(const Plan &pl, int mode, int64_t n, bool extra_pos, bool phi, const Plan &plp) {
+size_t force_bytes(const Plan &pl, int mode, int64_t n, bool extra_pos, const PhiPlan *phi) {
   Carver c;
   c.take<double>(part_doubles(pl, n, 3));
   if (split_like(mode)) c.take<float>(6 * (size_t)n);
   if (extra_pos) c.take<double>(3 * (size_t)n);
-  if (phi) c.take<double>((size_t)plp.n_jc * n);
+  if (phi) c.take<double>(phi->out_doubles(n));
   return c.off + 256;
 }
 
@@ -482,14 +482,14 @@ nb_status nb_forces(const nb_params *params, const nb_system *sys, double *phi, 
   cudaStream_t st = (cudaStream_t)stream;
   const int mode = params->precision;
   const Plan pl = make_force_plan(n, mode, params->soft2);
-  const Plan plp = make_plan(n, MODE_FP64, 1);
+  const PhiPlan plp = make_phi_plan(n);
   Arena *a = nullptr;
-  NB_TRY(get_arena(st, force_bytes(pl, mode, n, false, phi != nullptr, plp), &a));
+  NB_TRY(get_arena(st, force_bytes(pl, mode, n, false, phi ? &plp : nullptr), &a));
   Carver cv;
   cv.base = a->buf;
   double *part = cv.take<double>(part_doubles(pl, n, 3));
   float *split = split_like(mode) ? cv.take<float>(6 * (size_t)n) : nullptr;
-  double *ppart = phi ? cv.take<double>((size_t)plp.n_jc * n) : nullptr;
+  double *ppart = phi ? cv.take<double>(plp.out_doubles(n)) : nullptr;
   const Phys p = to_phys(params);
   const StateView v = to_view(sys);
   const double t = params->t0 + (double)sys->step * params->dt;
@@ -497,9 +497,9 @@ nb_status nb_forces(const nb_params *params, const nb_system *sys, double *phi, 
   NB_CUDA_TRY(launch_epi_forces(p, v, part, pl.n_jc, flags, t, a->err, st));
   count_launches(1);
   if (phi) {
-    NB_CUDA_TRY(launch_pair_phi(plp, n, sys->x, sys->y, sys->z, sys->q, params->charge, params->soft2, ppart, st));
+    NB_CUDA_TRY(launch_phi(plp, n, sys->x, sys->y, sys->z, sys->q, params->charge, params->soft2, ppart, a->err, st));
     // the pair sums carry w_j = q_j, or 1 for a single species
-    NB_CUDA_TRY(launch_chunk_sum1(n, ppart, plp.n_jc, sys->q ? 1.0 : params->charge, phi, st));
+    NB_CUDA_TRY(launch_chunk_sum1(n, ppart, plp.n_slots, sys->q ? 1.0 : params->charge, phi, st));
     count_launches(2);
   }
   return NB_OK;
@@ -534,7 +534,7 @@ nb_status nb_step(const nb_params *params, nb_system *sys, int64_t nsteps, void 
     sys->step += nsteps;
     return NB_OK;
   }
-  NB_TRY(get_arena(st, force_bytes(pl, mode, n, true, false, pl), &a));
+  NB_TRY(get_arena(st, force_bytes(pl, mode, n, true, nullptr), &a));
   Carver cv;
   cv.base = a->buf;
   double *part = cv.take<double>(part_doubles(pl, n, 3));
@@ -594,23 +594,23 @@ nb_status nb_energy(const nb_params *params, const nb_system *sys, double out[4]
     return NB_OK;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  const Plan pl = make_plan(n, MODE_FP64, 1);
+  const PhiPlan pl = make_phi_plan(n);
   Carver need;
-  need.take<double>((size_t)pl.n_jc * n);
+  need.take<double>(pl.out_doubles(n));
   need.take<double>(3 * ENERGY_BLOCKS);
   need.take<double>(4);
   Arena *a = nullptr;
   NB_TRY(get_arena(st, need.off + 256, &a));
   Carver cv;
   cv.base = a->buf;
-  double *ppart = cv.take<double>((size_t)pl.n_jc * n);
+  double *ppart = cv.take<double>(pl.out_doubles(n));
   double *bpart = cv.take<double>(3 * ENERGY_BLOCKS);
   double *out4 = cv.take<double>(4);
   const Phys p = to_phys(params);
   const StateView v = to_view(sys);
   const double t = params->t0 + (double)sys->step * params->dt;
-  NB_CUDA_TRY(launch_pair_phi(pl, n, sys->x, sys->y, sys->z, sys->q, params->charge, params->soft2, ppart, st));
-  NB_CUDA_TRY(launch_energy(p, v, ppart, pl.n_jc, t, bpart, out4, st));
+  NB_CUDA_TRY(launch_phi(pl, n, sys->x, sys->y, sys->z, sys->q, params->charge, params->soft2, ppart, a->err, st));
+  NB_CUDA_TRY(launch_energy(p, v, ppart, pl.n_slots, t, bpart, out4, st));
   count_launches(3);
   NB_CUDA_TRY(cudaMemcpyAsync(out, out4, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
   NB_CUDA_TRY(cudaStreamSynchronize(st));
@@ -1009,20 +1009,20 @@ extern "C" nb_status nb_traj_forward(const nb_params *params, nb_system *sys, in
     const int64_t len = std::min(every, nsteps - seg * every);
     if (len > 0) NB_TRY(nb_step(params, sys, len, stream));
   }
-  const Plan plp = make_plan(n, MODE_FP64, 1);
+  const PhiPlan plp = make_phi_plan(n);
   Carver need;
-  need.take<double>((size_t)plp.n_jc * n);
+  need.take<double>(plp.out_doubles(n));
   need.take<double>(ADJ_PART_BLOCKS);
   Arena *a = nullptr;
   NB_TRY(get_arena(st, need.off + 256, &a));
   Carver cv;
   cv.base = a->buf;
-  double *ppart = cv.take<double>((size_t)plp.n_jc * n);
+  double *ppart = cv.take<double>(plp.out_doubles(n));
   double *bpart = cv.take<double>(ADJ_PART_BLOCKS);
   const double *xT[3] = {sys->x, sys->y, sys->z};
   const double *tg[3] = {target, target + n, target + 2 * n};
-  NB_CUDA_TRY(launch_pair_phi(plp, n, sys->x, sys->y, sys->z, sys->q, params->charge, params->soft2, ppart, st));
-  NB_CUDA_TRY(launch_loss(to_phys(params), n, sys->q, xT, tg, ppart, plp.n_jc, bpart, loss, st));
+  NB_CUDA_TRY(launch_phi(plp, n, sys->x, sys->y, sys->z, sys->q, params->charge, params->soft2, ppart, a->err, st));
+  NB_CUDA_TRY(launch_loss(to_phys(params), n, sys->q, xT, tg, ppart, plp.n_slots, bpart, loss, st));
   count_launches(3);
   return NB_OK;
 }

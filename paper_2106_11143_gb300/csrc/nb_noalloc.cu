@@ -19,18 +19,19 @@
 // ordering) race on it and give wrong results; serialise them.  Each call
 // overwrites every scratch word it reads before reading it, so nothing has
 // to start at zero and the contents left by the previous call do not matter.
+#include <cstring>
 #include <mutex>
 
-#include "nb_common.cuh"
+#include "nb_tri.cuh"
 
 namespace nb {
 
 // Scratch capacity: 8 MiB of doubles.  It bounds n through the launch plan of
-// the potential kernel: n_jc * n + 3 * ENERGY_BLOCKS + 4 doubles must fit.
-// With the default plan on a 152-SM GB300 that holds for every n up to about
-// 1,000,000 (n_jc * n is about the SM count times the plan's blocks per SM
-// times its block size); a potential-kernel tuning override (nb_set_tuning
-// kind 1) or a GPU with more SMs can lower the limit.
+// the potential kernel: its output (n_slots * n doubles and, from n = 1500, the
+// half-pair schedule's counters) + 3 * ENERGY_BLOCKS + 5 doubles must fit.
+// With the default plan that holds for every n up to about 1,040,000
+// (make_phi_plan keeps its partials below 1,000,000 doubles and needs n above);
+// a potential-kernel tuning override (nb_set_tuning kind 1) can lower the limit.
 constexpr size_t NOALLOC_SCRATCH_DOUBLES = (size_t)1 << 20;
 static __device__ __align__(256) double g_noalloc_scratch[NOALLOC_SCRATCH_DOUBLES];
 
@@ -76,8 +77,8 @@ extern "C" nb_status nb_energy_noalloc(const nb_params *params, const nb_system 
     out[0] = out[1] = out[2] = out[3] = 0.0;
     return NB_OK;
   }
-  const Plan pl = make_plan(n, MODE_FP64, 1);
-  const size_t need = (size_t)pl.n_jc * (size_t)n + 3 * ENERGY_BLOCKS + 4;
+  const PhiPlan pl = make_phi_plan(n);
+  const size_t need = pl.out_doubles(n) + 3 * ENERGY_BLOCKS + 5;
   if (need > NOALLOC_SCRATCH_DOUBLES)
     return fail(NB_EINVAL,
                 "nb_energy_noalloc: n = %lld needs %zu scratch doubles, above its fixed %zu "
@@ -89,20 +90,28 @@ extern "C" nb_status nb_energy_noalloc(const nb_params *params, const nb_system 
     return fail(NB_ECUDA, "nb_energy_noalloc: cudaGetSymbolAddress of the scratch array failed: %s",
                 cudaGetErrorString(e));
   double *ppart = scratch;
-  double *bpart = ppart + (size_t)pl.n_jc * (size_t)n;
-  double *out4 = bpart + 3 * ENERGY_BLOCKS;
+  double *bpart = ppart + pl.out_doubles(n);
+  double *out4 = bpart + 3 * ENERGY_BLOCKS;  // and a device error word in its fifth double
+  unsigned *err = reinterpret_cast<unsigned *>(out4 + 4);
   const Phys p = to_phys(params);
   const StateView v = to_view(sys);
   const double t = params->t0 + (double)sys->step * params->dt;
   cudaStream_t st = (cudaStream_t)stream;
-  e = launch_pair_phi(pl, n, sys->x, sys->y, sys->z, sys->q, params->charge, params->soft2, ppart, st);
-  if (e == cudaSuccess) e = launch_energy(p, v, ppart, pl.n_jc, t, bpart, out4, st);
+  double h[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  e = cudaMemsetAsync(err, 0, sizeof(double), st);
+  if (e == cudaSuccess)
+    e = launch_phi(pl, n, sys->x, sys->y, sys->z, sys->q, params->charge, params->soft2, ppart, err, st);
+  if (e == cudaSuccess) e = launch_energy(p, v, ppart, pl.n_slots, t, bpart, out4, st);
   if (e == cudaSuccess) {
     count_launches(3);
-    e = cudaMemcpyAsync(out, out4, 4 * sizeof(double), cudaMemcpyDeviceToHost, st);
+    e = cudaMemcpyAsync(h, out4, sizeof(h), cudaMemcpyDeviceToHost, st);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess)
     return fail(NB_ECUDA, "nb_energy_noalloc: %s", cudaGetErrorString(e));
+  unsigned word;
+  std::memcpy(&word, &h[4], sizeof(word));
+  if (word & ERR_TIMEOUT) return fail(NB_ETIMEOUT, "nb_energy_noalloc: a bounded device wait gave up");
+  for (int k = 0; k < 4; ++k) out[k] = h[k];
   return NB_OK;
 }

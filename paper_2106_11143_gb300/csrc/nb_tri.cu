@@ -52,10 +52,6 @@
 
 namespace nb {
 
-// A staged tile: word k of entry e (64 entries, the tile twice) at
-// [k * 64 + e], the weight's high and low parts in the w of words 0 and 1.
-constexpr int TRI_TILE4 = 3 * 64;
-
 // The tile step of the literal mixed form, operation for operation that of the
 // FP64-difference kernel (sym_step_mixed and the diagonal loop of nb_sym.cu):
 // the displacement rounded once to FP32 (h + l is exact, so RN(h + l) is), the
@@ -139,52 +135,6 @@ __device__ __noinline__ void tri_tile_fp64(int64_t n, const double *x, const dou
       if (!ONE) accQ[c * ldq + lane] += b[c] * sc;
     }
   }
-}
-
-// The item's scale: the largest biased exponent of a coordinate in em, the
-// weights' in ew; false when the item is left to FP64.  Ends with a barrier.
-template <int NT, bool QARR>
-__device__ __forceinline__ bool tri_scale(int64_t p0, int np, int64_t q0, int nq, const double *x, const double *y,
-                                          const double *z, const double *q, double soft2, int &em, int &ew) {
-  __shared__ int red[3][NT / 32];
-  int mx = 0, wx = 0, wn = 0x7fffffff;
-  for (int i = threadIdx.x; i < np + nq; i += NT) {
-    const int64_t g = i < np ? p0 + i : q0 + (i - np);
-    mx = max(mx, __double2hiint(x[g]) & 0x7fffffff);
-    mx = max(mx, __double2hiint(y[g]) & 0x7fffffff);
-    mx = max(mx, __double2hiint(z[g]) & 0x7fffffff);
-    if (QARR) {
-      const int w = __double2hiint(q[g]) & 0x7fffffff;
-      wx = max(wx, w);
-      if (q[g] != 0.0) wn = min(wn, w);
-    }
-  }
-  mx = __reduce_max_sync(0xffffffffu, mx);
-  if (QARR) {
-    wx = __reduce_max_sync(0xffffffffu, wx);
-    wn = __reduce_min_sync(0xffffffffu, wn);
-  }
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    red[0][w] = mx;
-    red[1][w] = wx;
-    red[2][w] = wn;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < NT / 32; ++k) {
-    mx = max(mx, red[0][k]);
-    wx = max(wx, red[1][k]);
-    wn = min(wn, red[2][k]);
-  }
-  em = mx >> 20;
-  ew = 1023;
-  bool ok = tri_scale_ok(em, soft2);
-  if (QARR) {
-    ew = wx >> 20;
-    ok = ok && ew >= 1023 - 400 && ew <= 1023 + 400 && ew - (wn >> 20) <= TRI_WSPREAD;
-  }
-  return ok;
 }
 
 // The item's in-place output of the mixed form (sym_commit, nb_symsched.cuh,
@@ -282,35 +232,7 @@ __global__ void __launch_bounds__(NT, NB)
   const int pt = warp % PT, grp = warp / PT;
   TriIons<V> p;
   int low = 0;  // an l word is set
-  if (fast) {
-    for (int i = tid; i < BI; i += NT) {
-      float w0[4], w1[4], w2[4];
-      tri_ion<QARR>(q0 + i, i < nq, x, y, z, q, em, ew, -TRI_FAR, w0, w1, w2);
-      float4 *e = qs + (i >> 5) * TRI_TILE4 + (i & 31);
-      e[0] = e[32] = make_float4(w0[0], w0[1], w0[2], w0[3]);
-      e[64] = e[96] = make_float4(w1[0], w1[1], w1[2], w1[3]);
-      e[128] = e[160] = make_float4(w2[0], w2[1], w2[2], w2[3]);
-      low |= w2[0] != 0.0f || w2[1] != 0.0f || w2[2] != 0.0f;
-    }
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      float w0[2][4], w1[2][4], w2[2][4];
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const int i = pt * PI + v * 64 + b * 32 + lane;
-        tri_ion<QARR>(p0 + i, i < np, x, y, z, q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
-        low |= w2[b][0] != 0.0f || w2[b][1] != 0.0f || w2[b][2] != 0.0f;
-      }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        p.h[v][c] = pk(w0[0][c], w0[1][c]);
-        p.m[v][c] = pk(w1[0][c], w1[1][c]);
-        p.l[v][c] = pk(w2[0][c], w2[1][c]);
-      }
-      p.wh[v] = pk(w0[0][3], w0[1][3]);
-      p.wl[v] = pk(w1[0][3], w1[1][3]);
-    }
-  }
+  if (fast) low = tri_load<V, QARR, NT>(p, qs, BI, pt, p0, np, q0, nq, x, y, z, q, em, ew);
   for (int i = tid; i < 3 * BI; i += NT) accQ[i] = 0.0;
   for (int i = tid; i < NW * 3 * PI; i += NT) accP[i] = 0.0;
   // FP32 rounding of d leaves the 2^-69 L cut far behind at any distance (MIX)

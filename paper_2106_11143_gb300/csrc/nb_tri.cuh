@@ -94,6 +94,14 @@ __device__ __forceinline__ void tri_words(double x, int em, float w[3]) {
   w[2] = (float)(int)(((w1 & 0x7ffffu) << 5) | (w2 >> 27)) * (sg * 0x1p-69f);
 }
 
+// Whether the words of x hold it exactly: none of its bits lies below 2^-69.
+__device__ __forceinline__ bool tri_exact(double x, int em) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int s = em - (int)((hi >> 20) & 0x7ffu);
+  const int tz = lo ? __ffs((int)lo) - 1 : 31 + __ffs((int)((hi & 0xfffffu) | 0x100000u));
+  return s <= 16 || ((hi << 1) | lo) == 0 || tz >= s - 16;
+}
+
 // A padding ion's coordinate, in units of L: far enough that every term with
 // it underflows to zero (y^3 < 2^-149), near enough that r^2 stays finite.  The
 // two sides use opposite signs, so two padding ions never coincide.
@@ -321,6 +329,94 @@ __device__ __forceinline__ void tri_ion(int64_t g, bool real, const double *x, c
   }
 }
 
+// A staged tile: word k of entry e (64 entries, the tile twice) at
+// [k * 64 + e], the weight's high and low parts in the w of words 0 and 1.
+constexpr int TRI_TILE4 = 3 * 64;
+
+// The item's scale: the largest biased exponent of a coordinate in em, the
+// weights' in ew; false when the item is left to FP64.  Ends with a barrier.
+template <int NT, bool QARR>
+__device__ __forceinline__ bool tri_scale(int64_t p0, int np, int64_t q0, int nq, const double *x, const double *y,
+                                          const double *z, const double *q, double soft2, int &em, int &ew) {
+  __shared__ int red[3][NT / 32];
+  int mx = 0, wx = 0, wn = 0x7fffffff;
+  for (int i = threadIdx.x; i < np + nq; i += NT) {
+    const int64_t g = i < np ? p0 + i : q0 + (i - np);
+    mx = max(mx, __double2hiint(x[g]) & 0x7fffffff);
+    mx = max(mx, __double2hiint(y[g]) & 0x7fffffff);
+    mx = max(mx, __double2hiint(z[g]) & 0x7fffffff);
+    if (QARR) {
+      const int w = __double2hiint(q[g]) & 0x7fffffff;
+      wx = max(wx, w);
+      if (q[g] != 0.0) wn = min(wn, w);
+    }
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (QARR) {
+    wx = __reduce_max_sync(0xffffffffu, wx);
+    wn = __reduce_min_sync(0xffffffffu, wn);
+  }
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    red[0][w] = mx;
+    red[1][w] = wx;
+    red[2][w] = wn;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NT / 32; ++k) {
+    mx = max(mx, red[0][k]);
+    wx = max(wx, red[1][k]);
+    wn = min(wn, red[2][k]);
+  }
+  em = mx >> 20;
+  ew = 1023;
+  bool ok = tri_scale_ok(em, soft2);
+  if (QARR) {
+    ew = wx >> 20;
+    ok = ok && ew >= 1023 - 400 && ew <= 1023 + 400 && ew - (wn >> 20) <= TRI_WSPREAD;
+  }
+  return ok;
+}
+
+// Cuts the Q block's ions into words in shared memory (BI entries) and loads the
+// lane's ions of P-tile pt; returns whether any l word is set.
+template <int V, bool QARR, int NT>
+__device__ __forceinline__ int tri_load(TriIons<V> &p, float4 *qs, int BI, int pt, int64_t p0, int np, int64_t q0,
+                                        int nq, const double *x, const double *y, const double *z, const double *q,
+                                        int em, int ew) {
+  const int lane = threadIdx.x & 31;
+  int low = 0;
+  for (int i = threadIdx.x; i < BI; i += NT) {
+    float w0[4], w1[4], w2[4];
+    tri_ion<QARR>(q0 + i, i < nq, x, y, z, q, em, ew, -TRI_FAR, w0, w1, w2);
+    float4 *e = qs + (i >> 5) * TRI_TILE4 + (i & 31);
+    e[0] = e[32] = make_float4(w0[0], w0[1], w0[2], w0[3]);
+    e[64] = e[96] = make_float4(w1[0], w1[1], w1[2], w1[3]);
+    e[128] = e[160] = make_float4(w2[0], w2[1], w2[2], w2[3]);
+    low |= w2[0] != 0.0f || w2[1] != 0.0f || w2[2] != 0.0f;
+  }
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    float w0[2][4], w1[2][4], w2[2][4];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int i = pt * 64 * V + v * 64 + b * 32 + lane;
+      tri_ion<QARR>(p0 + i, i < np, x, y, z, q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
+      low |= w2[b][0] != 0.0f || w2[b][1] != 0.0f || w2[b][2] != 0.0f;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      p.h[v][c] = pk(w0[0][c], w0[1][c]);
+      p.m[v][c] = pk(w1[0][c], w1[1][c]);
+      p.l[v][c] = pk(w2[0][c], w2[1][c]);
+    }
+    p.wh[v] = pk(w0[0][3], w0[1][3]);
+    p.wl[v] = pk(w1[0][3], w1[1][3]);
+  }
+  return low;
+}
+
 // The plan of a force evaluation: make_plan's, with this file's kernel's own
 // block sizes where it serves the call (nb_tri.cu).
 Plan make_force_plan(int64_t n, int mode, double soft2);
@@ -328,5 +424,21 @@ Plan make_force_plan(int64_t n, int mode, double soft2);
 bool tri_serves(const Plan &pl, int mode, double soft2);
 cudaError_t launch_pair_tri(const Plan &pl, int mode, int64_t n, const double *x, const double *y, const double *z,
                             const double *q, double soft2, double *part, unsigned *err, cudaStream_t st);
+
+
+// The potential by the same arithmetic (nb_phi.cu): blocks of 32 G ions, the
+// block count and the output mode of a call at n ions (G = 0: the one-sided
+// kernel of make_plan(n, mode, 1)); out[jc * n + i], out_doubles in all.
+struct PhiPlan {
+  int G = 0, nbk = 0;
+  Plan one;  // the one-sided plan
+  int n_slots = 0;  // partial slots of the output
+  size_t out_doubles(int64_t n) const {
+    return (size_t)n_slots * (size_t)n + (G ? (size_t)(nbk + 2) / 2 : 0);  // and the schedule's counters
+  }
+};
+PhiPlan make_phi_plan(int64_t n);
+cudaError_t launch_phi(const PhiPlan &pl, int64_t n, const double *x, const double *y, const double *z,
+                       const double *q, double charge, double soft2, double *part, unsigned *err, cudaStream_t st);
 
 }  // namespace nb

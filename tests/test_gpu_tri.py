@@ -146,6 +146,87 @@ def test_softened_sums(nb, orc, n, soft, charges):
 
 
 # ---------------------------------------------------------------------------
+# The potential (csrc/nb_phi.cu) and the Jacobian product (csrc/nb_vjp.cu).
+
+
+@pytest.mark.parametrize("case", ["plain", "charges", "soft", "close", "tiny-weights"])
+@pytest.mark.parametrize("n", [1999, 2000, 2049, 9999, 10001, 16385, 31489])
+def test_potential(nb, orc, n, case):
+    """phi_i = sum_j q_j / s_ij at the edges of blocks, of the block sizes and of
+    the output mode (in place from 1e6 partials), against the oracle: relative to
+    sum_j |q_j| / s_ij within 1e-13 (FP64 rounding of n terms is 2^-52 sqrt(n),
+    1/r itself 2^-46)."""
+    pos, _ = W.random_cloud(n, seed=n + 5)
+    rng = np.random.default_rng(n)
+    q, soft2 = None, 0.0
+    if case == "charges":
+        q = W.E_CHARGE * rng.choice([-1.0, 1.0, 2.0, 0.0], size=n)
+    elif case == "tiny-weights":
+        q = W.E_CHARGE * 10.0 ** rng.uniform(-30, 30, size=n)
+    elif case == "soft":
+        soft2 = (1e-6) ** 2
+    elif case == "close":
+        pos[:, 40] = pos[:, 41] + np.array([1e-11, 0.0, 0.0])
+        pos[:, n - 1] = pos[:, 3] + np.array([0.0, 3e-12, 0.0])
+    phys = W.phys(soft2=soft2)
+    phi = nb.forces(nb.Params.from_phys(phys), nb.System(pos, q=q), want_phi=True).cpu().numpy()
+    nb.sync_status()
+    p = orc.make_params(**phys)
+    idx = np.unique(np.concatenate([np.arange(48), np.arange(n - 16, n), rng.integers(0, n, 64)]))
+    qq = np.full(n, W.E_CHARGE) if q is None else q
+    for i in idx:
+        ref = orc.coulomb(p, *pos, q=q, i0=int(i), i1=int(i) + 1, want_phi=True)[3][0]
+        mag = np.abs(qq) @ np.where(np.arange(n) == i, 0.0, 1.0 / np.sqrt(
+            np.maximum(np.sum((pos - pos[:, [i]]) ** 2, axis=0) + soft2, 1e-300)))
+        assert abs(phi[i] - ref) <= 1e-13 * mag, (n, case, i)
+
+
+def vjp_bound(pos, lam, q, i):
+    d = pos[:, [i]] - pos
+    r = np.sqrt(np.sum(d * d, axis=0))
+    dl = np.sqrt(np.sum((lam[:, [i]] - lam) ** 2, axis=0))
+    with np.errstate(divide="ignore", invalid="ignore"):
+        return np.sum(np.where(r > 0, 4.0 * np.abs(q) * dl / r ** 3, 0.0))
+
+
+@pytest.mark.parametrize("case", ["plain", "charges", "soft", "zero", "uniform", "local", "decades", "close"])
+@pytest.mark.parametrize("n", [2500, 2561, 4100, 16385])
+def test_jacobian_product(nb, orc, n, case):
+    """Edges of blocks and the two block sizes; cotangents that vanish, that are
+    one constant plus a part 2^-30 of it, that decay over six decades across the
+    cloud and that spread over twelve decades; close pairs.  Gate per ion: 1e-12
+    of a bound on the sum of its term magnitudes (|T| <= 4 |dl| r^-3)."""
+    pos, _ = W.random_cloud(n, seed=n + 9)
+    rng = np.random.default_rng(n)
+    lam = rng.standard_normal((3, n))
+    q, soft2 = None, 0.0
+    if case == "charges":
+        q = W.E_CHARGE * rng.choice([-1.0, 1.0, 2.0], size=n)
+    elif case == "soft":
+        soft2 = (2e-6) ** 2
+    elif case == "zero":
+        lam[:] = 0.0
+    elif case == "uniform":
+        lam = np.array([[1.0], [-2.0], [0.0]]) + 2.0 ** -30 * lam
+    elif case == "local":
+        lam *= np.exp(-14.0 * np.abs(pos[2]) / np.max(np.abs(pos[2])))
+    elif case == "decades":
+        lam *= 10.0 ** rng.uniform(-6, 6, size=n)
+    elif case == "close":
+        pos[:, 40] = pos[:, 41] + np.array([1e-11, 0.0, 0.0])
+        pos[:, n - 1] = pos[:, 3] + np.array([0.0, 3e-10, 0.0])
+    phys = W.phys(soft2=soft2)
+    g = nb.forces_vjp(nb.Params.from_phys(phys), nb.System(pos, q=q), lam).cpu().numpy()
+    nb.sync_status()
+    ref = np.stack(orc.forces_vjp(orc.make_params(**phys), 0.0, *pos, *lam, q=q))
+    qq = np.full(n, W.E_CHARGE) if q is None else q
+    idx = np.unique(np.concatenate([np.arange(48), np.arange(n - 16, n), rng.integers(0, n, 100)]))
+    for i in idx:
+        bound = W.K_COULOMB * abs(qq[i]) / W.MASS_40U * vjp_bound(pos, lam, qq, i)
+        assert np.linalg.norm(g[:, i] - ref[:, i]) <= 1e-12 * bound, (n, case, i)
+
+
+# ---------------------------------------------------------------------------
 # The ensemble kernel's force phase (csrc/nb_batched.cu).
 
 
