@@ -14,25 +14,29 @@
 //
 // Half-pair kernel (k_vjp_sym): T changes sign under i <-> j (both d and dl
 // do), so one evaluation serves both ions: g_i += w_j T and g_j -= w_i T.  The
-// work is organised as in the force kernel (nb_sym.cu): block pairs (P, Q),
+// work is organised as in the force kernel (nb_tri.cu): block pairs (P, Q),
 // P <= Q, of BI = 32 G ions, drawn from the round-robin schedule of
-// nb_symsched.cuh; each warp takes Q-tiles and visits the P-tiles in the
-// staggered order pt = (qs + k) mod G, one per barrier-separated step, so the
-// warps hold distinct P-tiles and update their shared-memory accumulators
-// without atomics.  A lane holds one P-ion (position, weight and lam in
-// registers); the Q-tile (64 B per ion) sits twice in shared memory, so the
-// entry (lane + r) mod 32 of rotation r is a fixed offset from the lane's
-// base; only the Q side's block-floating sums (six floats and their unit)
-// rotate, by warp shuffle.  Diagonal items (P == Q) are one-sided.  Output:
-// each item adds its sums into acc[c * n + i] in round order
-// (nb_symsched.cuh): bitwise reproducible with no partial buffer.
+// nb_symsched.cuh; a warp owns a P-tile of 64 ions, one packed pair per lane,
+// and visits the Q-tiles; positions and cotangents are three FP32 words each on
+// the item's two grids (nb_tri.cuh), so d and dl are exact differences on the
+// FP32 pipe, and T and the tile sums are double-floats in packed .f32x2
+// instructions, added to FP64 sums after each tile.  A tile with a pair too close
+// for the words, or an item of unusual scales, takes the pair's-own-units form of
+// the one-sided kernel (vjp_tile_units).
 //
-// Four warps per block and 128-ion blocks at n < 16384 give enough items to
-// fill the GPU at the adjoint's sizes (528 items at n = 4096).
+// What bounds it: the FMA pipe, 225 lane-cycles per evaluation (21 for d, 30 for
+// the normalised dl, 18 for r^2, 16 for r^-3 and r^-2, 28 for d . dl, 7 for its
+// product with 3 r^-2, 48 for T, 48 for the sums, 9 to keep them normalised), 80 %
+// busy at n = 32768 with issue at 52 %.  The kernel it replaces formed d and dl
+// with six FP64 subtractions per evaluation and scaled every pair's term to
+// block-floating sums: 2.83 -> 1.55 ms at n = 20000, 16.6 -> 9.0 ms at 50000, 164
+// -> 106 us at 4096 (per nb_forces_vjp call); conditioned error rms 2^-48.5
+// against 2^-47.4.
 #include <mutex>
 
-#include "nb_vjpterm.cuh"
 #include "nb_symsched.cuh"
+#include "nb_tri.cuh"
+#include "nb_vjpterm.cuh"
 
 namespace nb {
 
@@ -169,128 +173,384 @@ __global__ void __launch_bounds__(256) k_pair_vjp(int64_t n, int64_t jchunk, con
 // ---------------------------------------------------------------------------
 // Half-pair kernel.
 
-// Where an item keeps its finished Q sums (and a diagonal item its block's
-// sums): at the start of the Q-tile's own 4 KB of staged entries (64 of 64 B
-// in the doubled layout), read only by the warp that owns the tile.  Sum c
-// of ion i of the block: double [i / 32][c][i mod 32] with a 512-double
-// stride per tile.
-__device__ __forceinline__ double &vqsum(VD8 *posQ, int c, int i) {
-  return reinterpret_cast<double *>(posQ)[(i >> 5) * 512 + c * 32 + (i & 31)];
+// A staged Q-ion: words 0-2 of the position (with the weight's high and low
+// parts in the w of 0 and 1), then of the cotangent; word k of ion e at
+// [k * 32 + e].  Stored once: twice (a fixed offset per rotation) would leave
+// room for three blocks per SM instead of four.
+constexpr int VJP_TILE4 = 6 * 32;
+
+struct VjpIons {  // the lane's two P-ions
+  TriIons<1> r, lam;
+};
+
+// r^-3 as the double-float (sh, sl) and r^-2 as (w, wl) from r^2 = h + l and the
+// seed y: with the residual rho = 1 - (h + l) y^2, r^-3 = y^3 (1 + 3/2 rho + 15/8
+// rho^2) and r^-2 = y^2 (1 + rho + rho^2).
+__device__ __forceinline__ void vjp_rinv(f32x2 h, f32x2 l, f32x2 y, f32x2 &sh, f32x2 &sl, f32x2 &w, f32x2 &wl) {
+  w = pmul(y, y);
+  const f32x2 nw = pneg(w);
+  const f32x2 e = pfma(y, y, nw);
+  const f32x2 rho = psub(pfma(h, nw, pk1(1.0f)), pfma(l, w, pmul(h, e)));
+  wl = pfma(w, pfma(rho, rho, rho), e);
+  const f32x2 t = pfma(pmul(rho, pk1(1.25f)), rho, rho);
+  sh = pmul(w, y);
+  const f32x2 low = pfma(e, y, pfma(w, y, pneg(sh)));
+  sl = pfma(sh, t, pfma(pmul(sh, pk1(0.5f)), t, low));
+  pfast2(sh, sl);
 }
 
-// 32 rotations of a Q-tile against the lane's P-ion: the P side's sums in
-// (ah, al, ea), the Q side's rotating with their ions.
-template <bool W>
-__device__ __forceinline__ void vjp_tile_pair(const VD8 &pp, const VD8 *qd, int lane, double soft2, double a[3],
-                                              double b[3]) {
-  float ah[3] = {0.0f, 0.0f, 0.0f}, al[3] = {0.0f, 0.0f, 0.0f};
-  float bh[3] = {0.0f, 0.0f, 0.0f}, bl[3] = {0.0f, 0.0f, 0.0f};
-  int ea = VJP_BF_EMPTY, eb = VJP_BF_EMPTY;
-#pragma unroll 2
-  for (int r = 0; r < 32; ++r) {
-    vjp_eval<W, true>(pp, qd[r], soft2, ah, al, ea, bh, bl, eb);
+// One tile step (tri_tile's conventions; qt: the tile): a += w_q T per P-ion, b
+// -= w_p T per Q-ion, T = r^-3 (dl - 3 r^-2 (d . dl) d).  emin: the smallest
+// |dl| met (its largest component).
+template <bool W, bool ONE, bool SOFT>
+__device__ __forceinline__ float vjp_tile(const VjpIons &p, const float4 *qt, int lane, int self, f32x2 s2h,
+                                          f32x2 s2l, TriSums<1> &t, float &emin) {
+  float ymax = 0.0f, rmin = __int_as_float(0x7f800000);
+  emin = rmin;
+  const int next = (lane + 1) & 31;
+#pragma unroll 1
+  for (int r0 = 0; r0 < 32; r0 += 2) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      bh[c] = __shfl_sync(0xffffffffu, bh[c], (lane + 1) & 31);
-      bl[c] = __shfl_sync(0xffffffffu, bl[c], (lane + 1) & 31);
-    }
-    eb = __shfl_sync(0xffffffffu, eb, (lane + 1) & 31);
-  }
-  bf_widen(ah, al, ea, a);
-  bf_widen(bh, bl, eb, b);
-}
-
-template <bool QARR, bool INPLACE>
-__global__ void __launch_bounds__(VJP_THREADS, 4) k_vjp_sym(int64_t n, int nbk, int G,
-                                                         const double *__restrict__ x,
-                                                         const double *__restrict__ y,
-                                                         const double *__restrict__ z,
-                                                         const double *__restrict__ q,
-                                                         const double *__restrict__ lx,
-                                                         const double *__restrict__ ly,
-                                                         const double *__restrict__ lz, double soft2,
-                                                         double *__restrict__ acc,
-                                                         int *__restrict__ sync, unsigned *err) {
-  constexpr bool inplace = INPLACE;  // the output mode, fixed at compile time
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int BI = 32 * G;
-  VD8 *posP = reinterpret_cast<VD8 *>(smem_raw);
-  VD8 *posQ = posP + BI;                                      // 2 BI entries (dup)
-  double *accP = reinterpret_cast<double *>(posQ + 2 * BI);  // [3][BI]
-  const SymItem it = sym_block_item(inplace, sync, nbk);
-  const int P = it.P, Q = it.Q;
-  const int64_t p0 = (int64_t)P * BI, q0 = (int64_t)Q * BI;
-  const int np = (int)min((int64_t)BI, n - p0), nq = (int)min((int64_t)BI, n - q0);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int i = tid; i < BI; i += VJP_THREADS) {
-    vjp_stage<QARR>(posP, i, p0 + i, n, x, y, z, q, lx, ly, lz, false);
-    if (P != Q) vjp_stage<QARR>(posQ, i, q0 + i, n, x, y, z, q, lx, ly, lz, true);
-    accP[i] = 0.0;
-    accP[BI + i] = 0.0;
-    accP[2 * BI + i] = 0.0;
-  }
-  __syncthreads();
-
-  if (P == Q) {  // the block's own pairs, one-sided (the self pair gives T = 0)
-    for (int i = tid; i < np; i += VJP_THREADS) {
-      const VD8 pi = posP[i];
-      double a[3] = {0.0, 0.0, 0.0};
-      for (int j0 = 0; j0 < np; j0 += 32) {  // tiles of 32 partners, as off the diagonal
-        float ah[3] = {0.0f, 0.0f, 0.0f}, al[3] = {0.0f, 0.0f, 0.0f};
-        int ea = VJP_BF_EMPTY, eb = VJP_BF_EMPTY;
-        for (int j = j0; j < min(np, j0 + 32); ++j)
-          vjp_eval<QARR, false>(pi, posP[j], soft2, ah, al, ea, nullptr, nullptr, eb);
-        double t[3];
-        bf_widen(ah, al, ea, t);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) a[c] += t[c];
+    for (int s = 0; s < 2; ++s) {
+      const float4 *qe = qt + ((lane + r0 + s) & 31);
+      const float4 q0 = qe[0], q1 = qe[32], q2 = qe[64], u0 = qe[96], u1 = qe[128], u2 = qe[160];
+      f32x2 dh[3], dl[3], eh[3], el[3], h, l, sh, sl, wh, wl;
+      tri_diff(p.r.h[0][0], p.r.m[0][0], p.r.l[0][0], pk1(q0.x), pk1(q1.x), pk1(q2.x), dh[0], dl[0]);
+      tri_diff(p.r.h[0][1], p.r.m[0][1], p.r.l[0][1], pk1(q0.y), pk1(q1.y), pk1(q2.y), dh[1], dl[1]);
+      tri_diff(p.r.h[0][2], p.r.m[0][2], p.r.l[0][2], pk1(q0.z), pk1(q1.z), pk1(q2.z), dh[2], dl[2]);
+      tri_r2(dh, dl, h, l);
+      float ha, hb;
+      upk(h, ha, hb);
+      const bool me0 = ONE && s == 0 && r0 == 0 && self == 0, me1 = ONE && s == 0 && r0 == 0 && self == 1;
+      if (SOFT) {
+        rmin = fminf(rmin, fminf(me0 ? rmin : ha, me1 ? rmin : hb));
+        f32x2 e;
+        ptwo_sum(h, s2h, h, e);
+        l = padd(l, padd(e, s2l));
+        upk(h, ha, hb);
       }
+      float ya = rsqrt_approx(ha), yb = rsqrt_approx(hb);
+      if (!SOFT) ymax = fmaxf(ymax, fmaxf(me0 ? 0.0f : ya, me1 ? 0.0f : yb));
+      if (ONE) {
+        ya = fminf(ya, 0x1p30f);
+        yb = fminf(yb, 0x1p30f);
+      }
+      vjp_rinv(h, l, pk(ya, yb), sh, sl, wh, wl);
+      // the cotangents' difference: normalised, since it may be tiny beside either
+      tri_diff(p.lam.h[0][0], p.lam.m[0][0], p.lam.l[0][0], pk1(u0.x), pk1(u1.x), pk1(u2.x), eh[0], el[0]);
+      tri_diff(p.lam.h[0][1], p.lam.m[0][1], p.lam.l[0][1], pk1(u0.y), pk1(u1.y), pk1(u2.y), eh[1], el[1]);
+      tri_diff(p.lam.h[0][2], p.lam.m[0][2], p.lam.l[0][2], pk1(u0.z), pk1(u1.z), pk1(u2.z), eh[2], el[2]);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) vqsum(posQ, c, i) = a[c];
-    }
-    __syncthreads();
-    sym_output<VJP_THREADS>(inplace, it, n, p0, np, q0, nq, acc, sync, err,
-                            [&](int c, int i) { return vqsum(posQ, c, i); }, [&](int c, int i) { return 0.0; });
-    return;
-  }
-
-  const bool weighted = QARR || np < BI || nq < BI;
-  for (int qs = warp; qs < G; qs += VJP_W) {
-    const VD8 *qd = posQ + qs * 64 + lane;
-    double aq[3] = {0.0, 0.0, 0.0};
-    for (int k = 0; k < G; ++k) {
-      const int pt = (qs + k) % G;
-      __syncthreads();  // all warps are at step k: their P-tiles are distinct
-      const int ip = pt * 32 + lane;
-      const VD8 pp = posP[ip];
-      double a[3], b[3];
-      if (weighted)
-        vjp_tile_pair<true>(pp, qd, lane, soft2, a, b);
-      else
-        vjp_tile_pair<false>(pp, qd, lane, soft2, a, b);
+      for (int c = 0; c < 3; ++c) pfast2(eh[c], el[c]);
+      float m0[3], m1[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) upk(eh[c], m0[c], m1[c]);
+      const float e0 = fmaxf(fmaxf(fabsf(m0[0]), fabsf(m0[1])), fabsf(m0[2]));
+      const float e1 = fmaxf(fmaxf(fabsf(m1[0]), fabsf(m1[1])), fabsf(m1[2]));
+      emin = fminf(emin, fminf(me0 ? emin : e0, me1 ? emin : e1));
+      // d . dl
+      const f32x2 p0 = pmul(dh[0], eh[0]), p1 = pmul(dh[1], eh[1]), p2 = pmul(dh[2], eh[2]);
+      f32x2 low = padd(pfma(dh[0], eh[0], pneg(p0)), padd(pfma(dh[1], eh[1], pneg(p1)), pfma(dh[2], eh[2], pneg(p2))));
+      f32x2 uh, ul, x1, x2;
+      ptwo_sum(p0, p1, uh, x1);
+      ptwo_sum(uh, p2, uh, x2);
+      low = padd(low, padd(x1, x2));
+#pragma unroll
+      for (int c = 0; c < 3; ++c) low = pfma(dh[c], el[c], pfma(dl[c], eh[c], low));
+      // k = 3 r^-2 (d . dl)
+      ptwo_prod(uh, low, wh, wl, uh, ul);
+      const f32x2 kh = pmul(pk1(3.0f), uh);
+      const f32x2 kl = pfma(pk1(3.0f), ul, pfma(pk1(3.0f), uh, pneg(kh)));
+      f32x2 sph = sh, spl = sl, sqh = sh, sql = sl;
+      if (W) ptwo_prod(sh, sl, pk1(q0.w), pk1(q1.w), sph, spl);
+      if (W && !ONE) ptwo_prod(sh, sl, p.r.wh[0], p.r.wl[0], sqh, sql);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        accP[c * BI + ip] += a[c];
-        aq[c] += b[c];
+        f32x2 xh, xl, vh, vl, th, tl;
+        ptwo_prod(dh[c], dl[c], kh, kl, xh, xl);
+        ptwo_diff(eh[c], xh, vh, vl);
+        vl = padd(vl, psub(el[c], xl));
+        ptwo_prod(vh, vl, sph, spl, th, tl);
+        pacc(t.ah[0][c], t.al[0][c], th, tl);
+        if (!ONE) {
+          if (W) ptwo_prod(vh, vl, sqh, sql, th, tl);
+          pacc_sub(t.bh[c], t.bl[c], th, tl);
+        }
+        if (s == 1) {
+          pfast2(t.ah[0][c], t.al[0][c]);
+          if (!ONE) pfast2(t.bh[c], t.bl[c]);
+        }
       }
-    }
-    __syncwarp();  // every lane is done reading the tile
+      if (!ONE)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) vqsum(posQ, c, qs * 32 + lane) = aq[c];
+        for (int c = 0; c < 3; ++c) {
+          t.bh[c] = pshfl(t.bh[c], next);
+          t.bl[c] = pshfl(t.bl[c], next);
+        }
+    }
   }
-  __syncthreads();
-  sym_output<VJP_THREADS>(inplace, it, n, p0, np, q0, nq, acc, sync, err,
-                          [&](int c, int i) { return accP[c * BI + i]; },
-                          [&](int c, int i) { return vqsum(posQ, c, i); });
+  return SOFT ? rsqrt_approx(rmin) : ymax;
 }
 
-static size_t vjp_smem_bytes(int G) { return (size_t)32 * G * (3 * sizeof(VD8) + 3 * sizeof(double)); }
+// The same tile step with each pair in its own units and block-floating sums, as
+// in the one-sided kernel: ions i0 .. i0 + 63 against j0 .. j0 + 31.
+template <bool QARR>
+__device__ __noinline__ void vjp_tile_units(int64_t n, const double *x, const double *y, const double *z,
+                                            const double *q, const double *lx, const double *ly, const double *lz,
+                                            double soft2, int64_t i0, int64_t j0, bool one, double sc, double *accP,
+                                            int ldp, double *accQ, int ldq) {
+  const int lane = threadIdx.x & 31;
+  for (int u = 0; u < 64; u += 32) {
+    VD8 pp;
+    vjp_stage<QARR>(&pp, 0, i0 + u + lane, n, x, y, z, q, lx, ly, lz, false);
+    float ah[3] = {0.0f, 0.0f, 0.0f}, al[3] = {0.0f, 0.0f, 0.0f};
+    float bh[3] = {0.0f, 0.0f, 0.0f}, bl[3] = {0.0f, 0.0f, 0.0f};
+    int ea = VJP_BF_EMPTY, eb = VJP_BF_EMPTY;
+    for (int r = 0; r < 32; ++r) {
+      const int64_t j = j0 + ((lane + r) & 31);
+      VD8 pq;
+      vjp_stage<QARR>(&pq, 0, j, n, x, y, z, q, lx, ly, lz, false);
+      if (i0 + u + lane < n && j < n) vjp_eval<QARR, true>(pp, pq, soft2, ah, al, ea, bh, bl, eb);
+      for (int c = 0; c < 3; ++c) {
+        bh[c] = __shfl_sync(0xffffffffu, bh[c], (lane + 1) & 31);
+        bl[c] = __shfl_sync(0xffffffffu, bl[c], (lane + 1) & 31);
+      }
+      eb = __shfl_sync(0xffffffffu, eb, (lane + 1) & 31);
+    }
+    double a[3], b[3];
+    bf_widen(ah, al, ea, a);
+    bf_widen(bh, bl, eb, b);
+    for (int c = 0; c < 3; ++c) {
+      accP[c * ldp + u + lane] += a[c] * sc;
+      if (!one) accQ[c * ldq + lane] += b[c] * sc;
+    }
+  }
+}
 
-cudaError_t launch_vjp_sym(int64_t n, int nbk, int G, const double *x, const double *y,
-                           const double *z, const double *q, const double *lx, const double *ly,
-                           const double *lz, double soft2, double *part, int *sync, unsigned *err,
-                           bool inplace, cudaStream_t st) {
-  if (G != 4 && G != 8) return cudaErrorInvalidValue;
+// The item's scales: the largest biased exponents of a coordinate, of each
+// component of a cotangent and of a weight; false when the item is left to
+// vjp_tile_units (lengths or cotangents beyond 2^+-100 and 2^+-200, components
+// more than 2^40 apart, weights as in nb_tri.cuh, a softening far above the
+// cloud).  Ends with a barrier.
+template <bool QARR>
+__device__ __forceinline__ bool vjp_scale(int64_t p0, int np, int64_t q0, int nq, const double *x, const double *y,
+                                          const double *z, const double *q, const double *lx, const double *ly,
+                                          const double *lz, double soft2, int &em, int el[3], int &ew) {
+  __shared__ int red[6][VJP_W];
+  int mx = 0, lm[3] = {0, 0, 0}, wx = 0, wn = 0x7fffffff;
+  auto mag = [](double v) { return __double2hiint(v) & 0x7fffffff; };
+  for (int i = threadIdx.x; i < np + nq; i += VJP_THREADS) {
+    const int64_t g = i < np ? p0 + i : q0 + (i - np);
+    mx = max(mx, max(mag(x[g]), max(mag(y[g]), mag(z[g]))));
+    lm[0] = max(lm[0], mag(lx[g]));
+    lm[1] = max(lm[1], mag(ly[g]));
+    lm[2] = max(lm[2], mag(lz[g]));
+    if (QARR && q[g] != 0.0) {
+      wx = max(wx, mag(q[g]));
+      wn = min(wn, mag(q[g]));
+    }
+  }
+  const int w = threadIdx.x >> 5;
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  wx = __reduce_max_sync(0xffffffffu, wx);
+  wn = __reduce_min_sync(0xffffffffu, wn);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) lm[c] = __reduce_max_sync(0xffffffffu, lm[c]);
+  if ((threadIdx.x & 31) == 0) {
+    red[0][w] = mx;
+    red[1][w] = wx;
+    red[2][w] = wn;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) red[3 + c][w] = lm[c];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < VJP_W; ++k) {
+    mx = max(mx, red[0][k]);
+    wx = max(wx, red[1][k]);
+    wn = min(wn, red[2][k]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) lm[c] = max(lm[c], red[3 + c][k]);
+  }
+  em = mx >> 20;
+  const int top = max(lm[0], max(lm[1], lm[2])) >> 20;
+  bool ok = tri_scale_ok(em, soft2) && em >= 1023 - 100 && em <= 1023 + 100 && top <= 1023 + 200;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    el[c] = lm[c] ? lm[c] >> 20 : (top ? top : 1023);  // no cotangent at all: any unit
+    ok = ok && el[c] >= 1023 - 200 && el[c] >= top - 40;
+  }
+  ew = QARR ? wx >> 20 : 1023;
+  if (QARR) ok = ok && ew >= 1023 - 400 && ew <= 1023 + 400 && ew - (wn >> 20) <= TRI_WSPREAD;
+  return ok;
+}
+
+// A cotangent's component more than 2^16 below the largest of its kind may lose
+// bits below 2^-69 of that largest.  In an item where one does, a tile keeps to
+// its words if no pair's |dl| is below 2^-24 of the largest cotangent: the loss
+// is then at most 2^-45 of the pair's own term.
+constexpr float VJP_EMIN_CUT = 0x1p-24f;
+// Without a set l word only FP32's range limits a tile's 1/r.
+constexpr float VJP_YMAX_GRID = 0x1p24f;
+
+// The words of ion g's cotangent (zeros past the end) on the components' own
+// grids, in the unit of the largest; returns whether one is not exact.
+__device__ __forceinline__ int vjp_lam(int64_t g, bool real, const double *lx, const double *ly, const double *lz,
+                                       const int el[3], int top, float w0[3], float w1[3], float w2[3]) {
+  int cut = 0;
+  const double *l[3] = {lx, ly, lz};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float t[3] = {0.0f, 0.0f, 0.0f};
+    if (real) {
+      tri_words(l[c][g], el[c], t);
+      cut |= !tri_exact(l[c][g], el[c]);
+    }
+    const float f = __int_as_float((127 + el[c] - top) << 23);
+    w0[c] = t[0] * f;
+    w1[c] = t[1] * f;
+    w2[c] = t[2] * f;
+  }
+  return cut;
+}
+
+template <bool QARR, bool INPLACE, bool SOFT>
+__global__ void __launch_bounds__(VJP_THREADS, 4)
+    k_vjp_sym(int64_t n, int nbk, int G, const double *__restrict__ x, const double *__restrict__ y,
+              const double *__restrict__ z, const double *__restrict__ q, const double *__restrict__ lx,
+              const double *__restrict__ ly, const double *__restrict__ lz, double soft2, double *__restrict__ acc,
+              int *__restrict__ sync, unsigned *err) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int BI = 32 * G;
+  float4 *qs = reinterpret_cast<float4 *>(smem_raw);              // [G][VJP_TILE4]
+  double *accQ = reinterpret_cast<double *>(qs + G * VJP_TILE4);  // [3][BI]
+  double *accP = accQ + 3 * BI;                                   // [VJP_W][3][64]
+  const SymItem it = sym_block_item(INPLACE, sync, nbk);
+  const int64_t p0 = (int64_t)it.P * BI, q0 = (int64_t)it.Q * BI;
+  const int np = (int)min((int64_t)BI, n - p0), nq = (int)min((int64_t)BI, n - q0);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool diag = it.P == it.Q;
+  int em, el[3], ew;
+  const bool fast = vjp_scale<QARR>(p0, np, q0, diag ? 0 : nq, x, y, z, q, lx, ly, lz, soft2, em, el, ew);
+  const int ee = max(el[0], max(el[1], el[2]));
+  // units: lengths 2^kl, cotangents 2^ke, weights 2^kw; T in 2^(ke - 3 kl + kw)
+  const int kt = fast ? (ee - 1022) - 3 * (em - 1022) + (ew - 1023) : 0;
+  const int PT = G >> 1, NG = VJP_W / PT, nqt = G / NG;  // P-tiles of 64 ions, warps and Q-tiles per P-tile
+  const int pt = warp % PT, grp = warp / PT;
+  VjpIons p;
+  int low = 0;  // an l word of a position is set
+  int cut = 0;  // a cotangent is not exact in its words
+  if (fast) {
+    float w0[2][4], w1[2][4], w2[2][4];
+    for (int i = tid; i < BI; i += VJP_THREADS) {
+      const int64_t g = q0 + i;
+      float4 *e = qs + (i >> 5) * VJP_TILE4 + (i & 31);
+      tri_ion<QARR>(g, i < nq, x, y, z, q, em, ew, -TRI_FAR, w0[0], w1[0], w2[0]);
+      e[0] = make_float4(w0[0][0], w0[0][1], w0[0][2], w0[0][3]);
+      e[32] = make_float4(w1[0][0], w1[0][1], w1[0][2], w1[0][3]);
+      e[64] = make_float4(w2[0][0], w2[0][1], w2[0][2], 0.0f);
+      low |= w2[0][0] != 0.0f || w2[0][1] != 0.0f || w2[0][2] != 0.0f;
+      cut |= vjp_lam(g, i < nq, lx, ly, lz, el, ee, w0[0], w1[0], w2[0]);
+      e[96] = make_float4(w0[0][0], w0[0][1], w0[0][2], 0.0f);
+      e[128] = make_float4(w1[0][0], w1[0][1], w1[0][2], 0.0f);
+      e[160] = make_float4(w2[0][0], w2[0][1], w2[0][2], 0.0f);
+    }
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int i = pt * 64 + b * 32 + lane;
+      tri_ion<QARR>(p0 + i, i < np, x, y, z, q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
+      low |= w2[b][0] != 0.0f || w2[b][1] != 0.0f || w2[b][2] != 0.0f;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      p.r.h[0][c] = pk(w0[0][c], w0[1][c]);
+      p.r.m[0][c] = pk(w1[0][c], w1[1][c]);
+      p.r.l[0][c] = pk(w2[0][c], w2[1][c]);
+    }
+    p.r.wh[0] = pk(w0[0][3], w0[1][3]);
+    p.r.wl[0] = pk(w1[0][3], w1[1][3]);
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int i = pt * 64 + b * 32 + lane;
+      cut |= vjp_lam(p0 + i, i < np, lx, ly, lz, el, ee, w0[b], w1[b], w2[b]);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      p.lam.h[0][c] = pk(w0[0][c], w0[1][c]);
+      p.lam.m[0][c] = pk(w1[0][c], w1[1][c]);
+      p.lam.l[0][c] = pk(w2[0][c], w2[1][c]);
+    }
+  }
+  for (int i = tid; i < 3 * BI; i += VJP_THREADS) accQ[i] = 0.0;
+  for (int i = tid; i < VJP_W * 3 * 64; i += VJP_THREADS) accP[i] = 0.0;
+  const float ylim = __syncthreads_or(low) ? TRI_YMAX : VJP_YMAX_GRID;
+  const float elim = __syncthreads_or(cut) ? VJP_EMIN_CUT : 0.0f;
+  f32x2 s2h = 0, s2l = 0;
+  if (SOFT) {
+    float sh, sl;
+    split_f64_scaled(soft2, 2 * (em - 1022), sh, sl);
+    s2h = pk1(sh);
+    s2l = pk1(sl);
+  }
+  double *aP = accP + warp * 3 * 64;
+  const double back = pow2d(-kt), fwd = pow2d(kt);
+  const bool live = pt * 64 < np;
+  for (int k = 0; k < nqt; ++k) {
+    const int t = grp * nqt + (k + pt) % nqt;  // distinct over the P-tiles of a step: nqt >= PT
+    if (k > 0) __syncthreads();                // the Q sums of the last step are written
+    if (!live || t * 32 >= nq) continue;
+    double *aQ = accQ + t * 32;
+    bool done = false;
+    if (fast) {
+      TriSums<1> ts;
+      const f32x2 zero = pk1(0.0f);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) ts.ah[0][c] = ts.al[0][c] = ts.bh[c] = ts.bl[c] = zero;
+      const float4 *qt = qs + t * VJP_TILE4;
+      float emin;
+      const int u = t - 2 * pt;  // the lane's own ion in this Q-tile, if any
+      const float ymax = diag ? vjp_tile<QARR, true, SOFT>(p, qt, lane, u == 0 || u == 1 ? u : -1, s2h, s2l, ts, emin)
+                              : vjp_tile<QARR, false, SOFT>(p, qt, lane, -1, s2h, s2l, ts, emin);
+      done = !__any_sync(0xffffffffu, !(ymax <= ylim) || !(emin >= elim));
+      if (done) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          float h0, h1, l0, l1;
+          upk(ts.ah[0][c], h0, h1);
+          upk(ts.al[0][c], l0, l1);
+          aP[c * 64 + lane] += (double)h0 + (double)l0;
+          aP[c * 64 + 32 + lane] += (double)h1 + (double)l1;
+          if (!diag) {
+            upk(ts.bh[c], h0, h1);
+            upk(ts.bl[c], l0, l1);
+            aQ[c * BI + lane] += ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
+          }
+        }
+      }
+    }
+    if (!done)
+      vjp_tile_units<QARR>(n, x, y, z, q, lx, ly, lz, soft2, p0 + pt * 64, q0 + t * 32, diag, back, aP, 64, aQ, BI);
+  }
+  __syncthreads();
+  sym_output<VJP_THREADS>(INPLACE, it, n, p0, np, q0, nq, acc, sync, err,
+                          [&](int c, int i) {
+                            double v = 0.0;
+                            for (int g = 0; g < NG; ++g) v += accP[(g * PT + i / 64) * 192 + c * 64 + i % 64];
+                            return v * fwd;
+                          },
+                          [&](int c, int i) { return accQ[c * BI + i] * fwd; });
+}
+
+static size_t vjp_smem_bytes(int G) {
+  return (size_t)G * VJP_TILE4 * sizeof(float4) + (size_t)3 * 32 * G * sizeof(double) +
+         (size_t)VJP_W * 3 * 64 * sizeof(double);
+}
+
+template <bool SOFT>
+static cudaError_t launch_vjp_t(int64_t n, int nbk, int G, const double *x, const double *y,
+                                const double *z, const double *q, const double *lx, const double *ly,
+                                const double *lz, double soft2, double *part, int *sync, unsigned *err,
+                                bool inplace, cudaStream_t st) {
   static std::mutex mu;
   static bool done[64] = {false};
   int dev = 0;
@@ -301,8 +561,8 @@ cudaError_t launch_vjp_sym(int64_t n, int nbk, int G, const double *x, const dou
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!done[dev]) {
       const int lim = (int)vjp_smem_bytes(8);
-      const void *fns[4] = {(const void *)k_vjp_sym<true, false>, (const void *)k_vjp_sym<false, false>,
-                            (const void *)k_vjp_sym<true, true>, (const void *)k_vjp_sym<false, true>};
+      const void *fns[4] = {(const void *)k_vjp_sym<true, false, SOFT>, (const void *)k_vjp_sym<false, false, SOFT>,
+                            (const void *)k_vjp_sym<true, true, SOFT>, (const void *)k_vjp_sym<false, true, SOFT>};
       for (int k = 0; k < 4 && e == cudaSuccess; ++k)
         e = cudaFuncSetAttribute(fns[k], cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
       if (e != cudaSuccess) return e;
@@ -315,8 +575,8 @@ cudaError_t launch_vjp_sym(int64_t n, int nbk, int G, const double *x, const dou
   }
   const int items = nbk * (nbk + 1) / 2;
   const size_t smem = vjp_smem_bytes(G);
-#define NB_VJP_LAUNCH(QA, IP)                                                                                  \
-  k_vjp_sym<QA, IP><<<items, VJP_THREADS, smem, st>>>(n, nbk, G, x, y, z, q, lx, ly, lz, soft2, part, sync, err)
+#define NB_VJP_LAUNCH(QA, IP) \
+  k_vjp_sym<QA, IP, SOFT><<<items, VJP_THREADS, smem, st>>>(n, nbk, G, x, y, z, q, lx, ly, lz, soft2, part, sync, err)
   if (inplace) {
     if (q) NB_VJP_LAUNCH(true, true); else NB_VJP_LAUNCH(false, true);
   } else {
@@ -324,6 +584,15 @@ cudaError_t launch_vjp_sym(int64_t n, int nbk, int G, const double *x, const dou
   }
 #undef NB_VJP_LAUNCH
   return cudaGetLastError();
+}
+
+cudaError_t launch_vjp_sym(int64_t n, int nbk, int G, const double *x, const double *y,
+                           const double *z, const double *q, const double *lx, const double *ly,
+                           const double *lz, double soft2, double *part, int *sync, unsigned *err,
+                           bool inplace, cudaStream_t st) {
+  if (G != 4 && G != 8) return cudaErrorInvalidValue;
+  return soft2 != 0.0 ? launch_vjp_t<true>(n, nbk, G, x, y, z, q, lx, ly, lz, soft2, part, sync, err, inplace, st)
+                      : launch_vjp_t<false>(n, nbk, G, x, y, z, q, lx, ly, lz, soft2, part, sync, err, inplace, st);
 }
 
 cudaError_t launch_pair_vjp(const Plan &pl, int64_t n, const double *x, const double *y,
