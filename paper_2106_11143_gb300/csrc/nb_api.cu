@@ -16,6 +16,7 @@
 #include <utility>
 
 #include "nb_common.cuh"
+#include "nb_epi.cuh"
 #include "nb_symsched.cuh"
 #include "nb_tri.cuh"
 
@@ -232,14 +233,17 @@ cudaError_t launch_pairs(const Plan &pl, int mode, int64_t n, const double *x, c
   return launch_pair_force(pl, mode, n, x, y, z, q, pf, soft2, part, err, st);
 }
 
-// Force evaluation at positions (x, y, z) into `part`.
+// Force evaluation at positions (x, y, z) into `part`; `ready`: the kernel that
+// wrote the positions has stored their FP32 parts in `split` too.
 nb_status pair_forces(const Plan &pl, int mode, int64_t n, const double *x, const double *y,
                       const double *z, const double *q, double soft2, double *part, float *split,
-                      unsigned *err, cudaStream_t st) {
+                      unsigned *err, cudaStream_t st, bool ready = false) {
   PosF32 pf{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   if (split_like(mode)) {
-    NB_CUDA_TRY(launch_split_positions(n, x, y, z, split, st));
-    count_launches(1);
+    if (!ready) {
+      NB_CUDA_TRY(launch_split_positions(n, x, y, z, split, st));
+      count_launches(1);
+    }
     pf = PosF32{split, split + n, split + 2 * n, split + 3 * n, split + 4 * n, split + 5 * n};
   }
   timing_begin(st);
@@ -404,13 +408,13 @@ nb_status capture_window(Arena *a, const Plan &pl, int mode, const Phys &p, cons
   for (int64_t k = 1; k <= STEP_WINDOW && rc == NB_OK && e == cudaSuccess; ++k) {
     double *const *P = (k % 2) ? A : B;
     double *const *Nx = (k % 2) ? B : A;
-    rc = pair_forces(pl, mode, v.n, P[0], P[1], P[2], v.q, soft2, part, split, a->err, cs);
+    rc = pair_forces(pl, mode, v.n, P[0], P[1], P[2], v.q, soft2, part, split, a->err, cs, true);
     if (rc != NB_OK) break;
     const int64_t *cin = k == 1 ? c : c + 1;
     const int64_t soff = k == 1 ? 1 : k - STEP_WINDOW;
     int64_t *cout = k == 1 ? c + 1 : (k == STEP_WINDOW ? c : nullptr);
     const int64_t cout_off = k == 1 ? STEP_WINDOW : 0;
-    e = launch_epi_step(p, v, P[0], P[1], P[2], part, pl.n_jc, soff, Nx[0], Nx[1], Nx[2], a->err, cs,
+    e = launch_epi_step_split(p, v, P[0], P[1], P[2], part, pl.n_jc, soff, Nx[0], Nx[1], Nx[2], split, a->err, cs,
                         cin, cout, cout_off);
     count_launches(1);
   }
@@ -555,15 +559,15 @@ nb_status nb_step(const nb_params *params, nb_system *sys, int64_t nsteps, void 
   const int64_t reps = windows ? (nsteps - 1 - pre) / STEP_WINDOW : 0;
   int64_t *ctr = step_counters(a);
   double **b0 = buf(0);
-  NB_CUDA_TRY(launch_drift(p, v, b0[0], b0[1], b0[2], st));
+  NB_CUDA_TRY(launch_drift_split(p, v, b0[0], b0[1], b0[2], split, st));
   count_launches(1);
   for (int64_t s = 0; s < pre; ++s) {
     double **P = buf(s), **Nx = buf(s + 1);
-    NB_TRY(pair_forces(pl, mode, n, P[0], P[1], P[2], sys->q, params->soft2, part, split, a->err, st));
+    NB_TRY(pair_forces(pl, mode, n, P[0], P[1], P[2], sys->q, params->soft2, part, split, a->err, st, true));
     const int64_t snew = sys->step + s + 1;
     int64_t *cout = (windows && s + 1 == pre) ? ctr : nullptr;  // the windows' starting index
-    NB_CUDA_TRY(launch_epi_step(p, v, P[0], P[1], P[2], part, pl.n_jc, snew, Nx[0], Nx[1], Nx[2], a->err, st,
-                                nullptr, cout, snew));
+    NB_CUDA_TRY(launch_epi_step_split(p, v, P[0], P[1], P[2], part, pl.n_jc, snew, Nx[0], Nx[1], Nx[2], split, a->err,
+                                      st, nullptr, cout, snew));
     count_launches(1);
   }
   if (reps > 0) {
@@ -575,7 +579,7 @@ nb_status nb_step(const nb_params *params, nb_system *sys, int64_t nsteps, void 
     count_launches(wg->kernels * (uint64_t)reps);
   }
   double **P = buf(nsteps - 1);
-  NB_TRY(pair_forces(pl, mode, n, P[0], P[1], P[2], sys->q, params->soft2, part, split, a->err, st));
+  NB_TRY(pair_forces(pl, mode, n, P[0], P[1], P[2], sys->q, params->soft2, part, split, a->err, st, true));
   NB_CUDA_TRY(launch_epi_step(p, v, P[0], P[1], P[2], part, pl.n_jc, sys->step + nsteps, nullptr, nullptr, nullptr,
                               a->err, st));
   count_launches(1);

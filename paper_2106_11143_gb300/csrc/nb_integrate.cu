@@ -1,7 +1,7 @@
 // nb_integrate.cu -- O(N) kernels of libnb.so: the epilogues that turn the
 // pair partial sums into accelerations (Eq. 1), the velocity-Verlet kick and
 // drift (Sec. II), the Langevin kick, and the energy reduction.
-#include "nb_verlet.cuh"
+#include "nb_epi.cuh"
 
 namespace nb {
 
@@ -23,59 +23,15 @@ __device__ __forceinline__ void chunk_sum3(const double *__restrict__ part, int 
   slot_sum3(n_jc, [&](int jc, int c) { return __ldcs(p + ((int64_t)jc * 3 + c) * n); }, out);
 }
 
-// The epilogues run with EPI_THREADS threads per block, one of two ways:
-//  - one thread per ion, adding its chunk partials with chunk_sum3;
-//  - eight threads per ion (the default): warp u of a block forms slot_sum3's
-//    running sum u (chunks u, u+8, ...) for the block's 32 ions, and the
-//    eight sums go through shared memory to the first warp, which adds them in
-//    slot_sum3's pairing and finishes one ion per lane.  The dependent chain
-//    of the sum is spread over eight threads, each warp load reads 256
-//    contiguous bytes, and the FP64 tail still serves 32 ions per warp
-//    instruction.
-// Both give the same sums, bit for bit.  epi_sums returns false for threads
-// without an ion (the caller then returns); it holds a block barrier in the
-// eight-lane form, so every thread of the block must call it.
+// The epilogues run one of two ways:
+//  - one thread per ion, EPI_THREADS per block, adding its chunk partials with
+//    chunk_sum3;
+//  - eight threads per ion (the default with eight slots or more): warp u of a
+//    block forms slot_sum3's running sum u for the block's 32 ions (nb_epi.cuh)
+//    and a ninth warp adds the eight in slot_sum3's pairing and finishes one ion
+//    per lane.
+// Both give the same sums, bit for bit.
 constexpr int EPI_THREADS = 256;
-
-template <bool EIGHT>
-__device__ __forceinline__ bool epi_sums(const double *__restrict__ part, int n_jc, int64_t n,
-                                         int64_t &i, double cs[3]) {
-  if (!EIGHT) {
-    i = (int64_t)blockIdx.x * EPI_THREADS + threadIdx.x;
-    if (i >= n) return false;
-    chunk_sum3(part, n_jc, n, i, cs);
-    return true;
-  }
-  // Warp u of the block forms running sum u (slots u, u+8, ...) for the
-  // block's 32 ions, one ion per lane: each load of a warp reads one slot of
-  // 32 consecutive ions, 256 contiguous bytes (two L1 lines).
-  static_assert(EPI_THREADS == 256, "eight warps, one per running sum");
-  const int u = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const int64_t g = (int64_t)blockIdx.x * 32 + l;
-  const int64_t ig = g < n ? g : n - 1;  // every warp reaches the barrier
-  cs[0] = cs[1] = cs[2] = 0.0;
-  const double *pi = part + ig;
-  for (int jc = u; jc < n_jc; jc += 8) {
-    const double *q = pi + (int64_t)jc * 3 * n;
-    cs[0] += __ldcs(q);
-    cs[1] += __ldcs(q + n);
-    cs[2] += __ldcs(q + 2 * n);
-  }
-  __shared__ double csum[3][8][32];
-  csum[0][u][l] = cs[0];
-  csum[1][u][l] = cs[1];
-  csum[2][u][l] = cs[2];
-  __syncthreads();
-  if (threadIdx.x >= 32) return false;
-  i = g;
-  if (i >= n) return false;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {  // slot_sum3's pairing of the eight running sums
-    const double(*s)[32] = csum[c];
-    cs[c] = ((s[0][l] + s[1][l]) + (s[2][l] + s[3][l])) + ((s[4][l] + s[5][l]) + (s[6][l] + s[7][l]));
-  }
-  return true;
-}
 
 // Eight threads per ion unless tuning kind 8 says one (R = 0) for this n:
 // measured on GB300 the eight-thread form was faster at every n up to 1e5
@@ -89,7 +45,26 @@ static bool epi_eight(int64_t n, int n_jc) {
   if (tuning_lookup(8, 0, n, &tb, &tr, &tbps)) return tr == 1;
   return n_jc >= 8;
 }
-static int epi_blocks(int64_t n, bool eight) { return blocks_for(eight ? 8 * n : n, EPI_THREADS); }
+static int epi_blocks(int64_t n, bool eight) { return blocks_for(n, eight ? EPI8_IONS : EPI_THREADS); }
+
+// The ion and its three sums in either form; false for threads without an ion
+// to finish.  Holds a block barrier in the eight-thread form.
+template <bool EIGHT>
+__device__ __forceinline__ bool epi_sums(const double *__restrict__ part, int n_jc, int64_t n, int64_t &i,
+                                         double cs[3]) {
+  if (!EIGHT) {
+    i = (int64_t)blockIdx.x * EPI_THREADS + threadIdx.x;
+    if (i >= n) return false;
+    chunk_sum3(part, n_jc, n, i, cs);
+    return true;
+  }
+  i = (int64_t)blockIdx.x * EPI8_IONS + (threadIdx.x & 31);
+  const bool last = epi8_slots(part, n_jc, n);
+  __syncthreads();
+  if (!last || i >= n) return false;
+  epi8_total(cs);
+  return true;
+}
 
 // ---------------------------------------------------------------------------
 template <bool EIGHT>
@@ -120,7 +95,7 @@ __global__ void __launch_bounds__(EPI_THREADS)
                  unsigned *err) {
   epi_forces<false>(p, s, part, n_jc, flags, t, err);
 }
-__global__ void __launch_bounds__(EPI_THREADS)
+__global__ void __launch_bounds__(EPI8_THREADS)
     k_epi_forces8(Phys p, StateView s, const double *__restrict__ part, int n_jc, int flags, double t,
                   unsigned *err) {
   epi_forces<true>(p, s, part, n_jc, flags, t, err);
@@ -130,7 +105,7 @@ cudaError_t launch_epi_forces(const Phys &p, const StateView &s, const double *p
                               int flags, double t, unsigned *err, cudaStream_t st) {
   const bool eight = epi_eight(s.n, n_jc);
   if (eight)
-    k_epi_forces8<<<epi_blocks(s.n, true), EPI_THREADS, 0, st>>>(p, s, part, n_jc, flags, t, err);
+    k_epi_forces8<<<epi_blocks(s.n, true), EPI8_THREADS, 0, st>>>(p, s, part, n_jc, flags, t, err);
   else
     k_epi_forces<<<epi_blocks(s.n, false), EPI_THREADS, 0, st>>>(p, s, part, n_jc, flags, t, err);
   return cudaGetLastError();
@@ -165,7 +140,7 @@ __global__ void __launch_bounds__(EPI_THREADS)
               double *gz, int flags, double t) {
   epi_vjp<false>(p, s, part, n_jc, lx, ly, lz, gx, gy, gz, flags, t);
 }
-__global__ void __launch_bounds__(EPI_THREADS)
+__global__ void __launch_bounds__(EPI8_THREADS)
     k_epi_vjp8(Phys p, StateView s, const double *__restrict__ part, int n_jc, const double *__restrict__ lx,
                const double *__restrict__ ly, const double *__restrict__ lz, double *gx, double *gy,
                double *gz, int flags, double t) {
@@ -176,7 +151,7 @@ cudaError_t launch_epi_vjp(const Phys &p, const StateView &s, const double *part
                            const double *lx, const double *ly, const double *lz, double *gx,
                            double *gy, double *gz, int flags, double t, cudaStream_t st) {
   if (epi_eight(s.n, n_jc))
-    k_epi_vjp8<<<epi_blocks(s.n, true), EPI_THREADS, 0, st>>>(p, s, part, n_jc, lx, ly, lz, gx, gy, gz, flags, t);
+    k_epi_vjp8<<<epi_blocks(s.n, true), EPI8_THREADS, 0, st>>>(p, s, part, n_jc, lx, ly, lz, gx, gy, gz, flags, t);
   else
     k_epi_vjp<<<epi_blocks(s.n, false), EPI_THREADS, 0, st>>>(p, s, part, n_jc, lx, ly, lz, gx, gy, gz, flags, t);
   return cudaGetLastError();
@@ -184,21 +159,29 @@ cudaError_t launch_epi_vjp(const Phys &p, const StateView &s, const double *part
 
 // ---------------------------------------------------------------------------
 // First drift of a run: r+ = r + v dt + a dt^2/2 into (px, py, pz), which may
-// alias (x, y, z) (each thread touches only its own ion).
-__global__ void k_drift(Phys p, StateView s, double *px, double *py, double *pz) {
+// alias (x, y, z) (each thread touches only its own ion), and with `split` its
+// FP32 parts.
+__global__ void k_drift(Phys p, StateView s, double *px, double *py, double *pz, float *split) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= s.n) return;
   const double dt = p.dt;
-  px[i] = verlet_drift(s.x[i], s.vx[i], s.ax[i], dt);
-  py[i] = verlet_drift(s.y[i], s.vy[i], s.ay[i], dt);
-  pz[i] = verlet_drift(s.z[i], s.vz[i], s.az[i], dt);
+  const double r[3] = {verlet_drift(s.x[i], s.vx[i], s.ax[i], dt), verlet_drift(s.y[i], s.vy[i], s.ay[i], dt),
+                       verlet_drift(s.z[i], s.vz[i], s.az[i], dt)};
+  px[i] = r[0];
+  py[i] = r[1];
+  pz[i] = r[2];
+  if (split) store_split(split, s.n, i, r);
 }
 
+cudaError_t launch_drift_split(const Phys &p, const StateView &s, double *px, double *py, double *pz, float *split,
+                               cudaStream_t st) {
+  const int T = 256;
+  k_drift<<<blocks_for(s.n, T), T, 0, st>>>(p, s, px, py, pz, split);
+  return cudaGetLastError();
+}
 cudaError_t launch_drift(const Phys &p, const StateView &s, double *px, double *py, double *pz,
                          cudaStream_t st) {
-  const int T = 256;
-  k_drift<<<blocks_for(s.n, T), T, 0, st>>>(p, s, px, py, pz);
-  return cudaGetLastError();
+  return launch_drift_split(p, s, px, py, pz, nullptr, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -213,27 +196,56 @@ cudaError_t launch_drift(const Phys &p, const StateView &s, double *px, double *
 // there.  The counter form lets one captured graph of steps be replayed with
 // a step index that advances from replay to replay (cin and cout are never
 // the same word, so no thread reads what another writes).
+//
+// In the eight-thread form the ninth warp has everything that does not depend
+// on the sums in registers before the barrier: its ion's state, the kick's
+// constants (three FP64 divisions), the trap's factors (an FP64 cosine in the RF
+// trap) and the Langevin draws, all of it formed while the other warps wait for
+// their slots.  With `split`, the next positions' FP32 (hi, lo) parts are stored
+// beside them (six floats per ion, as k_split_positions forms them), which saves
+// the split modes that kernel's launch.
 template <bool EIGHT>
 __device__ __forceinline__ void epi_step(const Phys &p, const StateView &s, const double *cx,
                                          const double *cy, const double *cz, const double *part, int n_jc,
                                          int64_t soff, const int64_t *cin, int64_t *cout, int64_t cout_off,
-                                         double *nx, double *ny, double *nz, unsigned *err) {
-  int64_t i;
+                                         double *nx, double *ny, double *nz, float *split, unsigned *err) {
+  const int64_t i = EIGHT ? (int64_t)blockIdx.x * EPI8_IONS + (threadIdx.x & 31)
+                          : (int64_t)blockIdx.x * EPI_THREADS + threadIdx.x;
+  const bool last = !EIGHT || epi8_slots(part, n_jc, s.n);
+  if (!EIGHT && i >= s.n) return;
+  double r[3], v[3], a[3], xi[3];
+  KickConst kc;
+  TrapFactors tf;
+  const bool own = last && i < s.n;
+  int64_t base = 0;
+  if (own) {
+    r[0] = cx[i]; r[1] = cy[i]; r[2] = cz[i];
+    v[0] = s.vx[i]; v[1] = s.vy[i]; v[2] = s.vz[i];
+    a[0] = s.ax[i]; a[1] = s.ay[i]; a[2] = s.az[i];
+    base = cin ? *cin : 0;
+    kc = kick_consts(p, s, i);
+    tf = trap_factors(p, base + soff);
+    kick_noise(p, s.ion0 + i, base + soff, xi);
+  }
   double cs[3];
-  if (!epi_sums<EIGHT>(part, n_jc, s.n, i, cs)) return;
-  const int64_t base = cin ? *cin : 0;
-  const int64_t snew = base + soff;
+  if (EIGHT) {
+    __syncthreads();
+    if (!own) return;
+    epi8_total(cs);
+  } else {
+    chunk_sum3(part, n_jc, s.n, i, cs);
+  }
   if (cout && i == 0) *cout = base + cout_off;
-  const double r[3] = {cx[i], cy[i], cz[i]};
-  double v[3] = {s.vx[i], s.vy[i], s.vz[i]};
-  double a[3] = {s.ax[i], s.ay[i], s.az[i]};
-  const bool bad = verlet_kick(p, s, i, snew, r, cs, v, a);
+  const bool bad = verlet_kick(p.dt, kc, tf, xi, r, cs, v, a);
   s.vx[i] = v[0]; s.vy[i] = v[1]; s.vz[i] = v[2];
   s.ax[i] = a[0]; s.ay[i] = a[1]; s.az[i] = a[2];
   if (nx) {
-    nx[i] = verlet_drift(r[0], v[0], a[0], p.dt);
-    ny[i] = verlet_drift(r[1], v[1], a[1], p.dt);
-    nz[i] = verlet_drift(r[2], v[2], a[2], p.dt);
+    const double rn[3] = {verlet_drift(r[0], v[0], a[0], p.dt), verlet_drift(r[1], v[1], a[1], p.dt),
+                          verlet_drift(r[2], v[2], a[2], p.dt)};
+    nx[i] = rn[0];
+    ny[i] = rn[1];
+    nz[i] = rn[2];
+    if (split) store_split(split, s.n, i, rn);
   } else {
     s.x[i] = r[0]; s.y[i] = r[1]; s.z[i] = r[2];
   }
@@ -243,28 +255,34 @@ __global__ void __launch_bounds__(EPI_THREADS)
     k_epi_step(Phys p, StateView s, const double *__restrict__ cx, const double *__restrict__ cy,
                const double *__restrict__ cz, const double *__restrict__ part, int n_jc, int64_t soff,
                const int64_t *cin, int64_t *cout, int64_t cout_off, double *nx, double *ny, double *nz,
-               unsigned *err) {
-  epi_step<false>(p, s, cx, cy, cz, part, n_jc, soff, cin, cout, cout_off, nx, ny, nz, err);
+               float *split, unsigned *err) {
+  epi_step<false>(p, s, cx, cy, cz, part, n_jc, soff, cin, cout, cout_off, nx, ny, nz, split, err);
 }
-__global__ void __launch_bounds__(EPI_THREADS)
+__global__ void __launch_bounds__(EPI8_THREADS)
     k_epi_step8(Phys p, StateView s, const double *__restrict__ cx, const double *__restrict__ cy,
                 const double *__restrict__ cz, const double *__restrict__ part, int n_jc, int64_t soff,
                 const int64_t *cin, int64_t *cout, int64_t cout_off, double *nx, double *ny, double *nz,
-                unsigned *err) {
-  epi_step<true>(p, s, cx, cy, cz, part, n_jc, soff, cin, cout, cout_off, nx, ny, nz, err);
+                float *split, unsigned *err) {
+  epi_step<true>(p, s, cx, cy, cz, part, n_jc, soff, cin, cout, cout_off, nx, ny, nz, split, err);
 }
 
+cudaError_t launch_epi_step_split(const Phys &p, const StateView &s, const double *cx, const double *cy,
+                                  const double *cz, const double *part, int n_jc, int64_t snew,
+                                  double *nx, double *ny, double *nz, float *split, unsigned *err, cudaStream_t st,
+                                  const int64_t *cin, int64_t *cout, int64_t cout_off) {
+  if (epi_eight(s.n, n_jc))
+    k_epi_step8<<<epi_blocks(s.n, true), EPI8_THREADS, 0, st>>>(p, s, cx, cy, cz, part, n_jc, snew, cin, cout,
+                                                                 cout_off, nx, ny, nz, split, err);
+  else
+    k_epi_step<<<epi_blocks(s.n, false), EPI_THREADS, 0, st>>>(p, s, cx, cy, cz, part, n_jc, snew, cin, cout,
+                                                                cout_off, nx, ny, nz, split, err);
+  return cudaGetLastError();
+}
 cudaError_t launch_epi_step(const Phys &p, const StateView &s, const double *cx, const double *cy,
                             const double *cz, const double *part, int n_jc, int64_t snew,
                             double *nx, double *ny, double *nz, unsigned *err, cudaStream_t st,
                             const int64_t *cin, int64_t *cout, int64_t cout_off) {
-  if (epi_eight(s.n, n_jc))
-    k_epi_step8<<<epi_blocks(s.n, true), EPI_THREADS, 0, st>>>(p, s, cx, cy, cz, part, n_jc, snew, cin, cout,
-                                                                cout_off, nx, ny, nz, err);
-  else
-    k_epi_step<<<epi_blocks(s.n, false), EPI_THREADS, 0, st>>>(p, s, cx, cy, cz, part, n_jc, snew, cin, cout,
-                                                                cout_off, nx, ny, nz, err);
-  return cudaGetLastError();
+  return launch_epi_step_split(p, s, cx, cy, cz, part, n_jc, snew, nx, ny, nz, nullptr, err, st, cin, cout, cout_off);
 }
 
 // ---------------------------------------------------------------------------

@@ -116,11 +116,14 @@ __device__ __forceinline__ void stage_ion(D4 *pos, float4 *sp, const StateView &
   }
 }
 
+// One warp beyond the SMALL_THREADS of the pair items forms the trap's factors.
+constexpr int SMALL_BLOCK = SMALL_THREADS + 32;
+
 // nsteps steps from (x, v, a) at step index step0; thread i < n owns ion i.
 // Per step: [barrier] pair items -> chunk partials [barrier] kick and next
 // drift of the own ion.  Writes x, v, a back at the end.
 template <int MODE, bool QARR>
-__global__ void __launch_bounds__(SMALL_THREADS, 1)
+__global__ void __launch_bounds__(SMALL_BLOCK, 1)
     k_small_steps(Phys p, StateView s, int tile, int jchunk, int n_jc, int64_t step0, int64_t nsteps,
                   unsigned *err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -129,6 +132,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1)
   D4 *pos = reinterpret_cast<D4 *>(smem_raw);
   float4 *sp = reinterpret_cast<float4 *>(pos + n);
   double *part = reinterpret_cast<double *>(sp + (split_like(MODE) ? 2 * n : 0));
+  TrapFactors *tf = reinterpret_cast<TrapFactors *>(part + 3 * n * n_jc);
   const bool own = tid < n;
   const double dt = p.dt;
   const float soft2f = (float)p.soft2;
@@ -149,20 +153,27 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1)
   const int items = n * n_jc;
   for (int64_t st = 0; st < nsteps; ++st) {
     __syncthreads();  // this step's positions are staged; last step's partials are read
-    for (int it = tid; it < items; it += SMALL_THREADS) {
-      const int jc = it / n;
-      const int i = it - jc * n;
-      const int jb = jc * jchunk;
-      double o[3];
-      chunk_partial<MODE, QARR>(pos, sp, i, jb, min(jb + jchunk, n), tile, p.soft2, soft2f, s2h, s2l, o);
+    if (tid >= SMALL_THREADS) {  // the trap's factors at the new time, beside the pair sums
+      const TrapFactors f = trap_factors(p, step0 + st + 1);
+      if (tid == SMALL_THREADS) *tf = f;
+    } else {
+      for (int it = tid; it < items; it += SMALL_THREADS) {
+        const int jc = it / n;
+        const int i = it - jc * n;
+        const int jb = jc * jchunk;
+        double o[3];
+        chunk_partial<MODE, QARR>(pos, sp, i, jb, min(jb + jchunk, n), tile, p.soft2, soft2f, s2h, s2l, o);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) part[(jc * 3 + c) * n + i] = o[c];
+        for (int c = 0; c < 3; ++c) part[(jc * 3 + c) * n + i] = o[c];
+      }
     }
     __syncthreads();  // partials complete; nobody reads the positions until the next barrier
     if (own) {
       double cs[3];
       slot_sum3(n_jc, [&](int jc, int c) { return part[(jc * 3 + c) * n + tid]; }, cs);
-      bad |= verlet_kick_k(p, kc, tid, step0 + st + 1, r, cs, v, a);
+      double xi[3];
+      kick_noise(p, tid, step0 + st + 1, xi);
+      bad |= verlet_kick(dt, kc, *tf, xi, r, cs, v, a);
       if (st + 1 < nsteps) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) r[c] = verlet_drift(r[c], v[c], a[c], dt);
@@ -180,7 +191,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1)
 
 size_t small_smem_bytes(const Plan &pl, int mode, int64_t n) {
   return (size_t)n * sizeof(D4) + (split_like(mode) ? (size_t)n * 2 * sizeof(float4) : 0) +
-         (size_t)pl.n_jc * 3 * (size_t)n * sizeof(double);
+         (size_t)pl.n_jc * 3 * (size_t)n * sizeof(double) + sizeof(TrapFactors);
 }
 
 template <int MODE>
@@ -206,10 +217,10 @@ static cudaError_t launch_small_m(const Plan &pl, const Phys &p, const StateView
   }
   const size_t smem = small_smem_bytes(pl, MODE, s.n);
   if (s.q)
-    k_small_steps<MODE, true><<<1, SMALL_THREADS, smem, st>>>(p, s, pl.block, (int)pl.jchunk, pl.n_jc,
+    k_small_steps<MODE, true><<<1, SMALL_BLOCK, smem, st>>>(p, s, pl.block, (int)pl.jchunk, pl.n_jc,
                                                               step0, nsteps, err);
   else
-    k_small_steps<MODE, false><<<1, SMALL_THREADS, smem, st>>>(p, s, pl.block, (int)pl.jchunk, pl.n_jc,
+    k_small_steps<MODE, false><<<1, SMALL_BLOCK, smem, st>>>(p, s, pl.block, (int)pl.jchunk, pl.n_jc,
                                                                step0, nsteps, err);
   return cudaGetLastError();
 }

@@ -115,45 +115,49 @@ __device__ __forceinline__ KickConst kick_consts(const Phys &p, const StateView 
   return k;
 }
 
-// Kick of ion i at positions r (step index snew, time t0 + snew dt), given
-// its pair sum cs = sum_j w_j (r_i - r_j) / s_ij^3 and its constants kc:
+// The trap acceleration (Eq. 1) is linear in the position: a_k = f_k(t) r_k for
+// the reference species, with the products of trap_accel.  The factors depend on
+// the time alone; the RF trap's take an FP64 cosine, a long dependent chain, so a
+// kernel forms them beside the pair sums, not after them.
+struct TrapFactors {
+  double f[3];
+};
+__device__ __forceinline__ TrapFactors trap_factors(const Phys &p, int64_t snew) {
+  TrapFactors tf;
+  const double t = p.t0 + (double)snew * p.dt;
+  trap_accel(p, t, 1.0, 1.0, 1.0, tf.f[0], tf.f[1], tf.f[2]);
+  return tf;
+}
+
+// The Langevin draws of ion i at step snew (zeros without noise).
+__device__ __forceinline__ void kick_noise(const Phys &p, int64_t i, int64_t snew, double xi[3]) {
+  xi[0] = xi[1] = xi[2] = 0.0;
+  if (p.noise_T > 0.0) normals3(p.seed, p.instance, snew, i, xi);
+}
+
+// Kick of an ion at positions r (step index snew, time t0 + snew dt), given
+// its pair sum cs = sum_j w_j (r_i - r_j) / s_ij^3, its constants kc, the trap's
+// factors at that time and its draws xi:
 //   a+_cons = k_C q_i/m_i cs + trap(r, t)   (Eq. 1)
 //   v+ = (v + (a + a+_cons) dt/2) * [1 / (1 + gamma dt/(2 m_i))]  [+ Langevin kick]
 //   a+ = a+_cons - (gamma/m_i) v+
 // v and a hold the ion's velocity and acceleration on entry and the new ones
 // on return.  Returns true if any of them is not finite.
-__device__ __forceinline__ bool verlet_kick_k(const Phys &p, const KickConst &kc, int64_t i,
-                                              int64_t snew, const double r[3], const double cs[3],
-                                              double v[3], double a[3]) {
-  const double dt = p.dt;
-  const double t = p.t0 + (double)snew * dt;
-  double tr[3];
-  trap_accel(p, t, r[0], r[1], r[2], tr[0], tr[1], tr[2]);
-  tr[0] *= kc.ts;
-  tr[1] *= kc.ts;
-  tr[2] *= kc.ts;
-  double xi[3] = {0.0, 0.0, 0.0};
-  if (p.noise_T > 0.0) normals3(p.seed, p.instance, snew, i, xi);
+__device__ __forceinline__ bool verlet_kick(double dt, const KickConst &kc, const TrapFactors &tf, const double xi[3],
+                                            const double r[3], const double cs[3], double v[3], double a[3]) {
   bool bad = false;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const double ucons = kc.pref * cs[k] + tr[k];
-    double vn = (v[k] + 0.5 * dt * (a[k] + ucons)) * kc.inv;
-    vn += kc.sig * xi[k];
-    const double an = ucons - kc.g * vn;
+    const double tr = __dmul_rn(__dmul_rn(tf.f[k], r[k]), kc.ts);
+    const double ucons = __fma_rn(kc.pref, cs[k], tr);
+    double vn = __fma_rn(0.5 * dt, a[k] + ucons, v[k]) * kc.inv;
+    vn = __fma_rn(kc.sig, xi[k], vn);
+    const double an = __fma_rn(-kc.g, vn, ucons);
     v[k] = vn;
     a[k] = an;
     bad |= not_finite(vn) || not_finite(an);
   }
   return bad;
-}
-
-// The kick with its constants formed on the spot; ion i of the view is ion
-// s.ion0 + i of the system, which keys its Langevin draws.
-__device__ __forceinline__ bool verlet_kick(const Phys &p, const StateView &s, int64_t i,
-                                            int64_t snew, const double r[3], const double cs[3],
-                                            double v[3], double a[3]) {
-  return verlet_kick_k(p, kick_consts(p, s, i), s.ion0 + i, snew, r, cs, v, a);
 }
 
 }  // namespace nb
