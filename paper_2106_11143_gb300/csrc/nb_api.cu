@@ -230,6 +230,7 @@ cudaError_t launch_pairs(const Plan &pl, int mode, int64_t n, const double *x, c
                          const double *q, const PosF32 &pf, double soft2, double *part, unsigned *err,
                          cudaStream_t st) {
   if (tri_serves(pl, mode, soft2)) return launch_pair_tri(pl, mode, n, x, y, z, q, soft2, part, err, st);
+  if (one_serves(pl, mode, n)) return launch_pair_one(pl, n, 0, n, x, y, z, q, soft2, part, st);
   return launch_pair_force(pl, mode, n, x, y, z, q, pf, soft2, part, err, st);
 }
 
@@ -670,8 +671,11 @@ nb_status range_pair_sums(const nb_params *params, const nb_system *sys, int64_t
     pf = PosF32{split, split + n, split + 2 * n, split + 3 * n, split + 4 * n, split + 5 * n};
   }
   timing_begin(st);
-  NB_CUDA_TRY(launch_pair_force_range(pl, mode, n, i0, ni, sys->x, sys->y, sys->z, sys->q, pf, params->soft2,
-                                      part, st));
+  if (one_serves(pl, mode, n))
+    NB_CUDA_TRY(launch_pair_one(pl, n, i0, ni, sys->x, sys->y, sys->z, sys->q, params->soft2, part, st));
+  else
+    NB_CUDA_TRY(launch_pair_force_range(pl, mode, n, i0, ni, sys->x, sys->y, sys->z, sys->q, pf, params->soft2,
+                                        part, st));
   timing_end(st);
   count_launches(1);
   *part_out = part;

@@ -425,6 +425,10 @@ bool tri_serves(const Plan &pl, int mode, double soft2);
 cudaError_t launch_pair_tri(const Plan &pl, int mode, int64_t n, const double *x, const double *y, const double *z,
                             const double *q, double soft2, double *part, unsigned *err, cudaStream_t st);
 
+// The same for the one-sided sums of ions [i0, i0 + ni) (nb_one.cu).
+bool one_serves(const Plan &pl, int mode, int64_t n);
+cudaError_t launch_pair_one(const Plan &pl, int64_t n, int64_t i0, int64_t ni, const double *x, const double *y,
+                            const double *z, const double *q, double soft2, double *part, cudaStream_t st);
 
 // The potential by the same arithmetic (nb_phi.cu): blocks of 32 G ions, the
 // block count and the output mode of a call at n ions (G = 0: the one-sided
