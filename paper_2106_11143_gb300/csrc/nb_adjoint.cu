@@ -55,56 +55,58 @@ __global__ void k_adj_init(Phys p, int64_t n, CVec3 xT, CVec3 aT, CVec3 tgt, Vec
 //   g = J^T ab;  xb += g;  wacc += ab (-2 w x);
 // and unless `last`:  vb' = vb + dt xb;  ab = dt/2 vb + dt^2/2 xb (+ dt/2 vb'
 // when `more`, the next iteration's first line);  vb = vb'.
-// With EIGHT (eight slots or more) eight threads per ion sum them (nb_epi.cuh)
-// and a ninth warp, its state loaded before the barrier, finishes; otherwise one
-// thread per ion does both.  The slots are added in the same order either way.
-// Loss and gradient of 20 steps at n = 4096 (32 slots): 5.17 ms with one thread
-// per ion adding them in a chain, 4.82 ms with eight.
+// With EIGHT (eight slots or more) eight threads per ion sum them and warp 8 + c,
+// its state loaded before the barrier, finishes component c (nb_epi.cuh);
+// otherwise one thread per ion does it all.  The slots are added in the same
+// order either way.  Loss and gradient of 20 steps at n = 4096 (32 slots): 5.17 ms
+// with one thread per ion adding them in a chain, 4.82 ms with one finishing warp,
+// 4.74 with three.
 template <bool EIGHT>
-__global__ void __launch_bounds__(EIGHT ? EPI8_THREADS : 256)
+__global__ void __launch_bounds__(EIGHT ? EPI8_THREADS_COMP : 256)
     k_adj_epi(Phys p, int64_t n, const double *q, CVec3 x, const double *__restrict__ part, int n_jc, Vec3 xb, Vec3 vb,
               Vec3 ab, Vec3 wacc, int last, int more) {
+  constexpr int NC = EIGHT ? 1 : 3;
   const int64_t i = EIGHT ? (int64_t)blockIdx.x * EPI8_IONS + (threadIdx.x & 31)
                           : (int64_t)blockIdx.x * 256 + threadIdx.x;
-  const bool own = (!EIGHT || epi8_slots(part, n_jc, n)) && i < n;
-  const double *xs[3] = {x.x, x.y, x.z};
-  double *xbs[3] = {xb.x, xb.y, xb.z}, *vbs[3] = {vb.x, vb.y, vb.z}, *abs_[3] = {ab.x, ab.y, ab.z};
-  double *ws[3] = {wacc.x, wacc.y, wacc.z};
-  double lam[3], xbo[3], wo[3], vbo[3], xo[3], pref = 0.0;
+  const int fin = EIGHT ? epi8_slots(part, n_jc, n) : 0;
+  const bool own = fin >= 0 && i < n;
+  const double *const xs[3] = {x.x, x.y, x.z};
+  double *const xbs[3] = {xb.x, xb.y, xb.z}, *const vbs[3] = {vb.x, vb.y, vb.z};
+  double *const abs_[3] = {ab.x, ab.y, ab.z}, *const ws[3] = {wacc.x, wacc.y, wacc.z};
+  double lam[NC], xbo[NC], wo[NC], vbo[NC], xo[NC], om[NC], pref = 0.0;
   if (own) {
     pref = pref_of(p, q, i);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      lam[k] = abs_[k][i];
-      xbo[k] = xbs[k][i];
-      wo[k] = ws[k][i];
-      vbo[k] = vbs[k][i];
-      xo[k] = xs[k][i];
+    for (int k = 0; k < NC; ++k) {
+      const int c = EIGHT ? fin : k;
+      lam[k] = (c == 0 ? abs_[0] : c == 1 ? abs_[1] : abs_[2])[i];
+      xbo[k] = (c == 0 ? xbs[0] : c == 1 ? xbs[1] : xbs[2])[i];
+      wo[k] = (c == 0 ? ws[0] : c == 1 ? ws[1] : ws[2])[i];
+      vbo[k] = (c == 0 ? vbs[0] : c == 1 ? vbs[1] : vbs[2])[i];
+      xo[k] = (c == 0 ? xs[0] : c == 1 ? xs[1] : xs[2])[i];
+      om[k] = c == 0 ? p.omega[0] : c == 1 ? p.omega[1] : p.omega[2];
     }
   }
   if (EIGHT) __syncthreads();
   if (!own) return;
-  double cs[3];
-  if (EIGHT) {
-    epi8_total(cs);
-  } else {
-    const double *pi = part + i;
-    slot_sum3(n_jc, [&](int jc, int c) { return pi[((int64_t)jc * 3 + c) * n]; }, cs);
-  }
   const double dt = p.dt;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const double w2 = p.omega[k] * p.omega[k];
-    const double g = pref * cs[k] - w2 * lam[k];
+  for (int k = 0; k < NC; ++k) {
+    const int c = EIGHT ? fin : k;
+    const double *pi = part + i;
+    const double cs = EIGHT ? epi8_total(c)
+                            : slot_sum1(n_jc, [&](int jc) { return __ldcs(pi + ((int64_t)jc * 3 + c) * n); });
+    const double w2 = om[k] * om[k];
+    const double g = pref * cs - w2 * lam[k];
     const double xbn = xbo[k] + g;
-    ws[k][i] = wo[k] + lam[k] * (-2.0 * p.omega[k] * xo[k]);
-    xbs[k][i] = xbn;
+    (c == 0 ? ws[0] : c == 1 ? ws[1] : ws[2])[i] = wo[k] + lam[k] * (-2.0 * om[k] * xo[k]);
+    (c == 0 ? xbs[0] : c == 1 ? xbs[1] : xbs[2])[i] = xbn;
     if (!last) {
       const double vbn = vbo[k] + dt * xbn;
       double a = 0.5 * dt * vbo[k] + 0.5 * dt * dt * xbn;
       if (more) a += 0.5 * dt * vbn;
-      abs_[k][i] = a;
-      vbs[k][i] = vbn;
+      (c == 0 ? abs_[0] : c == 1 ? abs_[1] : abs_[2])[i] = a;
+      (c == 0 ? vbs[0] : c == 1 ? vbs[1] : vbs[2])[i] = vbn;
     }
   }
 }
@@ -217,7 +219,7 @@ cudaError_t launch_adj_epi(const Phys &p, int64_t n, const double *q, const doub
                            double *const ab[3], double *const wacc[3], int last, int more,
                            cudaStream_t st) {
   if (n_jc >= 8)
-    k_adj_epi<true><<<nblk(n, EPI8_IONS), EPI8_THREADS, 0, st>>>(p, n, q, CVec3{x[0], x[1], x[2]}, part, n_jc,
+    k_adj_epi<true><<<nblk(n, EPI8_IONS), EPI8_THREADS_COMP, 0, st>>>(p, n, q, CVec3{x[0], x[1], x[2]}, part, n_jc,
         Vec3{xb[0], xb[1], xb[2]}, Vec3{vb[0], vb[1], vb[2]},
         Vec3{ab[0], ab[1], ab[2]}, Vec3{wacc[0], wacc[1], wacc[2]},
         last, more);

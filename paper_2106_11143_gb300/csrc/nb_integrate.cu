@@ -16,20 +16,21 @@ __device__ __forceinline__ double chunk_sum(const double *__restrict__ part, int
 }
 
 // The three components of ion i's chunk partials, part[(jc*3 + c)*n + i],
-// summed by slot_sum3 with streaming loads (the partials are read once).
+// summed in slot_sum1's order with streaming loads (the partials are read once).
 __device__ __forceinline__ void chunk_sum3(const double *__restrict__ part, int n_jc, int64_t n,
                                            int64_t i, double out[3]) {
   const double *p = part + i;
-  slot_sum3(n_jc, [&](int jc, int c) { return __ldcs(p + ((int64_t)jc * 3 + c) * n); }, out);
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    out[c] = slot_sum1(n_jc, [&](int jc) { return __ldcs(p + ((int64_t)jc * 3 + c) * n); });
 }
 
 // The epilogues run one of two ways:
 //  - one thread per ion, EPI_THREADS per block, adding its chunk partials with
 //    chunk_sum3;
 //  - eight threads per ion (the default with eight slots or more): warp u of a
-//    block forms slot_sum3's running sum u for the block's 32 ions (nb_epi.cuh)
-//    and a ninth warp adds the eight in slot_sum3's pairing and finishes one ion
-//    per lane.
+//    block forms slot_sum1's running sum u for the block's 32 ions, further warps
+//    add the eight in slot_sum1's pairing and finish one ion per lane (nb_epi.cuh).
 // Both give the same sums, bit for bit.
 constexpr int EPI_THREADS = 256;
 
@@ -59,10 +60,11 @@ __device__ __forceinline__ bool epi_sums(const double *__restrict__ part, int n_
     return true;
   }
   i = (int64_t)blockIdx.x * EPI8_IONS + (threadIdx.x & 31);
-  const bool last = epi8_slots(part, n_jc, n);
+  const bool last = epi8_slots(part, n_jc, n) == 0;
   __syncthreads();
   if (!last || i >= n) return false;
-  epi8_total(cs);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) cs[c] = epi8_total(c);
   return true;
 }
 
@@ -170,7 +172,8 @@ __global__ void k_drift(Phys p, StateView s, double *px, double *py, double *pz,
   px[i] = r[0];
   py[i] = r[1];
   pz[i] = r[2];
-  if (split) store_split(split, s.n, i, r);
+  if (split)
+    for (int c = 0; c < 3; ++c) store_split(split, s.n, i, c, r[c]);
 }
 
 cudaError_t launch_drift_split(const Phys &p, const StateView &s, double *px, double *py, double *pz, float *split,
@@ -197,85 +200,120 @@ cudaError_t launch_drift(const Phys &p, const StateView &s, double *px, double *
 // a step index that advances from replay to replay (cin and cout are never
 // the same word, so no thread reads what another writes).
 //
-// In the eight-thread form the ninth warp has everything that does not depend
-// on the sums in registers before the barrier: its ion's state, the kick's
-// constants (three FP64 divisions), the trap's factors (an FP64 cosine in the RF
-// trap) and the Langevin draws, all of it formed while the other warps wait for
-// their slots.  With `split`, the next positions' FP32 (hi, lo) parts are stored
-// beside them (six floats per ion, as k_split_positions forms them), which saves
-// the split modes that kernel's launch.
+// In the eight-thread form warp 8 + c finishes component c, with everything that
+// does not depend on the sums formed before the barrier, while the other warps
+// wait for their slots: its component's state, its trap factor (an FP64 cosine in
+// the RF trap) and the Langevin draws.  The kick's constants (four FP64 divisions,
+// 2800 cycles of one warp) come from the host (kc) unless the ions have charges or
+// masses of their own (own_kc); then each finishing warp forms a part of them.
+// The one-thread form takes the trap's factors from its block's first warp.
+// With `split`, the next positions' FP32 (hi, lo) parts are stored beside them
+// (six floats per ion, as k_split_positions forms them), which saves the split
+// modes that kernel's launch.
 template <bool EIGHT>
-__device__ __forceinline__ void epi_step(const Phys &p, const StateView &s, const double *cx,
+__device__ __forceinline__ void epi_step(const Phys &p, const StateView &s, KickConst kc, bool own_kc, const double *cx,
                                          const double *cy, const double *cz, const double *part, int n_jc,
                                          int64_t soff, const int64_t *cin, int64_t *cout, int64_t cout_off,
                                          double *nx, double *ny, double *nz, float *split, unsigned *err) {
-  const int64_t i = EIGHT ? (int64_t)blockIdx.x * EPI8_IONS + (threadIdx.x & 31)
-                          : (int64_t)blockIdx.x * EPI_THREADS + threadIdx.x;
-  const bool last = !EIGHT || epi8_slots(part, n_jc, s.n);
-  if (!EIGHT && i >= s.n) return;
-  double r[3], v[3], a[3], xi[3];
-  KickConst kc;
-  TrapFactors tf;
-  const bool own = last && i < s.n;
-  int64_t base = 0;
-  if (own) {
-    r[0] = cx[i]; r[1] = cy[i]; r[2] = cz[i];
-    v[0] = s.vx[i]; v[1] = s.vy[i]; v[2] = s.vz[i];
-    a[0] = s.ax[i]; a[1] = s.ay[i]; a[2] = s.az[i];
-    base = cin ? *cin : 0;
-    kc = kick_consts(p, s, i);
-    tf = trap_factors(p, base + soff);
-    kick_noise(p, s.ion0 + i, base + soff, xi);
+  constexpr int NC = EIGHT ? 1 : 3;
+  __shared__ KickConst s_kc[EIGHT ? EPI8_IONS : 1];
+  __shared__ TrapFactors s_tf;
+  const int lane = threadIdx.x & 31;
+  const int64_t i = EIGHT ? (int64_t)blockIdx.x * EPI8_IONS + lane : (int64_t)blockIdx.x * EPI_THREADS + threadIdx.x;
+  const int fin = EIGHT ? epi8_slots(part, n_jc, s.n) : 0;
+  const bool own = fin >= 0 && i < s.n;
+  const double *const cs_[3] = {cx, cy, cz};
+  double *const vs[3] = {s.vx, s.vy, s.vz}, *const as[3] = {s.ax, s.ay, s.az}, *const xs[3] = {s.x, s.y, s.z};
+  double *const ns[3] = {nx, ny, nz};
+  double r[NC], v[NC], a[NC], xi[NC], tf[NC];
+  const int64_t base = cin ? *cin : 0;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    const int c = EIGHT ? fin : k;
+    xi[k] = tf[k] = 0.0;
+    if (!own) continue;
+    r[k] = (c == 0 ? cs_[0] : c == 1 ? cs_[1] : cs_[2])[i];
+    v[k] = (c == 0 ? vs[0] : c == 1 ? vs[1] : vs[2])[i];
+    a[k] = (c == 0 ? as[0] : c == 1 ? as[1] : as[2])[i];
   }
+  if (EIGHT && fin >= 0) tf[0] = trap_factor1(p, base + soff, fin);
+  if (!EIGHT && threadIdx.x < 32) {
+    const TrapFactors f = trap_factors(p, base + soff);
+    if (lane == 0) s_tf = f;
+  }
+  if (own && p.noise_T > 0.0) {
+    double all[3];
+    kick_noise(p, s.ion0 + i, base + soff, all);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) xi[k] = !EIGHT ? all[k] : (fin == 0 ? all[0] : fin == 1 ? all[1] : all[2]);
+  }
+  if (own && own_kc) {
+    if (!EIGHT) {
+      kc = kick_consts(p, s, i);
+    } else if (fin == 0) {
+      s_kc[lane].pref = coulomb_pref(p, s, i);
+    } else if (fin == 1) {
+      s_kc[lane].inv = kick_inv(p, ion_mass(p, s, i));
+      s_kc[lane].sig = kick_sig(p, ion_mass(p, s, i));
+    } else {
+      s_kc[lane].ts = trap_scale(p, s, i);
+      s_kc[lane].g = p.gamma / ion_mass(p, s, i);
+    }
+  }
+  __syncthreads();
+  if (!own) return;
+  if (EIGHT && own_kc) kc = s_kc[lane];
   double cs[3];
-  if (EIGHT) {
-    __syncthreads();
-    if (!own) return;
-    epi8_total(cs);
-  } else {
+  if (EIGHT)
+    cs[0] = epi8_total(fin);
+  else
     chunk_sum3(part, n_jc, s.n, i, cs);
-  }
-  if (cout && i == 0) *cout = base + cout_off;
-  const bool bad = verlet_kick(p.dt, kc, tf, xi, r, cs, v, a);
-  s.vx[i] = v[0]; s.vy[i] = v[1]; s.vz[i] = v[2];
-  s.ax[i] = a[0]; s.ay[i] = a[1]; s.az[i] = a[2];
-  if (nx) {
-    const double rn[3] = {verlet_drift(r[0], v[0], a[0], p.dt), verlet_drift(r[1], v[1], a[1], p.dt),
-                          verlet_drift(r[2], v[2], a[2], p.dt)};
-    nx[i] = rn[0];
-    ny[i] = rn[1];
-    nz[i] = rn[2];
-    if (split) store_split(split, s.n, i, rn);
-  } else {
-    s.x[i] = r[0]; s.y[i] = r[1]; s.z[i] = r[2];
+  if (cout && i == 0 && fin == 0) *cout = base + cout_off;
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    const int c = EIGHT ? fin : k;
+    if (!EIGHT) tf[k] = s_tf.f[k];
+    bad |= verlet_kick1(p.dt, kc, tf[k], xi[k], r[k], cs[k], v[k], a[k]);
+    (c == 0 ? vs[0] : c == 1 ? vs[1] : vs[2])[i] = v[k];
+    (c == 0 ? as[0] : c == 1 ? as[1] : as[2])[i] = a[k];
+    if (nx) {
+      const double rn = verlet_drift(r[k], v[k], a[k], p.dt);
+      (c == 0 ? ns[0] : c == 1 ? ns[1] : ns[2])[i] = rn;
+      if (split) store_split(split, s.n, i, c, rn);
+    } else {
+      (c == 0 ? xs[0] : c == 1 ? xs[1] : xs[2])[i] = r[k];
+    }
   }
   if (bad) atomicOr(err, ERR_NONFINITE);
 }
 __global__ void __launch_bounds__(EPI_THREADS)
-    k_epi_step(Phys p, StateView s, const double *__restrict__ cx, const double *__restrict__ cy,
-               const double *__restrict__ cz, const double *__restrict__ part, int n_jc, int64_t soff,
-               const int64_t *cin, int64_t *cout, int64_t cout_off, double *nx, double *ny, double *nz,
+    k_epi_step(Phys p, StateView s, KickConst kc, int own_kc, const double *__restrict__ cx,
+               const double *__restrict__ cy, const double *__restrict__ cz, const double *__restrict__ part, int n_jc,
+               int64_t soff, const int64_t *cin, int64_t *cout, int64_t cout_off, double *nx, double *ny, double *nz,
                float *split, unsigned *err) {
-  epi_step<false>(p, s, cx, cy, cz, part, n_jc, soff, cin, cout, cout_off, nx, ny, nz, split, err);
+  epi_step<false>(p, s, kc, own_kc, cx, cy, cz, part, n_jc, soff, cin, cout, cout_off, nx, ny, nz, split, err);
 }
-__global__ void __launch_bounds__(EPI8_THREADS)
-    k_epi_step8(Phys p, StateView s, const double *__restrict__ cx, const double *__restrict__ cy,
-                const double *__restrict__ cz, const double *__restrict__ part, int n_jc, int64_t soff,
-                const int64_t *cin, int64_t *cout, int64_t cout_off, double *nx, double *ny, double *nz,
+__global__ void __launch_bounds__(EPI8_THREADS_COMP)
+    k_epi_step8(Phys p, StateView s, KickConst kc, int own_kc, const double *__restrict__ cx,
+                const double *__restrict__ cy, const double *__restrict__ cz, const double *__restrict__ part, int n_jc,
+                int64_t soff, const int64_t *cin, int64_t *cout, int64_t cout_off, double *nx, double *ny, double *nz,
                 float *split, unsigned *err) {
-  epi_step<true>(p, s, cx, cy, cz, part, n_jc, soff, cin, cout, cout_off, nx, ny, nz, split, err);
+  epi_step<true>(p, s, kc, own_kc, cx, cy, cz, part, n_jc, soff, cin, cout, cout_off, nx, ny, nz, split, err);
 }
 
 cudaError_t launch_epi_step_split(const Phys &p, const StateView &s, const double *cx, const double *cy,
                                   const double *cz, const double *part, int n_jc, int64_t snew,
                                   double *nx, double *ny, double *nz, float *split, unsigned *err, cudaStream_t st,
                                   const int64_t *cin, int64_t *cout, int64_t cout_off) {
+  const bool own_kc = s.q || s.m;
+  const KickConst kc = own_kc ? KickConst{} : uniform_kick_consts(p);
   if (epi_eight(s.n, n_jc))
-    k_epi_step8<<<epi_blocks(s.n, true), EPI8_THREADS, 0, st>>>(p, s, cx, cy, cz, part, n_jc, snew, cin, cout,
-                                                                 cout_off, nx, ny, nz, split, err);
+    k_epi_step8<<<epi_blocks(s.n, true), EPI8_THREADS_COMP, 0, st>>>(p, s, kc, own_kc, cx, cy, cz, part, n_jc, snew,
+                                                                      cin, cout, cout_off, nx, ny, nz, split, err);
   else
-    k_epi_step<<<epi_blocks(s.n, false), EPI_THREADS, 0, st>>>(p, s, cx, cy, cz, part, n_jc, snew, cin, cout,
-                                                                cout_off, nx, ny, nz, split, err);
+    k_epi_step<<<epi_blocks(s.n, false), EPI_THREADS, 0, st>>>(p, s, kc, own_kc, cx, cy, cz, part, n_jc, snew, cin,
+                                                                cout, cout_off, nx, ny, nz, split, err);
   return cudaGetLastError();
 }
 cudaError_t launch_epi_step(const Phys &p, const StateView &s, const double *cx, const double *cy,

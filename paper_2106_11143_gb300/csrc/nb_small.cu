@@ -14,7 +14,7 @@
 // plan: ion i against the partners of j-chunk jc, in tiles of the plan's
 // block size, with the same pair term and the same per-tile flushes
 // (nb_pairterm.cuh).  It keeps the chunk partials in shared memory and adds
-// them in the epilogue's order (slot_sum3).  It then applies the same kick
+// them in the epilogue's order (slot_sum1).  It then applies the same kick
 // and drift (nb_verlet.cuh).  Each ion's result is therefore bitwise that of
 // the multi-kernel path.
 #include <mutex>
@@ -116,30 +116,6 @@ __device__ __forceinline__ void stage_comp(D4 *pos, float4 *sp, int i, int c, do
     reinterpret_cast<float *>(sp + 2 * i)[c] = h;
     reinterpret_cast<float *>(sp + 2 * i + 1)[c] = __double2float_rn(r - (double)h);
   }
-}
-
-// slot_sum3 for one component, with the same bits and fewer FP64 adds: its
-// 0 + v of a running sum's first slot is v with -0 made +0, and adding a running
-// sum that no slot went to changes nothing (none is ever -0).
-template <class LD>
-__device__ __forceinline__ double slot_sum1(int n_jc, LD ld) {
-  double s[8];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    double v = u < n_jc ? ld(u) : 0.0;
-    if (__double2hiint(v) == (int)0x80000000 && __double2loint(v) == 0) v = 0.0;
-    s[u] = v;
-  }
-  for (int jc = 8; jc < n_jc; jc += 8)
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (jc + u < n_jc) s[u] += ld(jc + u);
-#pragma unroll
-  for (int w = 1; w < 8; w <<= 1)
-#pragma unroll
-    for (int u = 0; u < 8; u += 2 * w)
-      if (u + w < n_jc) s[u] += s[u + w];
-  return s[0];
 }
 
 // One warp beyond the SMALL_THREADS of the pair items holds the trap's factors.

@@ -6,6 +6,8 @@
 // an ion given the same inputs gets the same bits on every path.
 #pragma once
 
+#include <cmath>
+
 #include "nb_common.cuh"
 
 namespace nb {
@@ -51,43 +53,32 @@ __device__ __forceinline__ double coulomb_pref(const Phys &p, const StateView &s
   return s.q ? p.k_coulomb * s.q[i] / m : p.k_coulomb * p.charge * p.charge / m;
 }
 
-// Sum of the n_jc chunk partials (x, y, z) of one ion, as eight interleaved
-// running sums (chunk jc goes to sum jc mod 8) added pairwise at the end.
-// The dependent chain is n_jc/8 + 3 FP64 adds instead of n_jc: at small n the
-// latency of that chain, not the bandwidth, bounds the epilogue.  ld(jc, c)
-// returns component c of chunk jc; the loads of eight chunks are issued
-// before their adds.
+// Sum of the n_jc chunk partials of one component of an ion, as eight interleaved
+// running sums (chunk jc goes to sum jc mod 8, from zero) added pairwise at the
+// end.  The dependent chain is n_jc/8 + 3 FP64 adds instead of n_jc: at small n
+// the latency of that chain, not the bandwidth, bounds the epilogue.  ld(jc)
+// returns chunk jc; the loads of eight chunks are issued before their adds.
+// FP64 adds of zeros are left out (64 cycles of an SMSP each): 0 + v is v with -0
+// made +0, and adding a running sum that no slot went to changes nothing, since
+// none is ever -0.
+__device__ __forceinline__ double no_neg_zero(double v) {
+  return __double2hiint(v) == (int)0x80000000 && __double2loint(v) == 0 ? 0.0 : v;
+}
 template <class LD>
-__device__ __forceinline__ void slot_sum3(int n_jc, LD ld, double out[3]) {
-  double s[8][3];
+__device__ __forceinline__ double slot_sum1(int n_jc, LD ld) {
+  double s[8];
 #pragma unroll
-  for (int u = 0; u < 8; ++u) s[u][0] = s[u][1] = s[u][2] = 0.0;
-  int jc = 0;
-  for (; jc + 8 <= n_jc; jc += 8) {
-    double v[8][3];
+  for (int u = 0; u < 8; ++u) s[u] = u < n_jc ? no_neg_zero(ld(u)) : 0.0;
+  for (int jc = 8; jc < n_jc; jc += 8)
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      v[u][0] = ld(jc + u, 0);
-      v[u][1] = ld(jc + u, 1);
-      v[u][2] = ld(jc + u, 2);
-    }
+    for (int u = 0; u < 8; ++u)
+      if (jc + u < n_jc) s[u] += ld(jc + u);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      s[u][0] += v[u][0];
-      s[u][1] += v[u][1];
-      s[u][2] += v[u][2];
-    }
-  }
+  for (int w = 1; w < 8; w <<= 1)
 #pragma unroll
-  for (int u = 0; u < 7; ++u)
-    if (jc + u < n_jc) {
-      s[u][0] += ld(jc + u, 0);
-      s[u][1] += ld(jc + u, 1);
-      s[u][2] += ld(jc + u, 2);
-    }
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-    out[c] = ((s[0][c] + s[1][c]) + (s[2][c] + s[3][c])) + ((s[4][c] + s[5][c]) + (s[6][c] + s[7][c]));
+    for (int u = 0; u < 8; u += 2 * w)
+      if (u + w < n_jc) s[u] += s[u + w];
+  return s[0];
 }
 
 // Drift of one coordinate: r + v dt + a dt^2/2.
@@ -104,14 +95,27 @@ __device__ __forceinline__ double verlet_drift(double r, double v, double a, dou
 struct KickConst {
   double pref, ts, inv, g, sig;
 };
+__device__ __forceinline__ double kick_inv(const Phys &p, double mi) {
+  return 1.0 / (1.0 + p.gamma * p.dt / (2.0 * mi));
+}
+__device__ __forceinline__ double kick_sig(const Phys &p, double mi) {
+  return p.noise_T > 0.0 ? sqrt(2.0 * p.gamma * KB * p.noise_T * p.dt) / mi : 0.0;
+}
 __device__ __forceinline__ KickConst kick_consts(const Phys &p, const StateView &s, int64_t i) {
-  KickConst k;
-  k.pref = coulomb_pref(p, s, i);
-  k.ts = trap_scale(p, s, i);
   const double mi = ion_mass(p, s, i);
-  k.inv = 1.0 / (1.0 + p.gamma * p.dt / (2.0 * mi));
-  k.g = p.gamma / mi;
-  k.sig = p.noise_T > 0.0 ? sqrt(2.0 * p.gamma * KB * p.noise_T * p.dt) / mi : 0.0;
+  return KickConst{coulomb_pref(p, s, i), trap_scale(p, s, i), kick_inv(p, mi), p.gamma / mi, kick_sig(p, mi)};
+}
+
+// The same for all ions where they have the reference charge and mass, formed on
+// the host: every operation is correctly rounded and none is an a b + c to fuse,
+// so the bits are kick_consts'.
+inline KickConst uniform_kick_consts(const Phys &p) {
+  KickConst k;
+  k.pref = p.k_coulomb * p.charge * p.charge / p.mass;
+  k.ts = 1.0;
+  k.inv = 1.0 / (1.0 + p.gamma * p.dt / (2.0 * p.mass));
+  k.g = p.gamma / p.mass;
+  k.sig = p.noise_T > 0.0 ? std::sqrt(2.0 * p.gamma * KB * p.noise_T * p.dt) / p.mass : 0.0;
   return k;
 }
 
@@ -127,6 +131,11 @@ __device__ __forceinline__ TrapFactors trap_factors(const Phys &p, int64_t snew)
   const double t = p.t0 + (double)snew * p.dt;
   trap_accel(p, t, 1.0, 1.0, 1.0, tf.f[0], tf.f[1], tf.f[2]);
   return tf;
+}
+// Component c of them: a branch that a warp of one component takes as one.
+__device__ __forceinline__ double trap_factor1(const Phys &p, int64_t snew, int c) {
+  const TrapFactors tf = trap_factors(p, snew);
+  return c == 0 ? tf.f[0] : c == 1 ? tf.f[1] : tf.f[2];
 }
 
 // The Langevin draws of ion i at step snew (zeros without noise).
