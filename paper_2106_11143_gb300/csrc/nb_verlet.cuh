@@ -68,7 +68,10 @@ template <class LD>
 __device__ __forceinline__ double slot_sum1(int n_jc, LD ld) {
   double s[8];
 #pragma unroll
-  for (int u = 0; u < 8; ++u) s[u] = u < n_jc ? no_neg_zero(ld(u)) : 0.0;
+  for (int u = 0; u < 8; ++u) {
+    const double v = u < n_jc ? ld(u) : 0.0;
+    s[u] = no_neg_zero(v);
+  }
   for (int jc = 8; jc < n_jc; jc += 8)
 #pragma unroll
     for (int u = 0; u < 8; ++u)
