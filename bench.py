@@ -39,15 +39,18 @@ FLOPS_PER_PAIR = 20
 # displacement and the widening of r^-3); everything else runs on the FP32 pipe.
 FP64_FLOPS_PER_EVAL_SYM = 2 * 6 + 4
 SM_COUNT = 152
-# The pipe whose rate bounds each path's pair kernel, and the probe kind that
-# measures it (nb_pipe_probe; 2 flops per FMA lane).
+# The pipe whose rate bounds each path's pair kernel of nb_sym.cu and nb_pair.cu,
+# and the probe kind that measures it (nb_pipe_probe; 2 flops per FMA lane).  The
+# kernels of nb_tri.cu and nb_one.cu (pair_kernel) are all bound by the FP32 pipe.
 PATH_PIPE = {"fp64": "dfma", "df64": "ffma", "mixed": "ffma", "mixed_split": "ffma", "mixed_split_rsq": "ffma"}
 DTYPE = {"fp64": "f64", "df64": "f32x2+f64", "mixed": "f32+f64", "mixed_split": "f32+f64", "mixed_split_rsq": "f32+f64"}
 ACCURACY_GATE = {"fp64": 1e-12, "df64": 1e-12, "mixed": 1e-6, "mixed_split": 1e-6, "mixed_split_rsq": 1e-6}
 PATHS = ("fp64", "df64", "mixed", "mixed_split", "mixed_split_rsq")
 PROFILES = os.path.join(ROOT, "profiles")
-# Kernel sources a recorded DRAM-traffic figure is valid for.
+# Kernel sources a recorded DRAM-traffic figure is valid for: those of the kernels
+# of nb_sym.cu and nb_pair.cu, and those of nb_tri.cu's (k_pair_sym_tri).
 KERNEL_SOURCES = ("nb_sym.cu", "nb_symsched.cuh", "nb_pair.cu", "nb_common.cuh", "nb_pairterm.cuh")
+TRI_SOURCES = ("nb_tri.cu", "nb_tri.cuh", "nb_symsched.cuh", "nb_common.cuh")
 L2_FLUSH_BYTES = 256 << 20
 
 
@@ -328,24 +331,38 @@ def evaluations(nb, precision, n):
     return (n * n + full * bi * bi + rem * rem) // 2, "k_pair_sym<%s>" % precision
 
 
-def kernel_source_sha():
+def pair_kernel(nb, precision, n):
+    """The kernel a default force evaluation launches where it is one of those
+    on three-word positions: nb_tri.cu's in the half-pair plans of fp64, df64
+    and, from 2000 ions, mixed; nb_one.cu's in the one-sided fp64 and df64 plans
+    above 512 ions; None elsewhere (nb_sym.cu and nb_pair.cu)."""
+    sym = nb.plan_info("force", precision, n)["symmetric"]
+    if sym and (precision in ("fp64", "df64") or (precision == "mixed" and n >= 2000)):
+        return "k_pair_sym_tri"
+    if not sym and precision in ("fp64", "df64") and 512 < n <= 4096:
+        return "k_pair_one"
+    return None
+
+
+def kernel_source_sha(kernel=None):
     import hashlib
     h = hashlib.sha256()
-    for f in KERNEL_SOURCES:
+    for f in TRI_SOURCES if kernel == "k_pair_sym_tri" else KERNEL_SOURCES:
         with open(os.path.join(ROOT, "paper_2106_11143_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:12]
 
 
-def recorded_counters(precision, n):
+def recorded_counters(precision, n, kernel=None):
     """ncu counters of the pair kernel per launch, from the summaries under
     profiles/: a line `traffic: precision=P n=N bytes=B [inst=I] source=S`
     records one capture of this bench's command: B the DRAM bytes (read +
     write), I the warp instructions executed (smsp__inst_executed.sum), S
-    the kernel sources' hash when it was taken.  ({}, None) when there is no
-    capture for this case or the kernel has changed since."""
+    the kernel sources' hash when it was taken; a field kernel=K names
+    pair_kernel's kernels.  ({}, None) when there is no capture for this case or
+    the kernel has changed since."""
     import glob
-    want = kernel_source_sha()
+    want = kernel_source_sha(kernel)
     out, src = {}, None
     for path in sorted(glob.glob(os.path.join(PROFILES, "*.md"))):
         for line in open(path):
@@ -353,7 +370,8 @@ def recorded_counters(precision, n):
             if not line.startswith("traffic: "):
                 continue
             kv = dict(t.split("=", 1) for t in line.split()[1:])
-            if kv.get("precision") == precision and int(kv.get("n", -1)) == n and kv.get("source") == want:
+            if (kv.get("precision") == precision and int(kv.get("n", -1)) == n and kv.get("source") == want
+                    and kv.get("kernel") == kernel):
                 for k in ("bytes", "inst", "fp64_inst"):  # the first summary naming a counter wins
                     if k in kv and k not in out:
                         out[k] = int(kv[k])
@@ -364,7 +382,7 @@ def recorded_counters(precision, n):
 OPMIX_KINDS = ("dadd", "dfma", "dmul", "fadd", "ffma", "fmul", "fadd2", "ffma2", "fmul2")
 
 
-def recorded_opmix(precision):
+def recorded_opmix(precision, kernel=None):
     """Lane-instructions per pair evaluation of the pair kernel in this
     precision, by kind (FP64 "dadd", "dfma", "dmul"; FP32 "fadd", "ffma",
     "fmul" and the packed "fadd2", "ffma2", "fmul2"), from an `opmix:` line
@@ -373,14 +391,14 @@ def recorded_opmix(precision):
     bench's with the same kernel configuration); {} when unrecorded or the
     kernel sources have changed since."""
     import glob
-    want = kernel_source_sha()
+    want = kernel_source_sha(kernel)
     for path in sorted(glob.glob(os.path.join(PROFILES, "*.md"))):
         for line in open(path):
             line = line.strip()
             if not line.startswith("opmix: "):
                 continue
             kv = dict(t.split("=", 1) for t in line.split()[1:])
-            if kv.get("precision") == precision and kv.get("source") == want:
+            if kv.get("precision") == precision and kv.get("source") == want and kv.get("kernel") == kernel:
                 return {k: float(kv[k]) for k in OPMIX_KINDS if k in kv}
     return {}
 
@@ -392,18 +410,21 @@ def recorded_traffic(precision, n):
     return c.get("bytes"), src
 
 
-def roofline(nb, path, n, kernel_ms, peaks, sm_mhz):
+def roofline(nb, path, n, kernel_ms, peaks, sm_mhz, kernel=None):
     """Roofline of the pair kernel: convention-A flops (20 per evaluation) on
     the evaluations the kernel performs, over its measured duration, against
     the measured rate of the pipe that bounds it at the SM clock sampled
-    during the timed steps."""
+    during the timed steps.  kernel: one of pair_kernel's, which the default plan
+    launches; None for nb_sym.cu's and nb_pair.cu's."""
     evals, kname = evaluations(nb, path, n)
     pipe = PATH_PIPE[path]
+    if kernel:
+        kname, pipe = "%s<%s>" % (kernel, path), "ffma"
     lanes = peaks[pipe]["lanes_per_clk_per_sm"]
     mhz = sm_mhz or peaks[pipe]["sm_mhz"]
     peak = 2 * lanes * SM_COUNT * mhz * 1e6 / 1e12
     achieved = FLOPS_PER_PAIR * evals / (kernel_ms / 1e3) / 1e12
-    counters, src = recorded_counters(path, n)
+    counters, src = recorded_counters(path, n, kernel)
     traffic = counters.get("bytes")
     r = {"bound": "alu", "pipe": "FP64 FMA" if pipe == "dfma" else "FP32 FMA",
          "achieved": round(achieved, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
@@ -444,7 +465,7 @@ def roofline(nb, path, n, kernel_ms, peaks, sm_mhz):
         # the pipe's attainable rate for this kernel's own mix of FP64 adds,
         # FMAs and multiplies, each at its measured rate (an add retires at
         # about 0.84 of an FMA's rate on this GPU)
-        mix = recorded_opmix(path)
+        mix = recorded_opmix(path, kernel)
         kinds = [k for k in ("dadd", "dfma", "dmul") if mix.get(k, 0.0) > 0.0]
         if kinds and all(k in peaks for k in kinds):
             tot = sum(mix[k] for k in kinds)
@@ -456,7 +477,7 @@ def roofline(nb, path, n, kernel_ms, peaks, sm_mhz):
             r["fp64_pipe"]["mix_note"] = ("ceiling = the kernel's FP64 lane-instructions per evaluation by kind "
                                           "(opmix, profiles/) at the measured rate of each kind: %.3f lanes/clk/SM"
                                           % lanes_mix)
-    mix = recorded_opmix(path)
+    mix = recorded_opmix(path, kernel)
     if pipe == "ffma" and all(k in mix for k in ("fadd", "ffma", "fmul", "fadd2", "ffma2", "fmul2")):
         # the FMA pipe by the work it does: each FP32 add, multiply or FMA
         # one lane-cycle, each packed .f32x2 one two lane-cycles (it holds
@@ -489,7 +510,7 @@ def roofline(nb, path, n, kernel_ms, peaks, sm_mhz):
         units.append(("FMA pipe", r["fma_pipe"]["frac"]))
     if len(units) > 1:
         r["binding"] = max(units, key=lambda u: u[1])[0]
-    if path == "fp64" and kname.startswith("k_pair_sym"):
+    if path == "fp64" and kname.startswith("k_pair_sym<"):
         b = FP64_FLOPS_PER_EVAL_SYM * evals / (kernel_ms / 1e3) / 1e12
         r["conv_B"] = {"achieved": round(b, 3), "frac": round(b / peak, 4),
                        "note": "executed FP64 flops, 2 x 6 DFMA + 4 DADD per evaluation, over the FP64 FMA peak"}
@@ -529,7 +550,8 @@ def main_ours(args):
             paths[pth] = {"value": round(n * n / (r["ms_per_step"] / 1e3) / 1e9, 3), "unit": UNIT,
                           "ms_per_step": round(r["ms_per_step"], 4),
                           "kernel_ms": round(r["kernel_ms"], 4),
-                          "roofline": roofline(nb, pth, n, r["kernel_ms"], peaks, sm_mhz)}
+                          "roofline": roofline(nb, pth, n, r["kernel_ms"], peaks, sm_mhz,
+                                                   pair_kernel(nb, pth, n))}
         paths["speedup_mixed_over_fp64"] = round(paths["fp64"]["ms_per_step"] / paths["mixed"]["ms_per_step"], 3)
         paths["speedup_mixed_split_over_fp64"] = round(
             paths["fp64"]["ms_per_step"] / paths["mixed_split"]["ms_per_step"], 3)
@@ -555,7 +577,8 @@ def main_ours(args):
                    "n": n, "precision": args.precision, "pairs_per_step": n * n,
                    "l2": "flushed between timed steps (256 MB write outside the timed events)",
                    "parallelism": "replicas" if world > 1 else "single GPU"},
-        "roofline": roofline(nb, args.precision, n, head["kernel_ms"], peaks, sm_mhz),
+        "roofline": roofline(nb, args.precision, n, head["kernel_ms"], peaks, sm_mhz,
+                             pair_kernel(nb, args.precision, n)),
         "peaks": peaks,
         "cpu_baseline": cpu,
         "e2e": e2e,

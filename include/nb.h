@@ -54,21 +54,33 @@ typedef enum {
 } nb_status;
 
 /* Arithmetic of the pair interaction (the O(N^2) inner loop).
- *  NB_FP64       -- FP64 displacement and FP64 accumulation of the forces.
- *                   In between, r^2, 1/sqrt(r^2) and r^-3 run on the FP32
- *                   pipe: the displacement is split into exponent-scaled
- *                   FP32 (hi, lo) pairs, r^2 is a double-float, the FP32
- *                   hardware reciprocal square root (MUFU) is refined by a
- *                   Newton residual formed in compensated FP32 (Sec. IV:
- *                   approximate 1/sqrt refined by Newton-Raphson), and one
- *                   FP64 add widens r^-3.  This is FP64-class, not IEEE FP64
- *                   per pair: r^-3 carries a relative error of up to 1.1e-13
- *                   (about 500 ulp; measured over displacements from 1 nm to
- *                   1 km and every exponent) where an IEEE FP64 evaluation
- *                   would be within a few ulp.  Forces meet the 1e-12
- *                   conditioned-error contract (measured 3.4e-14 at
- *                   N = 1e5).  NB_FP64_RSQ_NR2 is the plain FP64 Newton form.
- *  NB_MIXED      -- pair displacements in FP64, cast to FP32; r^2, rsqrt,
+ *  NB_FP64       -- FP64-class forces in two forms, chosen by the size.
+ *                   Half-pair plans, one-sided plans of 513 to 4096 ions and
+ *                   ensembles of at most 4096-ion instances: each coordinate
+ *                   is cut, in units of a power of two above those it is
+ *                   paired with, into three FP32 words (68 bits); the
+ *                   displacement is the words' exact difference as an FP32
+ *                   (hi, lo) pair, and r^2, r^-3, the products and the sums
+ *                   over up to 32 partners are double-floats, added in FP64.
+ *                   Pairs closer than 2^-20 of that unit, and units or
+ *                   weights far from the ordinary, take the second form:
+ *                   FP64 displacement and FP64 accumulation, with r^2,
+ *                   1/sqrt(r^2) and r^-3 on the FP32 pipe: the displacement
+ *                   is split into exponent-scaled FP32 (hi, lo) pairs, r^2 is
+ *                   a double-float, the FP32 hardware reciprocal square root
+ *                   (MUFU) is refined by a Newton residual formed in
+ *                   compensated FP32 (Sec. IV: approximate 1/sqrt refined by
+ *                   Newton-Raphson), and one FP64 add widens r^-3.  Both are
+ *                   FP64-class, not IEEE FP64 per pair: r^-3 of the second
+ *                   carries a relative error of up to 1.1e-13 (about 500 ulp;
+ *                   measured over displacements from 1 nm to 1 km and every
+ *                   exponent; nb_rinv3_probe), the first is at or below it.
+ *                   Forces meet the 1e-12 conditioned-error contract
+ *                   (measured 2.9e-14 at N = 1e5).  NB_FP64_RSQ_NR2 is the
+ *                   plain FP64 Newton form.
+ *  NB_MIXED      -- pair displacements to FP64 accuracy (an FP64 subtraction,
+ *                   or in half-pair plans from 2000 ions the exact difference
+ *                   of three-word positions), cast to FP32; r^2, rsqrt,
  *                   r^-3 and the products in FP32; per-tile FP32 partial
  *                   sums added into FP64 accumulators with compensation.
  *  NB_MIXED_SPLIT -- as NB_MIXED, but each position is carried as an FP32
@@ -83,7 +95,8 @@ typedef enum {
  *                   FP32 rounding (relative 2^-48 |r| / |r_i - r_j|, 1e-6 at
  *                   |r| / |r_i - r_j| ~ 3e8).  No FP64 instruction in the
  *                   pair loop.
- *  NB_DF64       -- FP64-class accuracy from FP32 arithmetic: FP64
+ *  NB_DF64       -- FP64-class accuracy from FP32 arithmetic.  Where NB_FP64
+ *                   has its first form this is the same kernel; else FP64
  *                   displacement split into an FP32 (hi, lo) pair; r^2,
  *                   r^-3 and the force products as double-floats (FP32
  *                   pairs with exact products and TwoSum); per-tile
@@ -435,8 +448,9 @@ nb_status nb_energy_noalloc(const nb_params *params, const nb_system *sys,
 /* out[i] = the r^-3 that precision mode `precision` (an nb_precision value)
  * forms for one pair with FP64 displacement (dx[i], dy[i], dz[i]) and
  * softening soft2 >= 0: r^2 = dx^2 + dy^2 + dz^2 + soft2, then the mode's
- * 1/sqrt and cube -- the same device functions as the pair kernels, before the
- * charge weight.  NB_MIXED and NB_MIXED_SPLIT share their FP32 bulk; here
+ * 1/sqrt and cube -- the same device functions as the pair kernels that form
+ * FP64 displacements, before the charge weight (the kernels on three-word
+ * positions form r^-3 from the words' difference, to the same class).  NB_MIXED and NB_MIXED_SPLIT share their FP32 bulk; here
  * both start from the displacement rounded to FP32 (the split mode's own
  * displacement comes from FP32 position pairs instead).  NB_DF64 returns
  * its double-float result summed into one double.  r^2 == 0 gives 0 in the
