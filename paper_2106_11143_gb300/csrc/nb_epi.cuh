@@ -3,6 +3,7 @@
 // slots, the FP32 parts of a position, and the step's launches.
 #pragma once
 
+#include "nb_pdl.cuh"
 #include "nb_verlet.cuh"
 
 namespace nb {

@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(EPI8_THREADS_COMP)
                 const double *__restrict__ cy, const double *__restrict__ cz, const double *__restrict__ part, int n_jc,
                 int64_t soff, const int64_t *cin, int64_t *cout, int64_t cout_off, double *nx, double *ny, double *nz,
                 float *split, unsigned *err) {
+  pdl_wait();
   epi_step<true>(p, s, kc, own_kc, cx, cy, cz, part, n_jc, soff, cin, cout, cout_off, nx, ny, nz, split, err);
 }
 
@@ -309,10 +310,9 @@ cudaError_t launch_epi_step_split(const Phys &p, const StateView &s, const doubl
   const bool own_kc = s.q || s.m;
   const KickConst kc = own_kc ? KickConst{} : uniform_kick_consts(p);
   if (epi_eight(s.n, n_jc))
-    k_epi_step8<<<epi_blocks(s.n, true), EPI8_THREADS_COMP, 0, st>>>(p, s, kc, own_kc, cx, cy, cz, part, n_jc, snew,
-                                                                      cin, cout, cout_off, nx, ny, nz, split, err);
-  else
-    k_epi_step<<<epi_blocks(s.n, false), EPI_THREADS, 0, st>>>(p, s, kc, own_kc, cx, cy, cz, part, n_jc, snew, cin,
+    return launch_pdl(k_epi_step8, dim3(epi_blocks(s.n, true)), dim3(EPI8_THREADS_COMP), 0, st, p, s, kc, (int)own_kc,
+                      cx, cy, cz, part, n_jc, snew, cin, cout, cout_off, nx, ny, nz, split, err);
+  k_epi_step<<<epi_blocks(s.n, false), EPI_THREADS, 0, st>>>(p, s, kc, own_kc, cx, cy, cz, part, n_jc, snew, cin,
                                                                 cout, cout_off, nx, ny, nz, split, err);
   return cudaGetLastError();
 }

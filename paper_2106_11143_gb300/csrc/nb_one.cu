@@ -18,6 +18,7 @@
 // reason the scale L is taken over all n ions, not over the block's: up to 4096
 // ions that scan is at most 96 loads per thread.
 #include "nb_pairterm.cuh"
+#include "nb_pdl.cuh"
 #include "nb_tri.cuh"
 
 namespace nb {
@@ -48,6 +49,7 @@ __global__ void __launch_bounds__(ONE_NT, 4)
                const double *__restrict__ y, const double *__restrict__ z, const double *__restrict__ q, double soft2,
                double *__restrict__ part) {
   __shared__ __align__(16) float qs[ONE_J / 2 * ONE_PAIR];
+  pdl_wait();
   const int tid = threadIdx.x;
   const int64_t i = (int64_t)blockIdx.x * ONE_NT + tid;
   const bool own = i < ni;
@@ -178,14 +180,10 @@ bool one_serves(const Plan &pl, int mode, int64_t n) {
 cudaError_t launch_pair_one(const Plan &pl, int64_t n, int64_t i0, int64_t ni, const double *x, const double *y,
                             const double *z, const double *q, double soft2, double *part, cudaStream_t st) {
   const dim3 grid((unsigned)((ni + ONE_NT - 1) / ONE_NT), (unsigned)pl.n_jc);
-#define NB_ONE(QA, SO) k_pair_one<QA, SO><<<grid, ONE_NT, 0, st>>>(n, pl.jchunk, i0, ni, x, y, z, q, soft2, part)
-  if (soft2 != 0.0) {
-    if (q) NB_ONE(true, true); else NB_ONE(false, true);
-  } else {
-    if (q) NB_ONE(true, false); else NB_ONE(false, false);
-  }
+#define NB_ONE(QA, SO) launch_pdl(k_pair_one<QA, SO>, grid, dim3(ONE_NT), 0, st, n, pl.jchunk, i0, ni, x, y, z, q, soft2, part)
+  if (soft2 != 0.0) return q ? NB_ONE(true, true) : NB_ONE(false, true);
+  return q ? NB_ONE(true, false) : NB_ONE(false, false);
 #undef NB_ONE
-  return cudaGetLastError();
 }
 
 }  // namespace nb
