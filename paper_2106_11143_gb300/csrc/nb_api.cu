@@ -912,9 +912,9 @@ nb_status nb_plan_info(int32_t kind, int32_t precision, int64_t n, int64_t out[8
 }
 
 nb_status nb_sym_schedule(int32_t nbk, int32_t *P, int32_t *Q, int32_t *round) {
-  if (nbk < 1 || nbk > 60000) return fail(NB_EINVAL, "nbk must be in 1..60000");
+  if (nbk < 1 || nbk > SYM_MAX_BLOCKS) return fail(NB_EINVAL, "nbk must be in 1..60000");
   if (!P || !Q || !round) return fail(NB_EINVAL, "output arrays must not be NULL");
-  const int64_t items = (int64_t)nbk * (nbk + 1) / 2;
+  const int64_t items = sym_items(nbk);
   for (int64_t t = 0; t < items; ++t) {
     const SymItem it = sym_item((int)t, nbk);
     P[t] = it.P;

@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "nb_pairterm.cuh"
+#include "nb_symsched.cuh"
 
 namespace nb {
 
@@ -365,9 +366,6 @@ bool tuning_lookup(int kind, int mode, int64_t n, int *block, int *R, int *bps) 
   return false;
 }
 
-// The symmetric kernels number their work items with an int: at most
-// SYM_MAX_BLOCKS blocks (nbk (nbk + 1) / 2 items).
-constexpr int64_t SYM_MAX_BLOCKS = 60000;
 // Output mode of the symmetric kernels (nb_symsched.cuh): the round-ordered
 // in-place adds from SYM_INPLACE_BLOCKS blocks on (at least about 4600
 // items, ten waves of three items per SM on 152 SMs, so the chain of nbk

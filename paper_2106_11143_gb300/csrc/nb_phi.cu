@@ -264,7 +264,7 @@ static cudaError_t launch_phi_t(int64_t n, int nbk, int G, const double *x, cons
     e = cudaMemsetAsync(sync, 0, sizeof(int) * sym_sync_ints(nbk), st);
     if (e != cudaSuccess) return e;
   }
-  const int items = nbk * (nbk + 1) / 2;
+  const unsigned items = (unsigned)sym_items(nbk);
   const size_t smem = smem_of(G);
 #define NB_PHI_LAUNCH(QA, IP) \
   k_phi_sym_tri<V, QA, NT, NB, IP, SOFT><<<items, NT, smem, st>>>(n, nbk, G, x, y, z, q, soft2, part, sync, err)
@@ -297,8 +297,8 @@ PhiPlan make_phi_plan(int64_t n) {
   auto blocks = [&](int g) { return (n + 32 * g - 1) / (32 * g); };
   int G = n < 10000 ? 4 : 8;
   if (blocks(G) * n > PHI_SLOT_DOUBLES && blocks(16) * n <= PHI_SLOT_DOUBLES) G = 16;
-  while (G < 16 && blocks(G) > 60000) G *= 2;
-  if (blocks(G) > 60000) return pl;
+  while (G < 16 && blocks(G) > SYM_MAX_BLOCKS) G *= 2;
+  if (blocks(G) > SYM_MAX_BLOCKS) return pl;
   pl.G = G;
   pl.nbk = (int)blocks(G);
   pl.n_slots = blocks(G) * n > PHI_SLOT_DOUBLES ? 1 : pl.nbk;

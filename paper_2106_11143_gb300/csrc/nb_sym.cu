@@ -863,7 +863,7 @@ static cudaError_t launch_sym_rot(int64_t n, int nbk, const double *x, const dou
     cudaError_t e = cudaMemsetAsync(sync, 0, sizeof(int) * sym_sync_ints(nbk), st);
     if (e != cudaSuccess) return e;
   }
-  const int items = nbk * (nbk + 1) / 2;
+  const unsigned items = (unsigned)sym_items(nbk);
   const size_t smem = sym_rot_smem_bytes(MODE);
   if (q && inplace)
     k_pair_sym_rot<MODE, true, RW, true><<<items, 32 * RW, smem, st>>>(n, nbk, x, y, z, q, pf, soft2, part, sync, err);
@@ -917,7 +917,7 @@ static cudaError_t launch_sym_m(int64_t n, int nbk, int G, const double *x, cons
     e = cudaMemsetAsync(sync, 0, sizeof(int) * sym_sync_ints(nbk), st);
     if (e != cudaSuccess) return e;
   }
-  const int items = nbk * (nbk + 1) / 2;
+  const unsigned items = (unsigned)sym_items(nbk);
   const size_t smem = sym_smem_bytes(G, MODE);
   if (q && inplace)
     k_pair_sym<MODE, true, P2, NT, true><<<items, NT, smem, st>>>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err);

@@ -49,6 +49,13 @@ constexpr int SYM_SPIN_LIMIT = 1 << 23;
 // Number of ints of sync state for nbk blocks.
 __host__ __device__ constexpr int64_t sym_sync_ints(int64_t nbk) { return nbk + 1; }
 
+// Items of a schedule of nbk blocks, which are also its grid.  From nbk = 46341
+// the product passes 2^31 before it is halved; the items themselves fit an int up
+// to SYM_MAX_BLOCKS blocks.
+constexpr int64_t SYM_MAX_BLOCKS = 60000;
+__host__ __device__ constexpr int64_t sym_items(int64_t nbk) { return nbk * (nbk + 1) / 2; }
+static_assert(sym_items(SYM_MAX_BLOCKS) <= 0x7fffffff, "items are numbered with an int and launched as grid.x");
+
 struct SymItem {
   int P, Q, round;
 };

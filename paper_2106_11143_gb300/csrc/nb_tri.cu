@@ -367,7 +367,7 @@ static cudaError_t launch_tri(int64_t n, int nbk, int G, int SB, const double *x
     e = cudaMemsetAsync(sync, 0, sizeof(int) * sym_sync_ints(nbk), st);
     if (e != cudaSuccess) return e;
   }
-  const int items = nbk * (nbk + 1) / 2;
+  const unsigned items = (unsigned)sym_items(nbk);
   const size_t smem = tri_smem<V, NT>(G);
 #define NB_TRI_LAUNCH(QA, IP) \
   k_pair_sym_tri<MIX, V, QA, NT, NB, IP, SOFT><<<items, NT, smem, st>>>(n, nbk, G, SB, x, y, z, q, soft2, part, sync, err)
@@ -403,7 +403,7 @@ Plan make_force_plan(int64_t n, int mode, double soft2) {
   if (!tri_sums(pl, mode, soft2) || (mode == MODE_MIXED && n < 2000) || tuning_lookup(4, mode, n, &tb, &tr, &tbps)) return pl;
   int G = n > 12160 ? 8 : (n >= 2800 ? 4 : 2);
   if (mode == MODE_MIXED) G = n >= 60000 ? 16 : (n > 12160 ? 8 : (n >= 3000 ? 4 : 2));
-  while (G < 32 && (n + 32 * G - 1) / (32 * G) > 60000) G *= 2;  // the schedule's block limit
+  while (G < 32 && (n + 32 * G - 1) / (32 * G) > SYM_MAX_BLOCKS) G *= 2;  // the schedule's block limit
   pl.G = G;
   pl.nbk = (int)((n + 32 * G - 1) / (32 * G));
   // the output rule of the half-pair kernels: in place from 96 blocks or 1 GB of partials

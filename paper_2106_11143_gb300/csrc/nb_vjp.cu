@@ -573,7 +573,7 @@ static cudaError_t launch_vjp_t(int64_t n, int nbk, int G, const double *x, cons
     e = cudaMemsetAsync(sync, 0, sizeof(int) * sym_sync_ints(nbk), st);
     if (e != cudaSuccess) return e;
   }
-  const int items = nbk * (nbk + 1) / 2;
+  const unsigned items = (unsigned)sym_items(nbk);
   const size_t smem = vjp_smem_bytes(G);
 #define NB_VJP_LAUNCH(QA, IP) \
   k_vjp_sym<QA, IP, SOFT><<<items, VJP_THREADS, smem, st>>>(n, nbk, G, x, y, z, q, lx, ly, lz, soft2, part, sync, err)
