@@ -259,7 +259,11 @@ nb_status nb_step_range_kick(const nb_params *params, nb_system *sys, int64_t i0
  *   Coulomb = (k_C/2) sum_i q_i sum_{j != i} q_j / sqrt(r_ij^2 + soft2).
  * FP64 differences and sums regardless of params->precision; the pair term
  * 1/sqrt(r^2 + soft2) is formed as in NB_FP64 (FP32-pipe double-float,
- * widened to FP64).  Synchronises the stream before returning.            */
+ * widened to FP64).  Synchronises the stream before returning.  Large systems
+ * (above about 22 600 ions) add their pair sums in a fixed order with bounded
+ * waits: NB_ETIMEOUT, with out[] left as it was, if one gave up in this call or
+ * in an earlier one of the stream that nb_sync_status has not reported yet (it
+ * still reports it).                                                       */
 nb_status nb_energy(const nb_params *params, const nb_system *sys,
                     double out[4], void *stream);
 

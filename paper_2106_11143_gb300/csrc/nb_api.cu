@@ -603,22 +603,30 @@ nb_status nb_energy(const nb_params *params, const nb_system *sys, double out[4]
   Carver need;
   need.take<double>(pl.out_doubles(n));
   need.take<double>(3 * ENERGY_BLOCKS);
-  need.take<double>(4);
+  need.take<double>(5);
   Arena *a = nullptr;
   NB_TRY(get_arena(st, need.off + 256, &a));
   Carver cv;
   cv.base = a->buf;
   double *ppart = cv.take<double>(pl.out_doubles(n));
   double *bpart = cv.take<double>(3 * ENERGY_BLOCKS);
-  double *out4 = cv.take<double>(4);
+  double *out4 = cv.take<double>(5);  // and the error word in the fifth
   const Phys p = to_phys(params);
   const StateView v = to_view(sys);
   const double t = params->t0 + (double)sys->step * params->dt;
   NB_CUDA_TRY(launch_phi(pl, n, sys->x, sys->y, sys->z, sys->q, params->charge, params->soft2, ppart, a->err, st));
-  NB_CUDA_TRY(launch_energy(p, v, ppart, pl.n_slots, t, bpart, out4, st));
+  NB_CUDA_TRY(launch_energy(p, v, ppart, pl.n_slots, t, bpart, out4, st, a->err));
   count_launches(3);
-  NB_CUDA_TRY(cudaMemcpyAsync(out, out4, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
+  double h[5];
+  NB_CUDA_TRY(cudaMemcpyAsync(h, out4, sizeof(h), cudaMemcpyDeviceToHost, st));
   NB_CUDA_TRY(cudaStreamSynchronize(st));
+  // The in-place potential waits for other items' adds: a wait that gave up (a set
+  // word makes any later one give up too) leaves a part of the sum out.
+  unsigned word;
+  std::memcpy(&word, &h[4], sizeof(word));
+  if (pl.G && pl.n_slots == 1 && (word & ERR_TIMEOUT))
+    return fail(NB_ETIMEOUT, "nb_energy: a bounded device wait gave up");
+  std::memcpy(out, h, 4 * sizeof(double));
   return NB_OK;
 }
 

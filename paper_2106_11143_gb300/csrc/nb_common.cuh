@@ -547,10 +547,12 @@ cudaError_t launch_loss(const Phys &p, int64_t n, const double *q, const double 
                         double *loss, cudaStream_t st);
 constexpr int ADJ_PART_BLOCKS = 128;
 
-// Energies: block partials then one final block; out4 is device memory.
+// Energies: block partials then one final block; out4 is device memory, and with
+// err the error word follows in a fifth double.
 constexpr int ENERGY_BLOCKS = 128;
 constexpr int ENERGY_THREADS = 256;
 cudaError_t launch_energy(const Phys &p, const StateView &s, const double *phi_part, int n_jc,
-                          double t, double *block_part, double *out4, cudaStream_t st);
+                          double t, double *block_part, double *out4, cudaStream_t st,
+                          const unsigned *err = nullptr);
 
 }  // namespace nb

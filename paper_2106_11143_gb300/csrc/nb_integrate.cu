@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(ENERGY_THREADS) k_energy_part(Phys p, StateVie
 }
 
 __global__ void __launch_bounds__(ENERGY_THREADS) k_energy_final(const double *__restrict__ block_part,
-                                                                 double *out4) {
+                                                                 double *out4, const unsigned *err) {
   __shared__ double sh[3 * ENERGY_THREADS];
   double acc[3] = {0.0, 0.0, 0.0};
   for (int b = threadIdx.x; b < ENERGY_BLOCKS; b += ENERGY_THREADS)
@@ -385,15 +385,16 @@ __global__ void __launch_bounds__(ENERGY_THREADS) k_energy_final(const double *_
     out4[1] = acc[1];
     out4[2] = acc[2];
     out4[3] = acc[0] + acc[1] + acc[2];
+    if (err) *reinterpret_cast<unsigned *>(out4 + 4) = *err;
   }
 }
 
 cudaError_t launch_energy(const Phys &p, const StateView &s, const double *phi_part, int n_jc,
-                          double t, double *block_part, double *out4, cudaStream_t st) {
+                          double t, double *block_part, double *out4, cudaStream_t st, const unsigned *err) {
   k_energy_part<<<ENERGY_BLOCKS, ENERGY_THREADS, 0, st>>>(p, s, phi_part, n_jc, t, block_part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_energy_final<<<1, ENERGY_THREADS, 0, st>>>(block_part, out4);
+  k_energy_final<<<1, ENERGY_THREADS, 0, st>>>(block_part, out4, err);
   return cudaGetLastError();
 }
 

@@ -57,3 +57,21 @@ def test_wait_probe_rejects_bad_arguments(nb):
     ok = C.c_int32()
     assert L.nb_sym_wait_probe(-1, 0, C.byref(ok), None) == 1
     assert L.nb_sym_wait_probe(0, 0, None, None) == 1
+
+
+def test_energy_reports_a_wait_that_gave_up(nb):
+    """From 1e6 partials (about 22 700 ions) the potential is summed in place with
+    bounded waits, which give up early once the stream's error word holds a
+    timeout: nb_energy must not return such a sum as good."""
+    w = W.cloud_large(n=40000)
+    par = nb.Params.from_phys(w["phys"])
+    s = nb.System(w["pos"], w["vel"])
+    before = nb.energy(par, s)
+    assert nb.sym_wait_probe(0, 1) is False  # sets the word; nobody has read it
+    with pytest.raises(nb.NBError) as e:
+        nb.energy(par, s)
+    assert e.value.status == 4  # NB_ETIMEOUT
+    with pytest.raises(nb.NBError) as e:
+        nb.sync_status()  # the status is still the stream's to report
+    assert e.value.status == 4
+    assert np.array_equal(nb.energy(par, s), before)
