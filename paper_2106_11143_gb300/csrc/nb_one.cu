@@ -71,8 +71,7 @@ __global__ void __launch_bounds__(ONE_NT, 4)
       s2l = pk1(l);
     }
     float w0[4], w1[4], w2[4];
-    tri_ion<false>(g, own, x, y, z, q, em, ew, TRI_FAR, w0, w1, w2);
-    const bool mylow = w2[0] != 0.0f || w2[1] != 0.0f || w2[2] != 0.0f;
+    const bool mylow = tri_ion<false>(g, own, x, y, z, q, em, ew, TRI_FAR, w0, w1, w2);
     f32x2 ph[3], pm[3], pl[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -86,7 +85,7 @@ __global__ void __launch_bounds__(ONE_NT, 4)
       if (jb > c0) __syncthreads();
       for (int j = tid; j < padded; j += ONE_NT) {
         float v0[4], v1[4], v2[4];
-        tri_ion<QARR>(jb + j, j < cnt, x, y, z, q, em, ew, -TRI_FAR, v0, v1, v2);
+        low |= tri_ion<QARR>(jb + j, j < cnt, x, y, z, q, em, ew, -TRI_FAR, v0, v1, v2);
         float *e = qs + (j >> 1) * ONE_PAIR + (j & 1);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -96,7 +95,6 @@ __global__ void __launch_bounds__(ONE_NT, 4)
         }
         e[18] = v0[3];
         e[20] = v1[3];
-        low |= v2[0] != 0.0f || v2[1] != 0.0f || v2[2] != 0.0f;
       }
       low = __syncthreads_or(low);
       const int self = (int)(g - jb);  // the ion's own place among the staged partners, if any

@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(NT, NB)
   const int PT = BI / PI, NG = NW / PT, nqt = G / NG;  // P-tiles, warps per P-tile, Q-tiles per warp
   const int pt = warp % PT, grp = warp / PT;
   TriIons<V> p;
-  int low = 0;  // an l word is set
+  int low = 0;  // a coordinate has bits in or below its l word
   if (fast) low = tri_load<V, QARR, NT>(p, qs, BI, pt, p0, np, q0, nq, x, y, z, q, em, ew);
   for (int i = tid; i < 3 * BI; i += NT) accQ[i] = 0.0;
   for (int i = tid; i < NW * 3 * PI; i += NT) accP[i] = 0.0;

@@ -17,8 +17,8 @@
 // A pair closer than 2^-20 L (where the 2^-69 L cut would pass 2^-49 of the
 // distance, and dl stops being small against dm) makes its tile fall back to
 // FP64 arithmetic; the test is the smallest r^2 met, one FMNMX per pair.  When
-// no coordinate of the item has bits in l (positions on a grid), d is exact
-// and normal at any distance, and only FP32's range sets a limit, 2^-40 L.
+// no coordinate of the item has bits in l or below it (positions on a grid), d
+// is exact and normal at any distance, and only FP32's range sets a limit, 2^-40 L.
 // Items whose scale or weights are far from the ordinary (below) take the
 // FP64 path as a whole.
 #pragma once
@@ -305,9 +305,11 @@ __device__ __forceinline__ float tri_tile(const TriIons<V> &p, LD ld, int lane, 
   return SOFT ? rsqrt_approx(rmin) : ymax;
 }
 
-// Words of ion g (or a padding ion on side `far`) with its weight.
+// Words of ion g (or a padding ion on side `far`) with its weight; returns whether
+// an l word is set or the words do not hold a coordinate exactly (bits below 2^-69
+// leave no trace in l).
 template <bool QARR>
-__device__ __forceinline__ void tri_ion(int64_t g, bool real, const double *x, const double *y, const double *z,
+__device__ __forceinline__ bool tri_ion(int64_t g, bool real, const double *x, const double *y, const double *z,
                                         const double *q, int em, int ew, float far, float w0[4], float w1[4],
                                         float w2[4]) {
   w0[3] = w1[3] = w2[3] = 0.0f;
@@ -320,12 +322,15 @@ __device__ __forceinline__ void tri_ion(int64_t g, bool real, const double *x, c
     tri_words(z[g], em, t);
     w0[2] = t[0]; w1[2] = t[1]; w2[2] = t[2];
     if (QARR && q[g] != 0.0) split_f64_scaled(q[g], ew - 1023, w0[3], w1[3]);
+    return w2[0] != 0.0f || w2[1] != 0.0f || w2[2] != 0.0f || !tri_exact(x[g], em) || !tri_exact(y[g], em) ||
+           !tri_exact(z[g], em);
   } else {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       w0[c] = far;
       w1[c] = w2[c] = 0.0f;
     }
+    return false;
   }
 }
 
@@ -380,7 +385,7 @@ __device__ __forceinline__ bool tri_scale(int64_t p0, int np, int64_t q0, int nq
 }
 
 // Cuts the Q block's ions into words in shared memory (BI entries) and loads the
-// lane's ions of P-tile pt; returns whether any l word is set.
+// lane's ions of P-tile pt; returns whether tri_ion did for any.
 template <int V, bool QARR, int NT>
 __device__ __forceinline__ int tri_load(TriIons<V> &p, float4 *qs, int BI, int pt, int64_t p0, int np, int64_t q0,
                                         int nq, const double *x, const double *y, const double *z, const double *q,
@@ -389,12 +394,11 @@ __device__ __forceinline__ int tri_load(TriIons<V> &p, float4 *qs, int BI, int p
   int low = 0;
   for (int i = threadIdx.x; i < BI; i += NT) {
     float w0[4], w1[4], w2[4];
-    tri_ion<QARR>(q0 + i, i < nq, x, y, z, q, em, ew, -TRI_FAR, w0, w1, w2);
+    low |= tri_ion<QARR>(q0 + i, i < nq, x, y, z, q, em, ew, -TRI_FAR, w0, w1, w2);
     float4 *e = qs + (i >> 5) * TRI_TILE4 + (i & 31);
     e[0] = e[32] = make_float4(w0[0], w0[1], w0[2], w0[3]);
     e[64] = e[96] = make_float4(w1[0], w1[1], w1[2], w1[3]);
     e[128] = e[160] = make_float4(w2[0], w2[1], w2[2], w2[3]);
-    low |= w2[0] != 0.0f || w2[1] != 0.0f || w2[2] != 0.0f;
   }
 #pragma unroll
   for (int v = 0; v < V; ++v) {
@@ -402,8 +406,7 @@ __device__ __forceinline__ int tri_load(TriIons<V> &p, float4 *qs, int BI, int p
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int i = pt * 64 * V + v * 64 + b * 32 + lane;
-      tri_ion<QARR>(p0 + i, i < np, x, y, z, q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
-      low |= w2[b][0] != 0.0f || w2[b][1] != 0.0f || w2[b][2] != 0.0f;
+      low |= tri_ion<QARR>(p0 + i, i < np, x, y, z, q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {

@@ -438,18 +438,17 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
   const int PT = G >> 1, NG = VJP_W / PT, nqt = G / NG;  // P-tiles of 64 ions, warps and Q-tiles per P-tile
   const int pt = warp % PT, grp = warp / PT;
   VjpIons p;
-  int low = 0;  // an l word of a position is set
+  int low = 0;  // a position has bits in or below its l word
   int cut = 0;  // a cotangent is not exact in its words
   if (fast) {
     float w0[2][4], w1[2][4], w2[2][4];
     for (int i = tid; i < BI; i += VJP_THREADS) {
       const int64_t g = q0 + i;
       float4 *e = qs + (i >> 5) * VJP_TILE4 + (i & 31);
-      tri_ion<QARR>(g, i < nq, x, y, z, q, em, ew, -TRI_FAR, w0[0], w1[0], w2[0]);
+      low |= tri_ion<QARR>(g, i < nq, x, y, z, q, em, ew, -TRI_FAR, w0[0], w1[0], w2[0]);
       e[0] = make_float4(w0[0][0], w0[0][1], w0[0][2], w0[0][3]);
       e[32] = make_float4(w1[0][0], w1[0][1], w1[0][2], w1[0][3]);
       e[64] = make_float4(w2[0][0], w2[0][1], w2[0][2], 0.0f);
-      low |= w2[0][0] != 0.0f || w2[0][1] != 0.0f || w2[0][2] != 0.0f;
       cut |= vjp_lam(g, i < nq, lx, ly, lz, el, ee, w0[0], w1[0], w2[0]);
       e[96] = make_float4(w0[0][0], w0[0][1], w0[0][2], 0.0f);
       e[128] = make_float4(w1[0][0], w1[0][1], w1[0][2], 0.0f);
@@ -458,8 +457,7 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int i = pt * 64 + b * 32 + lane;
-      tri_ion<QARR>(p0 + i, i < np, x, y, z, q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
-      low |= w2[b][0] != 0.0f || w2[b][1] != 0.0f || w2[b][2] != 0.0f;
+      low |= tri_ion<QARR>(p0 + i, i < np, x, y, z, q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
