@@ -327,31 +327,6 @@ __device__ __noinline__ void bsym_forces(const BIons v, double *acc, int npad, d
 // counters the FP64 adds of all 16 warps coincided: 18.8 ms.
 constexpr int BTRI_PI = 128;
 
-// A tile of a task in FP64 (nb_tri.cuh's limits): the P side's 128 ions
-// against tile q0 .. q0 + 31, added to acc.
-template <bool QARR>
-__device__ __noinline__ void btri_tile_fp64(const BIons v, int p0, int q0, bool one, double soft2, double sc,
-                                            double *acc, int npad) {
-  const int lane = threadIdx.x & 31;
-  for (int u = 0; u < BTRI_PI; u += 32) {
-    const int i = p0 + u + lane;
-    double a[3] = {0.0, 0.0, 0.0}, b[3] = {0.0, 0.0, 0.0};
-    for (int r = 0; r < 32; ++r) {
-      const int j = q0 + ((lane + r) & 31);
-      if (i < v.n && j < v.n && i != j) {
-        const BD4 pi = bion<QARR, false>(v, i), pj = bion<QARR, false>(v, j);
-        bsym_eval<QARR>(pi, pj, soft2, a, b);
-      }
-      for (int c = 0; c < 3; ++c) b[c] = bshfl_next(b[c], lane);
-    }
-    for (int c = 0; c < 3; ++c) {
-      if (i < v.n) acc[c * npad + i] += a[c] * sc;
-      __syncwarp();
-      if (!one && q0 + lane < v.n) acc[c * npad + q0 + lane] += b[c] * sc;
-    }
-  }
-}
-
 // Bounded wait of a warp for counter c to reach v (about a second).
 constexpr int BTRI_SPIN_LIMIT = 1 << 24;
 __device__ __forceinline__ bool btri_wait(const int *c, int v) {
@@ -365,28 +340,91 @@ __device__ __forceinline__ bool btri_wait(const int *c, int v) {
   __threadfence_block();
   return ok;
 }
+// A task's turn: the counters of A and (two super-tiles) B and what to wait for.
+struct BTurn {
+  const int *a, *b;
+  int va, vb;
+  __device__ __forceinline__ bool wait(bool one) const {
+    const bool ok = btri_wait(a, va);
+    return (one || btri_wait(b, vb)) && ok;
+  }
+};
+
+// A task in FP64 (nb_tri.cuh's limits): the P side's np ions (a multiple of 32, at
+// most 128) against tile q0 .. q0 + 31, all of it before its turn.
+template <bool QARR>
+__device__ __noinline__ bool btri_task_fp64(const BIons v, int p0, int np, int q0, bool one, double soft2, double *acc,
+                                            int npad, const BTurn turn) {
+  const int lane = threadIdx.x & 31;
+  double a[4][3], b[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    a[u][0] = a[u][1] = a[u][2] = 0.0;
+    if (32 * u >= np) continue;
+    const int i = p0 + 32 * u + lane;
+#pragma unroll 1
+    for (int r = 0; r < 32; ++r) {
+      const int j = q0 + ((lane + r) & 31);
+      if (i < v.n && j < v.n && i != j) {
+        const BD4 pi = bion<QARR, false>(v, i), pj = bion<QARR, false>(v, j);
+        bsym_eval<QARR>(pi, pj, soft2, a[u], b);
+      }
+      for (int c = 0; c < 3; ++c) b[c] = bshfl_next(b[c], lane);
+    }
+  }
+  if (!turn.wait(one)) return false;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int i = p0 + 32 * u + lane;
+    if (32 * u < np && i < v.n)
+      for (int c = 0; c < 3; ++c) acc[c * npad + i] += a[u][c];
+  }
+  if (!one && q0 + lane < v.n)
+    for (int c = 0; c < 3; ++c) acc[c * npad + q0 + lane] += b[c];
+  return true;
+}
 
 // One task: the pair arithmetic of the P side's 64 V ions from p0 against tile
-// q0 .. q0 + 31, then, in its turn, the adds to acc.  wait() takes the turn
-// (false: it gave up); self as in tri_tile, or -1 for two super-tiles.
-template <int V, bool QARR, class WAIT>
-__device__ __forceinline__ bool btri_task(const BIons &v, double *acc, int npad, float4 *st, int em, int ew,
-                                          double soft2, int p0, int q0, int self, WAIT wait) {
+// q0 .. q0 + 31, then, in its turn, the adds to acc.  The units are the task's
+// own, from its 64 V + 32 ions: an ion far out, or a coordinate small beside its
+// instance's, concerns the tasks that hold it alone.  False: the wait gave up.
+// self as in tri_tile, or -1 for two super-tiles.
+template <int V, bool QARR>
+__device__ __forceinline__ bool btri_task(const BIons &v, double *acc, int npad, float4 *st, int ew, double soft2, int p0,
+                                          int q0, int self, const BTurn &turn) {
   const int lane = threadIdx.x & 31, n = v.n;
   const bool one = self >= 0;
+  TriScale sc;
+  sc.ew = ew;
+  int mx[3] = {0, 0, 0};
+  auto grow = [&](int i) {
+    if (i < n) {
+      mx[0] = max(mx[0], __double2hiint(v.x[i]) & 0x7fffffff);
+      mx[1] = max(mx[1], __double2hiint(v.y[i]) & 0x7fffffff);
+      mx[2] = max(mx[2], __double2hiint(v.z[i]) & 0x7fffffff);
+    }
+  };
+  grow(q0 + lane);
+#pragma unroll
+  for (int u = 0; u < 2 * V; ++u) grow(p0 + 32 * u + lane);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) mx[c] = __reduce_max_sync(0xffffffffu, mx[c]);
+  bool done = tri_axes<QARR>(mx, soft2, sc);
   float w0[2][4], w1[2][4], w2[2][4];
   __syncwarp();  // every lane is done with the last tile
-  tri_ion<QARR>(q0 + lane, q0 + lane < n, v.x, v.y, v.z, v.q, em, ew, -TRI_FAR, w0[0], w1[0], w2[0]);
+  const int qf = tri_ion<QARR, TRI_NEAR, false>(q0 + lane, q0 + lane < n, v.x, v.y, v.z, v.q, sc, -TRI_FAR, w0[0], w1[0],
+                                                w2[0]);
   st[lane] = make_float4(w0[0][0], w0[0][1], w0[0][2], w0[0][3]);
   st[32 + lane] = make_float4(w1[0][0], w1[0][1], w1[0][2], w1[0][3]);
   st[64 + lane] = make_float4(w2[0][0], w2[0][1], w2[0][2], w2[0][3]);
+  int pf = 0;
   TriIons<V> p;
 #pragma unroll
   for (int u = 0; u < V; ++u) {
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int i = p0 + u * 64 + b * 32 + lane;
-      tri_ion<QARR>(i, i < n, v.x, v.y, v.z, v.q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
+      pf |= tri_ion<QARR, TRI_NEAR, false>(i, i < n, v.x, v.y, v.z, v.q, sc, TRI_FAR, w0[b], w1[b], w2[b]);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -397,37 +435,50 @@ __device__ __forceinline__ bool btri_task(const BIons &v, double *acc, int npad,
     p.wh[u] = pk(w0[0][3], w0[1][3]);
     p.wl[u] = pk(w1[0][3], w1[1][3]);
   }
+  int fl = __reduce_or_sync(0xffffffffu, pf | qf << 6);
+  if (done && ((fl >> 3) & (fl >> 9) & 7)) {  // both sides near on one axis: is one cut?
+    auto place = [&](int i) {
+      return i < n ? tri_place<TRI_NEAR>(v.x[i], sc.ex[0], 0) | tri_place<TRI_NEAR>(v.y[i], sc.ex[1], 1) |
+                         tri_place<TRI_NEAR>(v.z[i], sc.ex[2], 2)
+                   : 0;
+    };
+    fl = place(q0 + lane) << 6;
+#pragma unroll 1
+    for (int u = 0; u < 2 * V; ++u) fl |= place(p0 + 32 * u + lane);
+    fl = __reduce_or_sync(0xffffffffu, fl);
+    done = !tri_fault(fl, fl >> 6);
+  }
   TriSums<V> ts;
-  const f32x2 zero = pk1(0.0f);
+  if (done) {
+    const f32x2 zero = pk1(0.0f);
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    ts.bh[c] = ts.bl[c] = zero;
+    for (int c = 0; c < 3; ++c) {
+      ts.bh[c] = ts.bl[c] = zero;
 #pragma unroll
-    for (int u = 0; u < V; ++u) ts.ah[u][c] = ts.al[u][c] = zero;
+      for (int u = 0; u < V; ++u) ts.ah[u][c] = ts.al[u][c] = zero;
+    }
+    __syncwarp();
+    auto ld = [&](int r, float4 &f0, float4 &f1, float4 &f2) {
+      const float4 *e = st + ((lane + r) & 31);
+      f0 = e[0];
+      f1 = e[32];
+      f2 = e[64];
+    };
+    float ymax;
+    if (soft2 != 0.0) {
+      float sh, sl;
+      split_f64_scaled(soft2, 2 * (sc.em - 1022), sh, sl);
+      ymax = one ? tri_tile<V, QARR, true, true>(p, ld, lane, self, pk1(sh), pk1(sl), ts)
+                 : tri_tile<V, QARR, false, true>(p, ld, lane, -1, pk1(sh), pk1(sl), ts);
+    } else {
+      ymax = one ? tri_tile<V, QARR, true, false>(p, ld, lane, self, zero, zero, ts)
+                 : tri_tile<V, QARR, false, false>(p, ld, lane, -1, zero, zero, ts);
+    }
+    done = !__any_sync(0xffffffffu, !(ymax <= TRI_YMAX_GRID));
   }
-  __syncwarp();
-  auto ld = [&](int r, float4 &f0, float4 &f1, float4 &f2) {
-    const float4 *e = st + ((lane + r) & 31);
-    f0 = e[0];
-    f1 = e[32];
-    f2 = e[64];
-  };
-  float ymax;
-  if (soft2 != 0.0) {
-    float sh, sl;
-    split_f64_scaled(soft2, 2 * (em - 1022), sh, sl);
-    ymax = one ? tri_tile<V, QARR, true, true>(p, ld, lane, self, pk1(sh), pk1(sl), ts)
-               : tri_tile<V, QARR, false, true>(p, ld, lane, -1, pk1(sh), pk1(sl), ts);
-  } else {
-    ymax = one ? tri_tile<V, QARR, true, false>(p, ld, lane, self, zero, zero, ts)
-               : tri_tile<V, QARR, false, false>(p, ld, lane, -1, zero, zero, ts);
-  }
-  const bool done = !__any_sync(0xffffffffu, !(ymax <= TRI_YMAX));
-  if (!wait()) return false;
-  if (!done) {
-    btri_tile_fp64<QARR>(v, p0, q0, one, soft2, pow2d(2 * (em - 1022) - (ew - 1023)), acc, npad);
-    return true;
-  }
+  if (!done) return btri_task_fp64<QARR>(v, p0, 64 * V, q0, one, soft2, acc, npad, turn);
+  if (!turn.wait(one)) return false;
+  const double fwd = pow2d((ew - 1023) - 2 * (sc.em - 1022));  // from the task's units
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     float h0, h1, l0, l1;
@@ -436,20 +487,21 @@ __device__ __forceinline__ bool btri_task(const BIons &v, double *acc, int npad,
       upk(ts.ah[u][c], h0, h1);
       upk(ts.al[u][c], l0, l1);
       const int i = p0 + u * 64 + lane;
-      if (i < n) acc[c * npad + i] += (double)h0 + (double)l0;
-      if (i + 32 < n) acc[c * npad + i + 32] += (double)h1 + (double)l1;
+      if (i < n) acc[c * npad + i] = fma((double)h0 + (double)l0, fwd, acc[c * npad + i]);
+      if (i + 32 < n) acc[c * npad + i + 32] = fma((double)h1 + (double)l1, fwd, acc[c * npad + i + 32]);
     }
     if (!one && q0 + lane < n) {
       upk(ts.bh[c], h0, h1);
       upk(ts.bl[c], l0, l1);
-      acc[c * npad + q0 + lane] += ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
+      double &a = acc[c * npad + q0 + lane];
+      a = fma(((double)h0 + (double)l0) + ((double)h1 + (double)l1), fwd, a);
     }
   }
   return true;
 }
 
 template <bool QARR>
-__device__ __forceinline__ void btri_forces(const BIons &v, double *acc, int npad, float4 *stage, int *cnt, int em,
+__device__ __forceinline__ void btri_forces(const BIons &v, double *acc, int npad, float4 *stage, int *cnt,
                                             int ew, double soft2, unsigned *err) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5;
   const int n = v.n, S = (n + BTRI_PI - 1) / BTRI_PI, odd = S & 1;
@@ -468,20 +520,17 @@ __device__ __forceinline__ void btri_forces(const BIons &v, double *acc, int npa
     const bool one = A == B;
     // rounds before this one that X has taken part in: all but its own bye
     auto before = [&](int X) { return rd - (odd && X < rd - 1 ? 1 : 0); };
-    auto wait = [&]() {
-      const bool a = btri_wait(cnt + A, 4 * before(A) + k);
-      return (one || btri_wait(cnt + B, 4 * before(B))) && a;
-    };
+    const BTurn turn{cnt + A, cnt + B, 4 * before(A) + k, 4 * before(B)};
     // a super-tile of at most 64 ions (the last one, or a small instance) has
     // one pair of P-ions per lane: 8.9 to 6.1 ms for 50 steps of 1024 instances
     // of 16 .. 64 ions
     bool ok;
     if (q0 >= n)
-      ok = wait();
+      ok = turn.wait(one);
     else if (p0 + 64 < n)
-      ok = btri_task<2, QARR>(v, acc, npad, st, em, ew, soft2, p0, q0, one ? k : -1, wait);
+      ok = btri_task<2, QARR>(v, acc, npad, st, ew, soft2, p0, q0, one ? k : -1, turn);
     else
-      ok = btri_task<1, QARR>(v, acc, npad, st, em, ew, soft2, p0, q0, one ? k : -1, wait);
+      ok = btri_task<1, QARR>(v, acc, npad, st, ew, soft2, p0, q0, one ? k : -1, turn);
     if (!ok && lane == 0) atomicOr(err, ERR_TIMEOUT);
     __threadfence_block();
     __syncwarp();
@@ -514,7 +563,7 @@ __global__ void __launch_bounds__(512, 1) k_batched(Phys pall, const Phys *__res
   double *acc = sz + npad;                                       // SYM: [3][npad]
   float4 *stage = reinterpret_cast<float4 *>(acc + 3 * npad);    // SYM: BTRI_STAGE4 per warp
   double *sw = sz + npad;                                        // one-sided: the weights
-  __shared__ int red[3][BATCH_THREADS_MAX / 32];
+  __shared__ int red[2][BATCH_THREADS_MAX / 32];
   __shared__ int cnt[BATCH_SYM_N / BTRI_PI];  // tasks that have added to each super-tile
   const int T = blockDim.x;
   const int tid = threadIdx.x;
@@ -570,7 +619,6 @@ __global__ void __launch_bounds__(512, 1) k_batched(Phys pall, const Phys *__res
       const int64_t snew = step0 + st + 1;
       const double t = p.t0 + (double)snew * dt;
       // drift: r+ = r + v dt + a dt^2/2 (each thread its own ions)
-      int mx = 0;
       if (SYM)
         for (int i = tid; i < BATCH_SYM_N / BTRI_PI; i += T) cnt[i] = 0;
       for (int i = tid; i < n; i += T) {
@@ -580,24 +628,15 @@ __global__ void __launch_bounds__(512, 1) k_batched(Phys pall, const Phys *__res
         sx[i] = rx;
         sy[i] = ry;
         sz[i] = rz;
-        if (SYM) {
-          mx = max(mx, max(__double2hiint(rx) & 0x7fffffff,
-                           max(__double2hiint(ry) & 0x7fffffff, __double2hiint(rz) & 0x7fffffff)));
-          acc[i] = acc[npad + i] = acc[2 * npad + i] = 0.0;
-        }
+        if (SYM) acc[i] = acc[npad + i] = acc[2 * npad + i] = 0.0;
       }
+      __syncthreads();
       // forces at r+ and the kick
-      double fwd = 1.0;  // the accumulators' unit
       if (SYM) {
-        const int em = block_extreme<false>(mx, red[2]) >> 20;
-        if (tri_w && tri_scale_ok(em, soft2)) {
-          fwd = pow2d((ew - 1023) - 2 * (em - 1022));
-          btri_forces<QARR>(ions, acc, npad, stage, cnt, em, ew, soft2, err);
-        } else {
+        if (tri_w)
+          btri_forces<QARR>(ions, acc, npad, stage, cnt, ew, soft2, err);
+        else
           bsym_forces<QARR, DF>(ions, acc, npad, soft2, s2h, s2l);
-        }
-      } else {
-        __syncthreads();
       }
       for (int ib = 0; ib < n; ib += T) {
         const int i = ib + tid;
@@ -606,9 +645,9 @@ __global__ void __launch_bounds__(512, 1) k_batched(Phys pall, const Phys *__res
         double a0 = 0.0, a1 = 0.0, a2 = 0.0;
         if (SYM) {
           if (i < n) {
-            a0 = acc[i] * fwd;
-            a1 = acc[npad + i] * fwd;
-            a2 = acc[2 * npad + i] * fwd;
+            a0 = acc[i];
+            a1 = acc[npad + i];
+            a2 = acc[2 * npad + i];
           }
         } else if (DF) {
           float ah[3] = {0.0f, 0.0f, 0.0f}, al[3] = {0.0f, 0.0f, 0.0f};

@@ -49,19 +49,20 @@ __global__ void __launch_bounds__(ONE_NT, 4)
                const double *__restrict__ y, const double *__restrict__ z, const double *__restrict__ q, double soft2,
                double *__restrict__ part) {
   __shared__ __align__(16) float qs[ONE_J / 2 * ONE_PAIR];
+  __shared__ int qf[ONE_J / 32];  // places of each 32 staged partners
   pdl_wait();
   const int tid = threadIdx.x;
   const int64_t i = (int64_t)blockIdx.x * ONE_NT + tid;
   const bool own = i < ni;
   const int64_t g = i0 + i;
-  int em, ew;
-  const bool ok = tri_scale<ONE_NT, QARR>(0, 0, 0, (int)n, x, y, z, q, soft2, em, ew);
+  TriScale sc;
+  const bool ok = tri_scale<ONE_NT, QARR>(0, 0, 0, (int)n, x, y, z, q, soft2, sc);
   const int64_t c0 = (int64_t)blockIdx.y * jchunk, c1 = min(n, c0 + jchunk);
   double tot[3] = {0.0, 0.0, 0.0};
   if (!ok) {
     if (own) one_fp64<QARR>(x, y, z, q, soft2, g, c0, c1, tot);
   } else {
-    const int kl = em - 1022, kw = QARR ? ew - 1023 : 0;
+    const int kl = sc.em - 1022, kw = sc.ew - 1023;
     const double fwd = pow2d(kw - 2 * kl);
     f32x2 s2h = 0, s2l = 0;
     if (SOFT) {
@@ -71,7 +72,7 @@ __global__ void __launch_bounds__(ONE_NT, 4)
       s2l = pk1(l);
     }
     float w0[4], w1[4], w2[4];
-    const bool mylow = tri_ion<false>(g, own, x, y, z, q, em, ew, TRI_FAR, w0, w1, w2);
+    const int pf = tri_ion<false>(g, own, x, y, z, q, sc, TRI_FAR, w0, w1, w2);
     f32x2 ph[3], pm[3], pl[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -81,11 +82,12 @@ __global__ void __launch_bounds__(ONE_NT, 4)
     }
     for (int64_t jb = c0; jb < c1; jb += ONE_J) {
       const int cnt = (int)min((int64_t)ONE_J, c1 - jb), padded = (cnt + 3) & ~3;
-      int low = 0;
       if (jb > c0) __syncthreads();
-      for (int j = tid; j < padded; j += ONE_NT) {
+      for (int j = tid; j < ONE_J; j += ONE_NT) {  // a warp takes 32 partners
+        if ((j & ~31) >= padded) break;
         float v0[4], v1[4], v2[4];
-        low |= tri_ion<QARR>(jb + j, j < cnt, x, y, z, q, em, ew, -TRI_FAR, v0, v1, v2);
+        const int tf = __reduce_or_sync(0xffffffffu, tri_ion<QARR>(jb + j, j < cnt, x, y, z, q, sc, -TRI_FAR, v0, v1, v2));
+        if ((j & 31) == 0) qf[j >> 5] = tf;
         float *e = qs + (j >> 1) * ONE_PAIR + (j & 1);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -96,7 +98,9 @@ __global__ void __launch_bounds__(ONE_NT, 4)
         e[18] = v0[3];
         e[20] = v1[3];
       }
-      low = __syncthreads_or(low);
+      __syncthreads();
+      int cf = 0;  // the partners' places
+      for (int k = 0; k < padded; k += 32) cf |= qf[k >> 5];
       const int self = (int)(g - jb);  // the ion's own place among the staged partners, if any
       f32x2 ah[3] = {0, 0, 0}, al[3] = {0, 0, 0};
       float ymax = 0.0f, rmin = __int_as_float(0x7f800000);
@@ -108,9 +112,9 @@ __global__ void __launch_bounds__(ONE_NT, 4)
           const ulonglong2 *e = reinterpret_cast<const ulonglong2 *>(qs + (j >> 1) * ONE_PAIR);
           const ulonglong2 a = e[0], b = e[1], c2 = e[2], d = e[3], f = e[4];
           f32x2 dh[3], dl[3], h, l, sh, sl;
-          tri_diff(ph[0], pm[0], pl[0], a.x, b.y, d.x, dh[0], dl[0]);
-          tri_diff(ph[1], pm[1], pl[1], a.y, c2.x, d.y, dh[1], dl[1]);
-          tri_diff(ph[2], pm[2], pl[2], b.x, c2.y, f.x, dh[2], dl[2]);
+          tri_diff_n(ph[0], pm[0], pl[0], a.x, b.y, d.x, dh[0], dl[0]);
+          tri_diff_n(ph[1], pm[1], pl[1], a.y, c2.x, d.y, dh[1], dl[1]);
+          tri_diff_n(ph[2], pm[2], pl[2], b.x, c2.y, f.x, dh[2], dl[2]);
           tri_r2(dh, dl, h, l);
           float ha, hb;
           upk(h, ha, hb);
@@ -144,7 +148,6 @@ __global__ void __launch_bounds__(ONE_NT, 4)
         }
       }
       if (SOFT) ymax = rsqrt_approx(rmin);
-      const float ylim = low || mylow ? TRI_YMAX : TRI_YMAX_GRID;
       double r[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -153,7 +156,7 @@ __global__ void __launch_bounds__(ONE_NT, 4)
         upk(al[c], l0, l1);
         r[c] = ((f32_to_f64(h0) + f32_to_f64(h1)) + (f32_to_f64(l0) + f32_to_f64(l1))) * fwd;
       }
-      if (own && !(ymax <= ylim)) one_fp64<QARR>(x, y, z, q, soft2, g, jb, jb + cnt, r);
+      if (own && (tri_fault(pf, cf) || !(ymax <= TRI_YMAX_GRID))) one_fp64<QARR>(x, y, z, q, soft2, g, jb, jb + cnt, r);
 #pragma unroll
       for (int c = 0; c < 3; ++c) tot[c] += r[c];
     }

@@ -126,19 +126,20 @@ __global__ void __launch_bounds__(NT, NB)
   float4 *qs = reinterpret_cast<float4 *>(smem_raw);              // [G][TRI_TILE4]
   double *accQ = reinterpret_cast<double *>(qs + G * TRI_TILE4);  // [BI]
   double *accP = accQ + BI;                                       // [NW][PI]
+  __shared__ int qf[32];                                          // (the force kernel's; 1/r needs no component)
   const SymItem it = sym_block_item(INPLACE, sync, nbk);
   const int64_t p0 = (int64_t)it.P * BI, q0 = (int64_t)it.Q * BI;
   const int np = (int)min((int64_t)BI, n - p0), nq = (int)min((int64_t)BI, n - q0);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool diag = it.P == it.Q;
-  int em, ew;
-  const bool fast = tri_scale<NT, QARR>(p0, np, q0, diag ? 0 : nq, x, y, z, q, soft2, em, ew);
-  const int kl = fast ? em - 1022 : 0, kw = fast ? ew - 1023 : 0;  // units: L = 2^kl, weights 2^kw
+  TriScale sc;
+  const bool fast = tri_scale<NT, QARR>(p0, np, q0, diag ? 0 : nq, x, y, z, q, soft2, sc);
+  const int kl = fast ? sc.em - 1022 : 0, kw = fast ? sc.ew - 1023 : 0;  // units: L = 2^kl, weights 2^kw
   const int PT = BI / PI, NG = NW / PT, nqt = G / NG;
   const int pt = warp % PT, grp = warp / PT;
   TriIons<V> p;
-  int low = 0;
-  if (fast) low = tri_load<V, QARR, NT>(p, qs, BI, pt, p0, np, q0, nq, x, y, z, q, em, ew);
+  bool low = false;
+  if (fast) tri_load<V, QARR, NT, TRI_NEAR, true>(p, qs, qf, BI, pt, p0, np, q0, nq, x, y, z, q, sc, low);
   for (int i = tid; i < BI; i += NT) accQ[i] = 0.0;
   for (int i = tid; i < NW * PI; i += NT) accP[i] = 0.0;
   const float ylim = __syncthreads_or(low) ? TRI_YMAX : TRI_YMAX_GRID;

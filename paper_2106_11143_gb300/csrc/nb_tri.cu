@@ -218,25 +218,32 @@ __global__ void __launch_bounds__(NT, NB)
   float4 *qs = reinterpret_cast<float4 *>(smem_raw);                 // [G][TRI_TILE4]
   double *accQ = reinterpret_cast<double *>(qs + G * TRI_TILE4);     // [3][BI]
   double *accP = accQ + 3 * BI;                                      // [NW][3][PI]
+  __shared__ int qf[32];                                             // places of each Q-tile (G <= 32)
+  __shared__ int ex[3];                                              // the axes' exponents, for tri_tile_fault
   const SymItem it = sym_block_item(INPLACE, sync, nbk);
   const int64_t p0 = (int64_t)it.P * BI, q0 = (int64_t)it.Q * BI;
   const int np = (int)min((int64_t)BI, n - p0), nq = (int)min((int64_t)BI, n - q0);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool diag = it.P == it.Q;
-  int em, ew;
-  const bool fast = tri_scale<NT, QARR>(p0, np, q0, diag ? 0 : nq, x, y, z, q, soft2, em, ew);
+  TriScale sc;
+  const bool fast = tri_scale<NT, QARR>(p0, np, q0, diag ? 0 : nq, x, y, z, q, soft2, sc);
   // units: a coordinate is L X with L = 2^(em - 1022), a weight 2^(ew - 1023) w
-  const int kl = fast ? em - 1022 : 0, kw = fast ? ew - 1023 : 0;
+  const int kl = fast ? sc.em - 1022 : 0, kw = fast ? sc.ew - 1023 : 0;
 
   const int PT = BI / PI, NG = NW / PT, nqt = G / NG;  // P-tiles, warps per P-tile, Q-tiles per warp
   const int pt = warp % PT, grp = warp / PT;
   TriIons<V> p;
-  int low = 0;  // a coordinate has bits in or below its l word
-  if (fast) low = tri_load<V, QARR, NT>(p, qs, BI, pt, p0, np, q0, nq, x, y, z, q, em, ew);
+  int pf = 0;
+  bool low;
+  if (tid == 0) {
+    ex[0] = sc.ex[0];
+    ex[1] = sc.ex[1];
+    ex[2] = sc.ex[2];
+  }
+  if (fast) pf = tri_load<V, QARR, NT, MIX ? TRI_NEAR_MIX : TRI_NEAR, false>(p, qs, qf, BI, pt, p0, np, q0, nq, x, y, z, q, sc, low);
   for (int i = tid; i < 3 * BI; i += NT) accQ[i] = 0.0;
   for (int i = tid; i < NW * 3 * PI; i += NT) accP[i] = 0.0;
-  // FP32 rounding of d leaves the 2^-69 L cut far behind at any distance (MIX)
-  const float ylim = __syncthreads_or(low) && !MIX ? TRI_YMAX : TRI_YMAX_GRID;
+  __syncthreads();
   f32x2 s2h = 0, s2l = 0;
   if (SOFT) {
     float sh, sl;
@@ -261,7 +268,10 @@ __global__ void __launch_bounds__(NT, NB)
     const bool one = diag && (!MIX || sp == sq);
     if (MIX && diag && sp > sq) continue;
     bool done = false;
-    if (fast) {
+    bool words = fast;
+    if (fast && (pf & qf[t]))
+      words = !tri_tile_fault<MIX ? TRI_NEAR_MIX : TRI_NEAR>(n, x, y, z, p0 + pt * PI, PI, q0 + t * 32, ex);
+    if (words) {
       TriSums<V> ts;
       const f32x2 zero = pk1(0.0f);
 #pragma unroll
@@ -286,7 +296,7 @@ __global__ void __launch_bounds__(NT, NB)
         ymax = MIX ? tri_tile_mixed<V, QARR, false>(p, qt, lane, -1, ts)
                    : tri_tile<V, QARR, false, SOFT>(p, ld, lane, -1, s2h, s2l, ts);
       }
-      done = !__any_sync(0xffffffffu, !(ymax <= ylim));
+      done = !__any_sync(0xffffffffu, !(ymax <= TRI_YMAX_GRID));
       if (done) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {

@@ -3,24 +3,32 @@
 //
 // GB300's FP64 pipe retires 2 lanes per clock per SM against 128 on the FP32
 // pipe, so even the three FP64 subtractions of a displacement take longer than
-// about 100 FP32 instructions.  Here a work item (two blocks of ions) picks one
-// power of two L above every coordinate it touches and cuts each coordinate's
-// bits, in units of L, into
+// about 100 FP32 instructions.  Here a work item (two sets of ions) picks for
+// each axis a power of two L_c above every coordinate of that axis it touches
+// and cuts the coordinates' bits, in units of L_c, into
 //   h: a multiple of 2^-22,  m: a multiple of 2^-45 below 2^-22,
-//   l: a multiple of 2^-69 below 2^-45   (all with the coordinate's sign).
-// A FP64 coordinate of at least 2^-16 L is represented exactly, a smaller one
-// to 2^-69 L.  The words' differences are exact in FP32 (at most 24 bits on
-// the word's own grid), so d = dh + dm + dl is exact, and one Fast2Sum makes
-// it the double-float (RN(dh + dm), rest): 7 FP32 operations per component,
-// all of which exist as packed .f32x2 instructions.
+//   l: a multiple of 2^-69 below 2^-45   (all with the coordinate's sign),
+// which are then put in units of L = max L_c, an exact scaling.  The words'
+// differences are exact in FP32, so d = dh + dm + dl is exact, and two Fast2Sums
+// make it a double-float (RN(d), rest), whatever words it starts in: 10 FP32
+// operations per component, all of which exist as packed .f32x2 instructions.
+// Each component is right to 2^-48 of itself, as an FP64 difference is right to
+// 2^-53 of itself, which the transverse forces of a thin chain need: its y may be
+// 2^-40 of its z.  One unit for the three axes left y with its bits above 2^-69
+// of the largest z, and an unnormalised (dh + dm, dl) with FP32 accuracy where
+// dh and dm cancel.
 //
-// A pair closer than 2^-20 L (where the 2^-69 L cut would pass 2^-49 of the
-// distance, and dl stops being small against dm) makes its tile fall back to
-// FP64 arithmetic; the test is the smallest r^2 met, one FMNMX per pair.  When
-// no coordinate of the item has bits in l or below it (positions on a grid), d
-// is exact and normal at any distance, and only FP32's range sets a limit, 2^-40 L.
-// Items whose scale or weights are far from the ordinary (below) take the
-// FP64 path as a whole.
+// A coordinate of at least 2^-17 L_c is exact in its words, a smaller one if it
+// has no bits below 2^-68 L_c (grids, zeros); else it is cut.  Against a partner
+// of 2^-15 L_c or more a cut one is right to 2^-52 of the difference; a tile
+// (pairs of 32 .. 128 ions) that holds a cut coordinate on one side and one below
+// 2^-15 L_c of the same axis on the other is done in FP64 (tri_fault; 3 tiles in
+// 10 000 of a random cloud).
+//
+// What is left for FP32's range: pairs closer than 2^-40 L send their tile to
+// FP64 too (the smallest r^2 met, one FMNMX per pair), and items whose scale,
+// flatness or weights are far from the ordinary (below) take the FP64 path as a
+// whole.
 #pragma once
 
 #include "nb_common.cuh"
@@ -77,9 +85,9 @@ __device__ __forceinline__ void ptwo_diff(f32x2 a, f32x2 b, f32x2 &s, f32x2 &e) 
   e = psub(psub(a, psub(s, bb)), padd(b, bb));
 }
 
-// The words of coordinate x in units of L = 2^(em - 1022), em at least x's
-// biased exponent: w[0] + w[1] + w[2] = x / L to 2^-69.
-__device__ __forceinline__ void tri_words(double x, int em, float w[3]) {
+// The words of coordinate x in units of 2^(em - 1022), em at least x's biased
+// exponent, times f: w[0] + w[1] + w[2] = f x / 2^(em - 1022) to 2^-69 f.
+__device__ __forceinline__ void tri_words(double x, int em, float f, float w[3]) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int e = (int)((hi >> 20) & 0x7ffu);
   const unsigned t1 = e ? (0x80000000u | ((hi & 0xfffffu) << 11) | (lo >> 21)) : 0u, t0 = e ? lo << 11 : 0u;
@@ -88,18 +96,30 @@ __device__ __forceinline__ void tri_words(double x, int em, float w[3]) {
   const unsigned w0 = j == 0 ? a0 : 0u;
   const unsigned w1 = j == 0 ? a1 : (j == 1 ? a0 : 0u);
   const unsigned w2 = j == 0 ? a2 : (j == 1 ? a1 : (j == 2 ? a0 : 0u));
-  const float sg = __uint_as_float(0x3f800000u | (hi & 0x80000000u));
+  const float sg = __uint_as_float(__float_as_uint(f) | (hi & 0x80000000u));
   w[0] = (float)(int)(w0 >> 10) * (sg * 0x1p-22f);
   w[1] = (float)(int)(((w0 & 0x3ffu) << 13) | (w1 >> 19)) * (sg * 0x1p-45f);
   w[2] = (float)(int)(((w1 & 0x7ffffu) << 5) | (w2 >> 27)) * (sg * 0x1p-69f);
 }
 
-// Whether the words of x hold it exactly: none of its bits lies below 2^-69.
-__device__ __forceinline__ bool tri_exact(double x, int em) {
+// A coordinate's place on its axis's grid: bit 0, cut (it has bits below 2^-68,
+// counted so that the difference of two uncut ones fits the words' 24 bits also
+// where their signs differ, and is below 2^(-2 - NEAR)); bit 3, near the origin
+// (below 2^-NEAR).  Shifted by the axis, 0 .. 2.
+constexpr int TRI_NEAR = 15;      // a cut coordinate is right to 2^-52 of a difference
+constexpr int TRI_NEAR_MIX = 38;  // .. to 2^-29, for FP32 displacements
+template <int NEAR>
+__device__ __forceinline__ int tri_place(double x, int em, int c) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int s = em - (int)((hi >> 20) & 0x7ffu);
+  const int e = (int)((hi >> 20) & 0x7ffu), s = em - e;
+  if (s < NEAR) return 0;
   const int tz = lo ? __ffs((int)lo) - 1 : 31 + __ffs((int)((hi & 0xfffffu) | 0x100000u));
-  return s <= 16 || ((hi << 1) | lo) == 0 || tz >= s - 16;
+  const bool cut = s >= NEAR + 2 && ((hi << 1) | lo) != 0 && (e == 0 || tz < s - 15);
+  return (cut ? 1 << c : 0) | (8 << c);
+}
+// Whether a pair of the two sides (OR of their ions' places) may lose bits.
+__device__ __forceinline__ bool tri_fault(int p, int q) {
+  return (((p >> 3) & q) | (p & (q >> 3))) & 7;
 }
 
 // A padding ion's coordinate, in units of L: far enough that every term with
@@ -107,33 +127,67 @@ __device__ __forceinline__ bool tri_exact(double x, int em) {
 // two sides use opposite signs, so two padding ions never coincide.
 constexpr float TRI_FAR = 1e18f;
 
-// Largest 1/r (units of 1/L) of the FP32 path, and where no l word is set.
-constexpr float TRI_YMAX = 0x1p20f, TRI_YMAX_GRID = 0x1p40f;
+// Largest 1/r (units of 1/L) of the FP32 path: y^3 and its products stay in range.
+constexpr float TRI_YMAX_GRID = 0x1p40f;
+// The same where the displacement is left unnormalised (nb_phi.cu) and an l word
+// is set or a coordinate cut.
+constexpr float TRI_YMAX = 0x1p20f;
 
-// Scales the path accepts: L within 2^+-200 (so that L^2, L^-2 and their
-// products with a force stay far inside FP64), and weights within 2^40 of the
-// item's largest (so that a double-float weight keeps its 48 bits).
-constexpr int TRI_EMIN = 1023 - 200, TRI_EMAX = 1023 + 200, TRI_WSPREAD = 40;
+// Scales the path accepts: L within 2^+-150 (so that L^2, L^-2 and their products
+// with any force the FP64 path can form stay inside FP64), weights within 2^40 of
+// the item's largest (so that a double-float weight keeps its 48 bits), and an axis
+// at least 2^-64 of the longest: its words are exact down to FP32's 2^-149, and the
+// products' and sums' roundings there, 2^-149 each, are below 2^-57 of the terms its
+// largest coordinate has with far partners (less 16 with weights, less 24 with a
+// softening beyond L, by what these take off the terms).
+constexpr int TRI_EMIN = 1023 - 150, TRI_EMAX = 1023 + 150, TRI_FLAT = 64, TRI_WSPREAD = 40;
 // and a softening length up to 2^10 L (far above it the terms' low parts would
 // leave FP32's range).
 __device__ __forceinline__ bool tri_scale_ok(int em, double soft2) {
   return em >= TRI_EMIN && em <= TRI_EMAX && ((__double2hiint(soft2) >> 20) & 0x7ff) - 2 * (em - 1022) <= 1023 + 20;
 }
 
-// d = p - q as a double-float: the word differences are exact; Fast2Sum holds
-// because dh is 0 or at least 2^-22 > |dm|.
+// An item's scale: biased exponents of L and of the axes' L_c, and of the weights.
+struct TriScale {
+  int em, ex[3], ew;
+  __device__ __forceinline__ float f(int c) const { return __int_as_float((127 + ex[c] - em) << 23); }
+};
+// From the largest high words of the coordinates of each axis; false: FP64.
+template <bool QARR>
+__device__ __forceinline__ bool tri_axes(const int mx[3], double soft2, TriScale &s) {
+  s.em = max(mx[0], max(mx[1], mx[2])) >> 20;
+  bool ok = tri_scale_ok(s.em, soft2);
+  const int flat = TRI_FLAT - (QARR ? 16 : 0) - ((__double2hiint(soft2) >> 20) - 2 * (s.em - 1022) > 1023 ? 24 : 0);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    s.ex[c] = mx[c] ? mx[c] >> 20 : s.em;  // an axis of zeros: any unit
+    ok = ok && s.em - s.ex[c] <= flat;
+  }
+  return ok;
+}
+
+// s + e = a + b exactly for |a| >= |b|, or a a multiple of ulp(s) (Fast2Sum).
+__device__ __forceinline__ void pfast2(f32x2 &a, f32x2 &b) {
+  const f32x2 s = padd(a, b);
+  b = psub(b, psub(s, a));
+  a = s;
+}
+
+// d = p - q as an unnormalised double-float: the word differences are exact, and
+// so is the Fast2Sum of dh and dm: |dm| may reach 2^-21 (signs that differ), but
+// dh is 0 or a multiple of 2^-22 and thus of the sum's last place.
 __device__ __forceinline__ void tri_diff(f32x2 ph, f32x2 pm, f32x2 pl, f32x2 qh, f32x2 qm, f32x2 ql, f32x2 &h,
                                          f32x2 &l) {
   const f32x2 dh = psub(ph, qh), dm = psub(pm, qm), dl = psub(pl, ql);
   h = padd(dh, dm);
   l = padd(psub(dm, psub(h, dh)), dl);
 }
-
-// s + e = a + b exactly for |a| >= |b| (Fast2Sum).
-__device__ __forceinline__ void pfast2(f32x2 &a, f32x2 &b) {
-  const f32x2 s = padd(a, b);
-  b = psub(b, psub(s, a));
-  a = s;
+// The same with h = RN(d): where dh and dm cancel, the leading bits of d stand in
+// l, and a product with (h, l) would keep only 24 of them.
+__device__ __forceinline__ void tri_diff_n(f32x2 ph, f32x2 pm, f32x2 pl, f32x2 qh, f32x2 qm, f32x2 ql, f32x2 &h,
+                                           f32x2 &l) {
+  tri_diff(ph, pm, pl, qh, qm, ql, h, l);
+  pfast2(h, l);
 }
 
 // r^2 of the double-float displacement (dh, dl) as the double-float (h, l).
@@ -253,9 +307,9 @@ __device__ __forceinline__ float tri_tile(const TriIons<V> &p, LD ld, int lane, 
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         f32x2 dh[3], dl[3], h, l, sh, sl;
-        tri_diff(p.h[v][0], p.m[v][0], p.l[v][0], pk1(q0.x), pk1(q1.x), pk1(q2.x), dh[0], dl[0]);
-        tri_diff(p.h[v][1], p.m[v][1], p.l[v][1], pk1(q0.y), pk1(q1.y), pk1(q2.y), dh[1], dl[1]);
-        tri_diff(p.h[v][2], p.m[v][2], p.l[v][2], pk1(q0.z), pk1(q1.z), pk1(q2.z), dh[2], dl[2]);
+        tri_diff_n(p.h[v][0], p.m[v][0], p.l[v][0], pk1(q0.x), pk1(q1.x), pk1(q2.x), dh[0], dl[0]);
+        tri_diff_n(p.h[v][1], p.m[v][1], p.l[v][1], pk1(q0.y), pk1(q1.y), pk1(q2.y), dh[1], dl[1]);
+        tri_diff_n(p.h[v][2], p.m[v][2], p.l[v][2], pk1(q0.z), pk1(q1.z), pk1(q2.z), dh[2], dl[2]);
         tri_r2(dh, dl, h, l);
         float ha, hb;
         upk(h, ha, hb);
@@ -305,108 +359,121 @@ __device__ __forceinline__ float tri_tile(const TriIons<V> &p, LD ld, int lane, 
   return SOFT ? rsqrt_approx(rmin) : ymax;
 }
 
-// Words of ion g (or a padding ion on side `far`) with its weight; returns whether
-// an l word is set or the words do not hold a coordinate exactly (bits below 2^-69
-// leave no trace in l).
-template <bool QARR>
-__device__ __forceinline__ bool tri_ion(int64_t g, bool real, const double *x, const double *y, const double *z,
-                                        const double *q, int em, int ew, float far, float w0[4], float w1[4],
-                                        float w2[4]) {
+// Words of ion g (or a padding ion on side `far`) with its weight; returns its place
+// (without CUT, the bits of the axes it is near on alone: no branches).
+template <bool QARR, int NEAR = TRI_NEAR, bool CUT = true>
+__device__ __forceinline__ int tri_ion(int64_t g, bool real, const double *x, const double *y, const double *z,
+                                       const double *q, const TriScale &sc, float far, float w0[4], float w1[4],
+                                       float w2[4]) {
   w0[3] = w1[3] = w2[3] = 0.0f;
+  int place = 0;
   if (real) {
-    float t[3];
-    tri_words(x[g], em, t);
-    w0[0] = t[0]; w1[0] = t[1]; w2[0] = t[2];
-    tri_words(y[g], em, t);
-    w0[1] = t[0]; w1[1] = t[1]; w2[1] = t[2];
-    tri_words(z[g], em, t);
-    w0[2] = t[0]; w1[2] = t[1]; w2[2] = t[2];
-    if (QARR && q[g] != 0.0) split_f64_scaled(q[g], ew - 1023, w0[3], w1[3]);
-    return w2[0] != 0.0f || w2[1] != 0.0f || w2[2] != 0.0f || !tri_exact(x[g], em) || !tri_exact(y[g], em) ||
-           !tri_exact(z[g], em);
+    const double r[3] = {x[g], y[g], z[g]};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      float t[3];
+      tri_words(r[c], sc.ex[c], sc.f(c), t);
+      w0[c] = t[0];
+      w1[c] = t[1];
+      w2[c] = t[2];
+      if (CUT)
+        place |= tri_place<NEAR>(r[c], sc.ex[c], c);
+      else
+        place |= sc.ex[c] - ((__double2hiint(r[c]) >> 20) & 0x7ff) >= NEAR ? 8 << c : 0;
+    }
+    if (QARR && q[g] != 0.0) split_f64_scaled(q[g], sc.ew - 1023, w0[3], w1[3]);
   } else {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       w0[c] = far;
       w1[c] = w2[c] = 0.0f;
     }
-    return false;
   }
+  return place;
 }
 
 // A staged tile: word k of entry e (64 entries, the tile twice) at
 // [k * 64 + e], the weight's high and low parts in the w of words 0 and 1.
 constexpr int TRI_TILE4 = 3 * 64;
 
-// The item's scale: the largest biased exponent of a coordinate in em, the
-// weights' in ew; false when the item is left to FP64.  Ends with a barrier.
+// The item's scale over ions [p0, p0 + np) and [q0, q0 + nq); false when the item is
+// left to FP64.  Ends with a barrier.
 template <int NT, bool QARR>
 __device__ __forceinline__ bool tri_scale(int64_t p0, int np, int64_t q0, int nq, const double *x, const double *y,
-                                          const double *z, const double *q, double soft2, int &em, int &ew) {
-  __shared__ int red[3][NT / 32];
-  int mx = 0, wx = 0, wn = 0x7fffffff;
+                                          const double *z, const double *q, double soft2, TriScale &sc) {
+  __shared__ int red[5][NT / 32];
+  int mx[3] = {0, 0, 0}, wx = 0, wn = 0x7fffffff;
   for (int i = threadIdx.x; i < np + nq; i += NT) {
     const int64_t g = i < np ? p0 + i : q0 + (i - np);
-    mx = max(mx, __double2hiint(x[g]) & 0x7fffffff);
-    mx = max(mx, __double2hiint(y[g]) & 0x7fffffff);
-    mx = max(mx, __double2hiint(z[g]) & 0x7fffffff);
+    mx[0] = max(mx[0], __double2hiint(x[g]) & 0x7fffffff);
+    mx[1] = max(mx[1], __double2hiint(y[g]) & 0x7fffffff);
+    mx[2] = max(mx[2], __double2hiint(z[g]) & 0x7fffffff);
     if (QARR) {
       const int w = __double2hiint(q[g]) & 0x7fffffff;
       wx = max(wx, w);
       if (q[g] != 0.0) wn = min(wn, w);
     }
   }
-  mx = __reduce_max_sync(0xffffffffu, mx);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) mx[c] = __reduce_max_sync(0xffffffffu, mx[c]);
   if (QARR) {
     wx = __reduce_max_sync(0xffffffffu, wx);
     wn = __reduce_min_sync(0xffffffffu, wn);
   }
   const int w = threadIdx.x >> 5;
   if ((threadIdx.x & 31) == 0) {
-    red[0][w] = mx;
-    red[1][w] = wx;
-    red[2][w] = wn;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) red[c][w] = mx[c];
+    red[3][w] = wx;
+    red[4][w] = wn;
   }
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < NT / 32; ++k) {
-    mx = max(mx, red[0][k]);
-    wx = max(wx, red[1][k]);
-    wn = min(wn, red[2][k]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) mx[c] = max(mx[c], red[c][k]);
+    wx = max(wx, red[3][k]);
+    wn = min(wn, red[4][k]);
   }
-  em = mx >> 20;
-  ew = 1023;
-  bool ok = tri_scale_ok(em, soft2);
+  bool ok = tri_axes<QARR>(mx, soft2, sc);
+  sc.ew = 1023;
   if (QARR) {
-    ew = wx >> 20;
-    ok = ok && ew >= 1023 - 400 && ew <= 1023 + 400 && ew - (wn >> 20) <= TRI_WSPREAD;
+    sc.ew = wx >> 20;
+    ok = ok && sc.ew >= 1023 - 400 && sc.ew <= 1023 + 400 && sc.ew - (wn >> 20) <= TRI_WSPREAD;
   }
   return ok;
 }
 
-// Cuts the Q block's ions into words in shared memory (BI entries) and loads the
-// lane's ions of P-tile pt; returns whether tri_ion did for any.
-template <int V, bool QARR, int NT>
-__device__ __forceinline__ int tri_load(TriIons<V> &p, float4 *qs, int BI, int pt, int64_t p0, int np, int64_t q0,
-                                        int nq, const double *x, const double *y, const double *z, const double *q,
-                                        int em, int ew) {
+// Cuts the Q block's ions into words in shared memory (BI entries), with the OR of
+// each tile's places in qf, and loads the lane's ions of P-tile pt; returns the
+// OR of that tile's places (CUT as in tri_ion).  low, with CUT: an l word is set or
+// a coordinate cut.
+template <int V, bool QARR, int NT, int NEAR, bool CUT>
+__device__ __forceinline__ int tri_load(TriIons<V> &p, float4 *qs, int *qf, int BI, int pt, int64_t p0, int np,
+                                        int64_t q0, int nq, const double *x, const double *y, const double *z,
+                                        const double *q, const TriScale &sc, bool &low) {
   const int lane = threadIdx.x & 31;
-  int low = 0;
-  for (int i = threadIdx.x; i < BI; i += NT) {
+  low = false;
+  for (int i = threadIdx.x; i < BI; i += NT) {  // a warp takes a tile
     float w0[4], w1[4], w2[4];
-    low |= tri_ion<QARR>(q0 + i, i < nq, x, y, z, q, em, ew, -TRI_FAR, w0, w1, w2);
+    const int f = tri_ion<QARR, NEAR, CUT>(q0 + i, i < nq, x, y, z, q, sc, -TRI_FAR, w0, w1, w2);
     float4 *e = qs + (i >> 5) * TRI_TILE4 + (i & 31);
     e[0] = e[32] = make_float4(w0[0], w0[1], w0[2], w0[3]);
     e[64] = e[96] = make_float4(w1[0], w1[1], w1[2], w1[3]);
     e[128] = e[160] = make_float4(w2[0], w2[1], w2[2], w2[3]);
+    low |= w2[0] != 0.0f || w2[1] != 0.0f || w2[2] != 0.0f || (f & 7);
+    const int tf = __reduce_or_sync(0xffffffffu, f);
+    if (lane == 0) qf[i >> 5] = tf;
   }
+  int pf = 0;
 #pragma unroll
   for (int v = 0; v < V; ++v) {
     float w0[2][4], w1[2][4], w2[2][4];
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int i = pt * 64 * V + v * 64 + b * 32 + lane;
-      low |= tri_ion<QARR>(p0 + i, i < np, x, y, z, q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
+      pf |= tri_ion<QARR, NEAR, CUT>(p0 + i, i < np, x, y, z, q, sc, TRI_FAR, w0[b], w1[b], w2[b]);
+      low |= w2[b][0] != 0.0f || w2[b][1] != 0.0f || w2[b][2] != 0.0f;
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -417,7 +484,26 @@ __device__ __forceinline__ int tri_load(TriIons<V> &p, float4 *qs, int BI, int p
     p.wh[v] = pk(w0[0][3], w0[1][3]);
     p.wl[v] = pk(w1[0][3], w1[1][3]);
   }
-  return low;
+  low |= pf & 7;
+  return __reduce_or_sync(0xffffffffu, pf);
+}
+
+// Whether a tile whose sides are both near the origin on one axis may lose bits:
+// ions [i0, i0 + ni) against [j0, j0 + 32), those below n; ex: the axes' exponents.
+template <int NEAR>
+__device__ __noinline__ bool tri_tile_fault(int64_t n, const double *x, const double *y, const double *z, int64_t i0,
+                                            int ni, int64_t j0, const int *ex) {
+  const int lane = threadIdx.x & 31;
+  auto place = [&](int64_t g) {
+    return g < n ? tri_place<NEAR>(x[g], ex[0], 0) | tri_place<NEAR>(y[g], ex[1], 1) |
+                       tri_place<NEAR>(z[g], ex[2], 2)
+                 : 0;
+  };
+  int f = place(j0 + lane) << 6;
+#pragma unroll 1
+  for (int u = 0; u < ni; u += 32) f |= place(i0 + u + lane);
+  f = __reduce_or_sync(0xffffffffu, f);
+  return tri_fault(f, f >> 6);
 }
 
 // The plan of a force evaluation: make_plan's, with this file's kernel's own

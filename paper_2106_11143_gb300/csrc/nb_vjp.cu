@@ -215,9 +215,9 @@ __device__ __forceinline__ float vjp_tile(const VjpIons &p, const float4 *qt, in
       const float4 *qe = qt + ((lane + r0 + s) & 31);
       const float4 q0 = qe[0], q1 = qe[32], q2 = qe[64], u0 = qe[96], u1 = qe[128], u2 = qe[160];
       f32x2 dh[3], dl[3], eh[3], el[3], h, l, sh, sl, wh, wl;
-      tri_diff(p.r.h[0][0], p.r.m[0][0], p.r.l[0][0], pk1(q0.x), pk1(q1.x), pk1(q2.x), dh[0], dl[0]);
-      tri_diff(p.r.h[0][1], p.r.m[0][1], p.r.l[0][1], pk1(q0.y), pk1(q1.y), pk1(q2.y), dh[1], dl[1]);
-      tri_diff(p.r.h[0][2], p.r.m[0][2], p.r.l[0][2], pk1(q0.z), pk1(q1.z), pk1(q2.z), dh[2], dl[2]);
+      tri_diff_n(p.r.h[0][0], p.r.m[0][0], p.r.l[0][0], pk1(q0.x), pk1(q1.x), pk1(q2.x), dh[0], dl[0]);
+      tri_diff_n(p.r.h[0][1], p.r.m[0][1], p.r.l[0][1], pk1(q0.y), pk1(q1.y), pk1(q2.y), dh[1], dl[1]);
+      tri_diff_n(p.r.h[0][2], p.r.m[0][2], p.r.l[0][2], pk1(q0.z), pk1(q1.z), pk1(q2.z), dh[2], dl[2]);
       tri_r2(dh, dl, h, l);
       float ha, hb;
       upk(h, ha, hb);
@@ -236,12 +236,9 @@ __device__ __forceinline__ float vjp_tile(const VjpIons &p, const float4 *qt, in
         yb = fminf(yb, 0x1p30f);
       }
       vjp_rinv(h, l, pk(ya, yb), sh, sl, wh, wl);
-      // the cotangents' difference: normalised, since it may be tiny beside either
-      tri_diff(p.lam.h[0][0], p.lam.m[0][0], p.lam.l[0][0], pk1(u0.x), pk1(u1.x), pk1(u2.x), eh[0], el[0]);
-      tri_diff(p.lam.h[0][1], p.lam.m[0][1], p.lam.l[0][1], pk1(u0.y), pk1(u1.y), pk1(u2.y), eh[1], el[1]);
-      tri_diff(p.lam.h[0][2], p.lam.m[0][2], p.lam.l[0][2], pk1(u0.z), pk1(u1.z), pk1(u2.z), eh[2], el[2]);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) pfast2(eh[c], el[c]);
+      tri_diff_n(p.lam.h[0][0], p.lam.m[0][0], p.lam.l[0][0], pk1(u0.x), pk1(u1.x), pk1(u2.x), eh[0], el[0]);
+      tri_diff_n(p.lam.h[0][1], p.lam.m[0][1], p.lam.l[0][1], pk1(u0.y), pk1(u1.y), pk1(u2.y), eh[1], el[1]);
+      tri_diff_n(p.lam.h[0][2], p.lam.m[0][2], p.lam.l[0][2], pk1(u0.z), pk1(u1.z), pk1(u2.z), eh[2], el[2]);
       float m0[3], m1[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) upk(eh[c], m0[c], m1[c]);
@@ -327,91 +324,113 @@ __device__ __noinline__ void vjp_tile_units(int64_t n, const double *x, const do
   }
 }
 
-// The item's scales: the largest biased exponents of a coordinate, of each
-// component of a cotangent and of a weight; false when the item is left to
-// vjp_tile_units (lengths or cotangents beyond 2^+-100 and 2^+-200, components
-// more than 2^40 apart, weights as in nb_tri.cuh, a softening far above the
-// cloud).  Ends with a barrier.
+// The same in FP64, for the tiles of flat items (vjp_scale): a pair's own units lose
+// a component below 2^-74 of its largest.
+template <bool QARR>
+__device__ __noinline__ void vjp_tile_fp64(int64_t n, const double *x, const double *y, const double *z, const double *q,
+                                           const double *lx, const double *ly, const double *lz, double soft2,
+                                           int64_t i0, int64_t j0, bool one, double sc, double *accP, int ldp,
+                                           double *accQ, int ldq) {
+  const int lane = threadIdx.x & 31;
+  for (int u = 0; u < 64; u += 32) {
+    const int64_t i = i0 + u + lane;
+    double a[3] = {0.0, 0.0, 0.0}, b[3] = {0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int r = 0; r < 32; ++r) {
+      const int64_t j = j0 + ((lane + r) & 31);
+      if (i < n && j < n && i != j) {
+        const double d[3] = {x[i] - x[j], y[i] - y[j], z[i] - z[j]};
+        const double l[3] = {lx[i] - lx[j], ly[i] - ly[j], lz[i] - lz[j]};
+        const double s = rinv3_fp64(d[0], d[1], d[2], soft2), v = rinv1_fp64(d[0], d[1], d[2], soft2);
+        const double k = 3.0 * (v * v) * fma(d[0], l[0], fma(d[1], l[1], d[2] * l[2]));
+        for (int c = 0; c < 3; ++c) {
+          const double t = s * fma(-k, d[c], l[c]);
+          a[c] += QARR ? t * q[j] : t;
+          b[c] -= QARR ? t * q[i] : t;
+        }
+      }
+      for (int c = 0; c < 3; ++c) b[c] = __shfl_sync(0xffffffffu, b[c], (lane + 1) & 31);
+    }
+    for (int c = 0; c < 3; ++c) {
+      accP[c * ldp + u + lane] += a[c] * sc;
+      if (!one) accQ[c * ldq + lane] += b[c] * sc;
+    }
+  }
+}
+
+// The item's scales: those of the positions and weights (nb_tri.cuh) and the
+// largest biased exponents of the cotangents' components; false when the item is
+// left to vjp_tile_units (lengths or cotangents beyond 2^+-100 and 2^+-200,
+// components of a cotangent more than 2^40 apart, a position or weight scale that
+// nb_tri.cuh leaves to FP64).  deep: an axis of the positions or cotangents is
+// below 2^-30 of the longest, so that the tiles left to other forms need FP64.
+// Ends with a barrier.
 template <bool QARR>
 __device__ __forceinline__ bool vjp_scale(int64_t p0, int np, int64_t q0, int nq, const double *x, const double *y,
                                           const double *z, const double *q, const double *lx, const double *ly,
-                                          const double *lz, double soft2, int &em, int el[3], int &ew) {
-  __shared__ int red[6][VJP_W];
-  int mx = 0, lm[3] = {0, 0, 0}, wx = 0, wn = 0x7fffffff;
+                                          const double *lz, double soft2, TriScale &sc, int el[3], bool &deep) {
+  __shared__ int red[3][VJP_W];
+  int lm[3] = {0, 0, 0};
   auto mag = [](double v) { return __double2hiint(v) & 0x7fffffff; };
   for (int i = threadIdx.x; i < np + nq; i += VJP_THREADS) {
     const int64_t g = i < np ? p0 + i : q0 + (i - np);
-    mx = max(mx, max(mag(x[g]), max(mag(y[g]), mag(z[g]))));
     lm[0] = max(lm[0], mag(lx[g]));
     lm[1] = max(lm[1], mag(ly[g]));
     lm[2] = max(lm[2], mag(lz[g]));
-    if (QARR && q[g] != 0.0) {
-      wx = max(wx, mag(q[g]));
-      wn = min(wn, mag(q[g]));
-    }
   }
-  const int w = threadIdx.x >> 5;
-  mx = __reduce_max_sync(0xffffffffu, mx);
-  wx = __reduce_max_sync(0xffffffffu, wx);
-  wn = __reduce_min_sync(0xffffffffu, wn);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) lm[c] = __reduce_max_sync(0xffffffffu, lm[c]);
-  if ((threadIdx.x & 31) == 0) {
-    red[0][w] = mx;
-    red[1][w] = wx;
-    red[2][w] = wn;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) red[3 + c][w] = lm[c];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < VJP_W; ++k) {
-    mx = max(mx, red[0][k]);
-    wx = max(wx, red[1][k]);
-    wn = min(wn, red[2][k]);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) lm[c] = max(lm[c], red[3 + c][k]);
-  }
-  em = mx >> 20;
-  const int top = max(lm[0], max(lm[1], lm[2])) >> 20;
-  bool ok = tri_scale_ok(em, soft2) && em >= 1023 - 100 && em <= 1023 + 100 && top <= 1023 + 200;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
+    lm[c] = __reduce_max_sync(0xffffffffu, lm[c]);
+    if ((threadIdx.x & 31) == 0) red[c][threadIdx.x >> 5] = lm[c];
+  }
+  bool ok = tri_scale<VJP_THREADS, QARR>(p0, np, q0, nq, x, y, z, q, soft2, sc);  // holds the barrier
+#pragma unroll
+  for (int k = 0; k < VJP_W; ++k)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) lm[c] = max(lm[c], red[c][k]);
+  const int top = max(lm[0], max(lm[1], lm[2])) >> 20;
+  deep = false;
+  const bool plain = sc.em >= 1023 - 100 && sc.em <= 1023 + 100 && top >= 1023 - 200 && top <= 1023 + 200;
+  ok = ok && sc.em >= 1023 - 100 && sc.em <= 1023 + 100 && top <= 1023 + 200;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    deep = deep || (plain && (sc.em - sc.ex[c] > 30 || (lm[c] && top - (lm[c] >> 20) > 30)));
     el[c] = lm[c] ? lm[c] >> 20 : (top ? top : 1023);  // no cotangent at all: any unit
     ok = ok && el[c] >= 1023 - 200 && el[c] >= top - 40;
   }
-  ew = QARR ? wx >> 20 : 1023;
-  if (QARR) ok = ok && ew >= 1023 - 400 && ew <= 1023 + 400 && ew - (wn >> 20) <= TRI_WSPREAD;
   return ok;
 }
 
-// A cotangent's component more than 2^16 below the largest of its kind may lose
-// bits below 2^-69 of that largest.  In an item where one does, a tile keeps to
-// its words if no pair's |dl| is below 2^-24 of the largest cotangent: the loss
-// is then at most 2^-45 of the pair's own term.
+// Largest 1/r of the FP32 path.
+constexpr float VJP_YMAX = 0x1p24f;
+// Cotangents spread more than positions do (a loss that reads a few ions), so their
+// rule allows a loss of 2^-44 of a pair's dl: the two sides of a tile may not hold
+// a cut component below 2^-26 and one below 2^-24 of the largest, and in an item
+// with a cut component (below 2^-17) no pair's |dl| may be below 2^-24 of it.  With
+// the positions' rule a field that decays over six decades took 3.4 ms at n =
+// 20000 instead of 1.7.
+constexpr int VJP_NEAR = 24;
 constexpr float VJP_EMIN_CUT = 0x1p-24f;
-// Without a set l word only FP32's range limits a tile's 1/r.
-constexpr float VJP_YMAX_GRID = 0x1p24f;
 
 // The words of ion g's cotangent (zeros past the end) on the components' own
-// grids, in the unit of the largest; returns whether one is not exact.
+// grids, in the unit of the largest; returns its place there (tri_place), and in
+// bit 6 whether a component is cut.
 __device__ __forceinline__ int vjp_lam(int64_t g, bool real, const double *lx, const double *ly, const double *lz,
                                        const int el[3], int top, float w0[3], float w1[3], float w2[3]) {
-  int cut = 0;
+  int place = 0;
   const double *l[3] = {lx, ly, lz};
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     float t[3] = {0.0f, 0.0f, 0.0f};
     if (real) {
-      tri_words(l[c][g], el[c], t);
-      cut |= !tri_exact(l[c][g], el[c]);
+      tri_words(l[c][g], el[c], __int_as_float((127 + el[c] - top) << 23), t);
+      place |= tri_place<VJP_NEAR>(l[c][g], el[c], c) | (tri_place<TRI_NEAR>(l[c][g], el[c], 0) & 1) << 6;
     }
-    const float f = __int_as_float((127 + el[c] - top) << 23);
-    w0[c] = t[0] * f;
-    w1[c] = t[1] * f;
-    w2[c] = t[2] * f;
+    w0[c] = t[0];
+    w1[c] = t[1];
+    w2[c] = t[2];
   }
-  return cut;
+  return place;
 }
 
 template <bool QARR, bool INPLACE, bool SOFT>
@@ -430,26 +449,31 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
   const int np = (int)min((int64_t)BI, n - p0), nq = (int)min((int64_t)BI, n - q0);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool diag = it.P == it.Q;
-  int em, el[3], ew;
-  const bool fast = vjp_scale<QARR>(p0, np, q0, diag ? 0 : nq, x, y, z, q, lx, ly, lz, soft2, em, el, ew);
+  __shared__ int qf[8];  // places of each Q-tile (G <= 8): positions, cotangents from bit 6, bit 12 cut
+  TriScale sc;
+  int el[3];
+  bool deep;
+  const bool fast = vjp_scale<QARR>(p0, np, q0, diag ? 0 : nq, x, y, z, q, lx, ly, lz, soft2, sc, el, deep);
   const int ee = max(el[0], max(el[1], el[2]));
   // units: lengths 2^kl, cotangents 2^ke, weights 2^kw; T in 2^(ke - 3 kl + kw)
-  const int kt = fast ? (ee - 1022) - 3 * (em - 1022) + (ew - 1023) : 0;
+  const int kt = fast ? (ee - 1022) - 3 * (sc.em - 1022) + (sc.ew - 1023) : 0;
   const int PT = G >> 1, NG = VJP_W / PT, nqt = G / NG;  // P-tiles of 64 ions, warps and Q-tiles per P-tile
   const int pt = warp % PT, grp = warp / PT;
   VjpIons p;
-  int low = 0;  // a position has bits in or below its l word
-  int cut = 0;  // a cotangent is not exact in its words
+  int pf = 0;   // places of the warp's P-tile
+  int cut = 0;  // a cotangent of the Q side is cut
   if (fast) {
     float w0[2][4], w1[2][4], w2[2][4];
     for (int i = tid; i < BI; i += VJP_THREADS) {
       const int64_t g = q0 + i;
       float4 *e = qs + (i >> 5) * VJP_TILE4 + (i & 31);
-      low |= tri_ion<QARR>(g, i < nq, x, y, z, q, em, ew, -TRI_FAR, w0[0], w1[0], w2[0]);
+      int f = tri_ion<QARR>(g, i < nq, x, y, z, q, sc, -TRI_FAR, w0[0], w1[0], w2[0]);
       e[0] = make_float4(w0[0][0], w0[0][1], w0[0][2], w0[0][3]);
       e[32] = make_float4(w1[0][0], w1[0][1], w1[0][2], w1[0][3]);
       e[64] = make_float4(w2[0][0], w2[0][1], w2[0][2], 0.0f);
-      cut |= vjp_lam(g, i < nq, lx, ly, lz, el, ee, w0[0], w1[0], w2[0]);
+      f = __reduce_or_sync(0xffffffffu, f | vjp_lam(g, i < nq, lx, ly, lz, el, ee, w0[0], w1[0], w2[0]) << 6);
+      cut |= f >> 12;
+      if (lane == 0) qf[i >> 5] = f;
       e[96] = make_float4(w0[0][0], w0[0][1], w0[0][2], 0.0f);
       e[128] = make_float4(w1[0][0], w1[0][1], w1[0][2], 0.0f);
       e[160] = make_float4(w2[0][0], w2[0][1], w2[0][2], 0.0f);
@@ -457,7 +481,7 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int i = pt * 64 + b * 32 + lane;
-      low |= tri_ion<QARR>(p0 + i, i < np, x, y, z, q, em, ew, TRI_FAR, w0[b], w1[b], w2[b]);
+      pf |= tri_ion<QARR>(p0 + i, i < np, x, y, z, q, sc, TRI_FAR, w0[b], w1[b], w2[b]);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -470,7 +494,7 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int i = pt * 64 + b * 32 + lane;
-      cut |= vjp_lam(p0 + i, i < np, lx, ly, lz, el, ee, w0[b], w1[b], w2[b]);
+      pf |= vjp_lam(p0 + i, i < np, lx, ly, lz, el, ee, w0[b], w1[b], w2[b]) << 6;
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -478,15 +502,15 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
       p.lam.m[0][c] = pk(w1[0][c], w1[1][c]);
       p.lam.l[0][c] = pk(w2[0][c], w2[1][c]);
     }
+    pf = __reduce_or_sync(0xffffffffu, pf);
   }
   for (int i = tid; i < 3 * BI; i += VJP_THREADS) accQ[i] = 0.0;
   for (int i = tid; i < VJP_W * 3 * 64; i += VJP_THREADS) accP[i] = 0.0;
-  const float ylim = __syncthreads_or(low) ? TRI_YMAX : VJP_YMAX_GRID;
-  const float elim = __syncthreads_or(cut) ? VJP_EMIN_CUT : 0.0f;
+  const float elim = __syncthreads_or(cut | pf >> 12) ? VJP_EMIN_CUT : 0.0f;
   f32x2 s2h = 0, s2l = 0;
   if (SOFT) {
     float sh, sl;
-    split_f64_scaled(soft2, 2 * (em - 1022), sh, sl);
+    split_f64_scaled(soft2, 2 * (sc.em - 1022), sh, sl);
     s2h = pk1(sh);
     s2l = pk1(sl);
   }
@@ -499,17 +523,17 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
     if (!live || t * 32 >= nq) continue;
     double *aQ = accQ + t * 32;
     bool done = false;
-    if (fast) {
+    if (fast && !tri_fault(pf, qf[t]) && !tri_fault(pf >> 6, qf[t] >> 6)) {
       TriSums<1> ts;
       const f32x2 zero = pk1(0.0f);
 #pragma unroll
       for (int c = 0; c < 3; ++c) ts.ah[0][c] = ts.al[0][c] = ts.bh[c] = ts.bl[c] = zero;
       const float4 *qt = qs + t * VJP_TILE4;
-      float emin;
       const int u = t - 2 * pt;  // the lane's own ion in this Q-tile, if any
+      float emin;
       const float ymax = diag ? vjp_tile<QARR, true, SOFT>(p, qt, lane, u == 0 || u == 1 ? u : -1, s2h, s2l, ts, emin)
                               : vjp_tile<QARR, false, SOFT>(p, qt, lane, -1, s2h, s2l, ts, emin);
-      done = !__any_sync(0xffffffffu, !(ymax <= ylim) || !(emin >= elim));
+      done = !__any_sync(0xffffffffu, !(ymax <= VJP_YMAX) || !(emin >= elim));
       if (done) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -526,8 +550,12 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
         }
       }
     }
-    if (!done)
-      vjp_tile_units<QARR>(n, x, y, z, q, lx, ly, lz, soft2, p0 + pt * 64, q0 + t * 32, diag, back, aP, 64, aQ, BI);
+    if (!done) {
+      if (deep)
+        vjp_tile_fp64<QARR>(n, x, y, z, q, lx, ly, lz, soft2, p0 + pt * 64, q0 + t * 32, diag, back, aP, 64, aQ, BI);
+      else
+        vjp_tile_units<QARR>(n, x, y, z, q, lx, ly, lz, soft2, p0 + pt * 64, q0 + t * 32, diag, back, aP, 64, aQ, BI);
+    }
   }
   __syncthreads();
   sym_output<VJP_THREADS>(INPLACE, it, n, p0, np, q0, nq, acc, sync, err,

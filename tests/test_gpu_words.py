@@ -56,3 +56,94 @@ def test_bits_below_the_words_of_a_grid(nb, n):
     f, _, ref = pair_sums(pos, idx)  # that pair's term is all but the whole sum: 1e21 against 1e5
     assert np.all(np.linalg.norm(g[:, idx] - f, axis=0) <= 1e-12 * np.linalg.norm(f, axis=0))
     assert np.all(np.abs(phi[idx] - ref) <= 1e-13 * ref)
+
+
+# ---------------------------------------------------------------------------
+# Flat and offset clouds: every component within 1e-12 (mixed: 1e-6) of the sum of
+# its own terms' magnitudes, |d_c| r^-3.  The pair term is right to 2^-43 of itself
+# in FP64 arithmetic and to 2^-46 on the FP32 pipe, the host's sum to 2^-49.
+
+
+def flat(n, form, amp, seed=0):
+    """A chain along z, 6e-4 long, with a transverse amplitude: `plane` in x alone,
+    `spread` over 20 decades (most coordinates cut), `offset` on x = 1e-4, `seed`
+    one displaced ion, its neighbours following with the cube of the distance."""
+    rng = np.random.default_rng([n, seed])
+    pos = np.zeros((3, n))
+    pos[2] = np.sort(rng.uniform(-3e-4, 3e-4, n))
+    if form == "plane":
+        pos[0] = amp * rng.standard_normal(n)
+    elif form == "spread":
+        pos[:2] = amp * 10.0 ** rng.uniform(-20, 0, (2, n)) * rng.choice([-1.0, 1.0], (2, n))
+    elif form == "offset":
+        pos[0] = 1e-4 + amp * rng.standard_normal(n)
+        pos[1] = amp * rng.standard_normal(n)
+    else:
+        pos[1] = amp / np.maximum(1.0, np.abs(np.arange(n) - n // 3)) ** 3
+    return pos
+
+
+def sample(n):
+    rng = np.random.default_rng(n)
+    return np.unique(np.concatenate([np.arange(min(n, 40)), np.arange(n - 8, n), rng.integers(0, n, 200)]))
+
+
+def check_components(acc, pos, tol):
+    idx = sample(pos.shape[1])
+    f, a, _ = pair_sums(pos, idx)
+    err = np.abs(acc[:, idx] - f)
+    assert np.all(err <= tol * a), float(np.max(err[a > 0] / a[a > 0]))
+
+
+FORMS = [("plane", 1e-8), ("plane", 1e-12), ("plane", 1e-15), ("plane", 1e-18), ("plane", 1e-21), ("plane", 1e-24),
+         ("spread", 1e-9), ("offset", 1e-11), ("offset", 1e-15), ("seed", 1e-9), ("seed", 1e-20)]
+
+
+@pytest.mark.parametrize("form,amp", FORMS)
+@pytest.mark.parametrize("precision,n", [("fp64", 600), ("df64", 1900), ("fp64", 1600), ("df64", 2900), ("fp64", 12500),
+                                         ("mixed", 2100), ("mixed", 13000)])
+def test_components_of_a_flat_cloud(nb, precision, n, form, amp):
+    pos = flat(n, form, amp)
+    s = nb.System(pos)
+    nb.forces(nb.Params.from_phys(W.phys(**UNIT), precision=precision), s)
+    nb.sync_status()
+    check_components(s.acc().cpu().numpy(), pos, 1e-6 if precision == "mixed" else 1e-12)
+
+
+@pytest.mark.parametrize("form,amp", FORMS)
+@pytest.mark.parametrize("precision", ["fp64", "df64"])
+def test_components_of_a_flat_ensemble(nb, precision, form, amp):
+    """One step from rest without a trap: the acceleration is the pair sum at the
+    start's positions."""
+    sizes = [40, 129, 600, 1100]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    parts = [flat(n, form, amp, seed=k) for k, n in enumerate(sizes)]
+    s = nb.System(np.concatenate(parts, axis=1), np.zeros((3, off[-1])))
+    nb.step_batched(nb.Params.from_phys(W.phys(**UNIT), precision=precision), s, off, 1)
+    nb.sync_status()
+    acc = s.acc().cpu().numpy()
+    for k, pos in enumerate(parts):
+        check_components(acc[:, off[k]:off[k + 1]], pos, 1e-12)
+
+
+@pytest.mark.parametrize("form,amp", FORMS)
+@pytest.mark.parametrize("lam_form,lam_amp", [("plane", 1e-15), ("spread", 1.0), ("offset", 1e-9)])
+@pytest.mark.parametrize("n", [2500, 16500])
+def test_components_of_a_flat_jacobian_product(nb, n, lam_form, lam_amp, form, amp):
+    """g_c = sum_j (dl_c - 3 r^-2 (d . dl) d_c) r^-3, against the magnitudes |dl_c| r^-3
+    and 3 |d| |dl| |d_c| r^-5."""
+    pos, lam = flat(n, form, amp), flat(n, lam_form, lam_amp, seed=9)
+    g = nb.forces_vjp(nb.Params.from_phys(W.phys(**UNIT)), nb.System(pos), lam).cpu().numpy()
+    nb.sync_status()
+    idx = sample(n)
+    for k in range(0, len(idx), 64):
+        i = idx[k:k + 64]
+        d = pos[:, i, None] - pos[:, None, :]
+        dl = lam[:, i, None] - lam[:, None, :]
+        r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2]
+        with np.errstate(divide="ignore"):
+            y = np.where(r2 > 0.0, 1.0 / np.sqrt(r2), 0.0)
+        y3 = y * y * y
+        t = y3 * (dl - 3.0 * (y * y) * (d * dl).sum(0) * d)
+        mag = y3 * (np.abs(dl) + 3.0 * y * np.sqrt((dl * dl).sum(0)) * np.abs(d))
+        assert np.all(np.abs(g[:, i] - t.sum(-1)) <= 1e-12 * mag.sum(-1))
