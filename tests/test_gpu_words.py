@@ -147,3 +147,62 @@ def test_components_of_a_flat_jacobian_product(nb, n, lam_form, lam_amp, form, a
         t = y3 * (dl - 3.0 * (y * y) * (d * dl).sum(0) * d)
         mag = y3 * (np.abs(dl) + 3.0 * y * np.sqrt((dl * dl).sum(0)) * np.abs(d))
         assert np.all(np.abs(g[:, i] - t.sum(-1)) <= 1e-12 * mag.sum(-1))
+
+
+# ---------------------------------------------------------------------------
+# The ensemble's tasks left to FP64 (btri_task_fp64): every kind of pair of ions a
+# task can hold, in instances of one, two and more super-tiles of 128 ions.
+
+
+def ensemble_once(nb, pos, off, q, soft2, threads, precision):
+    """One step from rest without a trap: the pair sums at pos."""
+    nb.set_tuning("ensemble", precision, 0, 1 << 40, threads, R=1)
+    try:
+        s = nb.System(pos, np.zeros_like(pos), q=q)
+        nb.step_batched(nb.Params.from_phys(W.phys(soft2=soft2, **UNIT), precision=precision), s, off, 1)
+        nb.sync_status()
+    finally:
+        nb.set_tuning("ensemble", precision, 0, 0, 0)
+    return s.acc().cpu().numpy()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "df64"])
+@pytest.mark.parametrize("soft", [0.0, 2e-6])
+@pytest.mark.parametrize("charges", [False, True])
+@pytest.mark.parametrize("kind", ["close", "coincident", "cut"])
+def test_ensemble_tasks_left_to_fp64(nb, kind, charges, soft, precision):
+    """Pairs at 2^-42 of the cloud or at no distance, and pairs with a coordinate of
+    2^-40 of it: in one 32-ion tile, in one super-tile, across two and three, and in
+    an instance of at most 64 ions.  Conditioned error of every ion 1e-12, and the
+    bits of 1, 3 and 16 warps."""
+    sizes = [20, 64, 128, 200, 300, 513]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    rng = np.random.default_rng(8)
+    pos = rng.uniform(-1e-4, 1e-4, (3, off[-1]))
+    pos[:, off[:-1] + 1] = 1e-4  # so that every task of super-tile 0 has L > 1e-4
+    for k, n in enumerate(sizes):
+        for a, b in ((2, 9), (3, 40), (5, 127), (7, 130), (33, 199), (150, 299), (140, 260), (400, 512), (4, 512)):
+            if b >= n:
+                continue
+            i, j = off[k] + a, off[k] + b
+            if kind == "cut":
+                pos[0, i], pos[0, j] = rng.uniform(1.0, 2.0, 2) * 1e-4 * 2.0 ** -40
+            else:
+                pos[:, j] = pos[:, i]
+                if kind == "close":
+                    pos[:, j] += 1e-4 * 2.0 ** -42 * np.array([1.0, -1.0, 0.5])
+    q = rng.choice([-1.0, 1.0, 2.0, 0.0], size=off[-1]) if charges else None
+    acc = ensemble_once(nb, pos, off, q, soft * soft, 512, precision)
+    for threads in (32, 96):
+        assert np.array_equal(acc, ensemble_once(nb, pos, off, q, soft * soft, threads, precision))
+    for k, n in enumerate(sizes):
+        p = pos[:, off[k]:off[k + 1]]
+        w = np.ones(n) if q is None else q[off[k]:off[k + 1]]
+        d = p[:, :, None] - p[:, None, :]
+        r2 = (d * d).sum(0) + soft * soft
+        same = np.all(d == 0.0, axis=0)  # coincident ions exert no force on each other
+        y = np.where(same, 0.0, 1.0 / np.sqrt(np.where(same, 1.0, r2)))
+        t = w * w[:, None] * y ** 3 * d if q is not None else y ** 3 * d
+        ref, cond = t.sum(-1), np.sqrt((t * t).sum(0)).sum(-1)
+        err = np.sqrt(((acc[:, off[k]:off[k + 1]] - ref) ** 2).sum(0))
+        assert np.all(err <= 1e-12 * cond), (n, float(np.max(err / np.maximum(cond, 1e-300))))
