@@ -1,11 +1,12 @@
-// nb_sym.cu -- symmetric (half-pair) force kernel: each unordered pair of ions
+// nb_sym.cu -- symmetric (half-pair) force kernels: each unordered pair of ions
 // is evaluated once and its force is applied to both ions with opposite
-// signs (Newton's third law), halving the pair arithmetic of the FP64-pipe
-// bound precisions (fp64, df64).
+// signs (Newton's third law), halving the pair arithmetic.
 //
-// The split and literal mixed precisions use it too (FP32 pair arithmetic
-// with per-step FP32 partials added into FP64, or into double-float sums on
-// the FP32 pipe for split).  In the split path's large blocks (G >= 16) a
+// They serve the split precisions and the softened literal mixed form (FP32 pair
+// arithmetic with per-step FP32 partials added into FP64, or into double-float
+// sums on the FP32 pipe for split), and in 32-ion blocks (k_pair_sym_rot) every
+// precision; fp64, df64 and the literal mixed form run on nb_tri.cu's kernel in
+// larger blocks.  In the split path's large blocks (G >= 16) a
 // lane holds four P-ions, whose arithmetic runs as two packed pairs of FP32
 // (.f32x2) instructions: sym_offdiag_split4.
 //
@@ -405,7 +406,7 @@ __device__ __forceinline__ void sym_offdiag_split4(const SD4 *posP, SD4 *posQ, f
 // once the warp is done with its Q-tile.
 template <int MODE, bool W, int NW>
 __device__ __forceinline__ void sym_offdiag(const SD4 *posP, SD4 *posQ, double *accP, int G, int BI,
-                                            double soft2, float s2h, float s2l) {
+                                            double soft2) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float *accPf = reinterpret_cast<float *>(accP);
   for (int qs = warp; qs < G; qs += NW) {
@@ -417,41 +418,23 @@ __device__ __forceinline__ void sym_offdiag(const SD4 *posP, SD4 *posQ, double *
       __syncthreads();  // all warps are at step k: their P-tiles are distinct
       const SD4 pp = posP[pt * 32 + lane];
       const int ip = pt * 32 + lane;
-      if (MODE == MODE_MIXED || split_like(MODE)) {
-        float a[3] = {0, 0, 0}, b[3] = {0, 0, 0};
-        if (MODE == MODE_MIXED) {
-          sym_step_mixed<W>(pp, qh, (float)soft2, lane, a, b);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            accP[c * BI + ip] += f32_to_f64(a[c]);
-            aq[c] += f32_to_f64(b[c]);
-          }
-        } else {
-          const float4 *fP = reinterpret_cast<const float4 *>(posP);
-          const float4 *fQ = reinterpret_cast<const float4 *>(posQ);
-          sym_step_split<W, MODE == MODE_SPLIT_RSQ>(fP[ip], fP[BI + ip], fQ + qs * 64 + lane,
-                                                    fQ + 2 * BI + qs * 64 + lane, (float)soft2, lane, a, b);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            df_add(accPf[c * BI + ip], accPf[(3 + c) * BI + ip], a[c]);
-            df_add(qfh[c], qfl[c], b[c]);
-          }
-        }
-      } else if (MODE == MODE_DF64) {
-        float ah[3] = {0, 0, 0}, al[3] = {0, 0, 0}, bh[3] = {0, 0, 0}, bl[3] = {0, 0, 0};
-        sym_step_df64<W>(pp, qh, s2h, s2l, lane, ah, al, bh, bl);
+      float a[3] = {0, 0, 0}, b[3] = {0, 0, 0};
+      if (MODE == MODE_MIXED) {
+        sym_step_mixed<W>(pp, qh, (float)soft2, lane, a, b);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          accP[c * BI + ip] += f32_to_f64(ah[c]) + f32_to_f64(al[c]);
-          aq[c] += f32_to_f64(bh[c]) + f32_to_f64(bl[c]);
+          accP[c * BI + ip] += f32_to_f64(a[c]);
+          aq[c] += f32_to_f64(b[c]);
         }
       } else {
-        double a[3] = {0.0, 0.0, 0.0}, b[3] = {0.0, 0.0, 0.0};
-        sym_step_fp64<W>(pp, qh, soft2, lane, a, b);
+        const float4 *fP = reinterpret_cast<const float4 *>(posP);
+        const float4 *fQ = reinterpret_cast<const float4 *>(posQ);
+        sym_step_split<W, MODE == MODE_SPLIT_RSQ>(fP[ip], fP[BI + ip], fQ + qs * 64 + lane, fQ + 2 * BI + qs * 64 + lane,
+                                                  (float)soft2, lane, a, b);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          accP[c * BI + ip] += a[c];
-          aq[c] += b[c];
+          df_add(accPf[c * BI + ip], accPf[(3 + c) * BI + ip], a[c]);
+          df_add(qfh[c], qfl[c], b[c]);
         }
       }
     }
@@ -501,19 +484,20 @@ __device__ __forceinline__ void sym_stage(SD4 *dst, int i, int BI, int64_t g, in
   dst[i] = e;
 }
 
-// Register budgets: fp64 two 256-thread blocks per SM; the split path's
+// Register budgets: the split path's
 // packed four-ion step with 256 threads three blocks per SM, the number its
 // 72 KB of shared memory allows (80 registers, a few bytes of spills outside
 // the pair loop: 2.6 % faster at n = 1e5 than two blocks of 102 registers,
 // 0.5-1 % slower at n = 16384-40000).
 template <int MODE, bool QARR, bool P2, int NT, bool INPLACE>
-__global__ void __launch_bounds__(NT, MODE == MODE_FP64 ? 512 / NT : (P2 && NT == 256) ? 3 : 0) k_pair_sym(int64_t n, int nbk, int G,
+__global__ void __launch_bounds__(NT, (P2 && NT == 256) ? 3 : 0) k_pair_sym(int64_t n, int nbk, int G,
                                                          const double *__restrict__ x,
                                                          const double *__restrict__ y,
                                                          const double *__restrict__ z,
                                                          const double *__restrict__ q, PosF32 pf,
                                                          double soft2, double *__restrict__ acc,
                                                          int *__restrict__ sync, unsigned *err) {
+  static_assert(MODE == MODE_MIXED || split_like(MODE), "fp64 and df64: nb_tri.cu");
   constexpr bool inplace = INPLACE;  // the output mode, fixed at compile time
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int BI = 32 * G;
@@ -540,94 +524,44 @@ __global__ void __launch_bounds__(NT, MODE == MODE_FP64 ? 512 / NT : (P2 && NT =
       accP[5 * BI + i] = 0.0;
     }
   }
-  float s2h = 0.0f, s2l = 0.0f;
-  if (MODE == MODE_DF64) split_f64(soft2, s2h, s2l);
   __syncthreads();
 
   if (P == Q) {  // the block's own pairs, one-sided; sums into qsum (posQ is not staged)
     for (int i = tid; i < np; i += NT) {
       const SD4 pi = posP[i];
       double a[3] = {0.0, 0.0, 0.0};
-      if (MODE == MODE_MIXED || split_like(MODE)) {
-        float af[3] = {0, 0, 0};
-        const float4 *f = reinterpret_cast<const float4 *>(posP);
-        for (int j = 0; j < np; ++j) {
-          float fx, fy, fz, wj;
-          if (MODE == MODE_MIXED) {
-            const SD4 pj = posP[j];
-            fx = f64_to_f32_rn(pi.x - pj.x);
-            fy = f64_to_f32_rn(pi.y - pj.y);
-            fz = f64_to_f32_rn(pi.z - pj.z);
-            wj = wf32(pj.w);
-          } else {
-            const float4 ih = f[i], il = f[BI + i], jh = f[j], jl = f[BI + j];
-            fx = (ih.x - jh.x) + (il.x - jl.x);
-            fy = (ih.y - jh.y) + (il.y - jl.y);
-            fz = (ih.z - jh.z) + (il.z - jl.z);
-            wj = jh.w;
-          }
-          float sj = f32_rinv3<MODE == MODE_SPLIT_RSQ>(fx, fy, fz, (float)soft2);
-          if (QARR) sj *= wj;
-          af[0] = fmaf(fx, sj, af[0]);
-          af[1] = fmaf(fy, sj, af[1]);
-          af[2] = fmaf(fz, sj, af[2]);
-          if ((j & 31) == 31) {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-              a[k] += f32_to_f64(af[k]);
-              af[k] = 0.0f;
-            }
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) a[k] += f32_to_f64(af[k]);
-      } else if (MODE == MODE_DF64) {
-        float ah[3] = {0, 0, 0}, al[3] = {0, 0, 0};
-        for (int j = 0; j < np; ++j) {
+      float af[3] = {0, 0, 0};
+      const float4 *f = reinterpret_cast<const float4 *>(posP);
+      for (int j = 0; j < np; ++j) {
+        float fx, fy, fz, wj;
+        if (MODE == MODE_MIXED) {
           const SD4 pj = posP[j];
-          float dh[3], dl[3];
-          split_f64(pi.x - pj.x, dh[0], dl[0]);
-          split_f64(pi.y - pj.y, dh[1], dl[1]);
-          split_f64(pi.z - pj.z, dh[2], dl[2]);
-          float sh, sl;
-          df_rinv3(dh, dl, s2h, s2l, sh, sl);
-          if (QARR) {
-            float wh, wl;
-            split_f64(pj.w, wh, wl);
-            const float ph = sh * wh;
-            sl = fmaf(sh, wl, fmaf(sl, wh, fmaf(sh, wh, -ph)));
-            sh = ph;
-          }
+          fx = f64_to_f32_rn(pi.x - pj.x);
+          fy = f64_to_f32_rn(pi.y - pj.y);
+          fz = f64_to_f32_rn(pi.z - pj.z);
+          wj = wf32(pj.w);
+        } else {
+          const float4 ih = f[i], il = f[BI + i], jh = f[j], jl = f[BI + j];
+          fx = (ih.x - jh.x) + (il.x - jl.x);
+          fy = (ih.y - jh.y) + (il.y - jl.y);
+          fz = (ih.z - jh.z) + (il.z - jl.z);
+          wj = jh.w;
+        }
+        float sj = f32_rinv3<MODE == MODE_SPLIT_RSQ>(fx, fy, fz, (float)soft2);
+        if (QARR) sj *= wj;
+        af[0] = fmaf(fx, sj, af[0]);
+        af[1] = fmaf(fy, sj, af[1]);
+        af[2] = fmaf(fz, sj, af[2]);
+        if ((j & 31) == 31) {
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
-            const float ph = dh[k] * sh;
-            const float pl = fmaf(dh[k], sl, fmaf(dl[k], sh, fmaf(dh[k], sh, -ph)));
-            float s, tt;
-            two_sum_f(ah[k], ph, s, tt);
-            ah[k] = s;
-            al[k] += tt + pl;
+            a[k] += f32_to_f64(af[k]);
+            af[k] = 0.0f;
           }
-          if ((j & 255) == 255) {  // flush the double-float sum every 256 pairs
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-              a[k] += f32_to_f64(ah[k]) + f32_to_f64(al[k]);
-              ah[k] = al[k] = 0.0f;
-            }
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) a[k] += f32_to_f64(ah[k]) + f32_to_f64(al[k]);
-      } else {
-        for (int j = 0; j < np; ++j) {
-          const SD4 pj = posP[j];
-          const double dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
-          double s = rinv3_fp64(dx, dy, dz, soft2);
-          if (QARR) s *= pj.w;
-          a[0] = fma(dx, s, a[0]);
-          a[1] = fma(dy, s, a[1]);
-          a[2] = fma(dz, s, a[2]);
         }
       }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) a[k] += f32_to_f64(af[k]);
 #pragma unroll
       for (int c = 0; c < 3; ++c) qsum(posQ, c, i) = a[c];
     }
@@ -645,9 +579,9 @@ __global__ void __launch_bounds__(NT, MODE == MODE_FP64 ? 512 / NT : (P2 && NT =
     else
       sym_offdiag_split4<false, NT / 32, MODE == MODE_SPLIT_RSQ>(posP, posQ, accPf, G, BI, soft2);
   } else if (weighted) {
-    sym_offdiag<MODE, true, NT / 32>(posP, posQ, accP, G, BI, soft2, s2h, s2l);
+    sym_offdiag<MODE, true, NT / 32>(posP, posQ, accP, G, BI, soft2);
   } else {
-    sym_offdiag<MODE, false, NT / 32>(posP, posQ, accP, G, BI, soft2, s2h, s2l);
+    sym_offdiag<MODE, false, NT / 32>(posP, posQ, accP, G, BI, soft2);
   }
   __syncthreads();
   if (P2)  // two copies of the P sums, added in copy order
@@ -947,36 +881,19 @@ cudaError_t launch_pair_sym(int mode, int64_t n, int nbk, int G, const double *x
       default: return cudaErrorInvalidValue;
     }
   }
-  if (G <= 2) {  // 64-ion blocks at small n: one warp per 32-ion tile
+  if (G == 2) {  // 64-ion blocks at small n: one warp per 32-ion tile
     switch (mode) {
-      case MODE_FP64:
-        return G == 1 ? launch_sym_m<MODE_FP64, false, 32>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st)
-                      : launch_sym_m<MODE_FP64, false, 64>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
-      case MODE_DF64:
-        return G == 1 ? launch_sym_m<MODE_DF64, false, 32>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st)
-                      : launch_sym_m<MODE_DF64, false, 64>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
       case MODE_MIXED:
-        return G == 1 ? launch_sym_m<MODE_MIXED, false, 32>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st)
-                      : launch_sym_m<MODE_MIXED, false, 64>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
+        return launch_sym_m<MODE_MIXED, false, 64>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
       case MODE_SPLIT:
-        return G == 1 ? launch_sym_m<MODE_SPLIT, false, 32>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st)
-                      : launch_sym_m<MODE_SPLIT, false, 64>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
+        return launch_sym_m<MODE_SPLIT, false, 64>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
       case MODE_SPLIT_RSQ:
-        return G == 1 ? launch_sym_m<MODE_SPLIT_RSQ, false, 32>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err,
-                                                                inplace, st)
-                      : launch_sym_m<MODE_SPLIT_RSQ, false, 64>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err,
-                                                                inplace, st);
-      default: return cudaErrorInvalidValue;
+        return launch_sym_m<MODE_SPLIT_RSQ, false, 64>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
+      default: return cudaErrorInvalidValue;  // fp64 and df64: nb_tri.cu
     }
   }
   const bool small = G == 4;  // 4 warps for 128-ion blocks
   switch (mode) {
-    case MODE_FP64:
-      return small ? launch_sym_m<MODE_FP64, false, S>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st)
-                   : launch_sym_m<MODE_FP64, false, L>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
-    case MODE_DF64:
-      return small ? launch_sym_m<MODE_DF64, false, S>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st)
-                   : launch_sym_m<MODE_DF64, false, L>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
     case MODE_MIXED:
       return small ? launch_sym_m<MODE_MIXED, false, S>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st)
                    : launch_sym_m<MODE_MIXED, false, L>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
@@ -992,7 +909,7 @@ cudaError_t launch_pair_sym(int mode, int64_t n, int nbk, int G, const double *x
         return launch_sym_m<MODE_SPLIT_RSQ, true, 512>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
       return G >= 16 ? launch_sym_m<MODE_SPLIT_RSQ, true, L>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st)
                      : launch_sym_m<MODE_SPLIT_RSQ, false, L>(n, nbk, G, x, y, z, q, pf, soft2, part, sync, err, inplace, st);
-    default: return cudaErrorInvalidValue;
+    default: return cudaErrorInvalidValue;  // fp64 and df64: nb_tri.cu
   }
 }
 

@@ -154,8 +154,7 @@ __device__ __forceinline__ void kick_noise(const Phys &p, int64_t i, int64_t sne
 //   v+ = (v + (a + a+_cons) dt/2) * [1 / (1 + gamma dt/(2 m_i))]  [+ Langevin kick]
 //   a+ = a+_cons - (gamma/m_i) v+
 // v and a hold the ion's velocity and acceleration on entry and the new ones
-// on return.  Returns true if any of them is not finite.  verlet_kick1 is one
-// component of it.
+// on return, of one component.  Returns true if either is not finite.
 __device__ __forceinline__ bool verlet_kick1(double dt, const KickConst &kc, double tf, double xi, double r, double cs,
                                              double &v, double &a) {
   const double tr = __dmul_rn(__dmul_rn(tf, r), kc.ts);
@@ -167,12 +166,4 @@ __device__ __forceinline__ bool verlet_kick1(double dt, const KickConst &kc, dou
   a = an;
   return not_finite(vn) || not_finite(an);
 }
-__device__ __forceinline__ bool verlet_kick(double dt, const KickConst &kc, const TrapFactors &tf, const double xi[3],
-                                            const double r[3], const double cs[3], double v[3], double a[3]) {
-  bool bad = false;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) bad |= verlet_kick1(dt, kc, tf.f[k], xi[k], r[k], cs[k], v[k], a[k]);
-  return bad;
-}
-
 }  // namespace nb

@@ -84,14 +84,12 @@ __device__ __forceinline__ void vjp_eval(const VD8 &p, const VD8 &q, double soft
   }
 }
 
-// Staged entry i of a tile or block (g = global index).  Ions past n are
-// weight-0, lam-0 dummies far away.  dup: the half-pair kernel's Q-side
-// layout, each 32-ion tile stored twice back to back.
+// Staged entry i of a tile (g = global index).  Ions past n are weight-0, lam-0
+// dummies far away.
 template <bool QARR>
 __device__ __forceinline__ void vjp_stage(VD8 *dst, int i, int64_t g, int64_t n, const double *x,
                                           const double *y, const double *z, const double *q,
-                                          const double *lx, const double *ly, const double *lz,
-                                          bool dup) {
+                                          const double *lx, const double *ly, const double *lz) {
   VD8 e;
   float wh = 0.0f, wl = 0.0f;
   if (g < n) {
@@ -111,13 +109,7 @@ __device__ __forceinline__ void vjp_stage(VD8 *dst, int i, int64_t g, int64_t n,
   }
   *reinterpret_cast<float2 *>(&e.w) = make_float2(wh, wl);
   e.pad = 0;
-  if (dup) {
-    const int k = (i >> 5) * 64 + (i & 31);
-    dst[k] = e;
-    dst[k + 32] = e;
-  } else {
-    dst[i] = e;
-  }
+  dst[i] = e;
 }
 
 // ---------------------------------------------------------------------------
@@ -150,7 +142,7 @@ __global__ void __launch_bounds__(256) k_pair_vjp(int64_t n, int64_t jchunk, con
   double g[3] = {0.0, 0.0, 0.0};
   for (int64_t j0 = jb; j0 < je; j0 += B) {
     __syncthreads();
-    if (j0 + tid < je) vjp_stage<QARR>(sj, tid, j0 + tid, n, x, y, z, q, lx, ly, lz, false);
+    if (j0 + tid < je) vjp_stage<QARR>(sj, tid, j0 + tid, n, x, y, z, q, lx, ly, lz);
     __syncthreads();
     const int cnt = (int)min((int64_t)B, je - j0);
     for (int k0 = 0; k0 < cnt; k0 += 32) {
@@ -299,14 +291,14 @@ __device__ __noinline__ void vjp_tile_units(int64_t n, const double *x, const do
   const int lane = threadIdx.x & 31;
   for (int u = 0; u < 64; u += 32) {
     VD8 pp;
-    vjp_stage<QARR>(&pp, 0, i0 + u + lane, n, x, y, z, q, lx, ly, lz, false);
+    vjp_stage<QARR>(&pp, 0, i0 + u + lane, n, x, y, z, q, lx, ly, lz);
     float ah[3] = {0.0f, 0.0f, 0.0f}, al[3] = {0.0f, 0.0f, 0.0f};
     float bh[3] = {0.0f, 0.0f, 0.0f}, bl[3] = {0.0f, 0.0f, 0.0f};
     int ea = VJP_BF_EMPTY, eb = VJP_BF_EMPTY;
     for (int r = 0; r < 32; ++r) {
       const int64_t j = j0 + ((lane + r) & 31);
       VD8 pq;
-      vjp_stage<QARR>(&pq, 0, j, n, x, y, z, q, lx, ly, lz, false);
+      vjp_stage<QARR>(&pq, 0, j, n, x, y, z, q, lx, ly, lz);
       if (i0 + u + lane < n && j < n) vjp_eval<QARR, true>(pp, pq, soft2, ah, al, ea, bh, bl, eb);
       for (int c = 0; c < 3; ++c) {
         bh[c] = __shfl_sync(0xffffffffu, bh[c], (lane + 1) & 31);
