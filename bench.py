@@ -359,8 +359,10 @@ def recorded_counters(precision, n, kernel=None):
     records one capture of this bench's command: B the DRAM bytes (read +
     write), I the warp instructions executed (smsp__inst_executed.sum), S
     the kernel sources' hash when it was taken; a field kernel=K names
-    pair_kernel's kernels.  ({}, None) when there is no capture for this case or
-    the kernel has changed since."""
+    pair_kernel's kernels.  source=retired: the last capture of a kernel that no
+    longer runs, for times taken of it (main_ours asks for pair_kernel's).
+    ({}, None) when there is no capture for this case or the kernel has changed
+    since."""
     import glob
     want = kernel_source_sha(kernel)
     out, src = {}, None
@@ -370,7 +372,7 @@ def recorded_counters(precision, n, kernel=None):
             if not line.startswith("traffic: "):
                 continue
             kv = dict(t.split("=", 1) for t in line.split()[1:])
-            if (kv.get("precision") == precision and int(kv.get("n", -1)) == n and kv.get("source") == want
+            if (kv.get("precision") == precision and int(kv.get("n", -1)) == n and kv.get("source") in (want, "retired")
                     and kv.get("kernel") == kernel):
                 for k in ("bytes", "inst", "fp64_inst"):  # the first summary naming a counter wins
                     if k in kv and k not in out:
@@ -389,7 +391,7 @@ def recorded_opmix(precision, kernel=None):
     of the summaries under profiles/ (SASS op counters of one ncu capture,
     which take three passes, so they come from a case smaller than the
     bench's with the same kernel configuration); {} when unrecorded or the
-    kernel sources have changed since."""
+    kernel sources have changed since (source=retired as in recorded_counters)."""
     import glob
     want = kernel_source_sha(kernel)
     for path in sorted(glob.glob(os.path.join(PROFILES, "*.md"))):
@@ -398,7 +400,7 @@ def recorded_opmix(precision, kernel=None):
             if not line.startswith("opmix: "):
                 continue
             kv = dict(t.split("=", 1) for t in line.split()[1:])
-            if kv.get("precision") == precision and kv.get("source") == want and kv.get("kernel") == kernel:
+            if kv.get("precision") == precision and kv.get("source") in (want, "retired") and kv.get("kernel") == kernel:
                 return {k: float(kv[k]) for k in OPMIX_KINDS if k in kv}
     return {}
 

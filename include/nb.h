@@ -57,13 +57,18 @@ typedef enum {
  *  NB_FP64       -- FP64-class forces in two forms, chosen by the size.
  *                   Half-pair plans, one-sided plans of 513 to 4096 ions and
  *                   ensembles of at most 4096-ion instances: each coordinate
- *                   is cut, in units of a power of two above those it is
- *                   paired with, into three FP32 words (68 bits); the
- *                   displacement is the words' exact difference as an FP32
- *                   (hi, lo) pair, and r^2, r^-3, the products and the sums
- *                   over up to 32 partners are double-floats, added in FP64.
- *                   Pairs closer than 2^-20 of that unit, and units or
- *                   weights far from the ordinary, take the second form:
+ *                   is cut, in units of a power of two above those of its axis
+ *                   that it is paired with, into three FP32 words (68 bits);
+ *                   the displacement is the words' exact difference as a
+ *                   normalised FP32 (hi, lo) pair, right to 2^-48 of each
+ *                   component, and r^2, r^-3, the products and the sums over up
+ *                   to 32 partners (256 one-sided) are double-floats, added in
+ *                   FP64.  Charges keep 48 bits.
+ *                   Groups of pairs whose words would cut a coordinate that is
+ *                   small beside its axis (below 2^-17 on one side, the other
+ *                   side below 2^-15), pairs closer than 2^-40 of the unit, and
+ *                   units or weights far from the ordinary (an axis below 2^-64
+ *                   of the longest, weights 2^40 apart) take the second form:
  *                   FP64 displacement and FP64 accumulation, with r^2,
  *                   1/sqrt(r^2) and r^-3 on the FP32 pipe: the displacement
  *                   is split into exponent-scaled FP32 (hi, lo) pairs, r^2 is
@@ -79,10 +84,14 @@ typedef enum {
  *                   (measured 2.9e-14 at N = 1e5).  NB_FP64_RSQ_NR2 is the
  *                   plain FP64 Newton form.
  *  NB_MIXED      -- pair displacements to FP64 accuracy (an FP64 subtraction,
- *                   or in half-pair plans from 2000 ions the exact difference
- *                   of three-word positions), cast to FP32; r^2, rsqrt,
- *                   r^-3 and the products in FP32; per-tile FP32 partial
- *                   sums added into FP64 accumulators with compensation.
+ *                   or in half-pair plans from 2000 ions without softening the
+ *                   exact difference of three-word positions), cast to FP32;
+ *                   r^2, rsqrt, r^-3 and the products in FP32; per-tile FP32
+ *                   partial sums added into FP64 accumulators with compensation.
+ *                   On three-word positions, groups of pairs that hold one closer
+ *                   than 2^-40 of the unit, where the FP64 differences' FP32 seed
+ *                   is clamped, and what NB_FP64 leaves to its second form
+ *                   (coordinates from 2^-38 down), are done in FP64.
  *  NB_MIXED_SPLIT -- as NB_MIXED, but each position is carried as an FP32
  *                   (hi, lo) pair built from the FP64 value once per call,
  *                   and the displacement is (hi_i - hi_j) + (lo_i - lo_j)
@@ -272,14 +281,21 @@ nb_status nb_energy(const nb_params *params, const nb_system *sys,
  *   d = r_i - r_j, dl = lam_i - lam_j, s^2 = |d|^2 + soft2,
  * plus, with NB_ACC_TOTAL, the trap's diagonal term at the current time.
  * The Jacobian is symmetric, so this is also the Jacobian-vector product.
- * lam* and g* are device SoA arrays of n doubles.  FP64 differences d and
- * dl.  Each pair's term (with its r^-3, r^-5 and d . dl) is formed in
- * double-float on the FP32 pipe, in units of the pair's own exponents
- * (relative error about 2^-44 of the term), and an ion's terms are summed in
- * double-float with one exponent per sum, the largest unit met so far, and
- * widened into an FP64 sum every 32 partners.  Weights q_j keep 48 bits;
- * a subnormal weight counts as 0.  One arithmetic for every
- * params->precision (NB_FP64 and NB_DF64 give the same bits).             */
+ * lam* and g* are device SoA arrays of n doubles.  From n = 2500 positions and
+ * cotangents are cut into three FP32 words per component, as NB_FP64's first
+ * form does with positions (there also for what is left to other forms); d and
+ * dl are the words' differences, each pair's term (with its r^-3, r^-2 and d . dl)
+ * and the sums over 32 partners are double-floats, added in FP64.  A cotangent's
+ * component below 2^-24 of the largest it is paired with may lose bits below 2^-44
+ * of the pair's dl.  Below n = 2500, and where the words do not serve: FP64
+ * differences d and dl, each pair's term in double-float in units of its own
+ * exponents, an ion's terms summed in double-float with one exponent per sum,
+ * the largest unit met so far, and widened into an FP64 sum every 32 partners.
+ * Relative error about 2^-44 of the term in either; components far below the
+ * others' scale (2^-64 of positions, 2^-40 of cotangents) take FP64 arithmetic
+ * from n = 2500.  Weights q_j keep 48 bits; a subnormal weight counts as 0.  One
+ * arithmetic for every params->precision (NB_FP64 and NB_DF64 give the same
+ * bits).                                                                   */
 nb_status nb_forces_vjp(const nb_params *params, const nb_system *sys,
                         const double *lx, const double *ly, const double *lz,
                         double *gx, double *gy, double *gz, int flags,
@@ -437,9 +453,10 @@ nb_status nb_traj_backward(const nb_params *params, const nb_system *sys, int64_
  * stream).  Its scratch is one fixed 8 MiB device array inside the library,
  * held on every GPU that loads the library until the process exits; n above
  * what it can hold is rejected with NB_EINVAL and a message in
- * nb_last_error().  With the default plan on a 152-SM GB300 the limit is
- * about n = 1,000,000; a potential-kernel tuning override (nb_set_tuning
- * kind 1) or a GPU with more SMs can lower it.
+ * nb_last_error().  With the default plan the limit is about n = 1,040,000;
+ * a potential-kernel tuning override (nb_set_tuning kind 1) can lower it.
+ * Bounded waits as in nb_energy, with an error word of its own: NB_ETIMEOUT if
+ * one gave up in this call.
  * All calls share that array: calls that may overlap on the GPU (other
  * streams, unordered host threads) race and must be serialised.  The first
  * call on each device looks up the array's device address with that device

@@ -317,14 +317,18 @@ __device__ __noinline__ void bsym_forces(const BIons v, double *acc, int npad, d
 // ones, which warps take in order, so the lowest unfinished never waits; the
 // wait is bounded all the same (ERR_TIMEOUT).
 //
-// What bounds it: the FMA pipe, as in nb_tri.cu, with 16 warps per SM (the
-// registers' limit); the words are cut from the FP64 positions at every task
-// (450 instructions against 10 400 of pair arithmetic), diagonal super-tiles are
+// What bounds it: the FMA pipe, as in nb_tri.cu, 79 % busy with 152 instances of
+// 4096 (issue 55 %, FP64 pipe 23 %) and 16 warps per SM (the registers' limit);
+// units and words are formed from the FP64 positions at every task
+// (600 instructions against 11 000 of pair arithmetic), diagonal super-tiles are
 // one-sided, and below about 500 ions there are fewer tasks than warps.  Two
-// steps of 512 instances of 32 .. 4096 ions: 14.2 ms (421 G pairs/s) against
-// 59.9 (fp64) and 25.8 ms (df64) with bsym_forces; 152 instances of 4096: 10.7
+// steps of 512 instances of 32 .. 4096 ions: 15.5 ms (385 G pairs/s) against
+// 59.9 (fp64) and 25.8 ms (df64) with bsym_forces; 152 instances of 4096: 11.2
 // against 45.9 and 18.7 ms.  With the tasks' adds between barriers instead of
-// counters the FP64 adds of all 16 warps coincided: 18.8 ms.
+// counters the FP64 adds of all 16 warps coincided, a third slower.  With one
+// unit per instance an ion far out, or a few kicked ones, sent every task to FP64
+// (37.8 ms instead of 2.7 for 152 instances of 64 .. 2048 with one ion at 5 m; 3.7
+// now).
 constexpr int BTRI_PI = 128;
 
 // Bounded wait of a warp for counter c to reach v (about a second).
@@ -522,8 +526,8 @@ __device__ __forceinline__ void btri_forces(const BIons &v, double *acc, int npa
     auto before = [&](int X) { return rd - (odd && X < rd - 1 ? 1 : 0); };
     const BTurn turn{cnt + A, cnt + B, 4 * before(A) + k, 4 * before(B)};
     // a super-tile of at most 64 ions (the last one, or a small instance) has
-    // one pair of P-ions per lane: 8.9 to 6.1 ms for 50 steps of 1024 instances
-    // of 16 .. 64 ions
+    // one pair of P-ions per lane: a third less time for 1024 instances of 16 ..
+    // 64 ions
     bool ok;
     if (q0 >= n)
       ok = turn.wait(one);

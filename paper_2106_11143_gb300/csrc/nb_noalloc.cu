@@ -27,7 +27,7 @@
 namespace nb {
 
 // Scratch capacity: 8 MiB of doubles.  It bounds n through the launch plan of
-// the potential kernel: its output (n_slots * n doubles and, from n = 1500, the
+// the potential kernel: its output (n_slots * n doubles and, from n = 2000, the
 // half-pair schedule's counters) + 3 * ENERGY_BLOCKS + 5 doubles must fit.
 // With the default plan that holds for every n up to about 1,040,000
 // (make_phi_plan keeps its partials below 1,000,000 doubles and needs n above);

@@ -5,8 +5,9 @@
 // Why: the one-sided kernel of nb_pair.cu takes seven FP64 instructions per
 // evaluation (three subtractions, three FMAs, the widened r^-3), 16 cycles of
 // the FP64 pipe each for a warp, and is bound by them: 17.2 us of a 23 us
-// step at n = 1024.  Here an evaluation is about 94 lane-cycles of the FMA pipe
-// and none of the FP64 pipe.  100 steps at n = 1024: 2.31 -> 1.37 ms; with df64,
+// step at n = 1024.  Here an evaluation is about 103 lane-cycles of the FMA pipe
+// and none of the FP64 pipe; the pipe is 43 % busy at n = 1024, where two blocks
+// per SM leave latency bare.  100 steps at n = 1024: 2.31 -> 1.08 ms; with df64,
 // whose pair term took 3 FP64 subtractions, and at 1499 and 1999 ions the same
 // kernel; rms error 2^-49.2 of the sum of the magnitudes (the FP64 form 2^-48.9).
 //
@@ -299,10 +300,9 @@ __global__ void __launch_bounds__(ONE_NT, 4)
 // The kernel serves the one-sided FP64-class sums above the single-block steps'
 // limit, whose bits up to there are those of nb_pair.cu's kernel, to 4096 ions
 // (whole calls are half-pair from 1500 or 2000), unless a tuned launch shape asks
-// for that kernel.  us per
-// nb_forces call with its host part, FP64 kernel and this one: n = 513 30.2 and
-// 28.4, 1024 31.4 and 27.9, 1499 48.3 and 30.2 (df64 31.6 and 29.1), 1999 df64
-// 40.7 and 32.0.
+// for that kernel.  us a
+// step with the FP64 kernel and this one: 15.6 and 9.9 at n = 600 (df64 13.1),
+// 23.8 and 11.2 at 1024 (df64 16.6), 42.9 and 15.6 at 1499 (df64 25.9).
 bool one_serves(const Plan &pl, int mode, int64_t n) {
   int tb = 0, tr = 0, tbps = 0;
   return !pl.sym && (mode == MODE_FP64 || mode == MODE_DF64) && n > SMALL_MAX_N && n <= ONE_MAX_N &&

@@ -5,8 +5,9 @@
 // Both ions of a pair share 1/r, so each pair is evaluated once; the one-sided
 // kernel (nb_pair.cu: k_pair_phi, five FP64 instructions per ordered pair) does
 // it twice.  What bounds it: the FMA pipe, 68 lane-cycles per evaluation (21 for
-// d, 18 for r^2, 10 for 1/r, 16 for the two sums, 3 to keep them normalised).  An
-// nb_energy call at n = 65537 takes 4.77 ms against 41.6, at 4097 92 us against
+// d, 18 for r^2, 10 for 1/r, 16 for the two sums, 3 to keep them normalised; d is left unnormalised, since 1/r needs
+// no component), 77 % busy at n = 32768 with issue at 54 %.  An
+// nb_energy call at n = 65537 takes 4.81 ms against 41.6, at 4097 92 us against
 // 261; relative error of phi rms 5.3e-16 against 1.5e-15 at 65537.  Padding ions'
 // terms are 2^-60 of a real one's, below the rounding of any sum.
 //
@@ -283,12 +284,12 @@ static cudaError_t launch_phi_t(int64_t n, int nbk, int G, const double *x, cons
 // in-place output.
 constexpr int64_t PHI_SLOT_DOUBLES = 1000000;
 // From n = 2000, where its error is no larger than that of FP64 sums (rms 5.1e-16
-// against 5.5e-16 of phi; an nb_energy call takes 70 us against 104).
+// against 5.5e-16 of phi; an nb_energy call takes 75 us against 104).
 constexpr int64_t PHI_FROM = 2000;
 
 // Block sizes by measurement (us per nb_energy call): 128 ions below 10000 (92
 // against 117 with 256 at n = 4097, 153 against 164 at 8192), 256 above (252
-// against 275 at 12000, 4788 against 4994 with 512 at 65537).
+// against 275 with 128 at 12000, 4788 against 4994 with 512 at 65537).
 PhiPlan make_phi_plan(int64_t n) {
   PhiPlan pl;
   pl.one = make_plan(n, MODE_FP64, 1);

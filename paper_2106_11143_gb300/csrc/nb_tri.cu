@@ -17,15 +17,18 @@
 //
 // Diagonal items (P == Q) run the same tiles one-sided (ONE).
 //
-// What bounds it: the FMA pipe, 126 lane-cycles per evaluation (21 for d, 18
-// for r^2, 18 for r^-3, 12 for the products, 48 for the two ions' TwoSum sums,
-// 9 to keep them normalised), 76 % busy at n = 32768 with issue at 48 %, ALU
-// 9 % and the FP64 pipe 23 % (the tiles' sums into FP64); most stalls wait for
-// the FMA pipe.  The half-pair kernel on the FP64 pipe (nb_sym.cu: 10.3 FP64
-// instructions per evaluation in fp64, 3.4 in df64) took 91.0 ms (fp64) and
-// 34.0 ms (df64) at n = 1e5; this one takes 19.2 ms for both.  Conditioned
-// error over all ions at n = 1e5: rms 2^-50.4, largest 2^-45.2, against
-// 2^-50.1 and 2^-44.9 (fp64) and 2^-49.2 and 2^-43.9 (df64) there.
+// What bounds it: the FMA pipe, 135 lane-cycles per evaluation (30 for the
+// normalised d, 18 for r^2, 18 for r^-3, 12 for the products, 48 for the two ions'
+// TwoSum sums, 9 to keep them normalised), 81 % busy at n = 32768 with issue at
+// 51 %, ALU 10 % and the FP64 pipe 24 % (the tiles' sums into FP64).  A half-pair
+// kernel on the FP64 pipe (10.3 FP64 instructions per evaluation in fp64, 3.4 in
+// df64) took 91.0 ms (fp64) and 34.0 ms (df64) at n = 1e5; this one takes 20.7 ms
+// for both (19.2 with d unnormalised, whose small components lost bits: nb_tri.cuh).
+// Conditioned error over all ions at n = 1e5: rms 2^-50.4, largest 2^-45.2, against
+// 2^-50.1 and 2^-44.9 (fp64) and 2^-49.2 and 2^-43.9 (df64) there; norm of the error
+// over that of the force, which the closest pairs set, rms of 200 clouds of 700 ..
+// 5003 ions and 250 of 16384: 6.8, 7.1, 6.5 and 6.3e-15 against 8.6, 7.5, 6.7 and
+// 6.5e-15 (single clouds go either way by up to 2).
 //
 // Measured and not kept: one pair of P-ions per lane (V = 1: twice the
 // shuffles per evaluation, 5-8 % slower; kept for 64-ion blocks, which it
@@ -37,8 +40,8 @@
 // The literal mixed form (MIX) takes the same words: its displacement, formed
 // exactly and rounded once to FP32, is the FP64 difference cast to FP32, at 8
 // FMA lane-cycles per component.  With 38 lane-cycles per evaluation it runs
-// 6.95 ms at n = 1e5 (FMA pipe 69 % by that count), where three FP64
-// differences per evaluation took 31.9 ms (nb_sym.cu), and gives its sums to
+// 6.95 ms at n = 1e5 (FMA pipe 67 %), where three FP64 differences per evaluation
+// took 31.9 ms, and gives its sums to
 // FP64 rounding: every FP32 operation and partial sum is the same, in the same
 // order (norm of the difference at most 2e-11 of the result over n = 2000 ..
 // 1e5; FP32 ties of a displacement may round the other way).  A pairwise
@@ -144,7 +147,7 @@ __device__ __noinline__ void tri_tile_fp64(int64_t n, const double *x, const dou
 // At n = 40000 (157 rounds of 256-ion blocks) the chain of commits bounded the
 // mixed form: 24 % per evaluation against sym_commit.  The fp64
 // items are three times as long and hide the chain: there sym_commit, with
-// fewer registers, is faster (19.2 against 19.7 ms at n = 1e5).
+// fewer registers, is faster (19.2 against 19.7 ms at n = 1e5, before d was normalised).
 template <int NT, class FP, class FQ>
 __device__ __forceinline__ void tri_commit(const SymItem &it, int64_t n, int BI, int64_t p0, int np, int64_t q0,
                                            int nq, double *out, int *sync, unsigned *err, FP sumP, FQ sumQ) {
@@ -398,12 +401,12 @@ static bool tri_sums(const Plan &pl, int mode, double soft2) {
 }
 bool tri_serves(const Plan &pl, int mode, double soft2) { return tri_sums(pl, mode, soft2) && pl.G >= 2; }
 
-// Block sizes, the fastest measured over n = 1500 .. 150000 (us per nb_forces
-// call, fp64): 64 ions below 2800 (30.0 against 33.1 with 128 at n = 2000),
-// 128 up to 12160 (82 against 107 with 256 at 5003, 239 against 270 at 10000),
-// where 96 blocks would take the in-place output, whose chain of commits these
-// short items do not hide (628 against 454 at 14000), 256 above (19245 against
-// 19989 with 512 at 1e5).  The mixed form's lines lie close by, from n = 2000;
+// Block sizes, the fastest measured over n = 1500 .. 150000 (fp64): 64 ions below
+// 2800 (us a step: 22.1 against 24.4 with 128 at n = 2000, 27.7 and 33.3 at 2600,
+// 33.4 and 33.3 at 3000), 128 up to 12160 (us per nb_forces call: 87 against 114
+// with 256 at 5003, 255 against 292 at 10000), where 96 blocks would take the
+// in-place output, whose chain of commits these short items do not hide (741
+// against 482 at 14000), 256 above (20668 against 21563 with 512 at 1e5).  The mixed form's lines lie close by, from n = 2000;
 // its FP32 sums run one-sided within a diagonal block, so its block (or
 // sub-block, see launch_pair_tri) stays that of make_plan: 64 ions below 3000,
 // 128 below 32768, 256 below 60000, 512 above.

@@ -18,19 +18,20 @@
 // P <= Q, of BI = 32 G ions, drawn from the round-robin schedule of
 // nb_symsched.cuh; a warp owns a P-tile of 64 ions, one packed pair per lane,
 // and visits the Q-tiles; positions and cotangents are three FP32 words each on
-// the item's two grids (nb_tri.cuh), so d and dl are exact differences on the
-// FP32 pipe, and T and the tile sums are double-floats in packed .f32x2
+// the item's grids, one per axis (nb_tri.cuh), so d and dl are exact differences on
+// the FP32 pipe, and T and the tile sums are double-floats in packed .f32x2
 // instructions, added to FP64 sums after each tile.  A tile with a pair too close
-// for the words, or an item of unusual scales, takes the pair's-own-units form of
-// the one-sided kernel (vjp_tile_units).
+// or coordinates too small for the words, or an item of unusual scales, takes the
+// pair's-own-units form of the one-sided kernel (vjp_tile_units), or FP64 where an
+// axis is far shorter than the others (vjp_tile_fp64).
 //
-// What bounds it: the FMA pipe, 225 lane-cycles per evaluation (21 for d, 30 for
-// the normalised dl, 18 for r^2, 16 for r^-3 and r^-2, 28 for d . dl, 7 for its
-// product with 3 r^-2, 48 for T, 48 for the sums, 9 to keep them normalised), 80 %
+// What bounds it: the FMA pipe, 234 lane-cycles per evaluation (30 for d, 30 for
+// dl, 18 for r^2, 16 for r^-3 and r^-2, 28 for d . dl, 7 for its
+// product with 3 r^-2, 48 for T, 48 for the sums, 9 to keep them normalised), 81 %
 // busy at n = 32768 with issue at 52 %.  The kernel it replaces formed d and dl
 // with six FP64 subtractions per evaluation and scaled every pair's term to
-// block-floating sums: 2.83 -> 1.55 ms at n = 20000, 16.6 -> 9.0 ms at 50000, 164
-// -> 106 us at 4096 (per nb_forces_vjp call); conditioned error rms 2^-48.5
+// block-floating sums: 2.83 -> 1.61 ms at n = 20000, 16.6 -> 9.5 ms at 50000, 164
+// -> 110 us at 4096 (per nb_forces_vjp call); conditioned error rms 2^-48.5
 // against 2^-47.4.
 #include <mutex>
 
