@@ -64,11 +64,13 @@ typedef enum {
  *                   component, and r^2, r^-3, the products and the sums over up
  *                   to 32 partners (256 one-sided) are double-floats, added in
  *                   FP64.  Charges keep 48 bits.
- *                   Groups of pairs whose words would cut a coordinate that is
- *                   small beside its axis (below 2^-17 on one side, the other
- *                   side below 2^-15), pairs closer than 2^-40 of the unit, and
- *                   units or weights far from the ordinary (an axis below 2^-64
- *                   of the longest, weights 2^40 apart) take the second form:
+ *                   Where the words cut a coordinate that is small beside its
+ *                   axis (below 2^-17 on one side, below 2^-15 on the other),
+ *                   the force of what they leave out is added in FP64; groups
+ *                   with many such pairs, or with one closer than 2^-40 of the
+ *                   unit, and units or weights far from the ordinary (an axis
+ *                   below 2^-64 of the longest, weights 2^40 apart) take the
+ *                   second form:
  *                   FP64 displacement and FP64 accumulation, with r^2,
  *                   1/sqrt(r^2) and r^-3 on the FP32 pipe: the displacement
  *                   is split into exponent-scaled FP32 (hi, lo) pairs, r^2 is

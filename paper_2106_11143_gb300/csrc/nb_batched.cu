@@ -322,13 +322,13 @@ __device__ __noinline__ void bsym_forces(const BIons v, double *acc, int npad, d
 // units and words are formed from the FP64 positions at every task
 // (600 instructions against 11 000 of pair arithmetic), diagonal super-tiles are
 // one-sided, and below about 500 ions there are fewer tasks than warps.  Two
-// steps of 512 instances of 32 .. 4096 ions: 15.5 ms (385 G pairs/s) against
+// steps of 512 instances of 32 .. 4096 ions: 15.6 ms (383 G pairs/s) against
 // 59.9 (fp64) and 25.8 ms (df64) with bsym_forces; 152 instances of 4096: 11.2
 // against 45.9 and 18.7 ms.  With the tasks' adds between barriers instead of
 // counters the FP64 adds of all 16 warps coincided, a third slower.  With one
 // unit per instance an ion far out, or a few kicked ones, sent every task to FP64
 // (37.8 ms instead of 2.7 for 152 instances of 64 .. 2048 with one ion at 5 m; 3.7
-// now).
+// now).  Residues of cut coordinates (nb_tri.cuh) are formed before the turn too.
 constexpr int BTRI_PI = 128;
 
 // Bounded wait of a warp for counter c to reach v (about a second).
@@ -388,6 +388,15 @@ __device__ __noinline__ bool btri_task_fp64(const BIons v, int p0, int np, int q
   return true;
 }
 
+// A task's residues (tri_residues): rs[u] those of ion p0 + 32 u + lane, rs[np / 32]
+// those of ion q0 + lane.
+template <bool QARR>
+__device__ __noinline__ void btri_residues(const BIons v, int p0, int np, int q0, double soft2, const TriScale sc,
+                                           double (*rs)[3]) {
+  tri_residues<QARR, TRI_NEAR>(v.n, v.x, v.y, v.z, v.q, soft2, p0, np, q0, sc.ex, rs[np >> 5],
+                               [&](int u, int c, double w) { rs[u >> 5][c] = w; });
+}
+
 // One task: the pair arithmetic of the P side's 64 V ions from p0 against tile
 // q0 .. q0 + 31, then, in its turn, the adds to acc.  The units are the task's
 // own, from its 64 V + 32 ions: an ion far out, or a coordinate small beside its
@@ -439,18 +448,11 @@ __device__ __forceinline__ bool btri_task(const BIons &v, double *acc, int npad,
     p.wh[u] = pk(w0[0][3], w0[1][3]);
     p.wl[u] = pk(w1[0][3], w1[1][3]);
   }
-  int fl = __reduce_or_sync(0xffffffffu, pf | qf << 6);
-  if (done && ((fl >> 3) & (fl >> 9) & 7)) {  // both sides near on one axis: is one cut?
-    auto place = [&](int i) {
-      return i < n ? tri_place<TRI_NEAR>(v.x[i], sc.ex[0], 0) | tri_place<TRI_NEAR>(v.y[i], sc.ex[1], 1) |
-                         tri_place<TRI_NEAR>(v.z[i], sc.ex[2], 2)
-                   : 0;
-    };
-    fl = place(q0 + lane) << 6;
-#pragma unroll 1
-    for (int u = 0; u < 2 * V; ++u) fl |= place(p0 + 32 * u + lane);
-    fl = __reduce_or_sync(0xffffffffu, fl);
-    done = !tri_fault(fl, fl >> 6);
+  const int fl = __reduce_or_sync(0xffffffffu, pf | qf << 6);
+  int rot = 0;  // rotations with residues, where both sides are near on an axis
+  if (done && fl & fl >> 6) {
+    rot = tri_rotations<TRI_NEAR>(n, v.x, v.y, v.z, p0, 64 * V, q0, sc.ex);
+    done = 2 * rot <= 64 * V;
   }
   TriSums<V> ts;
   if (done) {
@@ -481,6 +483,8 @@ __device__ __forceinline__ bool btri_task(const BIons &v, double *acc, int npad,
     done = !__any_sync(0xffffffffu, !(ymax <= TRI_YMAX_GRID));
   }
   if (!done) return btri_task_fp64<QARR>(v, p0, 64 * V, q0, one, soft2, acc, npad, turn);
+  double rs[2 * V + 1][3];
+  if (rot) btri_residues<QARR>(v, p0, 64 * V, q0, soft2, sc, rs);
   if (!turn.wait(one)) return false;
   const double fwd = pow2d((ew - 1023) - 2 * (sc.em - 1022));  // from the task's units
 #pragma unroll
@@ -501,6 +505,13 @@ __device__ __forceinline__ bool btri_task(const BIons &v, double *acc, int npad,
       a = fma(((double)h0 + (double)l0) + ((double)h1 + (double)l1), fwd, a);
     }
   }
+  if (rot)
+#pragma unroll 1
+    for (int u = 0; u <= 2 * V; ++u) {
+      const int i = u < 2 * V ? p0 + 32 * u + lane : q0 + lane;
+      if (i < n && (u < 2 * V || !one))
+        for (int c = 0; c < 3; ++c) acc[c * npad + i] += rs[u][c];
+    }
   return true;
 }
 

@@ -22,7 +22,7 @@
 // TwoSum sums, 9 to keep them normalised), 81 % busy at n = 32768 with issue at
 // 51 %, ALU 10 % and the FP64 pipe 24 % (the tiles' sums into FP64).  A half-pair
 // kernel on the FP64 pipe (10.3 FP64 instructions per evaluation in fp64, 3.4 in
-// df64) took 91.0 ms (fp64) and 34.0 ms (df64) at n = 1e5; this one takes 20.7 ms
+// df64) took 91.0 ms (fp64) and 34.0 ms (df64) at n = 1e5; this one takes 20.8 ms
 // for both (19.2 with d unnormalised, whose small components lost bits: nb_tri.cuh).
 // Conditioned error over all ions at n = 1e5: rms 2^-50.4, largest 2^-45.2, against
 // 2^-50.1 and 2^-44.9 (fp64) and 2^-49.2 and 2^-43.9 (df64) there; norm of the error
@@ -140,6 +140,20 @@ __device__ __noinline__ void tri_tile_fp64(int64_t n, const double *x, const dou
   }
 }
 
+// Adds a tile's residues (tri_residues) to the accumulators.
+template <bool QARR, int NEAR>
+__device__ __noinline__ void tri_tile_residues(int64_t n, const double *x, const double *y, const double *z,
+                                               const double *q, double soft2, int64_t i0, int ni, int64_t j0,
+                                               const int *ex, bool one, double sc, double *accP, int ldp, double *accQ,
+                                               int ldq) {
+  const int lane = threadIdx.x & 31;
+  double b[3];
+  tri_residues<QARR, NEAR>(n, x, y, z, q, soft2, i0, ni, j0, ex, b,
+                           [&](int u, int c, double v) { accP[c * ldp + u + lane] += v * sc; });
+  if (!one)
+    for (int c = 0; c < 3; ++c) accQ[c * ldq + lane] += b[c] * sc;
+}
+
 // The item's in-place output of the mixed form (sym_commit, nb_symsched.cuh,
 // laid out for short items): the sums are formed before the wait for the
 // previous round, and all of a thread's old values are loaded before the first
@@ -222,7 +236,7 @@ __global__ void __launch_bounds__(NT, NB)
   double *accQ = reinterpret_cast<double *>(qs + G * TRI_TILE4);     // [3][BI]
   double *accP = accQ + 3 * BI;                                      // [NW][3][PI]
   __shared__ int qf[32];                                             // places of each Q-tile (G <= 32)
-  __shared__ int ex[3];                                              // the axes' exponents, for tri_tile_fault
+  __shared__ int ex[3];                                              // the axes' exponents, for tri_residues
   const SymItem it = sym_block_item(INPLACE, sync, nbk);
   const int64_t p0 = (int64_t)it.P * BI, q0 = (int64_t)it.Q * BI;
   const int np = (int)min((int64_t)BI, n - p0), nq = (int)min((int64_t)BI, n - q0);
@@ -271,10 +285,10 @@ __global__ void __launch_bounds__(NT, NB)
     const bool one = diag && (!MIX || sp == sq);
     if (MIX && diag && sp > sq) continue;
     bool done = false;
-    bool words = fast;
+    int rot = 0;  // rotations with residues, where both sides are near on an axis
     if (fast && (pf & qf[t]))
-      words = !tri_tile_fault<MIX ? TRI_NEAR_MIX : TRI_NEAR>(n, x, y, z, p0 + pt * PI, PI, q0 + t * 32, ex);
-    if (words) {
+      rot = tri_rotations<MIX ? TRI_NEAR_MIX : TRI_NEAR>(n, x, y, z, p0 + pt * PI, PI, q0 + t * 32, ex);
+    if (fast && 2 * rot <= PI) {
       TriSums<V> ts;
       const f32x2 zero = pk1(0.0f);
 #pragma unroll
@@ -321,6 +335,9 @@ __global__ void __launch_bounds__(NT, NB)
               aQ[c * BI + lane] += ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
           }
         }
+        if (rot)
+          tri_tile_residues<QARR, MIX ? TRI_NEAR_MIX : TRI_NEAR>(n, x, y, z, q, soft2, p0 + pt * PI, PI, q0 + t * 32, ex,
+                                                                 one, back, aP, PI, aQ, BI);
       }
     }
     if (!done) {
@@ -406,7 +423,7 @@ bool tri_serves(const Plan &pl, int mode, double soft2) { return tri_sums(pl, mo
 // 33.4 and 33.3 at 3000), 128 up to 12160 (us per nb_forces call: 87 against 114
 // with 256 at 5003, 255 against 292 at 10000), where 96 blocks would take the
 // in-place output, whose chain of commits these short items do not hide (741
-// against 482 at 14000), 256 above (20668 against 21563 with 512 at 1e5).  The mixed form's lines lie close by, from n = 2000;
+// against 482 at 14000), 256 above (4 % faster than 512 at 1e5).  The mixed form's lines lie close by, from n = 2000;
 // its FP32 sums run one-sided within a diagonal block, so its block (or
 // sub-block, see launch_pair_tri) stays that of make_plan: 64 ions below 3000,
 // 128 below 32768, 256 below 60000, 512 above.

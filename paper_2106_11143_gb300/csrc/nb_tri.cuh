@@ -20,10 +20,13 @@
 //
 // A coordinate of at least 2^-17 L_c is exact in its words, a smaller one if it
 // has no bits below 2^-68 L_c (grids, zeros); else it is cut.  Against a partner
-// of 2^-15 L_c or more a cut one is right to 2^-52 of the difference; a tile
-// (pairs of 32 .. 128 ions) that holds a cut coordinate on one side and one below
-// 2^-15 L_c of the same axis on the other is done in FP64 (tri_fault; 3 tiles in
-// 10 000 of a random cloud).
+// of 2^-15 L_c or more a cut one is right to 2^-52 of the difference; for a pair of
+// a cut one and one below 2^-15 L_c of the same axis, the force of what the words
+// leave out of d is added in FP64 (tri_residues; one tile of 128 x 32 ions in 3000 of a
+// random cloud has such a pair), and a tile where that would be more than half its
+// rotations is done in FP64 as a whole.  Doing every such tile in FP64 took longer
+// than the kernel's other tiles together below n = 5000: 62.3 against 55.7 us a step
+// at n = 4096.
 //
 // What is left for FP32's range: pairs closer than 2^-40 L send their tile to
 // FP64 too (the smallest r^2 met, one FMNMX per pair), and items whose scale,
@@ -360,7 +363,7 @@ __device__ __forceinline__ float tri_tile(const TriIons<V> &p, LD ld, int lane, 
 }
 
 // Words of ion g (or a padding ion on side `far`) with its weight; returns its place
-// (without CUT, the bits of the axes it is near on alone: no branches).
+// (without CUT the bits of the axes it is near on alone: no branches).
 template <bool QARR, int NEAR = TRI_NEAR, bool CUT = true>
 __device__ __forceinline__ int tri_ion(int64_t g, bool real, const double *x, const double *y, const double *z,
                                        const double *q, const TriScale &sc, float far, float w0[4], float w1[4],
@@ -488,22 +491,112 @@ __device__ __forceinline__ int tri_load(TriIons<V> &p, float4 *qs, int *qf, int 
   return __reduce_or_sync(0xffffffffu, pf);
 }
 
-// Whether a tile whose sides are both near the origin on one axis may lose bits:
-// ions [i0, i0 + ni) against [j0, j0 + 32), those below n; ex: the axes' exponents.
+// The part of coordinate x below its words' last place.
+__device__ __forceinline__ double tri_residue(double x, int em) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)(b >> 52) & 0x7ff, s = em - e;
+  if (s <= 16) return 0.0;
+  if (e == 0 || s >= 69) return x;
+  return x - __longlong_as_double(b & (long long)(~0ull << (s - 16)));
+}
+
+// The pairs of a cut coordinate and a near one in a tile: ions [i0, i0 + ni) against
+// [j0, j0 + 32), those below n; ex: the axes' exponents.  TriPlaces holds the Q
+// side's places; rotations() gives, for the lane's ion i0 + u + lane, bit r for such a
+// pair with Q-ion (lane + r) mod 32.
 template <int NEAR>
-__device__ __noinline__ bool tri_tile_fault(int64_t n, const double *x, const double *y, const double *z, int64_t i0,
-                                            int ni, int64_t j0, const int *ex) {
+struct TriPlaces {
+  unsigned cut[3], near[3];
+  __device__ __forceinline__ static int of(int64_t n, int64_t g, const double *x, const double *y, const double *z,
+                                           const int *ex) {
+    return g < n ? tri_place<NEAR>(x[g], ex[0], 0) | tri_place<NEAR>(y[g], ex[1], 1) | tri_place<NEAR>(z[g], ex[2], 2) : 0;
+  }
+  __device__ __forceinline__ TriPlaces(int q) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      cut[c] = __ballot_sync(0xffffffffu, q >> c & 1);
+      near[c] = __ballot_sync(0xffffffffu, q >> (3 + c) & 1);
+    }
+  }
+  __device__ __forceinline__ unsigned rotations(int p) const {
+    unsigned m = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) m |= (p >> (3 + c) & 1 ? cut[c] : 0u) | (p >> c & 1 ? near[c] : 0u);
+    return __funnelshift_r(m, m, threadIdx.x & 31);
+  }
+};
+
+// How many of the tile's ni rotations (32 for every 32 ions of the P side) hold such
+// pairs.
+template <int NEAR>
+__device__ __noinline__ int tri_rotations(int64_t n, const double *x, const double *y, const double *z, int64_t i0,
+                                          int ni, int64_t j0, const int *ex) {
   const int lane = threadIdx.x & 31;
-  auto place = [&](int64_t g) {
-    return g < n ? tri_place<NEAR>(x[g], ex[0], 0) | tri_place<NEAR>(y[g], ex[1], 1) |
-                       tri_place<NEAR>(z[g], ex[2], 2)
-                 : 0;
-  };
-  int f = place(j0 + lane) << 6;
+  const TriPlaces<NEAR> pl(TriPlaces<NEAR>::of(n, j0 + lane, x, y, z, ex));
+  int k = 0;
 #pragma unroll 1
-  for (int u = 0; u < ni; u += 32) f |= place(i0 + u + lane);
-  f = __reduce_or_sync(0xffffffffu, f);
-  return tri_fault(f, f >> 6);
+  for (int u = 0; u < ni; u += 32)
+    k += __popc(__reduce_or_sync(0xffffffffu, pl.rotations(TriPlaces<NEAR>::of(n, i0 + u + lane, x, y, z, ex))));
+  return k;
+}
+
+// What the words leave out of the tile's sums: over these pairs, with e the difference
+// of the residues, r^-3 (e - 3 r^-2 (d . e) d) (the second order is below 2^-56 of the
+// force at the closest pairs the words serve).  addP(u, c, v) takes what falls to ion i0 + u + lane; b:
+// the lane's Q-ion's sums.  Rotations without such pairs are skipped, and the Q
+// side's terms go home by shuffle.
+template <bool QARR, int NEAR, class ADD>
+__device__ __forceinline__ void tri_residues(int64_t n, const double *x, const double *y, const double *z,
+                                             const double *q, double soft2, int64_t i0, int ni, int64_t j0,
+                                             const int *ex, double b[3], ADD addP) {
+  const int lane = threadIdx.x & 31;
+  const TriPlaces<NEAR> pl(TriPlaces<NEAR>::of(n, j0 + lane, x, y, z, ex));
+  auto load = [&](int64_t g, double r[3], double e[3], double &w) {
+    r[0] = r[1] = r[2] = e[0] = e[1] = e[2] = w = 0.0;
+    if (g >= n) return;
+    r[0] = x[g];
+    r[1] = y[g];
+    r[2] = z[g];
+    if (QARR) w = q[g];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) e[c] = tri_residue(r[c], ex[c]);
+  };
+  double xq[3], eq[3], wq;
+  load(j0 + lane, xq, eq, wq);
+  b[0] = b[1] = b[2] = 0.0;
+#pragma unroll 1
+  for (int u = 0; u < ni; u += 32) {
+    const unsigned m = pl.rotations(TriPlaces<NEAR>::of(n, i0 + u + lane, x, y, z, ex));
+    double a[3] = {0.0, 0.0, 0.0};
+    unsigned w = __reduce_or_sync(0xffffffffu, m);
+    if (w) {
+      double xp[3], ep[3], wp;
+      load(i0 + u + lane, xp, ep, wp);
+      for (; w; w &= w - 1) {
+        const int r = __ffs((int)w) - 1, from = (lane + r) & 31, home = (lane - r) & 31;
+        double d[3], de[3], s = 0.0, k = 0.0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          d[c] = xp[c] - __shfl_sync(0xffffffffu, xq[c], from);
+          de[c] = ep[c] - __shfl_sync(0xffffffffu, eq[c], from);
+        }
+        const double wj = QARR ? __shfl_sync(0xffffffffu, wq, from) : 1.0;
+        if (m >> r & 1) {
+          s = rinv3_fp64(d[0], d[1], d[2], soft2);
+          const double v = rinv1_fp64(d[0], d[1], d[2], soft2);
+          k = 3.0 * (v * v) * fma(d[0], de[0], fma(d[1], de[1], d[2] * de[2]));
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const double t = s * fma(-k, d[c], de[c]);
+          a[c] += QARR ? t * wj : t;
+          b[c] -= __shfl_sync(0xffffffffu, QARR ? t * wp : t, home);
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) addP(u, c, a[c]);
+  }
 }
 
 // The plan of a force evaluation: make_plan's, with this file's kernel's own

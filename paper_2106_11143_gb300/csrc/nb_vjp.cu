@@ -20,8 +20,9 @@
 // and visits the Q-tiles; positions and cotangents are three FP32 words each on
 // the item's grids, one per axis (nb_tri.cuh), so d and dl are exact differences on
 // the FP32 pipe, and T and the tile sums are double-floats in packed .f32x2
-// instructions, added to FP64 sums after each tile.  A tile with a pair too close
-// or coordinates too small for the words, or an item of unusual scales, takes the
+// instructions, added to FP64 sums after each tile.  What the words cut of
+// small components is added in FP64 (vjp_tile_residues).  A tile with a pair too
+// close for the words or many cut components, or an item of unusual scales, takes the
 // pair's-own-units form of the one-sided kernel (vjp_tile_units), or FP64 where an
 // axis is far shorter than the others (vjp_tile_fp64).
 //
@@ -351,6 +352,84 @@ __device__ __noinline__ void vjp_tile_fp64(int64_t n, const double *x, const dou
   }
 }
 
+// Cotangents spread more than positions do (a loss that reads a few ions), so their
+// rule allows a loss of 2^-44 of a pair's dl: residues are added for the pairs of a
+// cut component below 2^-26 and one below 2^-24 of the largest, and in an item
+// with a cut component (below 2^-17) a tile with a pair of |dl| below 2^-24 of it
+// leaves its words.  A tile with residues in more than 16 of its 64 rotations (each
+// costs about as much as four of the pair's-own-units form) leaves them too.
+constexpr int VJP_NEAR = 24, VJP_ROT = 16;
+constexpr float VJP_EMIN_CUT = 0x1p-24f;
+
+// The same with the cotangents' places from bit 6 (ex: the positions' axes, then the
+// cotangents').
+struct VjpPlaces {
+  const TriPlaces<TRI_NEAR> r;
+  const TriPlaces<VJP_NEAR> l;
+  __device__ __forceinline__ explicit VjpPlaces(int q) : r(q), l(q >> 6) {}
+  __device__ __forceinline__ unsigned rotations(int p) const { return r.rotations(p) | l.rotations(p >> 6); }
+};
+__device__ __forceinline__ int vjp_places(int64_t n, int64_t g, const double *x, const double *y, const double *z,
+                                          const double *lx, const double *ly, const double *lz, const int *ex) {
+  return TriPlaces<TRI_NEAR>::of(n, g, x, y, z, ex) | TriPlaces<VJP_NEAR>::of(n, g, lx, ly, lz, ex + 3) << 6;
+}
+__device__ __noinline__ int vjp_rotations(int64_t n, const double *x, const double *y, const double *z, const double *lx,
+                                          const double *ly, const double *lz, int64_t i0, int64_t j0, const int *ex) {
+  const int lane = threadIdx.x & 31;
+  const VjpPlaces pl(vjp_places(n, j0 + lane, x, y, z, lx, ly, lz, ex));
+  int k = 0;
+#pragma unroll 1
+  for (int u = 0; u < 64; u += 32)
+    k += __popc(__reduce_or_sync(0xffffffffu, pl.rotations(vjp_places(n, i0 + u + lane, x, y, z, lx, ly, lz, ex))));
+  return k;
+}
+
+// What the words of a tile leave out (tri_residues): over the pairs of a cut
+// component of a position or cotangent and a near one, r^-3 (de - 3 r^-2 (d . dl) e)
+// with e and de the residues' differences.
+template <bool QARR>
+__device__ __noinline__ void vjp_tile_residues(int64_t n, const double *x, const double *y, const double *z,
+                                               const double *q, const double *lx, const double *ly, const double *lz,
+                                               double soft2, int64_t i0, int64_t j0, const int *ex, bool one, double sc,
+                                               double *accP, int ldp, double *accQ, int ldq) {
+  const int lane = threadIdx.x & 31;
+  const VjpPlaces pl(vjp_places(n, j0 + lane, x, y, z, lx, ly, lz, ex));
+  const double *const src[6] = {x, y, z, lx, ly, lz};
+  double b[3] = {0.0, 0.0, 0.0};
+#pragma unroll 1
+  for (int u = 0; u < 64; u += 32) {
+    const int64_t i = i0 + u + lane;
+    const unsigned m = pl.rotations(vjp_places(n, i, x, y, z, lx, ly, lz, ex));
+    double a[3] = {0.0, 0.0, 0.0};
+    for (unsigned w = __reduce_or_sync(0xffffffffu, m); w; w &= w - 1) {
+      const int r = __ffs((int)w) - 1, home = (lane - r) & 31;
+      const int64_t j = j0 + ((lane + r) & 31);
+      double t[3] = {0.0, 0.0, 0.0};
+      if (m >> r & 1) {  // both ions are below n
+        double d[6], e[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          d[c] = src[c][i] - src[c][j];
+          e[c] = tri_residue(src[c][i], ex[c]) - tri_residue(src[c][j], ex[c]);
+        }
+        const double s = rinv3_fp64(d[0], d[1], d[2], soft2), v = rinv1_fp64(d[0], d[1], d[2], soft2);
+        const double k = 3.0 * (v * v) * fma(d[0], d[3], fma(d[1], d[4], d[2] * d[5]));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          t[c] = s * fma(-k, e[c], e[c + 3]);
+          a[c] += QARR ? t[c] * q[j] : t[c];
+          if (QARR) t[c] *= q[i];
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) b[c] -= __shfl_sync(0xffffffffu, t[c], home);
+    }
+    for (int c = 0; c < 3; ++c) accP[c * ldp + u + lane] += a[c] * sc;
+  }
+  if (!one)
+    for (int c = 0; c < 3; ++c) accQ[c * ldq + lane] += b[c] * sc;
+}
+
 // The item's scales: those of the positions and weights (nb_tri.cuh) and the
 // largest biased exponents of the cotangents' components; false when the item is
 // left to vjp_tile_units (lengths or cotangents beyond 2^+-100 and 2^+-200,
@@ -396,14 +475,6 @@ __device__ __forceinline__ bool vjp_scale(int64_t p0, int np, int64_t q0, int nq
 
 // Largest 1/r of the FP32 path.
 constexpr float VJP_YMAX = 0x1p24f;
-// Cotangents spread more than positions do (a loss that reads a few ions), so their
-// rule allows a loss of 2^-44 of a pair's dl: the two sides of a tile may not hold
-// a cut component below 2^-26 and one below 2^-24 of the largest, and in an item
-// with a cut component (below 2^-17) no pair's |dl| may be below 2^-24 of it.  With
-// the positions' rule a field that decays over six decades took 3.4 ms at n =
-// 20000 instead of 1.7.
-constexpr int VJP_NEAR = 24;
-constexpr float VJP_EMIN_CUT = 0x1p-24f;
 
 // The words of ion g's cotangent (zeros past the end) on the components' own
 // grids, in the unit of the largest; returns its place there (tri_place), and in
@@ -443,6 +514,7 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool diag = it.P == it.Q;
   __shared__ int qf[8];  // places of each Q-tile (G <= 8): positions, cotangents from bit 6, bit 12 cut
+  __shared__ int ex[6];  // the axes' exponents, for vjp_tile_residues
   TriScale sc;
   int el[3];
   bool deep;
@@ -453,6 +525,12 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
   const int PT = G >> 1, NG = VJP_W / PT, nqt = G / NG;  // P-tiles of 64 ions, warps and Q-tiles per P-tile
   const int pt = warp % PT, grp = warp / PT;
   VjpIons p;
+  if (tid == 0)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      ex[c] = sc.ex[c];
+      ex[3 + c] = el[c];
+    }
   int pf = 0;   // places of the warp's P-tile
   int cut = 0;  // a cotangent of the Q side is cut
   if (fast) {
@@ -516,7 +594,10 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
     if (!live || t * 32 >= nq) continue;
     double *aQ = accQ + t * 32;
     bool done = false;
-    if (fast && !tri_fault(pf, qf[t]) && !tri_fault(pf >> 6, qf[t] >> 6)) {
+    int rot = 0;  // rotations with residues, where both sides are near on an axis
+    if (fast && (tri_fault(pf, qf[t]) || tri_fault(pf >> 6, qf[t] >> 6)))
+      rot = vjp_rotations(n, x, y, z, lx, ly, lz, p0 + pt * 64, q0 + t * 32, ex);
+    if (fast && rot <= VJP_ROT) {
       TriSums<1> ts;
       const f32x2 zero = pk1(0.0f);
 #pragma unroll
@@ -541,6 +622,9 @@ __global__ void __launch_bounds__(VJP_THREADS, 4)
             aQ[c * BI + lane] += ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
           }
         }
+        if (rot)
+          vjp_tile_residues<QARR>(n, x, y, z, q, lx, ly, lz, soft2, p0 + pt * 64, q0 + t * 32, ex, diag, back, aP, 64,
+                                  aQ, BI);
       }
     }
     if (!done) {

@@ -206,3 +206,62 @@ def test_ensemble_tasks_left_to_fp64(nb, kind, charges, soft, precision):
         ref, cond = t.sum(-1), np.sqrt((t * t).sum(0)).sum(-1)
         err = np.sqrt(((acc[:, off[k]:off[k + 1]] - ref) ** 2).sum(0))
         assert np.all(err <= 1e-12 * cond), (n, float(np.max(err / np.maximum(cond, 1e-300))))
+
+
+# ---------------------------------------------------------------------------
+# Residues: a few pairs of cut coordinates in tiles that keep to their words.
+
+
+def few_cut(n):
+    """A chain whose x is zero but for one ion at each end of the index range and six
+    close pairs at the edges of tiles and blocks, with x some 2^-40 of theirs; the
+    pairs are 3e-9 apart, so that their own x terms lead."""
+    rng = np.random.default_rng(n)
+    pos = np.zeros((3, n))
+    pos[2] = np.sort(rng.uniform(-3e-4, 3e-4, n))
+    pos[0, [0, n - 1, n // 2]] = 1e-6, -1.3e-6, 0.9e-6
+    pairs = [(5, 40), (31, 32), (63, 64), (100, n - 5), (n - 2, 127), (128, 129)]
+    for a, b in pairs:
+        pos[2, b] = pos[2, a] + 3e-9
+        pos[0, a], pos[0, b] = rng.uniform(1.0, 2.0, 2) * 1e-6 * 2.0 ** -40
+    return pos, np.unique(np.array(pairs))
+
+
+@pytest.mark.parametrize("charges", [False, True])
+@pytest.mark.parametrize("precision,n", [("fp64", 700), ("fp64", 1600), ("df64", 2900), ("fp64", 12500), ("mixed", 13000)])
+def test_residues_of_a_few_pairs(nb, precision, n, charges):
+    pos, idx = few_cut(n)
+    q = np.random.default_rng(n).choice([1.0, 2.0, -1.0], size=n) if charges else None
+    s = nb.System(pos, q=q)
+    nb.forces(nb.Params.from_phys(W.phys(**UNIT), precision=precision), s)
+    nb.sync_status()
+    g = s.acc().cpu().numpy()
+    w = np.ones(n) if q is None else q
+    for i in idx:
+        d = pos[:, [i]] - pos
+        r2 = (d * d).sum(0)
+        y = np.where(r2 > 0.0, 1.0 / np.sqrt(np.where(r2 > 0.0, r2, 1.0)), 0.0)
+        t = w[i] * w * y ** 3 * d
+        tol = 1e-6 if precision == "mixed" else 1e-12
+        assert np.all(np.abs(g[:, i] - t.sum(-1)) <= tol * np.abs(t).sum(-1)), i
+
+
+@pytest.mark.parametrize("charges", [False, True])
+@pytest.mark.parametrize("n", [2500, 16500])
+def test_residues_of_a_few_pairs_in_the_jacobian_product(nb, n, charges):
+    pos, idx = few_cut(n)
+    lam, _ = few_cut(n)
+    lam[2] = 1e-6 * np.random.default_rng(n).standard_normal(n)
+    lam[0] *= 1.7
+    q = np.random.default_rng(n).choice([1.0, 2.0, -1.0], size=n) if charges else None
+    g = nb.forces_vjp(nb.Params.from_phys(W.phys(**UNIT)), nb.System(pos, q=q), lam).cpu().numpy()
+    nb.sync_status()
+    w = np.ones(n) if q is None else q
+    for i in idx:
+        d, dl = pos[:, [i]] - pos, lam[:, [i]] - lam
+        r2 = (d * d).sum(0)
+        y = np.where(r2 > 0.0, 1.0 / np.sqrt(np.where(r2 > 0.0, r2, 1.0)), 0.0)
+        y3 = y * y * y
+        t = w[i] * w * y3 * (dl - 3.0 * (y * y) * (d * dl).sum(0) * d)
+        mag = np.abs(w[i] * w) * y3 * (np.abs(dl) + 3.0 * y * np.sqrt((dl * dl).sum(0)) * np.abs(d))
+        assert np.all(np.abs(g[:, i] - t.sum(-1)) <= 1e-12 * mag.sum(-1)), i
