@@ -22,7 +22,7 @@
 // TwoSum sums, 9 to keep them normalised), 81 % busy at n = 32768 with issue at
 // 51 %, ALU 10 % and the FP64 pipe 24 % (the tiles' sums into FP64).  A half-pair
 // kernel on the FP64 pipe (10.3 FP64 instructions per evaluation in fp64, 3.4 in
-// df64) took 91.0 ms (fp64) and 34.0 ms (df64) at n = 1e5; this one takes 20.8 ms
+// df64) took 91.0 ms (fp64) and 34.0 ms (df64) at n = 1e5; this one takes 20.6 ms
 // for both (19.2 with d unnormalised, whose small components lost bits: nb_tri.cuh).
 // Conditioned error over all ions at n = 1e5: rms 2^-50.4, largest 2^-45.2, against
 // 2^-50.1 and 2^-44.9 (fp64) and 2^-49.2 and 2^-43.9 (df64) there; norm of the error
@@ -420,13 +420,13 @@ bool tri_serves(const Plan &pl, int mode, double soft2) { return tri_sums(pl, mo
 
 // Block sizes, the fastest measured over n = 1500 .. 150000 (fp64): 64 ions below
 // 2800 (us a step: 22.1 against 24.4 with 128 at n = 2000, 27.7 and 33.3 at 2600,
-// 33.4 and 33.3 at 3000), 128 up to 12160 (us per nb_forces call: 87 against 114
-// with 256 at 5003, 255 against 292 at 10000), where 96 blocks would take the
-// in-place output, whose chain of commits these short items do not hide (741
-// against 482 at 14000), 256 above (4 % faster than 512 at 1e5).  The mixed form's lines lie close by, from n = 2000;
-// its FP32 sums run one-sided within a diagonal block, so its block (or
-// sub-block, see launch_pair_tri) stays that of make_plan: 64 ions below 3000,
-// 128 below 32768, 256 below 60000, 512 above.
+// 33.4 and 33.3 at 3000), 128 up to 12160 (us per nb_forces call: 90 against 115
+// with 256 at 5003, 257 against 297 at 10000), where 96 blocks would take the
+// in-place output, whose chain of commits these short items do not hide (631
+// against 485 at 14000), 256 above (4 % faster than 512 at 1e5).  The mixed form's
+// lines lie close by, from n = 2000; its FP32 sums run one-sided within a diagonal
+// block, so its block (or sub-block, see launch_pair_tri) stays that of make_plan:
+// 64 ions below 3000, 128 below 32768, 256 below 60000, 512 above.
 Plan make_force_plan(int64_t n, int mode, double soft2) {
   Plan pl = make_plan(n, mode, 0);
   int tb = 0, tr = 0, tbps = 0;
