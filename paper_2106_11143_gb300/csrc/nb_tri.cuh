@@ -491,13 +491,32 @@ __device__ __forceinline__ int tri_load(TriIons<V> &p, float4 *qs, int *qf, int 
   return __reduce_or_sync(0xffffffffu, pf);
 }
 
-// The part of coordinate x below its words' last place.
-__device__ __forceinline__ double tri_residue(double x, int em) {
+// The part of coordinate x below its words' last place, and its l word in units of
+// that place.
+struct TriRest {
+  double e = 0.0;
+  int l = 0;
+};
+__device__ __forceinline__ TriRest tri_residue(double x, int em) {
+  TriRest t;
   const long long b = __double_as_longlong(x);
   const int e = (int)(b >> 52) & 0x7ff, s = em - e;
-  if (s <= 16) return 0.0;
-  if (e == 0 || s >= 69) return x;
-  return x - __longlong_as_double(b & (long long)(~0ull << (s - 16)));
+  if (e == 0 || s >= 69) {
+    t.e = x;
+    return t;
+  }
+  const long long m = (b & 0xfffffffffffffll) | 1ll << 52;
+  if (s > 16) t.e = x - __longlong_as_double(b & (long long)(~0ull << (s - 16)));
+  t.l = (int)(s > 16 ? m >> (s - 16) : m << (16 - s)) & 0xffffff;
+  if (b < 0) t.l = -t.l;
+  return t;
+}
+// What the words leave out of p - q: the residues' difference, and the last bit of a
+// difference of l words of unlike sign, which has 25 (at 2^-42 L, the pairs' smallest
+// components that lead a sum, 2^-27 of it).
+__device__ __forceinline__ double tri_left_out(const TriRest &p, const TriRest &q, int em) {
+  const int l = p.l - q.l;
+  return p.e - q.e + (l - (int)(float)l) * pow2d(em - 1022 - 69);
 }
 
 // The pairs of a cut coordinate and a near one in a tile: ions [i0, i0 + ni) against
@@ -540,19 +559,19 @@ __device__ __noinline__ int tri_rotations(int64_t n, const double *x, const doub
   return k;
 }
 
-// What the words leave out of the tile's sums: over these pairs, with e the difference
-// of the residues, r^-3 (e - 3 r^-2 (d . e) d) (the second order is below 2^-56 of the
-// force at the closest pairs the words serve).  addP(u, c, v) takes what falls to ion i0 + u + lane; b:
-// the lane's Q-ion's sums.  Rotations without such pairs are skipped, and the Q
-// side's terms go home by shuffle.
+// What the words leave out of the tile's sums: over these pairs, with e what they leave
+// out of d, r^-3 (e - 3 r^-2 (d . e) (d - e)); what remains is below 2^-54 of each
+// component at the closest pairs the words serve.  addP(u, c, v) takes what falls to
+// ion i0 + u + lane; b: the lane's Q-ion's sums.  Rotations without such pairs are
+// skipped, and the Q side's terms go home by shuffle.
 template <bool QARR, int NEAR, class ADD>
 __device__ __forceinline__ void tri_residues(int64_t n, const double *x, const double *y, const double *z,
                                              const double *q, double soft2, int64_t i0, int ni, int64_t j0,
                                              const int *ex, double b[3], ADD addP) {
   const int lane = threadIdx.x & 31;
   const TriPlaces<NEAR> pl(TriPlaces<NEAR>::of(n, j0 + lane, x, y, z, ex));
-  auto load = [&](int64_t g, double r[3], double e[3], double &w) {
-    r[0] = r[1] = r[2] = e[0] = e[1] = e[2] = w = 0.0;
+  auto load = [&](int64_t g, double r[3], TriRest e[3], double &w) {
+    r[0] = r[1] = r[2] = w = 0.0;
     if (g >= n) return;
     r[0] = x[g];
     r[1] = y[g];
@@ -561,7 +580,8 @@ __device__ __forceinline__ void tri_residues(int64_t n, const double *x, const d
 #pragma unroll
     for (int c = 0; c < 3; ++c) e[c] = tri_residue(r[c], ex[c]);
   };
-  double xq[3], eq[3], wq;
+  double xq[3], wq;
+  TriRest eq[3];
   load(j0 + lane, xq, eq, wq);
   b[0] = b[1] = b[2] = 0.0;
 #pragma unroll 1
@@ -570,7 +590,8 @@ __device__ __forceinline__ void tri_residues(int64_t n, const double *x, const d
     double a[3] = {0.0, 0.0, 0.0};
     unsigned w = __reduce_or_sync(0xffffffffu, m);
     if (w) {
-      double xp[3], ep[3], wp;
+      double xp[3], wp;
+      TriRest ep[3];
       load(i0 + u + lane, xp, ep, wp);
       for (; w; w &= w - 1) {
         const int r = __ffs((int)w) - 1, from = (lane + r) & 31, home = (lane - r) & 31;
@@ -578,7 +599,10 @@ __device__ __forceinline__ void tri_residues(int64_t n, const double *x, const d
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           d[c] = xp[c] - __shfl_sync(0xffffffffu, xq[c], from);
-          de[c] = ep[c] - __shfl_sync(0xffffffffu, eq[c], from);
+          TriRest t;
+          t.e = __shfl_sync(0xffffffffu, eq[c].e, from);
+          t.l = __shfl_sync(0xffffffffu, eq[c].l, from);
+          de[c] = tri_left_out(ep[c], t, ex[c]);
         }
         const double wj = QARR ? __shfl_sync(0xffffffffu, wq, from) : 1.0;
         if (m >> r & 1) {
@@ -588,7 +612,7 @@ __device__ __forceinline__ void tri_residues(int64_t n, const double *x, const d
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const double t = s * fma(-k, d[c], de[c]);
+          const double t = s * fma(-k, d[c] - de[c], de[c]);
           a[c] += QARR ? t * wj : t;
           b[c] -= __shfl_sync(0xffffffffu, QARR ? t * wp : t, home);
         }

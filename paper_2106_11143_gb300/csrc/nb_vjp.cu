@@ -386,7 +386,7 @@ __device__ __noinline__ int vjp_rotations(int64_t n, const double *x, const doub
 
 // What the words of a tile leave out (tri_residues): over the pairs of a cut
 // component of a position or cotangent and a near one, r^-3 (de - 3 r^-2 (d . dl) e)
-// with e and de the residues' differences.
+// with e and de what they leave out of d and dl.
 template <bool QARR>
 __device__ __noinline__ void vjp_tile_residues(int64_t n, const double *x, const double *y, const double *z,
                                                const double *q, const double *lx, const double *ly, const double *lz,
@@ -410,7 +410,7 @@ __device__ __noinline__ void vjp_tile_residues(int64_t n, const double *x, const
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
           d[c] = src[c][i] - src[c][j];
-          e[c] = tri_residue(src[c][i], ex[c]) - tri_residue(src[c][j], ex[c]);
+          e[c] = tri_left_out(tri_residue(src[c][i], ex[c]), tri_residue(src[c][j], ex[c]), ex[c]);
         }
         const double s = rinv3_fp64(d[0], d[1], d[2], soft2), v = rinv1_fp64(d[0], d[1], d[2], soft2);
         const double k = 3.0 * (v * v) * fma(d[0], d[3], fma(d[1], d[4], d[2] * d[5]));

@@ -265,3 +265,57 @@ def test_residues_of_a_few_pairs_in_the_jacobian_product(nb, n, charges):
         t = w[i] * w * y3 * (dl - 3.0 * (y * y) * (d * dl).sum(0) * d)
         mag = np.abs(w[i] * w) * y3 * (np.abs(dl) + 3.0 * y * np.sqrt((dl * dl).sum(0)) * np.abs(d))
         assert np.all(np.abs(g[:, i] - t.sum(-1)) <= 1e-12 * mag.sum(-1)), i
+
+
+# Coordinates of unlike sign: their l words' difference has 25 bits, one more than
+# FP32.  The transverse terms lead where a pair is this close.
+
+
+def crossing(n, gap):
+    """A chain with pairs, gap apart, that straddle x = 0 at 2^-43 of the largest x; no
+    other ion is near x = 0."""
+    rng = np.random.default_rng([n, 1])
+    pos = np.zeros((3, n))
+    pos[2] = np.sort(rng.uniform(-3e-4, 3e-4, n))
+    pos[0] = rng.uniform(0.5, 1.0, n) * 1e-6 * rng.choice([-1.0, 1.0], n)
+    pairs = np.array([(5, 40), (31, 32), (63, 64), (100, n - 5), (n - 2, 127), (128, 129)])
+    pos[2, pairs[:, 1]] = pos[2, pairs[:, 0]] + gap
+    pos[0, pairs] = rng.uniform(1.0, 2.0, (6, 2)) * 1e-6 * 2.0 ** -43 * [1.0, -1.0]
+    return pos, np.unique(pairs)
+
+
+@pytest.mark.parametrize("charges", [False, True])
+@pytest.mark.parametrize("precision,n", [("fp64", 700), ("df64", 2900), ("fp64", 12500), ("ensemble", 700)])
+def test_pairs_across_an_axis(nb, precision, n, charges):
+    pos, idx = crossing(n, 4e-15)
+    q = np.random.default_rng(n).choice([1.0, 2.0, -1.0], size=n) if charges else None
+    if precision == "ensemble":
+        g = ensemble_once(nb, pos, np.array([0, n]), q, 0.0, 512, "fp64")
+    else:
+        s = nb.System(pos, q=q)
+        nb.forces(nb.Params.from_phys(W.phys(**UNIT), precision=precision), s)
+        nb.sync_status()
+        g = s.acc().cpu().numpy()
+    w = np.ones(n) if q is None else q
+    for i in idx:
+        d = pos[:, [i]] - pos
+        r2 = (d * d).sum(0)
+        y = np.where(r2 > 0.0, 1.0 / np.sqrt(np.where(r2 > 0.0, r2, 1.0)), 0.0)
+        t = w[i] * w * y ** 3 * d
+        assert np.all(np.abs(g[:, i] - t.sum(-1)) <= 1e-12 * np.abs(t).sum(-1)), i
+
+
+def test_pairs_across_an_axis_of_the_jacobian_product(nb):
+    n = 2500
+    pos, idx = crossing(n, 1e-10)
+    lam = pos * [[1.7], [0.0], [1.0]]
+    g = nb.forces_vjp(nb.Params.from_phys(W.phys(**UNIT)), nb.System(pos), lam).cpu().numpy()
+    nb.sync_status()
+    for i in idx:
+        d, dl = pos[:, [i]] - pos, lam[:, [i]] - lam
+        r2 = (d * d).sum(0)
+        y = np.where(r2 > 0.0, 1.0 / np.sqrt(np.where(r2 > 0.0, r2, 1.0)), 0.0)
+        y3 = y * y * y
+        t = y3 * (dl - 3.0 * (y * y) * (d * dl).sum(0) * d)
+        mag = y3 * (np.abs(dl) + 3.0 * y * np.sqrt((dl * dl).sum(0)) * np.abs(d))
+        assert np.all(np.abs(g[:, i] - t.sum(-1)) <= 1e-12 * mag.sum(-1)), i
